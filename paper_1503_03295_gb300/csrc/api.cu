@@ -62,8 +62,11 @@ DevParams make_dev_params(const sco_params& p) {
   P.inv_bD58_f = (float)P.inv_bD58;
   P.beta_f = (float)P.beta;
   P.bJ_f = (float)(P.beta * P.J);
+  P.bJ_h = P.bJ_f;
+  P.bJ_l = (float)(P.beta * P.J - (double)P.bJ_h);
   P.switching = P.bD > 0.0 ? 1 : 0;
   P.lx_magic = div_magic((unsigned long long)p.Lx);
+  P.lx_m32 = p.Lx > 1 ? (uint32_t)((1ull << 32) / (unsigned long long)p.Lx) : 0xFFFFFFFFu;
   P.key0 = p.seed;
   P.key1 = (uint64_t)(uint32_t)p.replica;
   const dd l2 = ln2_dd();
@@ -98,7 +101,9 @@ struct sco_ctx {
   int64_t launches = 0;
   Table tab;
   double* s = nullptr;
-  float4* s32 = nullptr;  // FP32 copy of the spins, one (x, y, z, 0) per site
+  float4* s32 = nullptr;    // FP32-guarded form: FP32 copy of the spins, one (x, y, z, 0) per site
+  SpinDf* sd = nullptr;     // FP64 form: float-float copy of the spins
+  SpinDf* propd = nullptr;  // FP64 form: the proposals of the step in float-float
   double* s_epoch = nullptr;
   SwitchBufs sw{};
   uint32_t* row_ptr = nullptr;
@@ -116,12 +121,6 @@ struct sco_ctx {
   bool colour_valid = false;
   uint32_t g = 1;
   uint64_t nnz = 0;
-  // FP64 form: the pair cache (hid parallel to col, keep records in SwitchBufs, upd per site);
-  // cache_state 0: the first halves hold the terms at the current spins; 1: the halves given by
-  // the parities of the last step hold them; 2: rebuild from the spins first
-  uint32_t* hid = nullptr;
-  uint8_t* upd = nullptr;
-  int cache_state = 0;
   bool dip_valid = false;  // cnt->max_degree_dip holds the dipolar Delta of the current graph
   int sticky = 0;
   unsigned long long ns_limit = 2000000000ull;  // bound of every device-side wait (2 s)
@@ -200,23 +199,6 @@ cudaError_t grow(T*& ptr, uint64_t& cap, uint64_t need) {
   return e;
 }
 
-bool cache_on(const sco_ctx* c) { return c->sw.keep != nullptr; }
-
-// The per-half-edge records of the pair cache for the current overflow capacity.
-cudaError_t alloc_keep(sco_ctx* c) {
-  cudaFree(c->sw.keep);
-  c->sw.keep = nullptr;
-  const size_t n = (size_t)c->P.N * kSlotCap + c->sw.ovf_cap;
-  return cudaMalloc(&c->sw.keep, n * sizeof(double4_32a));
-}
-
-PairCache pair_cache(sco_ctx* c) {
-  if (!cache_on(c)) return PairCache{};
-  // the last endpoint's term is needed only when the next step keeps this graph
-  const int carry = (c->t + 1) % c->p.n_sw != 0 ? 1 : 0;
-  return PairCache{c->hid, c->sw.keep, c->upd, carry, c->cache_state != 1 ? 1 : 0};
-}
-
 sco_status do_switch(sco_ctx* c, uint32_t epoch, const double* src, const float4* src32) {
   PhaseTimer tm(c, kPhSwitch);
   // per-switch counters: n_half, n_dip, ovf_n, nnz and max_degree, max_degree_dip
@@ -239,17 +221,6 @@ sco_status do_switch(sco_ctx* c, uint32_t epoch, const double* src, const float4
     c->sw.ovf = nullptr;
     SCO_TRY(cudaMalloc(&c->sw.ovf, 2 * need * sizeof(uint32_t)));
     c->sw.ovf_cap = (uint32_t)need;
-    if (cache_on(c)) {
-      // half-edge ids must stay below 2^32 for the cache: else run without it
-      if ((uint64_t)c->P.N * kSlotCap + need >= (1ull << 32)) {
-        cudaFree(c->sw.keep);
-        c->sw.keep = nullptr;
-        cudaFree(c->hid);
-        c->hid = nullptr;
-      } else {
-        SCO_TRY(alloc_keep(c));
-      }
-    }
     SCO_TRY(cudaMemsetAsync(c->cnt, 0, 4 * sizeof(unsigned long long), c->st));
     SCO_TRY(cudaMemsetAsync(&c->cnt->max_degree, 0, 2 * sizeof(unsigned), c->st));
     SCO_TRY(cudaMemsetAsync(&c->cnt->ovf_full, 0, sizeof(int), c->st));
@@ -261,19 +232,11 @@ sco_status do_switch(sco_ctx* c, uint32_t epoch, const double* src, const float4
     if (c->hcnt->ovf_n > c->sw.ovf_cap) return SCO_ECAPACITY;
   }
   c->nnz = c->hcnt->nnz;
-  if (c->col_cap < c->nnz) {
-    cudaFree(c->hid);
-    c->hid = nullptr;
-  }
   SCO_TRY(grow(c->col, c->col_cap, c->nnz > 0 ? c->nnz : 1));
-  if (cache_on(c) && !c->hid) SCO_TRY(cudaMalloc(&c->hid, c->col_cap * sizeof(uint32_t)));
   // rows are left unsorted (their order changes no result); getters sort their copies
-  SCO_TRY(csr_fill(c->P, c->sw, c->row_ptr, c->col, cache_on(c) ? c->hid : nullptr,
-                   c->hcnt->ovf_n > 0, false, c->cnt, c->st, &c->launches));
+  SCO_TRY(csr_fill(c->P, c->sw, c->row_ptr, c->col, c->hcnt->ovf_n > 0, false, c->cnt, c->st,
+                   &c->launches));
   c->dip_valid = false;
-  // the switch left the FP64 terms of the switching spins in the cache: valid now unless the
-  // graph was switched from other spins (the epoch start of a restored checkpoint)
-  c->cache_state = src == c->s ? 0 : 2;
   c->g = c->hcnt->max_degree + 1;
   c->graph_epoch = epoch;
   c->colour_valid = false;
@@ -328,6 +291,8 @@ void free_all(sco_ctx* c) {
   table_free(c->tab);
   cudaFree(c->s);
   cudaFree(c->s32);
+  cudaFree(c->sd);
+  cudaFree(c->propd);
   cudaFree(c->s_epoch);
   cudaFree(c->sw.hslot);
   cudaFree(c->sw.hcnt);
@@ -337,9 +302,6 @@ void free_all(sco_ctx* c) {
   cudaFree(c->sw.ocur);
   cudaFree(c->sw.ovf);
   cudaFree(c->sw.scan_tmp);
-  cudaFree(c->sw.keep);
-  cudaFree(c->hid);
-  cudaFree(c->upd);
   cudaFree(c->row_ptr);
   cudaFree(c->col);
   cudaFree(c->cb.word);
@@ -409,7 +371,12 @@ sco_status sco_init(const sco_params* p, void* stream, sco_ctx** out) {
   cudaError_t e = table_build(P, c->tab, c->st, &c->launches);
   if (e != cudaSuccess) return fail(from_cuda(e));
   e = cudaMalloc(&c->s, 3 * N * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&c->s32, N * sizeof(float4));
+  if (p->precision == SCO_FP64) {
+    if (e == cudaSuccess) e = cudaMalloc(&c->sd, N * sizeof(SpinDf));
+    if (e == cudaSuccess) e = cudaMalloc(&c->propd, N * sizeof(SpinDf));
+  } else if (e == cudaSuccess) {
+    e = cudaMalloc(&c->s32, N * sizeof(float4));
+  }
   if (e == cudaSuccess && p->n_sw > 1) e = cudaMalloc(&c->s_epoch, 3 * N * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->sw.hslot, N * kSlotCap * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&c->sw.hcnt, N * sizeof(uint32_t));
@@ -438,16 +405,9 @@ sco_status sco_init(const sco_params* p, void* stream, sco_ctx** out) {
   if (e == cudaSuccess) e = cudaMemsetAsync(c->cnt, 0, sizeof(DevCounters), c->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->acc, 0, N, c->st);
   if (e != cudaSuccess) return fail(from_cuda(e));
-  // the FP64 form keeps the pair cache while half-edge ids fit 32 bits
-  if (p->precision == SCO_FP64 && (uint64_t)N * kSlotCap + c->sw.ovf_cap < (1ull << 32)) {
-    e = alloc_keep(c);
-    if (e == cudaSuccess) e = cudaMalloc(&c->upd, N);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->upd, 0, N, c->st);
-    if (e != cudaSuccess) return fail(from_cuda(e));
-  }
   const uint64_t guess = (uint64_t)N * 24 + 1024;
   e = grow(c->col, c->col_cap, guess);
-  if (e == cudaSuccess) e = spins_init(P, c->s, c->s32, c->st, &c->launches);
+  if (e == cudaSuccess) e = spins_init(P, c->s, c->s32, c->sd, c->st, &c->launches);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
   if (e != cudaSuccess) return fail(from_cuda(e));
   *out = c;
@@ -488,12 +448,9 @@ sco_status sco_sweep(sco_ctx* c, int32_t n_mcs) {
     if (st != SCO_OK) return st;
     {
       PhaseTimer tm(c, kPhSweep);
-      if (cache_on(c) && c->cache_state == 2)
-        SCO_TRY(cache_build_run(c->P, c->tab, c->s, c->sw, c->cnt, c->st, &c->launches));
-      SCO_TRY(sweep_run(c->P, c->tab, c->s, c->s32, c->row_ptr, c->col, c->cb.perm, c->cb.off,
-                        c->g, (uint64_t)c->t, c->p.precision, c->acc, c->defer, c->cb.dcnt,
-                        c->prop, c->cnt, pair_cache(c), c->st, &c->launches));
-      c->cache_state = 1;
+      SCO_TRY(sweep_run(c->P, c->tab, c->s, c->s32, c->sd, c->row_ptr, c->col, c->cb.perm,
+                        c->cb.off, c->g, (uint64_t)c->t, c->p.precision, c->acc, c->defer,
+                        c->cb.dcnt, c->prop, c->propd, c->cnt, c->st, &c->launches));
     }
     c->t++;
   }
@@ -547,9 +504,8 @@ sco_status sco_set_spins(sco_ctx* c, const double* xyz, int32_t on_device) {
   if (!c || !xyz) return SCO_EINVAL;
   SCO_TRY(cudaMemcpyAsync(c->s, xyz, 3 * c->P.N * sizeof(double),
                           on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->st));
-  SCO_TRY(spins_to_f32(c->P.N, c->s, c->s32, c->st, &c->launches));
+  SCO_TRY(spins_copies(c->P.N, c->s, c->s32, c->sd, c->st, &c->launches));
   SCO_TRY(cudaStreamSynchronize(c->st));
-  c->cache_state = 2;  // the graph stays; its cached pair terms belong to the old spins
   return SCO_OK;
 }
 
@@ -681,7 +637,7 @@ sco_status sco_set_state(sco_ctx* c, const void* buf, size_t len) {
   if (len < need) return SCO_EINVAL;
   const char* body = (const char*)buf + sizeof(h);
   SCO_TRY(cudaMemcpyAsync(c->s, body, 3 * N * sizeof(double), cudaMemcpyHostToDevice, c->st));
-  SCO_TRY(spins_to_f32(N, c->s, c->s32, c->st, &c->launches));
+  SCO_TRY(spins_copies(N, c->s, c->s32, c->sd, c->st, &c->launches));
   c->t = h.t;
   c->graph_epoch = -1;
   c->colour_valid = false;
@@ -692,7 +648,7 @@ sco_status sco_set_state(sco_ctx* c, const void* buf, size_t len) {
                             cudaMemcpyHostToDevice, c->st));
     float4* tmp32 = nullptr;
     SCO_TRY(cudaMalloc(&tmp32, N * sizeof(float4)));
-    cudaError_t e = spins_to_f32(N, c->s_epoch, tmp32, c->st, &c->launches);
+    cudaError_t e = spins_copies(N, c->s_epoch, tmp32, nullptr, c->st, &c->launches);
     sco_status st = e == cudaSuccess
                         ? do_switch(c, (uint32_t)(c->t / c->p.n_sw), c->s_epoch, tmp32)
                         : from_cuda(e);

@@ -27,10 +27,12 @@ struct DevParams {
   float inv_bD58_f;       // its FP32 rounding
   float beta_f;           // fl32(beta), for the FP32 screens (no FP64 operation there)
   float bJ_f;             // fl32(fl(beta J))
+  float bJ_h, bJ_l;       // fl(beta J) in float-float
   int switching;          // 1 when beta D > 0 (pairs can be switched off)
   uint64_t key0, key1;    // Philox key: seed, replica
   double ln2_hi, ln2_lo;  // ln 2 as a double-double
   unsigned long long lx_magic;  // floor((2^64 - 1) / Lx) + 1 (0 when Lx = 1)
+  uint32_t lx_m32;              // floor(2^32 / Lx) (2^32 - 1 when Lx = 1), see site_xy
 };
 
 // floor(u / d) for 32-bit u and d >= 2 by one 64-bit high multiply with
@@ -46,6 +48,20 @@ __device__ __forceinline__ uint32_t div_by_magic(uint32_t u, unsigned long long 
 // Row y = i / Lx of site i, keeping 64-bit integer division out of the inner loops.
 __device__ __forceinline__ uint32_t site_row(uint32_t i, const DevParams& P) {
   return div_by_magic(i, P.lx_magic);
+}
+
+// Column x and row y of site j: umulhi(j, floor(2^32 / Lx)) is j / Lx or one less (the quotient
+// falls short of j / Lx by less than j / 2^32 < 1), corrected by one compare.  One 32-bit multiply
+// each way: site_row's 64-bit high multiply is four wide ones, which run at a quarter rate.
+__device__ __forceinline__ void site_xy(uint32_t j, const DevParams& P, int32_t& x, int32_t& y) {
+  uint32_t q = __umulhi(j, P.lx_m32);
+  uint32_t r = j - q * (uint32_t)P.Lx;
+  if (r >= (uint32_t)P.Lx) {
+    r -= (uint32_t)P.Lx;
+    ++q;
+  }
+  x = (int32_t)r;
+  y = (int32_t)q;
 }
 
 // Warp sum (lane 0 receives the total).

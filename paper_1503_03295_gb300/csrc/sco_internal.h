@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "df32.cuh"
 #include "sco_device.cuh"
 
 namespace sco {
@@ -53,6 +54,7 @@ struct Table {
   float4* xy32 = nullptr;    // by (|dx|, |dy|): FP32 copies {Dc, Vmax, 2 beta Vmax, q}
   Sw64* sw64 = nullptr;      // sweep, by (|dx|, |dy|): FP64 decision constants (see Sw64)
   float4* sw32 = nullptr;    // the same in FP32 (with its own c0)
+  PairDf* pdf = nullptr;     // sweep, by (|dx|, |dy|): the FP64 form's pair constants in float-float
   int32_t m_nn[2] = {-1, -1};
 };
 cudaError_t table_build(const DevParams& P, Table& t, cudaStream_t s, int64_t* launches);
@@ -64,9 +66,10 @@ void table_free(Table& t);
 void table_free_xy(Table& t);
 
 // ---- init / observables (spins.cu) ----
-cudaError_t spins_init(const DevParams& P, double* s, float4* s32, cudaStream_t st,
+// s32, sd: the FP32 and the float-float copies of the spins (either may be null)
+cudaError_t spins_init(const DevParams& P, double* s, float4* s32, SpinDf* sd, cudaStream_t st,
                        int64_t* launches);
-cudaError_t spins_to_f32(int64_t N, const double* s, float4* s32, cudaStream_t st,
+cudaError_t spins_copies(int64_t N, const double* s, float4* s32, SpinDf* sd, cudaStream_t st,
                          int64_t* launches);
 // largest dipolar degree of the current graph into cnt->max_degree_dip
 cudaError_t dip_degree_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* col,
@@ -87,27 +90,18 @@ struct SwitchBufs {
   uint32_t* ovf;    // 2 * ovf_cap (i, j | flag)
   uint32_t ovf_cap;
   uint64_t* scan_tmp;
-  // FP64 form only (else null): the pair cache, one 32-byte record per half-edge id h (slot
-  // i * kSlotCap + q of site i, then N * kSlotCap + overflow index), N * kSlotCap + ovf_cap of
-  // them, two halves of {1 - P_ij, x = beta (V - Vmax)}: one holds the pair at the current
-  // spins, the other the pair after the last proposed move of one endpoint (which half is which
-  // follows the endpoints' acceptance parities, see PairCache), so that every access of a pair
-  // touches one sector.  The switch writes the first half.
-  double4_32a* keep;
 };
 cudaError_t switch_run(const DevParams& P, const Table& t, const double* s, const float4* s32,
                        int precision, uint32_t epoch, SwitchBufs& b, DevCounters* cnt,
                        cudaStream_t st, int64_t* launches);
 cudaError_t csr_scan(const DevParams& P, SwitchBufs& b, uint32_t* row_ptr, DevCounters* cnt,
                      cudaStream_t st, int64_t* launches);
-// hid (optional, parallel to col): the half-edge id of every CSR entry (both entries of a pair
-// carry the id of its half-edge).  sort_rows (only without hid): sort every row by neighbour
-// index and record the largest dipolar degree; else a row holds its lower neighbours in the
-// order of their atomic slots, then its upper ones in switching order (no result depends on
-// the order inside a row).
+// sort_rows: sort every row by neighbour index and record the largest dipolar degree; else a row
+// holds its lower neighbours in the order of their atomic slots, then its upper ones in switching
+// order (no result depends on the order inside a row).
 cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, const uint32_t* row_ptr,
-                     uint32_t* col, uint32_t* hid, bool has_overflow, bool sort_rows,
-                     DevCounters* cnt, cudaStream_t st, int64_t* launches);
+                     uint32_t* col, bool has_overflow, bool sort_rows, DevCounters* cnt,
+                     cudaStream_t st, int64_t* launches);
 // out = col with every row sorted by neighbour index (the documented layout of the getters);
 // also records the largest dipolar degree in cnt.
 cudaError_t csr_sorted_copy(const DevParams& P, const uint32_t* row_ptr, const uint32_t* col,
@@ -146,30 +140,13 @@ cudaError_t bucket_run(const DevParams& P, uint32_t g, const uint32_t* row_ptr, 
                        DevCounters* cnt, cudaStream_t st, int64_t* launches);
 
 // ---- sweep.cu ----
-// The FP64 form's pair cache (see sweep_dev.cuh); hid null: no cache.
-struct PairCache {
-  const uint32_t* hid;  // per CSR entry: half-edge id of its pair
-  double4_32a* keep;    // per half-edge: the two halves of SwitchBufs::keep
-  // per site: bit 2 the parity p_i of its accepted moves since the halves were last written
-  // from the spins (the switch, or cache_build_run), bits 0-1 its decision in this MC step
-  // (0 not decided, 1 rejected, 2 accepted); an accepted move flips p_i as it is decided.  The
-  // current terms of pair (i, j) are in half p_i ^ p_j (0 after a reset): a site reads that
-  // half and writes its proposed-spin terms into the other, so an acceptance flips the half.
-  uint8_t* upd;
-  int carry;  // the next step uses this graph again: the endpoint decided last writes too
-  int reset;  // the halves were written from the spins: every parity starts at 0
-};
-cudaError_t sweep_run(const DevParams& P, const Table& t, double* s, float4* s32,
+// s32 (FP32-guarded form) or sd and propd (FP64 form): the working copies of the spins, and the
+// proposals of the step in float-float; the others may be null.
+cudaError_t sweep_run(const DevParams& P, const Table& t, double* s, float4* s32, SpinDf* sd,
                       const uint32_t* row_ptr, const uint32_t* col, const uint32_t* perm,
                       const uint32_t* off, uint32_t g, uint64_t step, int precision,
                       uint8_t* acc, uint32_t* defer, uint32_t* dcnt, double4_32a* prop,
-                      DevCounters* cnt, const PairCache& pc, cudaStream_t st,
-                      int64_t* launches);
-// Between two MC steps on the same graph after the spins changed outside the sweep: the pair
-// cache rebuilt from the spins (first halves; the next sweep resets the parities).
-cudaError_t cache_build_run(const DevParams& P, const Table& t, const double* s,
-                            const SwitchBufs& b, const DevCounters* cnt, cudaStream_t st,
-                            int64_t* launches);
+                      SpinDf* propd, DevCounters* cnt, cudaStream_t st, int64_t* launches);
 
 // ---- stats.cu ----
 // Graph diagnostics (see sco_get_graph_stats); copies 2 nb + 1 counts (survived, pairs, cross)

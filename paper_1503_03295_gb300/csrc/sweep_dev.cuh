@@ -28,10 +28,9 @@ struct SiteCtx {
 };
 
 // The pseudointeraction terms enter as sum_j [L_o,j - L_n,j] = log(prod z_o) - log(prod z_n)
-// with z = 1 - e^x = -expm1(x): one expm1 per pair energy and two logarithms per site (the
-// cached FP64 path compares the products instead: u prod z_o e^(sum dx) < prod z_n, see
-// accept_fp64_cached).  The products are renormalised by 2^kScale (exact) so that they never
-// underflow.
+// with z = 1 - e^x = -expm1(x): one expm1 per pair energy and two logarithms per site.  The
+// products are renormalised by 2^kScale (exact) so that they never underflow.  The FP64 form's
+// first decision, accept_df, compares products of e^-x - 1 instead and takes no logarithm.
 constexpr int kScale64 = 600;
 constexpr int kScale32 = 60;
 
@@ -143,136 +142,124 @@ __device__ __forceinline__ int accept_fp64(const DevParams& P, const SiteCtx& c,
   return 2;
 }
 
-// The pair cache of the FP64 form (single lattice).  For every surviving dipolar pair (half-edge
-// id h, carried by both CSR entries of the pair) record keep[h] holds two halves of
-// {1 - P = -expm1(x), x = beta (V - Vmax)}, each with the error of any FP64 evaluation of it
-// (|x error| <= c0 + 2^-52 |x|, relative error of the elementary function within
-// kExpm1RelErr6).  Half p_i ^ p_j holds the pair at the current spins, p_i being the parity of
-// site i's accepted moves since the switch (which leaves its FP64 values in the first half) or
-// a rebuild (PairCache::upd).  While a site is decided it reads that half and writes the pair
-// at its proposed spin into the other one: an acceptance flips its parity and so makes the
-// written half the current one, a rejection leaves the read half current.  The endpoint decided
-// last writes only when the next MC step keeps the graph.  So per pair endpoint one of the two
-// expm1 evaluations and one of the two dot products are read instead of computed, and nothing
-// has to be carried between the steps of an epoch.  A written 1 - P <= 0 (the proposed x not
-// strictly negative in FP64) makes every reader leave its decision to the double-double path,
-// which does not use the cache.
+// The FP64 form's decision (0: reject, 1: accept, 2: undecided) in float-float on the FP32 units
+// (df32.cuh), kG lanes of a warp per site; valid on the first lane of each group (sub = 0).
+//
+// What bounds it: FP32 issue (about 250 instructions per pair) and the gathers of the neighbours'
+// spins; in FP64 the same terms were bound by the 2 FP64 lanes of an SM per clock.
+//
+// With y = -x = beta (Vmax - V) >= 0 and z = 1 - e^-y, the acceptance u prod z_o e^(sum (x_n - x_o))
+// < prod z_n is u prod E_o < prod E_n for E = e^y - 1, since z / e^x = E: no sum of energies is
+// kept.  E = 2^k m with m in (0, 1.42) (df_expm1_scaled); the products of m are renormalised to
+// [1, 2) at every factor and the exponents summed as integers.
+//
+// Error bound of u prod E_o / prod E_n (relative, first order, doubled).  Per factor: kDfExpRelErr
+// (df_expm1_scaled given y), and dy / (1 - e^-y) <= 1.42 c0 / m with |dy| <= c0 = kYRelErr a1, where
+// c0 / m < 2^((d >> 23) + 1 - 40) for d the largest difference of the FP32 bit images of a1 and m
+// (a difference of 2^23 is a factor of two, off by at most 2^0.09); it has to stay below 2^-9, or
+// the site is left undecided (y <= 0 in float-float, or y >= 8192, likewise).  The products add
+// 2^-43 per factor, the exchange factor its argument's error and kDfExpRelErr.
+constexpr float kDfExpRelErr = 0x1p-31f;  // measured 2^-31.8 (y < 60), 20 M points
 
-// The site's PairCache::upd byte after its decision: an acceptance flips the parity (bit 2).
-__device__ __forceinline__ uint8_t upd_decided(uint32_t ui, bool accepted) {
-  return (uint8_t)(accepted ? ((ui & 4u) ^ 4u) | 2u : (ui & 4u) | 1u);
-}
-
-// accept_fp64 with the old-spin terms from the pair cache; writes the proposed-spin term of
-// every pair (the loop visits every pair, also when the decision is already undecided).
-__device__ __forceinline__ int accept_fp64_cached(const DevParams& P, const SiteCtx& c,
-                                                  const Sw64* __restrict__ sw,
-                                                  const double* __restrict__ s,
-                                                  const uint32_t* __restrict__ row_ptr,
-                                                  const uint32_t* __restrict__ col,
-                                                  const PairCache& pc, uint32_t ui) {
-  const double S0 = c.S[0], S1 = c.S[1], S2 = c.S[2];
-  const double N0 = c.Sn[0], N1 = c.Sn[1], N2 = c.Sn[2];
-  double bdv = 0.0, pz_o = 1.0, pz_n = 1.0;
-  unsigned long long c0m = 0;
-  int dmax = -2046;
-  int sc_o = 0, sc_n = 0, n = 0;
+template <int kG>
+__device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t yi,
+                                         const SpinDf& S, const SpinDf& N,
+                                         const PairDf* __restrict__ pdf, const SpinDf* sd,
+                                         const uint32_t* __restrict__ col, uint32_t e0,
+                                         uint32_t e1, uint32_t i, int sub) {
+  df pn = {1.f, 0.f}, po = {1.f, 0.f};
+  int K = 0, n = 0, dmax = -0x40000000;  // K: exponent of prod E_o / prod E_n beside po / pn
   bool bad = false;
-  const uint32_t e1 = row_ptr[c.i + 1];
-  for (uint32_t e = row_ptr[c.i]; e < e1; ++e) {
-    const uint32_t cj = col[e];
-    if (cj & kExchOnly) continue;
-    const int64_t j = cj;
-    const uint32_t h = pc.hid[e];
-    const uint32_t uj = pc.upd[j];
-    const uint32_t yj = site_row((uint32_t)j, P);
-    const int32_t dx = (int32_t)((uint32_t)j - yj * (uint32_t)P.Lx) - c.xi;
-    const int32_t dy = (int32_t)yj - c.yi;
-    const Sw64& t = sw[(int64_t)(dx < 0 ? -dx : dx) + (int64_t)P.Lx * (dy < 0 ? -dy : dy)];
-    const double fx = flip_if(t.ax, dx < 0), fy = flip_if(t.ay, dy < 0);
-    const double ax3 = flip_if(t.a3x, dx < 0), ay3 = flip_if(t.a3y, dy < 0);
-    const double a1 = t.a1, bvm = t.bvm;
-    const double bx = s[j], by = s[P.N + j], bz = s[2 * P.N + j];
-    // {1 - P, x} of the pair at the old spin: one 16-byte read of the record's sector, from
-    // the half given by the two parities (j's flipped already if it moved in this step)
-    double2* rec = reinterpret_cast<double2*>(&pc.keep[h]);
-    const uint32_t hf = ((ui ^ uj) >> 2) & 1u;
-    const double2 kv = rec[hf];
-    const double zo = kv.x, xo = kv.y;
-    // x = a1 (S'.S_j) - (S_j.a3 d)(S'.d) - bvm for the proposed spin S'
-    const double ns = N0 * bx + N1 * by + N2 * bz;
-    const double tp = bx * ax3 + by * ay3;
-    const double nd = N0 * fx + N1 * fy;
-    const double xn = fma(a1, ns, fma(-tp, nd, -bvm));
-    const bool okn = neg_strict(xn);
-    const double zn = okn ? neg_expm1_np6(xn) : -1.0;
-    if ((uj & 3u) == 0u || pc.carry) rec[hf ^ 1u] = make_double2(zn, xn);
-    // the cached term must be a positive number (a non-positive one marks an FP64 evaluation
-    // that could not be trusted)
-    if (!okn || !neg_strict(xo) || !(pos_bits(zo) - 1ull < 0x7FEFFFFFFFFFFFFFull)) {
+  for (uint32_t e = e0 + sub; e < e1; e += kG) {
+    const uint32_t j = col[e];
+    if (j & kExchOnly) continue;
+    int32_t xj, yj;
+    site_xy(j, P, xj, yj);
+    const int32_t dx = xj - xi, dy = yj - yi;
+    const SpinDf b = load32(sd + j);
+    const PairDf t = load32(pdf + (abs(dx) + (int64_t)P.Lx * abs(dy)));
+    const FieldDf g = df_field(t, dx < 0 ? -t.ax : t.ax, dy < 0 ? -t.ay : t.ay, b);
+    const df yn = df_pair_y(t, g, N), yo = df_pair_y(t, g, S);
+    if (!(fminf(yn.h, yo.h) > 0x1p-100f && fmaxf(yn.h, yo.h) < 8192.f)) {
       bad = true;
       continue;
     }
-    pz_n *= zn;
-    pz_o *= zo;
-    if (!renorm600(pz_n, sc_n) || !renorm600(pz_o, sc_o)) bad = true;
-    bdv += xn - xo;
-    dmax = max(dmax, exp_field(t.c0) - min(exp_field(zn), exp_field(zo)));
-    c0m = max(c0m, pos_bits(t.c0));
+    int kn, ko;
+    const df mn = df_expm1_scaled(yn, kn), mo = df_expm1_scaled(yo, ko);
+    dmax = max(dmax, __float_as_int(t.a1h) - __float_as_int(fminf(mn.h, mo.h)));
+    pn = df_mul(pn, mn);
+    po = df_mul(po, mo);
+    int xn = kn, xo = ko;
+    df_renorm(pn, xn);
+    df_renorm(po, xo);
+    K += xo - xn;
     ++n;
   }
+  if (kG > 1) {
+#pragma unroll
+    for (int o = kG / 2; o > 0; o >>= 1) {
+      const df qn = {__shfl_down_sync(0xffffffffu, pn.h, o, kG),
+                     __shfl_down_sync(0xffffffffu, pn.l, o, kG)};
+      const df qo = {__shfl_down_sync(0xffffffffu, po.h, o, kG),
+                     __shfl_down_sync(0xffffffffu, po.l, o, kG)};
+      pn = df_mul(pn, qn);
+      po = df_mul(po, qo);
+      K += __shfl_down_sync(0xffffffffu, K, o, kG);
+      n += __shfl_down_sync(0xffffffffu, n, o, kG);
+      dmax = max(dmax, __shfl_down_sync(0xffffffffu, dmax, o, kG));
+      bad |= __shfl_down_sync(0xffffffffu, (int)bad, o, kG) != 0;
+    }
+  }
+  if (sub != 0) return 0;
+  if (N.u_h == 0.f && N.u_l == 0.f) return 1;  // u = 0 accepts outright
   if (bad) return 2;
-  if (n > 0 && dmax + 2 + (32 - __clz(n)) > -10) return 2;  // n <= 2^(32 - clz n)
-  const double lin = n > 0 && dmax + 2 >= -1022
-                         ? (double)n * __longlong_as_double((long long)(dmax + 2 + 1023) << 52)
-                         : 0.0;
-  double tex = 0.0, bex = 0.0;
+  float bound = 0x1p-30f + (float)n * (2.f * kDfExpRelErr + 0x1p-42f);
+  if (n > 0) {
+    const int x = (dmax >> 23) + 1 - 40;
+    if (x > -9) return 2;
+    bound += 2.84f * (float)n * __int_as_float((max(x, -100) + 127) << 23);
+  }
+  df X = df_mul({N.u_h, N.u_l}, po);
   if (P.J != 0.0) {
-    double h0 = 0.0, h1 = 0.0, h2 = 0.0;
-    const int64_t nb[4] = {c.xi > 0 ? c.i - 1 : -1, c.xi + 1 < P.Lx ? c.i + 1 : -1,
-                           c.yi > 0 ? c.i - P.Lx : -1, c.yi + 1 < P.Ly ? c.i + P.Lx : -1};
+    // e^tex, tex = -beta J (S' - S) . (sum of the neighbours' spins)
+    df hx = {0.f, 0.f}, hy = hx, hz = hx;
+    const int32_t nb[4] = {xi > 0 ? -1 : 0, xi + 1 < P.Lx ? 1 : 0, yi > 0 ? -P.Lx : 0,
+                           yi + 1 < P.Ly ? P.Lx : 0};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      if (nb[q] < 0) continue;
-      h0 += s[nb[q]];
-      h1 += s[P.N + nb[q]];
-      h2 += s[2 * P.N + nb[q]];
+      if (nb[q] == 0) continue;
+      const SpinDf b = load32(sd + (int32_t)i + nb[q]);
+      hx = df_add(hx, {b.hx, b.lx});
+      hy = df_add(hy, {b.hy, b.ly});
+      hz = df_add(hz, {b.hz, b.lz});
     }
-    const double dot = (c.Sn[0] - c.S[0]) * h0 + (c.Sn[1] - c.S[1]) * h1 + (c.Sn[2] - c.S[2]) * h2;
-    tex = -(P.beta * P.J) * dot;
-    bex = 0x1p-44 * fabs(P.beta * P.J);
+    df w = df_mul(df_sub({N.hx, N.lx}, {S.hx, S.lx}), hx);
+    w = df_add(w, df_mul(df_sub({N.hy, N.ly}, {S.hy, S.ly}), hy));
+    w = df_add(w, df_mul(df_sub({N.hz, N.lz}, {S.hz, S.lz}), hz));
+    w = df_mul(w, {-P.bJ_h, -P.bJ_l});
+    w = df_fast(w.h, w.l);
+    const float aj = fabsf(P.bJ_h);
+    // |w error| <= 2^-40 beta J 4 (float-float sums of 12 terms below 2 each, scaled)
+    if (!(aj < 512.f)) return 2;
+    int k;
+    const df e = w.h < 0.f ? df_exp_core<true>(w, k) : df_exp_core<false>(w, k);
+    X = df_mul(X, df_add({1.f, 0.f}, e));
+    K += k;
+    bound += 0x1p-31f + 0x1p-38f * aj;
   }
-  // The decision in product form, without logarithms: mu < 0 is u Pz_o e^A < Pz_n with A = bdv +
-  // tex and Pz = pz 2^(-600 sc).  e^A = 2^k e^r, k = round(A / ln2) (|k| <= 2^20, else left
-  // undecided), e^r = 1 + r p(r) with p of expm1_np6 (relative error below 2^-32, the reduction's
-  // below 2^-34); X = u pz_o e^r and K = k + 600 (sc_n - sc_o), and X 2^K against pz_n is decided
-  // on the exponent fields when they differ by 2 or more, else by D = X 2^K - pz_n (X 2^K formed
-  // exactly from the bits).  delta bounds the relative errors of X 2^K and pz_n together,
-  // doubled: the terms of the logarithmic form's bound without its logarithms, and 2^-31 for e^r,
-  // its reduction, the two products and D.
-  const double A = bdv + tex;
-  const double t = fma(A, kExpInvLn2, 0x1.8p52);
-  const double kd = t - 0x1.8p52;
-  const int k = __double2loint(t);
-  if (k > (1 << 20) || k < -(1 << 20)) return 2;
-  const double r = fma(-kd, kExpLn2, A);
-  const double er = fma(r, expm1_poly6(r), 1.0);
-  const double X = (c.u * pz_o) * er;
-  const double c0s = (double)n * __longlong_as_double((long long)c0m);
-  const double delta = 2.0 * ((double)(n + 4) * c0s + 2.0 * lin +
-                              n * (4.0 * kExpm1RelErr6 + 0x1p-51) + bex +
-                              0x1p-51 * (fabs(tex) + fabs(bdv)) + 0x1p-31);
-  if (!(delta < 0.25)) return 2;
-  const int eX = exp_field(X), eY = exp_field(pz_n);
-  if (eX == 0) return 1;  // u = 0
-  const int dE = eX + k + kScale64 * (sc_n - sc_o) - eY;
-  if (dE >= 2) return 0;   // X 2^K >= 2^(eY + 2) > 2 pz_n
-  if (dE <= -2) return 1;  // X 2^K < 2^(eY - 1) <= pz_n / 2
-  const double Xs = __longlong_as_double(__double_as_longlong(X) + ((long long)(dE + eY - eX) << 52));
-  const double D = Xs - pz_n;
-  const long long oD = ord_bits(D), ol = ord_bits(delta * pz_n);
-  if (oD < -ol - 1) return 1;  // D < -delta pz_n
-  if (oD > ol) return 0;       // D > delta pz_n
+  bound *= 2.f;
+  if (!(bound < 0.25f)) return 2;
+  int kx = 0, kn = 0;
+  df_renorm(X, kx);
+  df_renorm(pn, kn);
+  K += kx - kn;
+  if (K >= 2) return 0;   // X 2^K >= 4 > 2 pn
+  if (K <= -2) return 1;  // X 2^K < 1/2 pn
+  const float f = K == 0 ? 1.f : (K > 0 ? 2.f : 0.5f);
+  const float D = (X.h * f - pn.h) + (X.l * f - pn.l);
+  const float lim = bound * pn.h;
+  if (D < -lim) return 1;
+  if (D > lim) return 0;
   return 2;
 }
 
@@ -414,38 +401,9 @@ __device__ __forceinline__ void write_site(const DevParams& P, const SiteCtx& c,
   acc[c.i] = ok ? 1 : 0;
 }
 
-// Product over the warp of the lanes' p 2^(-600 sc) (p a positive normal double): mantissa m in
-// [1, 2) and exponent e on every lane (the butterfly multiplies the same pairs on both lanes of
-// a step, so all lanes end with the same bits).
-__device__ __forceinline__ void warp_prod(double p, int sc, double& m, int& e) {
-  const unsigned long long b = pos_bits(p);
-  e = (int)(b >> 52) - 1023 - kScale64 * sc;
-  m = __longlong_as_double((long long)((b & 0xFFFFFFFFFFFFFull) | 0x3FF0000000000000ull));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    m *= __shfl_xor_sync(0xffffffffu, m, o);
-    e += __shfl_xor_sync(0xffffffffu, e, o);
-    const unsigned long long mb = pos_bits(m);
-    if ((mb >> 52) > 1023u) {  // m in [2, 4): halve it exactly
-      m = __longlong_as_double((long long)(mb - (1ull << 52)));
-      ++e;
-    }
-  }
-}
-
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ double warp_max_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ double warp_min_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
 __device__ __forceinline__ dd warp_sum_dd(dd v) {
@@ -537,110 +495,6 @@ __device__ int accept_fp64_warp(const DevParams& P, const SiteCtx& c,
                           0x1p-51 * (fabs(tex) + fabs(bdv) + fabs(mu)));
   if (mu < -B) return 1;
   if (mu > B) return 0;
-  return 2;
-}
-
-// accept_fp64_warp with the pair cache (see accept_fp64_cached); every lane writes the
-// proposed-spin terms of its pairs.
-__device__ int accept_fp64_warp_cached(const DevParams& P, const SiteCtx& c,
-                                       const Sw64* __restrict__ sw,
-                                       const double* __restrict__ s,
-                                       const uint32_t* __restrict__ row_ptr,
-                                       const uint32_t* __restrict__ col, const PairCache& pc,
-                                       uint32_t ui, int lane) {
-  double bdv = 0.0, pz_o = 1.0, pz_n = 1.0, c0s = 0.0;
-  int sc_o = 0, sc_n = 0, n = 0, bad = 0, dmax = -2046;
-  const uint32_t e1 = row_ptr[c.i + 1];
-  for (uint32_t e = row_ptr[c.i] + lane; e < e1; e += 32) {
-    const uint32_t cj = col[e];
-    if (cj & kExchOnly) continue;
-    const uint32_t j = cj;
-    const uint32_t h = pc.hid[e];
-    const uint32_t uj = pc.upd[j];
-    const uint32_t yj = site_row(j, P);
-    const int32_t dx = (int32_t)(j - yj * (uint32_t)P.Lx) - c.xi;
-    const int32_t dy = (int32_t)yj - c.yi;
-    const Sw64& t = sw[(int64_t)(dx < 0 ? -dx : dx) + (int64_t)P.Lx * (dy < 0 ? -dy : dy)];
-    const double fx = flip_if(t.ax, dx < 0), fy = flip_if(t.ay, dy < 0);
-    const double ax3 = flip_if(t.a3x, dx < 0), ay3 = flip_if(t.a3y, dy < 0);
-    const double bx = s[j], by = s[P.N + j], bz = s[2 * P.N + j];
-    double2* rec = reinterpret_cast<double2*>(&pc.keep[h]);
-    const uint32_t hf = ((ui ^ uj) >> 2) & 1u;
-    const double2 kv = rec[hf];
-    const double zo = kv.x, xo = kv.y;
-    const double ns = c.Sn[0] * bx + c.Sn[1] * by + c.Sn[2] * bz;
-    const double tp = bx * ax3 + by * ay3;
-    const double nd = c.Sn[0] * fx + c.Sn[1] * fy;
-    const double xn = fma(t.a1, ns, fma(-tp, nd, -t.bvm));
-    const bool okn = neg_strict(xn);
-    const double zn = okn ? neg_expm1_np6(xn) : -1.0;
-    if ((uj & 3u) == 0u || pc.carry) rec[hf ^ 1u] = make_double2(zn, xn);
-    if (!okn || !neg_strict(xo) || !(pos_bits(zo) - 1ull < 0x7FEFFFFFFFFFFFFFull)) {
-      bad = 1;
-      continue;
-    }
-    pz_n *= zn;
-    pz_o *= zo;
-    if (!renorm600(pz_n, sc_n) || !renorm600(pz_o, sc_o)) bad = 1;
-    bdv += xn - xo;
-    dmax = max(dmax, exp_field(t.c0) - min(exp_field(zn), exp_field(zo)));
-    c0s += t.c0;
-    ++n;
-  }
-  bdv = warp_sum_d(bdv);
-  c0s = warp_sum_d(c0s);
-  dmax = __reduce_max_sync(0xffffffffu, dmax);
-  n = __reduce_add_sync(0xffffffffu, n);
-  bad = __reduce_or_sync(0xffffffffu, bad);
-  if (bad) return 2;
-  if (n > 0 && dmax + 2 + (32 - __clz(n)) > -10) return 2;
-  double mo, mn;
-  int eo, en;
-  warp_prod(pz_o, sc_o, mo, eo);
-  warp_prod(pz_n, sc_n, mn, en);
-  const double lin = n > 0 && dmax + 2 >= -1022
-                         ? (double)n * __longlong_as_double((long long)(dmax + 2 + 1023) << 52)
-                         : 0.0;
-  double tex = 0.0, bex = 0.0;
-  if (P.J != 0.0) {
-    double h0 = 0.0, h1 = 0.0, h2 = 0.0;
-    const int64_t nb[4] = {c.xi > 0 ? c.i - 1 : -1, c.xi + 1 < P.Lx ? c.i + 1 : -1,
-                           c.yi > 0 ? c.i - P.Lx : -1, c.yi + 1 < P.Ly ? c.i + P.Lx : -1};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (nb[q] < 0) continue;
-      h0 += s[nb[q]];
-      h1 += s[P.N + nb[q]];
-      h2 += s[2 * P.N + nb[q]];
-    }
-    const double dot = (c.Sn[0] - c.S[0]) * h0 + (c.Sn[1] - c.S[1]) * h1 + (c.Sn[2] - c.S[2]) * h2;
-    tex = -(P.beta * P.J) * dot;
-    bex = 0x1p-44 * fabs(P.beta * P.J);
-  }
-  // the product form of accept_fp64_cached on the warp's products mo 2^eo and mn 2^en (the
-  // butterfly's ten products add 2^-49 to the 2^-31 term)
-  const double A = bdv + tex;
-  const double t = fma(A, kExpInvLn2, 0x1.8p52);
-  const double kd = t - 0x1.8p52;
-  const int k = __double2loint(t);
-  if (k > (1 << 20) || k < -(1 << 20)) return 2;
-  const double r = fma(-kd, kExpLn2, A);
-  const double er = fma(r, expm1_poly6(r), 1.0);
-  const double X = (c.u * mo) * er;
-  const double delta = 2.0 * ((double)(n + 4) * c0s + 2.0 * lin +
-                              n * (4.0 * kExpm1RelErr6 + 0x1p-51) + bex +
-                              0x1p-51 * (fabs(tex) + fabs(bdv)) + 0x1p-31);
-  if (!(delta < 0.25)) return 2;
-  const int eX = exp_field(X);
-  if (eX == 0) return 1;  // u = 0
-  const int dE = eX - 1023 + k + eo - en;  // mn in [1, 2)
-  if (dE >= 2) return 0;
-  if (dE <= -2) return 1;
-  const double Xs = __longlong_as_double(__double_as_longlong(X) + ((long long)(dE + 1023 - eX) << 52));
-  const double D = Xs - mn;
-  const long long oD = ord_bits(D), ol = ord_bits(delta * mn);
-  if (oD < -ol - 1) return 1;
-  if (oD > ol) return 0;
   return 2;
 }
 

@@ -340,10 +340,7 @@ __device__ __forceinline__ bool survives_fp32(const DevParams& P, float4 t32,
 
 // Where a site writes its upper neighbours: kSlotCap slots of its own (row `id` of hslot), then
 // an overflow list shared by all sites (entry: site id, j | flag).  indeg counts lower
-// neighbours per (local) site.  keep / keep_ovf (optional, FP64 form): the FP64 values of
-// 1 - P_ij and of x = beta (V - Vmax) of each surviving dipolar pair, written to the first half
-// of the pair-cache record at the same slot or overflow index (the cache that the FP64 sweep
-// starts from).
+// neighbours per (local) site.
 struct SwitchOut {
   uint32_t* hslot;
   uint32_t* indeg;
@@ -351,8 +348,6 @@ struct SwitchOut {
   uint32_t ovf_cap;
   unsigned long long* ovf_n;
   int* status;
-  double4_32a* keep = nullptr;
-  double4_32a* keep_ovf = nullptr;
 };
 
 // One site's walk along its half-plane list: the candidate search of Sec. 2.1 with the state it
@@ -374,17 +369,14 @@ struct SiteWalk {
 };
 
 __device__ __forceinline__ void switch_emit(const SwitchOut& o, uint32_t id, uint32_t& n_out,
-                                            uint32_t jv, double keep = 0.0, double xk = 0.0) {
+                                            uint32_t jv) {
   if (n_out < (uint32_t)kSlotCap) {
     o.hslot[(size_t)id * kSlotCap + n_out] = jv;
-    if (o.keep)
-      *reinterpret_cast<double2*>(&o.keep[(size_t)id * kSlotCap + n_out]) = make_double2(keep, xk);
   } else {
     const unsigned long long idx = atomicAdd(o.ovf_n, 1ull);
     if (idx < o.ovf_cap) {
       o.ovf[2 * idx] = id;
       o.ovf[2 * idx + 1] = jv;
-      if (o.keep) *reinterpret_cast<double2*>(&o.keep_ovf[idx]) = make_double2(keep, xk);
     } else {
       set_status(o.status, kStatusCapacity);
     }
@@ -466,7 +458,7 @@ __device__ __forceinline__ bool walk_step(const DevParams& P, const NearTable& T
                            keep, xk);
     }
     if (surv) {
-      switch_emit(o, a.id, a.n_out, (uint32_t)j, keep, xk);
+      switch_emit(o, a.id, a.n_out, (uint32_t)j);
       ++n_dip;
       if (k == mnn0) a.nn0 = true;
       if (k == mnn1) a.nn1 = true;

@@ -76,7 +76,8 @@ __global__ void k_hazard(int64_t K, const uint32_t* __restrict__ disp, uint64_t*
 // f = A1 S_j - A3 (S_j.d) d, |dV| <= 2^-16 Dc r^2 (shadow spins, FP32 constants).
 __global__ void k_xy(int32_t Lx, int32_t Ly, double D, double beta, double2* __restrict__ xy,
                      double* __restrict__ xyq, float4* __restrict__ xy32,
-                     Sw64* __restrict__ sw64, float4* __restrict__ sw32) {
+                     Sw64* __restrict__ sw64, float4* __restrict__ sw32,
+                     PairDf* __restrict__ pdf) {
   const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (q >= (int64_t)Lx * Ly) return;
   const int64_t ax = q % Lx, ay = q / Lx;
@@ -108,6 +109,8 @@ __global__ void k_xy(int32_t Lx, int32_t Ly, double D, double beta, double2* __r
   // each.  Doubled, and doubled again for the test against the larger of the two parts.
   t.bsw = 4.0 * (c64 + 0x1p-49) * (1.0 + 0x1p-20);
   sw64[q] = t;
+  const df d1 = df_split_const(t.a1), d3 = df_split_const(a3b), dv = df_split_const(bvm);
+  pdf[q] = PairDf{d1.h, d1.l, d3.h, d3.l, dv.h, dv.l, (float)ax, (float)ay};
   const double c32 = beta * (0x1p-16 * dc * (double)r2) + 0x1p-21 * bvm;
   sw32[q] = make_float4((float)a1, (float)a3, (float)bvm, (float)(c32 * (1.0 + 0x1p-20)));
 }
@@ -152,8 +155,9 @@ cudaError_t table_build_xy(const DevParams& P, Table& t, cudaStream_t s, int64_t
   if ((e = cudaMalloc(&t.xyq, nxy * sizeof(double))) != cudaSuccess) return e;
   if ((e = cudaMalloc(&t.sw64, nxy * sizeof(Sw64))) != cudaSuccess) return e;
   if ((e = cudaMalloc(&t.sw32, nxy * sizeof(float4))) != cudaSuccess) return e;
+  if ((e = cudaMalloc(&t.pdf, nxy * sizeof(PairDf))) != cudaSuccess) return e;
   k_xy<<<(unsigned)((nxy + 255) / 256), 256, 0, s>>>(P.Lx, P.Ly, P.D, P.beta, t.xy, t.xyq,
-                                                      t.xy32, t.sw64, t.sw32);
+                                                      t.xy32, t.sw64, t.sw32, t.pdf);
   ++*launches;
   // the FP64 candidate search's decay values, where this table owns the sorted list
   if (t.W && t.K > 0) {
@@ -224,6 +228,7 @@ void table_free_xy(Table& t) {
   cudaFree(t.xyq);
   cudaFree(t.sw64);
   cudaFree(t.sw32);
+  cudaFree(t.pdf);
   cudaFree(t.Ebits);
   t.Ebits = nullptr;
   t.xy = nullptr;
@@ -231,6 +236,7 @@ void table_free_xy(Table& t) {
   t.xyq = nullptr;
   t.sw64 = nullptr;
   t.sw32 = nullptr;
+  t.pdf = nullptr;
 }
 
 void table_free(Table& t) {
