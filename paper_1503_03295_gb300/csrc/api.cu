@@ -199,7 +199,8 @@ cudaError_t grow(T*& ptr, uint64_t& cap, uint64_t need) {
   return e;
 }
 
-sco_status do_switch(sco_ctx* c, uint32_t epoch, const double* src, const float4* src32) {
+sco_status do_switch(sco_ctx* c, uint32_t epoch, const double* src, const float4* src32,
+                     const SpinDf* srcd) {
   PhaseTimer tm(c, kPhSwitch);
   // per-switch counters: n_half, n_dip, ovf_n, nnz and max_degree, max_degree_dip
   SCO_TRY(cudaMemsetAsync(c->cnt, 0, 4 * sizeof(unsigned long long), c->st));
@@ -207,7 +208,7 @@ sco_status do_switch(sco_ctx* c, uint32_t epoch, const double* src, const float4
   if (c->p.n_sw > 1 && src == c->s)
     SCO_TRY(cudaMemcpyAsync(c->s_epoch, c->s, 3 * c->P.N * sizeof(double),
                             cudaMemcpyDeviceToDevice, c->st));
-  SCO_TRY(switch_run(c->P, c->tab, src, src32, c->p.precision, epoch, c->sw, c->cnt, c->st,
+  SCO_TRY(switch_run(c->P, c->tab, src, src32, srcd, c->p.precision, epoch, c->sw, c->cnt, c->st,
                      &c->launches));
   SCO_TRY(csr_scan(c->P, c->sw, c->row_ptr, c->cnt, c->st, &c->launches));
   sco_status st = read_counters(c);
@@ -224,8 +225,8 @@ sco_status do_switch(sco_ctx* c, uint32_t epoch, const double* src, const float4
     SCO_TRY(cudaMemsetAsync(c->cnt, 0, 4 * sizeof(unsigned long long), c->st));
     SCO_TRY(cudaMemsetAsync(&c->cnt->max_degree, 0, 2 * sizeof(unsigned), c->st));
     SCO_TRY(cudaMemsetAsync(&c->cnt->ovf_full, 0, sizeof(int), c->st));
-    SCO_TRY(switch_run(c->P, c->tab, src, src32, c->p.precision, epoch, c->sw, c->cnt, c->st,
-                       &c->launches));
+    SCO_TRY(switch_run(c->P, c->tab, src, src32, srcd, c->p.precision, epoch, c->sw, c->cnt,
+                       c->st, &c->launches));
     SCO_TRY(csr_scan(c->P, c->sw, c->row_ptr, c->cnt, c->st, &c->launches));
     st = read_counters(c);
     if (st != SCO_OK) return st;
@@ -280,7 +281,7 @@ sco_status do_colour(sco_ctx* c) {
 sco_status ensure_graph(sco_ctx* c) {
   const int64_t e = c->t / c->p.n_sw;
   if (c->graph_epoch != e) {
-    sco_status st = do_switch(c, (uint32_t)e, c->s, c->s32);
+    sco_status st = do_switch(c, (uint32_t)e, c->s, c->s32, c->sd);
     if (st != SCO_OK) return st;
   }
   if (!c->colour_valid) return do_colour(c);
@@ -424,7 +425,7 @@ void sco_destroy(sco_ctx* c) {
 sco_status sco_switch(sco_ctx* c) {
   if (!c) return SCO_EINVAL;
   if (c->sticky) return (sco_status)c->sticky;
-  return do_switch(c, (uint32_t)(c->t / c->p.n_sw), c->s, c->s32);
+  return do_switch(c, (uint32_t)(c->t / c->p.n_sw), c->s, c->s32, c->sd);
 }
 
 sco_status sco_colour(sco_ctx* c, int32_t* n_colours) {
@@ -646,14 +647,17 @@ sco_status sco_set_state(sco_ctx* c, const void* buf, size_t len) {
     if (!c->s_epoch) return SCO_ESTATE;
     SCO_TRY(cudaMemcpyAsync(c->s_epoch, body + 3 * N * sizeof(double), 3 * N * sizeof(double),
                             cudaMemcpyHostToDevice, c->st));
-    float4* tmp32 = nullptr;
-    SCO_TRY(cudaMalloc(&tmp32, N * sizeof(float4)));
-    cudaError_t e = spins_copies(N, c->s_epoch, tmp32, nullptr, c->st, &c->launches);
+    const bool f64 = c->p.precision == SCO_FP64;
+    void* tmp = nullptr;
+    SCO_TRY(cudaMalloc(&tmp, N * (f64 ? sizeof(SpinDf) : sizeof(float4))));
+    float4* t32 = f64 ? nullptr : (float4*)tmp;
+    SpinDf* td = f64 ? (SpinDf*)tmp : nullptr;
+    cudaError_t e = spins_copies(N, c->s_epoch, t32, td, c->st, &c->launches);
     sco_status st = e == cudaSuccess
-                        ? do_switch(c, (uint32_t)(c->t / c->p.n_sw), c->s_epoch, tmp32)
+                        ? do_switch(c, (uint32_t)(c->t / c->p.n_sw), c->s_epoch, t32, td)
                         : from_cuda(e);
     cudaStreamSynchronize(c->st);
-    cudaFree(tmp32);
+    cudaFree(tmp);
     if (st != SCO_OK) return st;
   }
   SCO_TRY(cudaStreamSynchronize(c->st));
@@ -711,7 +715,7 @@ sco_status sco_set_temperature(sco_ctx* c, double T) {
   c->P = make_dev_params(q);
   // the temperature-dependent tables (pair energies scaled by beta, candidate probabilities)
   table_free_xy(c->tab);
-  SCO_TRY(table_build_xy(c->P, c->tab, c->st, &c->launches));
+  SCO_TRY(table_build_xy(c->P, c->tab, c->tab, c->st, &c->launches));
   SCO_TRY(cudaStreamSynchronize(c->st));
   // the graph belongs to the old temperature: the next MC step switches again, same epoch
   c->graph_epoch = -1;

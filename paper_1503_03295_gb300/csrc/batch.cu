@@ -68,47 +68,34 @@ __global__ void __launch_bounds__(256) kb_clear(const BatchDev B) {
 template <int PREC>
 __global__ void __launch_bounds__(256, 4) kb_switch(const BatchDev B) {
   if (block_halted(B)) return;
-  __shared__ uint64_t sW[kNear];
-  __shared__ uint32_t sD[kNear];
+  __shared__ NearShared sh;
   __shared__ DevParams sP;
   const int r = block_replica(B);
   const RepDesc* d = B.desc + r;
   smem_copy(&sP, &d->P, sizeof(DevParams));
+  const NearTable T = near_table(d->search, sh);
   __syncthreads();
-  const int64_t K = sP.K;
-  const int64_t nnear = K < kNear ? K : kNear;
-  const uint64_t* W = d->W;
-  const uint32_t* disp = d->disp;
-  for (int q = threadIdx.x; q < nnear; q += blockDim.x) {
-    sW[q] = W[q];
-    sD[q] = disp[q];
-  }
-  __syncthreads();
-  const NearTable T{sW, sD, W, disp, nnear, K, nnear};
   const uint32_t base = d->base;
   const uint32_t i = (blockIdx.x - B.blk_start[r]) * kBatchBlock + threadIdx.x;
-  unsigned long long n_half = 0, n_dip = 0;
-  unsigned ghits = 0, g32 = 0;
+  unsigned n_half = 0, n_dip = 0, ghits = 0, g32 = 0;
   if (i < (uint32_t)sP.N) {
     const uint32_t gs = base + i;
-    const uint64_t Wtot = K > 0 ? __ldg(&W[K - 1]) : 0;
     const uint32_t epoch = (uint32_t)(B.ctl->step / (unsigned long long)B.n_sw);
     const SwitchOut o{B.hslot, B.indeg + base, B.ovf, B.ovf_cap, &B.ctl->ovf_n,
                       &B.ctl->ovf_full};
-    const size_t so = 3 * (size_t)base;
+    const SwitchIn in{d->pdf, d->qdf, d->xy32, B.s + 3 * (size_t)base,
+                      PREC == 1 ? B.s32 + base : nullptr, PREC == 0 ? B.sd + base : nullptr};
     const uint32_t n_out =
-        switch_site<PREC>(sP, T, Wtot, d->sw64, d->xyq, d->xy32, B.s + so, B.s32 + base, epoch,
-                          d->mnn0, d->mnn1, i, gs, o, n_dip, ghits, g32);
+        switch_site<PREC>(sP, T, in, epoch, d->mnn0, d->mnn1, i, gs, o, n_dip, ghits, g32);
     B.hcnt[gs] = n_out;
     n_half = n_out;
   }
-  n_half = warp_sum_u64(n_half);
-  n_dip = warp_sum_u64(n_dip);
+  const unsigned long long nh = warp_sum_u64(n_half), ndp = warp_sum_u64(n_dip);
   const unsigned long long gh = warp_sum_u64(ghits), gl = warp_sum_u64(g32);
   if ((threadIdx.x & 31) == 0) {
     DevCounters* c = B.cnt + r;
-    if (n_half) atomicAdd(&c->n_half, n_half);
-    if (n_dip) atomicAdd(&c->n_dip, n_dip);
+    if (nh) atomicAdd(&c->n_half, nh);
+    if (ndp) atomicAdd(&c->n_dip, ndp);
     if (gh) atomicAdd(&c->guard_fp64, gh);
     if (gl) atomicAdd(&c->guard_fp32, gl);
   }
@@ -472,6 +459,11 @@ __global__ void __launch_bounds__(256) kb_propose(const BatchDev B) {
   const bool ok = propose(d->P, c, B.ctl->step);
   B.prop[base + i] = ok ? make_double4_32a(c.Sn[0], c.Sn[1], c.Sn[2], c.u)
                         : make_double4_32a(0.0, 0.0, 1.0, -1.0);
+  if (B.propd) {
+    SpinDf p = spin_df(c.Sn[0], c.Sn[1], c.Sn[2], c.u);
+    if (!ok) p.u_h = -1.f;
+    B.propd[base + i] = p;
+  }
 }
 
 // Sites of class c (all replicas) one per thread; undecided ones go to the deferred list of
@@ -483,8 +475,8 @@ __global__ void __launch_bounds__(128, PREC == 1 ? 6 : 5) kb_sweep(const BatchDe
   extern __shared__ uint32_t wsm[];
   const int R = B.R;
   uint32_t* sbase = wsm;          // R + 1
-  uint32_t* sg1 = sbase + R + 1;  // R deferred by the first screen
-  uint32_t* sg2 = sg1 + R;        // R sent on to double-double (FP32-guarded form)
+  uint32_t* sg1 = sbase + R + 1;  // R deferred by the FP32 screen
+  uint32_t* sg2 = sg1 + R;        // R sent on to double-double
   for (int r = threadIdx.x; r <= R; r += blockDim.x) sbase[r] = B.site_start[r];
   for (int r = threadIdx.x; r < R; r += blockDim.x) {
     sg1[r] = 0;
@@ -504,26 +496,44 @@ __global__ void __launch_bounds__(128, PREC == 1 ? 6 : 5) kb_sweep(const BatchDe
       const uint32_t base = sbase[r];
       const RepDesc* d = B.desc + r;
       const DevParams& P = d->P;
-      const size_t so = 3 * (size_t)base;
-      double* s = B.s + so;
-      float4* s32 = B.s32 + base;
-      SiteCtx x;
-      load_site(P, x, gs - base, s);
-      if (!take_proposal(x, B.prop + base)) {
-        B.acc[gs] = 0;
-        continue;
-      }
-      int dec = 1;
-      if (x.u != 0.0) {
-        dec = PREC == 1 ? accept_fp32(P, x, d->sw32, s32, B.row_ptr + base, B.col)
-                        : accept_fp64(P, x, d->sw64, s, B.row_ptr + base, B.col);
+      double* s = B.s + 3 * (size_t)base;
+      const uint32_t i = gs - base;
+      int dec;
+      if (PREC == 0) {
+        const SpinDf N = load32(B.propd + gs);
+        if (N.u_h < 0.f) {
+          B.acc[gs] = 0;
+          continue;
+        }
+        int32_t xi, yi;
+        site_xy(i, P, xi, yi);
+        dec = accept_df<1>(P, xi, yi, load32(B.sd + gs), N, d->pdf, B.sd + base, B.col,
+                           B.row_ptr[gs], B.row_ptr[gs + 1], i, 0);
+        if (dec != 2) {
+          if (dec == 1) {
+            const double4_32a v = B.prop[gs];
+            s[i] = v.x;
+            s[P.N + i] = v.y;
+            s[2 * P.N + i] = v.z;
+            B.sd[gs] = N;
+          }
+          B.acc[gs] = (uint8_t)dec;
+        }
+      } else {
+        float4* s32 = B.s32 + base;
+        SiteCtx x;
+        load_site(P, x, i, s);
+        if (!take_proposal(x, B.prop + base)) {
+          B.acc[gs] = 0;
+          continue;
+        }
+        dec = x.u != 0.0 ? accept_fp32(P, x, d->sw32, s32, B.row_ptr + base, B.col) : 1;
+        if (dec != 2) write_site(P, x, dec == 1, s, s32, B.acc + base);
       }
       if (dec == 2) {
         B.defer[b + atomicAdd(&B.dcnt[c], 1u)] = gs;
-        atomicAdd(&sg1[r], 1u);
-        continue;
+        if (PREC == 1) atomicAdd(&sg1[r], 1u);
       }
-      write_site(P, x, dec == 1, s, PREC == 1 ? s32 : nullptr, B.acc + base);
     }
     if (!grid_sync(B.ctl->bar, &B.ctl->status, B.ns_limit)) break;
     const uint32_t nd = ld_u32_gpu(&B.dcnt[c]);
@@ -536,16 +546,18 @@ __global__ void __launch_bounds__(128, PREC == 1 ? 6 : 5) kb_sweep(const BatchDe
       const DevParams& P = d->P;
       const size_t so = 3 * (size_t)base;
       double* s = B.s + so;
-      float4* s32 = B.s32 + base;
       SiteCtx x;
       load_site(P, x, gs - base, s);
       take_proposal(x, B.prop + base);
-      int dec = PREC == 1 ? accept_fp64_warp(P, x, d->sw64, s, B.row_ptr + base, B.col, lane) : 2;
+      int dec = accept_fp64_warp(P, x, d->sw64, s, B.row_ptr + base, B.col, lane);
       if (dec == 2) {
-        if (PREC == 1 && lane == 0) atomicAdd(&sg2[r], 1u);
+        if (lane == 0) atomicAdd(&sg2[r], 1u);
         dec = accept_dd_warp(P, x, s, B.row_ptr + base, B.col, lane) ? 1 : 0;
       }
-      if (lane == 0) write_site(P, x, dec == 1, s, PREC == 1 ? s32 : nullptr, B.acc + base);
+      if (lane == 0) {
+        write_site(P, x, dec == 1, s, PREC == 1 ? B.s32 + base : nullptr, B.acc + base);
+        if (PREC == 0 && dec == 1) B.sd[gs] = B.propd[gs];
+      }
       __syncwarp();
     }
     if (!grid_sync(B.ctl->bar, &B.ctl->status, B.ns_limit)) break;
@@ -553,12 +565,8 @@ __global__ void __launch_bounds__(128, PREC == 1 ? 6 : 5) kb_sweep(const BatchDe
   __syncthreads();
   for (int r = threadIdx.x; r < R; r += blockDim.x) {
     DevCounters* cr = B.cnt + r;
-    if (PREC == 1) {
-      if (sg1[r]) atomicAdd(&cr->guard_fp32, (unsigned long long)sg1[r]);
-      if (sg2[r]) atomicAdd(&cr->guard_fp64, (unsigned long long)sg2[r]);
-    } else if (sg1[r]) {
-      atomicAdd(&cr->guard_fp64, (unsigned long long)sg1[r]);
-    }
+    if (sg1[r]) atomicAdd(&cr->guard_fp32, (unsigned long long)sg1[r]);
+    if (sg2[r]) atomicAdd(&cr->guard_fp64, (unsigned long long)sg2[r]);
   }
 }
 

@@ -22,10 +22,10 @@ constexpr int kBatchBlock = 256;  // sites per block of the per-site batch kerne
 // Constant description of replica r.
 struct RepDesc {
   DevParams P;
-  const uint64_t* W;  // hazard prefix of the lattice shape (shared between replicas)
-  const uint32_t* disp;
+  Search search;  // list of the lattice shape (shared between replicas), decay bits and guides
   const double2* xy;
-  const double* xyq;
+  const float2* qdf;
+  const PairDf* pdf;
   const float4* xy32;
   const Sw64* sw64;
   const float4* sw32;
@@ -74,7 +74,9 @@ struct BatchDev {
   int precision;
   int n_sw;
   double* s;
-  float4* s32;  // FP32 copy of the spins, one (x, y, z, 0) per site
+  float4* s32;    // FP32-guarded form: FP32 copy of the spins, one (x, y, z, 0) per site
+  SpinDf* sd;     // FP64 form: float-float copy
+  SpinDf* propd;  // FP64 form: Ntot proposals in float-float
   uint8_t* acc;
   uint32_t* hslot;
   uint32_t* hcnt;

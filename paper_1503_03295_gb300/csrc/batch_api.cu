@@ -26,6 +26,7 @@ struct sco_batch {
   std::vector<DevParams> P;
   std::vector<Table> lists;  // sorted list + hazard prefix, one per lattice shape
   std::vector<Table> xy;     // temperature-dependent tables, one per replica
+  std::vector<int> list_of;  // index of each replica's list
   std::vector<uint32_t> site_start, blk_start;
   std::vector<RepDesc> desc;
   BatchDev B{};
@@ -80,6 +81,8 @@ void free_all(sco_batch* b) {
   cudaFree((void*)B.site_start);
   cudaFree(B.s);
   cudaFree(B.s32);
+  cudaFree(B.sd);
+  cudaFree(B.propd);
   cudaFree(B.acc);
   cudaFree(B.hslot);
   cudaFree(B.hcnt);
@@ -288,6 +291,20 @@ bool valid_tuning(const sco_batch_tuning* t) {
          (t->kw_low_group == 1024 || t->kw_low_group == 2048 || t->kw_low_group == 4096);
 }
 
+// Replica r's parameters and tables in its description.
+void set_tables(sco_batch* b, int r) {
+  RepDesc& d = b->desc[r];
+  const Table& t = b->xy[r];
+  d.P = b->P[r];
+  d.search = table_search(t, b->lists[b->list_of[r]]);
+  d.xy = t.xy;
+  d.qdf = t.qdf;
+  d.pdf = t.pdf;
+  d.xy32 = t.xy32;
+  d.sw64 = t.sw64;
+  d.sw32 = t.sw32;
+}
+
 bool same_model(const sco_params& a, const sco_params& b) {
   return a.precision == b.precision && a.n_sw == b.n_sw;
 }
@@ -352,7 +369,8 @@ sco_status sco_batch_init(const sco_params* p, int32_t n, void* stream, sco_batc
   b->P.resize(n);
   b->xy.resize(n);
   b->desc.resize(n);
-  std::vector<int> list_of(n, -1);
+  b->list_of.assign(n, -1);
+  std::vector<int>& list_of = b->list_of;
   std::vector<std::pair<int32_t, int32_t>> shapes;
   for (int r = 0; r < n; ++r) {
     b->P[r] = make_dev_params(p[r]);
@@ -367,18 +385,11 @@ sco_status sco_batch_init(const sco_params* p, int32_t n, void* stream, sco_batc
     } else {
       list_of[r] = (int)(it - shapes.begin());
     }
-    const cudaError_t e = table_build_xy(b->P[r], b->xy[r], b->st, &b->launches);
-    if (e != cudaSuccess) return fail(from_cuda(e));
     const Table& L = b->lists[list_of[r]];
+    const cudaError_t e = table_build_xy(b->P[r], b->xy[r], L, b->st, &b->launches);
+    if (e != cudaSuccess) return fail(from_cuda(e));
     RepDesc& d = b->desc[r];
-    d.P = b->P[r];
-    d.W = L.W;
-    d.disp = L.disp;
-    d.xy = b->xy[r].xy;
-    d.xyq = b->xy[r].xyq;
-    d.xy32 = b->xy[r].xy32;
-    d.sw64 = b->xy[r].sw64;
-    d.sw32 = b->xy[r].sw32;
+    set_tables(b, r);
     d.mnn0 = L.m_nn[0];
     d.mnn1 = L.m_nn[1];
     d.base = b->site_start[r];
@@ -401,7 +412,12 @@ sco_status sco_batch_init(const sco_params* p, int32_t n, void* stream, sco_batc
   A(&B.cnt, n * sizeof(DevCounters));
   A(&B.ctl, sizeof(BatchCtl));
   A(&B.s, 3 * N * sizeof(double));
-  A(&B.s32, N * sizeof(float4));
+  if (B.precision == SCO_FP64) {
+    A(&B.sd, N * sizeof(SpinDf));
+    A(&B.propd, N * sizeof(SpinDf));
+  } else {
+    A(&B.s32, N * sizeof(float4));
+  }
   A(&B.acc, N);
   A(&B.hslot, N * kSlotCap * sizeof(uint32_t));
   A(&B.hcnt, N * sizeof(uint32_t));
@@ -441,7 +457,8 @@ sco_status sco_batch_init(const sco_params* p, int32_t n, void* stream, sco_batc
   if (e == cudaSuccess) e = cudaMemsetAsync(B.acc, 0, N, b->st);
   for (int r = 0; r < n && e == cudaSuccess; ++r) {
     const size_t so = 3 * (size_t)b->site_start[r];
-    e = spins_init(b->P[r], B.s + so, B.s32 + b->site_start[r], nullptr, b->st, &b->launches);
+    e = spins_init(b->P[r], B.s + so, B.s32 ? B.s32 + b->site_start[r] : nullptr,
+                   B.sd ? B.sd + b->site_start[r] : nullptr, b->st, &b->launches);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
   if (e != cudaSuccess) return fail(from_cuda(e));
@@ -643,8 +660,9 @@ sco_status sco_batch_set_spins(sco_batch* b, int32_t r, const double* xyz, int32
   const size_t N = (size_t)b->P[r].N, so = 3 * (size_t)b->site_start[r];
   SCO_TRY(cudaMemcpyAsync(b->B.s + so, xyz, 3 * N * sizeof(double),
                           on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, b->st));
-  SCO_TRY(spins_copies((int64_t)N, b->B.s + so, b->B.s32 + b->site_start[r], nullptr, b->st,
-                       &b->launches));
+  const uint32_t base = b->site_start[r];
+  SCO_TRY(spins_copies((int64_t)N, b->B.s + so, b->B.s32 ? b->B.s32 + base : nullptr,
+                       b->B.sd ? b->B.sd + base : nullptr, b->st, &b->launches));
   SCO_TRY(cudaStreamSynchronize(b->st));
   return SCO_OK;
 }
@@ -723,14 +741,9 @@ sco_status sco_batch_set_temperature(sco_batch* b, int32_t r, double T) {
   b->p[r] = q;
   b->P[r] = make_dev_params(q);
   table_free_xy(b->xy[r]);
-  SCO_TRY(table_build_xy(b->P[r], b->xy[r], b->st, &b->launches));
-  RepDesc& d = b->desc[r];
-  d.P = b->P[r];
-  d.xy = b->xy[r].xy;
-  d.xyq = b->xy[r].xyq;
-  d.xy32 = b->xy[r].xy32;
-  d.sw64 = b->xy[r].sw64;
-  d.sw32 = b->xy[r].sw32;
+  SCO_TRY(table_build_xy(b->P[r], b->xy[r], b->lists[b->list_of[r]], b->st, &b->launches));
+  set_tables(b, r);
+  const RepDesc& d = b->desc[r];
   SCO_TRY(cudaMemcpyAsync(const_cast<RepDesc*>(b->B.desc) + r, &d, sizeof(RepDesc),
                           cudaMemcpyHostToDevice, b->st));
   SCO_TRY(cudaStreamSynchronize(b->st));

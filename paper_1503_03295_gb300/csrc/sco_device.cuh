@@ -259,7 +259,6 @@ struct __align__(64) Sw64 {
   double ax, ay;    // |dx|, |dy|
   double bvm;       // fl(beta Vmax)
   double c0;        // bound on |error of x| not scaling with |x|, plus 2^-52 (2 beta Vmax)
-  double bsw;       // margin bound of the FP64 survival test of the switch (see table.cu)
 };
 
 // x with its sign flipped when neg (bit operation, no FP64 instruction)

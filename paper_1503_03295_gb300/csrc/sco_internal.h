@@ -41,28 +41,63 @@ cudaError_t scan_incl_u64(const uint64_t* in, uint64_t* out, int64_t n, uint64_t
                           uint64_t* total_dev, cudaStream_t s, int64_t* launches);
 
 // ---- table.cu ----
+// Guides into the decay bits E for the switch's candidate search (first k with E_k <= tb, on bit
+// images).  Near, tb >= e_near = E of the last head element: near[q], q = (bits of 1.0 - tb) >>
+// near_shift, is the first k with E_k at or below the largest target of cell q, so the candidate of
+// a target in cell q lies in [near[q], near[q + 1]].  Far, below: the same on q = (e_near - tb) >>
+// far_shift with far_n cells over the rest of the list.
+constexpr int kNear = 2048;       // head of the sorted list kept in shared memory (r <~ 25)
+constexpr int kNearGuide = 4096;  // 8 KB; at T = 0.6 D 64 cells per factor of two of E
+constexpr uint32_t kFarGuide = 65536;
+// Bits of 1.0: the decay value before the first element (W = 0).
+constexpr uint64_t kDecayStart = 0x3FF0000000000000ull;
+struct SearchHead {
+  uint64_t e_near, e_last;
+  int32_t near_shift, far_shift;
+};
+struct Search {
+  const uint64_t* E;
+  const uint64_t* W;
+  const uint32_t* disp;
+  const uint16_t* near;
+  const uint32_t* far;
+  const SearchHead* head;
+  int32_t K;
+  uint32_t far_n;
+};
 struct Table {
   int64_t K = 0;
   uint32_t* disp = nullptr;  // packed (dx & 0xFFFF) | (dy << 16), sorted by (r^2, dy, dx)
   uint64_t* W = nullptr;     // inclusive prefix of the integer hazards A_m
-  // by list index m: the bits of fl(exp(-beta D 2^-58 W_m)), the probability that a walk from
-  // the list's start passes m without a candidate (FP64 candidate search; temperature-dependent,
-  // built with the tables by (|dx|, |dy|) once the list exists)
+  // by list index m: the bits of exp(-beta D 2^-58 W_m), the probability that a walk from
+  // the list's start passes m without a candidate (candidate search; temperature-dependent)
   uint64_t* Ebits = nullptr;
+  SearchHead* head = nullptr;  // guides into Ebits (see Search)
+  uint16_t* near_g = nullptr;
+  uint32_t* far_g = nullptr;
+  uint32_t far_n = 0;
   double2* xy = nullptr;     // by (|dx|, |dy|): {fl(D c(r^2)), V_max = fl(fl(D A) 2^-59)}
-  double* xyq = nullptr;     // by (|dx|, |dy|): q = -expm1(-2 beta V_max), candidate probability
+  float2* qdf = nullptr;     // by (|dx|, |dy|): q = -expm1(-2 beta V_max), candidate probability
+                             // (float-float)
   float4* xy32 = nullptr;    // by (|dx|, |dy|): FP32 copies {Dc, Vmax, 2 beta Vmax, q}
   Sw64* sw64 = nullptr;      // sweep, by (|dx|, |dy|): FP64 decision constants (see Sw64)
   float4* sw32 = nullptr;    // the same in FP32 (with its own c0)
   PairDf* pdf = nullptr;     // sweep, by (|dx|, |dy|): the FP64 form's pair constants in float-float
+  void* pool = nullptr;      // the one allocation behind the temperature-dependent tables
   int32_t m_nn[2] = {-1, -1};
 };
 cudaError_t table_build(const DevParams& P, Table& t, cudaStream_t s, int64_t* launches);
-// the two halves: the temperature-dependent tables by (|dx|, |dy|), and the sorted list
-// with its hazard prefix (depends on Lx, Ly only; synchronises)
-cudaError_t table_build_xy(const DevParams& P, Table& t, cudaStream_t s, int64_t* launches);
+// the two halves: the temperature-dependent tables by (|dx|, |dy|) and over the sorted list `list`
+// (t's own, or one that several temperatures share), and the sorted list with its hazard prefix
+// (depends on Lx, Ly only; synchronises)
+cudaError_t table_build_xy(const DevParams& P, Table& t, const Table& list, cudaStream_t s,
+                           int64_t* launches);
 cudaError_t table_build_list(const DevParams& P, Table& t, cudaStream_t s, int64_t* launches);
 void table_free(Table& t);
+// t's temperature-dependent tables over `list` as the switch searches them
+inline Search table_search(const Table& t, const Table& list) {
+  return Search{t.Ebits, list.W, list.disp, t.near_g, t.far_g, t.head, (int32_t)list.K, t.far_n};
+}
 void table_free_xy(Table& t);
 
 // ---- init / observables (spins.cu) ----
@@ -92,7 +127,7 @@ struct SwitchBufs {
   uint64_t* scan_tmp;
 };
 cudaError_t switch_run(const DevParams& P, const Table& t, const double* s, const float4* s32,
-                       int precision, uint32_t epoch, SwitchBufs& b, DevCounters* cnt,
+                       const SpinDf* sd, int precision, uint32_t epoch, SwitchBufs& b, DevCounters* cnt,
                        cudaStream_t st, int64_t* launches);
 cudaError_t csr_scan(const DevParams& P, SwitchBufs& b, uint32_t* row_ptr, DevCounters* cnt,
                      cudaStream_t st, int64_t* launches);

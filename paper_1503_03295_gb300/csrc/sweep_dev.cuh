@@ -48,9 +48,7 @@ __device__ __forceinline__ bool renorm600(double& p, int& sc) {
 
 // Pair terms from the sweep table entry (Sw64): the beta-scaled field of S_j on site i,
 // f = a1 S_j - (S_j . a3 d) d, gives x = S.f - bvm = beta V(S) - beta Vmax for the old and the
-// new spin (7 + 2 x 3 FP64 operations); where only the proposed spin's term is formed (the pair
-// cache holds the old one), x = a1 (S'.S_j) - (S_j.a3 d)(S'.d) - bvm takes 9.  Either way the
-// rounding stays far inside c0.
+// new spin (7 + 2 x 3 FP64 operations); the rounding stays far inside c0.
 //
 // Error bound of the margin mu = ln u + beta dE' (first order, doubled):
 //   per pair, |dx| <= c0 + eps_r |x|, and c0 from the table already includes eps_r 2 beta Vmax;
@@ -61,86 +59,6 @@ __device__ __forceinline__ bool renorm600(double& p, int& sc) {
 //   each ratio is below 2^(e(c0_j) - e(z_j) + 1) with e the exponent field, so with two z per
 //   pair lin <= n 2^(dmax + 2), dmax the largest exponent difference, found with integer
 //   operations; it must stay below 2^-10 or the decision is left undecided.
-
-// FP64 decision (0: reject, 1: accept, 2: undecided).  eps_r = 2^-52 (unit roundoff, with
-// margin), eps_f = kLogRelErr for the library's log_np (inputs in (0, 1]), eps_z =
-// kExpm1RelErr6 for the library's expm1_np6 (two per pair, doubled: 4 eps_z).  Compares, minima
-// and renormalisation tests work on the bits of positive doubles (integer pipe).
-__device__ __forceinline__ int accept_fp64(const DevParams& P, const SiteCtx& c,
-                                           const Sw64* __restrict__ sw,
-                                           const double* __restrict__ s,
-                                           const uint32_t* __restrict__ row_ptr,
-                                           const uint32_t* __restrict__ col) {
-  const double S0 = c.S[0], S1 = c.S[1], S2 = c.S[2];
-  const double N0 = c.Sn[0], N1 = c.Sn[1], N2 = c.Sn[2];
-  double bdv = 0.0, pz_o = 1.0, pz_n = 1.0;
-  unsigned long long c0m = 0;  // bits of the largest c0 (n max c0 bounds their sum)
-  int dmax = -2046;  // largest e(c0_j) - e(z_j)
-  int sc_o = 0, sc_n = 0, n = 0;
-  const uint32_t e1 = row_ptr[c.i + 1];
-  for (uint32_t e = row_ptr[c.i]; e < e1; ++e) {
-    const uint32_t cj = col[e];
-    if (cj & kExchOnly) continue;
-    const int64_t j = cj;
-    const uint32_t yj = site_row((uint32_t)j, P);
-    const int32_t dx = (int32_t)((uint32_t)j - yj * (uint32_t)P.Lx) - c.xi;
-    const int32_t dy = (int32_t)yj - c.yi;
-    const Sw64& t = sw[(int64_t)(dx < 0 ? -dx : dx) + (int64_t)P.Lx * (dy < 0 ? -dy : dy)];
-    const double fx = flip_if(t.ax, dx < 0), fy = flip_if(t.ay, dy < 0);
-    const double ax3 = flip_if(t.a3x, dx < 0), ay3 = flip_if(t.a3y, dy < 0);
-    const double a1 = t.a1, bvm = t.bvm;
-    const double bx = s[j], by = s[P.N + j], bz = s[2 * P.N + j];
-    const double tp = bx * ax3 + by * ay3;
-    const double gx = a1 * bx - tp * fx;
-    const double gy = a1 * by - tp * fy;
-    const double gz = a1 * bz;
-    // three FMAs each; c0 covers the roundings (those touching bvm stay below 2^-51 bvm)
-    const double xn = fma(N0, gx, fma(N1, gy, fma(N2, gz, -bvm)));
-    const double xo = fma(S0, gx, fma(S1, gy, fma(S2, gz, -bvm)));
-    if (!neg_strict(xn) || !neg_strict(xo)) return 2;
-    const double zn = neg_expm1_np6(xn), zo = neg_expm1_np6(xo);
-    pz_n *= zn;
-    pz_o *= zo;
-    if (!renorm600(pz_n, sc_n) || !renorm600(pz_o, sc_o)) return 2;
-    bdv += xn - xo;
-    dmax = max(dmax, exp_field(t.c0) - min(exp_field(zn), exp_field(zo)));
-    c0m = max(c0m, pos_bits(t.c0));
-    ++n;
-  }
-  if (n > 0 && dmax + 2 + (32 - __clz(n)) > -10) return 2;  // n <= 2^(32 - clz n)
-  // n 2^(dmax + 2), the power of two from its bits (dmax + 2 <= -10 here; below -1022: 0)
-  const double lin = n > 0 && dmax + 2 >= -1022
-                         ? (double)n * __longlong_as_double((long long)(dmax + 2 + 1023) << 52)
-                         : 0.0;
-  double tex = 0.0, bex = 0.0;
-  if (P.J != 0.0) {
-    double h0 = 0.0, h1 = 0.0, h2 = 0.0;
-    const int64_t nb[4] = {c.xi > 0 ? c.i - 1 : -1, c.xi + 1 < P.Lx ? c.i + 1 : -1,
-                           c.yi > 0 ? c.i - P.Lx : -1, c.yi + 1 < P.Ly ? c.i + P.Lx : -1};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (nb[q] < 0) continue;
-      h0 += s[nb[q]];
-      h1 += s[P.N + nb[q]];
-      h2 += s[2 * P.N + nb[q]];
-    }
-    const double dot = (c.Sn[0] - c.S[0]) * h0 + (c.Sn[1] - c.S[1]) * h1 + (c.Sn[2] - c.S[2]) * h2;
-    tex = -(P.beta * P.J) * dot;
-    bex = 0x1p-44 * fabs(P.beta * P.J);
-  }
-  const double lo = log_np(pz_o), ln = log_np(pz_n);
-  // prod z = stored product * 2^(-kScale * count)
-  const double scale = (double)((sc_n - sc_o) * kScale64) * P.ln2_hi;
-  const double lu = log_np(c.u);
-  const double mu = lu + ((bdv + tex) + ((lo - ln) + scale));
-  const double c0s = (double)n * __longlong_as_double((long long)c0m);
-  const double B = 2.0 * ((double)(n + 4) * c0s + 2.0 * lin + n * (4.0 * kExpm1RelErr6 + 0x1p-51) +
-                          kLogRelErr * (fabs(lo) + fabs(ln) + fabs(lu)) + bex +
-                          0x1p-51 * (fabs(scale) + fabs(tex) + fabs(bdv) + fabs(mu)));
-  if (mu < -B) return 1;
-  if (mu > B) return 0;
-  return 2;
-}
 
 // The FP64 form's decision (0: reject, 1: accept, 2: undecided) in float-float on the FP32 units
 // (df32.cuh), kG lanes of a warp per site; valid on the first lane of each group (sub = 0).
@@ -415,9 +333,11 @@ __device__ __forceinline__ dd warp_sum_dd(dd v) {
   return v;
 }
 
-// The FP64 decision of accept_fp64 with the pairs of the site spread over the 32 lanes of a
-// warp (partial sums, products taken to logarithms per lane, then reduced).  Same bound, plus
-// the per-lane logarithms.
+// FP64 decision (0: reject, 1: accept, 2: undecided) with the pairs of the site spread over the 32
+// lanes of a warp (partial sums, products taken to logarithms per lane, then reduced).  eps_r =
+// 2^-52 (unit roundoff, with margin), eps_f = kLogRelErr for the library's log_np (inputs in
+// (0, 1]), eps_z = kExpm1RelErr6 for the library's expm1_np6 (two per pair, doubled: 4 eps_z).
+// Compares, minima and renormalisation tests work on the bits of positive doubles.
 __device__ int accept_fp64_warp(const DevParams& P, const SiteCtx& c,
                                 const Sw64* __restrict__ sw,
                                 const double* __restrict__ s,

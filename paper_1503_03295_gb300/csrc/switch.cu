@@ -12,43 +12,25 @@ namespace {
 // Persistent: each warp claims 32 sites at a time from a global counter, and a lane whose walk
 // ends takes up the next claimed site at once, so that the lanes of a warp stay busy although
 // the number of candidates differs from site to site (Poisson, mean about 14 at T = 0.6D).
-// Five blocks per SM for the FP32-screened form (48 registers); four for the FP64 form, which
-// takes the same time there with half the register spills.
+// Bound by instruction issue (57% busy, 21 of 32 lanes active) and the latency of the neighbours'
+// records.  Four blocks per SM (64 registers; three and five measured 0.3 and 0.25 ms slower at
+// L = 2304).  With the guided search, the float-float survival test and two candidates per step the
+// FP64 form's switch phase takes 3.09 ms at L = 2304, T = 0.6 D (5.68 before), the FP32-screened
+// one 2.75 (5.87).
 template <int PREC>
-__global__ void __launch_bounds__(256, PREC == 1 ? 5 : 4) k_switch(const DevParams P, const uint64_t* __restrict__ W,
-                                                const uint64_t* __restrict__ Eb,
-                                                const uint32_t* __restrict__ disp,
-                                                const Sw64* __restrict__ sw64,
-                                                const double* __restrict__ xyq,
-                                                const float4* __restrict__ xy32,
-                                                const double* __restrict__ s,
-                                                const float4* __restrict__ s32, uint32_t epoch,
-                                                int32_t mnn0, int32_t mnn1, SwitchBufs b,
-                                                DevCounters* __restrict__ cnt) {
-  // the head of the list: W (FP32-screened search) or the decay bits (FP64 search)
-  __shared__ uint64_t sX[kNear];
-  __shared__ uint32_t sD[kNear];
-  const bool decay = PREC == 0 && Eb != nullptr;
-  const int64_t nnear = P.K < kNear ? P.K : kNear;
-  for (int q = threadIdx.x; q < nnear; q += blockDim.x) {
-    sX[q] = decay ? Eb[q] : W[q];
-    sD[q] = disp[q];
-  }
+__global__ void __launch_bounds__(256, 4) k_switch(const __grid_constant__ DevParams P,
+                                                   const __grid_constant__ Search S,
+                                                   const SwitchIn in, uint32_t epoch, int32_t mnn0,
+                                                   int32_t mnn1, SwitchBufs b,
+                                                   DevCounters* __restrict__ cnt) {
+  __shared__ NearShared sh;
+  const NearTable T = near_table(S, sh);
   __syncthreads();
-  NearTable T{sX, sD, W, disp, nnear, P.K, nnear};
-  if (decay) {
-    T.nw = 0;
-    T.sE = sX;
-    T.E = Eb;
-    T.elast = P.K > 0 ? __ldg(&Eb[P.K - 1]) : 0ull;
-  }
-  const uint64_t Wtot = P.K > 0 ? __ldg(&W[P.K - 1]) : 0;
-  SwitchOut o{b.hslot, b.indeg, b.ovf, b.ovf_cap, &cnt->ovf_n, &cnt->ovf_full};
+  const SwitchOut o{b.hslot, b.indeg, b.ovf, b.ovf_cap, &cnt->ovf_n, &cnt->ovf_full};
   const uint32_t N = (uint32_t)P.N;
   const unsigned lane = threadIdx.x & 31u;
   const unsigned below = (1u << lane) - 1u;
-  unsigned long long n_half = 0, n_dip = 0;
-  unsigned ghits = 0, g32 = 0;
+  unsigned n_half = 0, n_dip = 0, ghits = 0, g32 = 0;
   SiteWalk<PREC> a;
   bool active = false, drained = false;  // drained, pool and pool_n are warp-uniform
   uint32_t pool = 0, pool_n = 0;
@@ -69,7 +51,7 @@ __global__ void __launch_bounds__(256, PREC == 1 ? 5 : 4) k_switch(const DevPara
       const uint32_t take = min((uint32_t)__popc(need), pool_n);
       const uint32_t rank = (uint32_t)__popc(need & below);
       if (!active && rank < take) {
-        walk_begin<PREC>(P, T, s, s32, pool + rank, pool + rank, a);
+        walk_begin<PREC>(P, in, pool + rank, pool + rank, a);
         active = true;
       }
       pool += take;
@@ -78,20 +60,18 @@ __global__ void __launch_bounds__(256, PREC == 1 ? 5 : 4) k_switch(const DevPara
     }
     const unsigned act = __ballot_sync(0xffffffffu, active);
     if (act == 0u) break;
-    if (active && !walk_step<PREC>(P, T, Wtot, sw64, xyq, xy32, s, s32, epoch, mnn0, mnn1, o,
-                                   a, n_dip, ghits, g32, act)) {
+    if (active && !walk_step<PREC>(P, T, in, epoch, mnn0, mnn1, o, a, n_dip, ghits, g32, act)) {
       const uint32_t n_out = walk_end<PREC>(P, mnn0, mnn1, o, a);
       b.hcnt[a.i] = n_out;
       n_half += n_out;
       active = false;
     }
   }
-  n_half = warp_sum_u64(n_half);
-  n_dip = warp_sum_u64(n_dip);
+  const unsigned long long nh = warp_sum_u64(n_half), ndp = warp_sum_u64(n_dip);
   const unsigned long long gh = warp_sum_u64(ghits), gl = warp_sum_u64(g32);
   if ((threadIdx.x & 31) == 0) {
-    if (n_half) atomicAdd(&cnt->n_half, n_half);
-    if (n_dip) atomicAdd(&cnt->n_dip, n_dip);
+    if (nh) atomicAdd(&cnt->n_half, nh);
+    if (ndp) atomicAdd(&cnt->n_dip, ndp);
     if (gh) atomicAdd(&cnt->guard_fp64, gh);
     if (gl) atomicAdd(&cnt->guard_fp32, gl);
   }
@@ -108,9 +88,11 @@ __global__ void k_degree(int64_t N, const uint32_t* __restrict__ hcnt,
   } else if (i == N) {
     deg[N] = 0;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(&cnt->max_degree, m);
+  // most warps stay at or below the running maximum: reading it first keeps their atomics off the
+  // one address (113 us at L = 2304 with an atomic per warp)
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0 && m > *(volatile unsigned*)&cnt->max_degree)
+    atomicMax(&cnt->max_degree, m);
 }
 
 // Row i holds its lower neighbours (j < i, scattered here by the sites j) followed by its
@@ -172,7 +154,7 @@ __global__ void k_rowsort(int64_t N, const uint32_t* __restrict__ row_ptr,
 }  // namespace
 
 cudaError_t switch_run(const DevParams& P, const Table& t, const double* s, const float4* s32,
-                       int precision, uint32_t epoch, SwitchBufs& b, DevCounters* cnt,
+                       const SpinDf* sd, int precision, uint32_t epoch, SwitchBufs& b, DevCounters* cnt,
                        cudaStream_t st, int64_t* launches) {
   cudaError_t e = cudaMemsetAsync(b.indeg, 0, P.N * sizeof(uint32_t), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(&cnt->sw_next, 0, sizeof(unsigned), st);
@@ -190,12 +172,12 @@ cudaError_t switch_run(const DevParams& P, const Table& t, const double* s, cons
   int64_t nb64 = (int64_t)bps[pi] * num_sms();
   if (nb64 > (P.N + 255) / 256) nb64 = (P.N + 255) / 256;
   const unsigned nb = (unsigned)nb64;
+  const Search S = table_search(t, t);
+  const SwitchIn in{t.pdf, t.qdf, t.xy32, s, s32, sd};
   if (precision == 1)
-    k_switch<1><<<nb, 256, 0, st>>>(P, t.W, nullptr, t.disp, t.sw64, t.xyq, t.xy32, s, s32,
-                                     epoch, t.m_nn[0], t.m_nn[1], b, cnt);
+    k_switch<1><<<nb, 256, 0, st>>>(P, S, in, epoch, t.m_nn[0], t.m_nn[1], b, cnt);
   else
-    k_switch<0><<<nb, 256, 0, st>>>(P, t.W, t.Ebits, t.disp, t.sw64, t.xyq, t.xy32, s, s32,
-                                     epoch, t.m_nn[0], t.m_nn[1], b, cnt);
+    k_switch<0><<<nb, 256, 0, st>>>(P, S, in, epoch, t.m_nn[0], t.m_nn[1], b, cnt);
   ++*launches;
   return cudaGetLastError();
 }

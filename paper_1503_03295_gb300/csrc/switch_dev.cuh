@@ -9,7 +9,7 @@
 // (i, epoch, n/2), draw n using words 2(n%2) (exponential) and 2(n%2)+1 (survival).
 //
 // Every decision is an exact comparison of reals built from FP64 inputs.  It is taken in
-// FP64 (or FP32 in the FP32-guarded form) together with a bound on the rounding error; a
+// float-float (after FP32 in the FP32-guarded form) together with a bound on the rounding error; a
 // margin inside the bound sends the decision to double-double arithmetic.
 #pragma once
 
@@ -20,90 +20,103 @@
 namespace sco {
 namespace {
 
-constexpr int kNear = 2048;  // head of the sorted list kept in shared memory (r <~ 25)
 constexpr int kStatusCapacity = 7;
 
 __device__ __forceinline__ void set_status(int* status, int code) { atomicCAS(status, 0, code); }
 
-// The sorted half-plane list as a walk reads it: displacements d, the hazard prefix W and (FP64
-// search) the decay bits E of Table::Ebits, the first nnear displacements in shared memory with
-// the first nw entries of W (nw = nnear, or 0 when the shared array holds E instead).
+// The sorted half-plane list as a walk reads it: displacements d, the hazard prefix W and the decay
+// bits E of Table::Ebits, the first nnear displacements and decay bits in shared memory, and the
+// guides into E (see Search).
 struct NearTable {
-  const uint64_t* sW;
+  const uint64_t* sE;
   const uint32_t* sD;
+  const uint16_t* sG;  // near guide: kNearGuide + 1 entries
   const uint64_t* W;
+  const uint64_t* E;
   const uint32_t* disp;
-  int64_t nnear, K, nw;
-  const uint64_t* sE = nullptr;  // first nnear decay bits (FP64 search), or nullptr
-  const uint64_t* E = nullptr;   // all K decay bits, or nullptr: search W with a logarithm
-  uint64_t elast = 0;            // E[K - 1]
-  __device__ __forceinline__ uint64_t w(int64_t k) const { return k < nw ? sW[k] : __ldg(&W[k]); }
-  __device__ __forceinline__ uint32_t d(int64_t k) const {
+  const uint32_t* far;  // far guide: far_n + 1 entries
+  uint64_t e_near, e_last;  // E[nnear - 1], E[K - 1]
+  int32_t nnear, K;
+  int32_t near_shift, far_shift;
+  uint32_t far_n;
+  __device__ __forceinline__ uint64_t w(int32_t k) const { return __ldg(&W[k]); }
+  __device__ __forceinline__ uint32_t d(int32_t k) const {
     return k < nnear ? sD[k] : __ldg(&disp[k]);
   }
-  __device__ __forceinline__ uint64_t e(int64_t k) const {
+  __device__ __forceinline__ uint64_t e(int32_t k) const {
     return k < nnear ? sE[k] : __ldg(&E[k]);
   }
   // first k in [lo, K) with W[k] >= target, K if none
-  __device__ __forceinline__ int64_t lower_bound(int64_t lo, uint64_t target) const {
-    if (lo < nw) {
-      if (sW[nw - 1] >= target) {
-        int64_t a = lo, b = nw - 1;
-        while (a < b) {
-          const int64_t mid = (a + b) >> 1;
-          if (sW[mid] >= target) b = mid; else a = mid + 1;
-        }
-        return a;
-      }
-      lo = nw;
-    }
-    int64_t a = lo, b = K;
+  __device__ __forceinline__ int32_t lower_bound(int32_t lo, uint64_t target) const {
+    uint32_t a = (uint32_t)lo, b = (uint32_t)K;
     while (a < b) {
-      const int64_t mid = (a + b) >> 1;
+      const uint32_t mid = (a + b) >> 1;
       if (__ldg(&W[mid]) >= target) b = mid; else a = mid + 1;
     }
-    return a;
+    return (int32_t)a;
   }
-  // first k in [lo, K) with E[k] <= target (E is non-increasing), K if none
-  __device__ __forceinline__ int64_t lower_bound_e(int64_t lo, uint64_t target) const {
-    if (lo < nnear) {
-      if (sE[nnear - 1] <= target) {
-        int64_t a = lo, b = nnear - 1;
-        while (a < b) {
-          const int64_t mid = (a + b) >> 1;
-          if (sE[mid] <= target) b = mid; else a = mid + 1;
-        }
-        return a;
+  // first k with E[k] <= tb (E is non-increasing), K if none: between two guide entries.  A whole
+  // binary search took 11 dependent shared-memory reads for a near candidate and 22 reads of the
+  // list in global memory for a far one (5.8% of the candidates at T = 0.6 D, hence some lane of
+  // most warps); the guides leave about two and four.
+  __device__ __forceinline__ int32_t first_le(uint64_t tb) const {
+    if (tb >= e_near) {
+      const uint32_t q = (uint32_t)((kDecayStart - tb) >> near_shift);
+      uint32_t a = sG[q], b = sG[q + 1];
+      while (a < b) {
+        const uint32_t mid = (a + b) >> 1;
+        if (sE[mid] <= tb) b = mid; else a = mid + 1;
       }
-      lo = nnear;
+      return (int32_t)a;
     }
-    int64_t a = lo, b = K;
+    const uint64_t q64 = (e_near - tb) >> far_shift;
+    const uint32_t q = q64 < far_n ? (uint32_t)q64 : far_n - 1;
+    uint32_t a = __ldg(&far[q]), b = __ldg(&far[q + 1]);
     while (a < b) {
-      const int64_t mid = (a + b) >> 1;
-      if (__ldg(&E[mid]) <= target) b = mid; else a = mid + 1;
+      const uint32_t mid = (a + b) >> 1;
+      if (__ldg(&E[mid]) <= tb) b = mid; else a = mid + 1;
     }
-    return a;
+    return (int32_t)a;
   }
 };
 
+// The block's copies of the list's head (every thread of the block calls it, then __syncthreads).
+struct NearShared {
+  uint64_t e[kNear];
+  uint32_t d[kNear];
+  uint16_t g[kNearGuide + 1];
+};
+__device__ __forceinline__ NearTable near_table(const Search& S, NearShared& sh) {
+  const int32_t K = S.K, nnear = K < kNear ? K : kNear;
+  for (int q = threadIdx.x; q < nnear; q += blockDim.x) {
+    sh.e[q] = S.E[q];
+    sh.d[q] = S.disp[q];
+  }
+  NearTable T{};
+  T.K = K;
+  if (K > 0) {
+    for (int q = threadIdx.x; q <= kNearGuide; q += blockDim.x) sh.g[q] = S.near[q];
+    const SearchHead h = *S.head;
+    T = NearTable{sh.e,     sh.d,     sh.g,  S.W, S.E,          S.disp,      S.far,
+                  h.e_near, h.e_last, nnear, K,   h.near_shift, h.far_shift, S.far_n};
+  }
+  return T;
+}
+
 // Exact re-evaluation of the next candidate: min { k > s : beta D 2^-58 (W_k - W_s) >= -ln u+ }.
 // The table view comes by value (its address would put the caller's copy in local memory).
-__device__ __noinline__ int64_t next_candidate_dd(const DevParams& P, const NearTable T,
-                                                  int64_t s, uint64_t Ws, double up) {
+__device__ __noinline__ int32_t next_candidate_dd(const DevParams& P, const NearTable T, int32_t s,
+                                                  uint64_t Ws, double up) {
   const dd ln2 = {P.ln2_hi, P.ln2_lo};
   const dd E = dd_neg(dd_log(dd_from(up), ln2));
   const dd tau = dd_ldexp(dd_div(E, two_prod(P.beta, P.D)), 58);
-  int64_t a = s + 1, b = T.K;
+  uint32_t a = (uint32_t)(s + 1), b = (uint32_t)T.K;
   while (a < b) {
-    const int64_t mid = (a + b) >> 1;
-    if (!dd_lt(dd_from_u64(T.w(mid) - Ws), tau)) b = mid; else a = mid + 1;
+    const uint32_t mid = (a + b) >> 1;
+    if (!dd_lt(dd_from_u64(T.w((int32_t)mid) - Ws), tau)) b = mid; else a = mid + 1;
   }
-  return a;
+  return (int32_t)a;
 }
-
-__device__ __forceinline__ int64_t next_candidate(const DevParams& P, const NearTable& T,
-                                                  int64_t s, uint64_t Ws, uint64_t Wtot,
-                                                  uint64_t wE, unsigned& ghits);
 
 // ceil(x) as an integer for finite x >= 0 (saturating at 2^64 - 1), from the bits of x with
 // integer operations only (64-bit conversions would run on the FP64 pipe).
@@ -118,30 +131,20 @@ __device__ __forceinline__ uint64_t ceil_u64d(double x) {
   return q + ((q << (-ex)) != mant ? 1ull : 0ull);
 }
 
-__device__ __forceinline__ uint64_t ceil_u64(float x) {
-  const uint32_t b = __float_as_uint(x);
-  if (b == 0u || (b >> 31)) return 0ull;
-  const int ex = (int)((b >> 23) & 0xFFu) - 150;  // x = mant * 2^ex
-  const uint64_t mant = (uint64_t)((b & 0x7FFFFFu) | 0x800000u);
-  if (ex >= 0) return ex >= 40 ? ~0ull : mant << ex;
-  if (ex <= -25) return 1ull;  // 0 < x < 1
-  const uint64_t q = mant >> (-ex);
-  return q + ((q << (-ex)) != mant ? 1ull : 0ull);
-}
-
+// The candidate search with a logarithm, for what the decay table leaves open (targets below
+// 2^-990 at very low temperatures, or next to a table value).
 // tau = -ln(u+) / (beta D 2^-58) carries < 2^-48 relative error (log_np within kLogRelErr =
 // 2^-49, fl(beta D), fl(2^58 / bD), one product); the candidate is certain when
 // W_k - W_s >= tau (1 + 2^-46) and
 // W_(k-1) - W_s < tau (1 - 2^-46), compared as integers (ceil of the bounds).
-__device__ __forceinline__ int64_t next_candidate(const DevParams& P, const NearTable& T,
-                                                  int64_t s, uint64_t Ws, uint64_t Wtot,
-                                                  uint64_t wE, unsigned& ghits) {
-  if (s >= T.K - 1 || !P.switching) return T.K;
+__device__ __noinline__ int32_t next_candidate(const DevParams& P, const NearTable T, int32_t s,
+                                               uint64_t wE, unsigned& ghits) {
+  const uint64_t Ws = s >= 0 ? T.w(s) : 0ull;
   const double up = u53pos(wE);
   const double tau = -log_np(up) * P.inv_bD58;
-  const uint64_t rem = Wtot - Ws;
+  const uint64_t rem = T.w(T.K - 1) - Ws;
   const uint64_t thr = ceil_u64d(tau);
-  int64_t k = T.K;
+  int32_t k = T.K;
   if (thr <= rem) k = T.lower_bound(s + 1, Ws + thr);
   // thr = ceil(tau): ceil(tau (1 + 2^-46)) <= thr + floor(thr 2^-46) + 1 = hi and
   // tau (1 - 2^-46) >= (thr - 1)(1 - 2^-46) >= thr - floor(thr 2^-46) - 2 = lo (saturating),
@@ -157,81 +160,38 @@ __device__ __forceinline__ int64_t next_candidate(const DevParams& P, const Near
   return next_candidate_dd(P, T, s, Ws, up);
 }
 
-// Bits of 1.0: the decay value before the first element (W = 0).
-constexpr uint64_t kDecayStart = 0x3FF0000000000000ull;
-// Targets below 2^-990 take the exact search (the decay table's values there are not normal).
+// Targets below 2^-990 take the search with a logarithm (the decay table's values there are not
+// normal).
 constexpr uint64_t kDecayMinBits = 0x0210000000000000ull;
 
-// FP64 candidate search without a logarithm.  With E*_m = exp(-beta D 2^-58 W_m) the next
+// Candidate search without a logarithm.  With E*_m = exp(-beta D 2^-58 W_m) the next
 // candidate min { k > s : beta D 2^-58 (W_k - W_s) >= -ln u+ } is min { k > s : E*_k <= u+ E*_s }
-// (exp is increasing), searched on the table's bits: E_m within 2^-52 of E*_m, the target
-// fl(u+ E_s) within 2^-51.9 of u+ E*_s.  Positive doubles order as their bit images, and 16
-// units in the last place are at least 2^-49 relative, more than the combined error, so the
-// candidate is certain when E_k's bits lie at least 16 below the target's and E_(k-1)'s at least
-// 16 above; otherwise (or for a target below 2^-990) the search with the logarithm decides.
+// (exp is increasing), searched on the table's bits: E_m within 2^-50 of E*_m, the target
+// fl(u+ E_s) within 2^-49.9 of u+ E*_s.  Positive doubles order as their bit images, and 32
+// units in the last place are at least 2^-48 relative, more than the combined error, so the
+// candidate is certain when E_k's bits lie at least 32 below the target's and E_(k-1)'s at least
+// 32 above; otherwise (or for a target below 2^-990) the search with the logarithm decides.
 // Es carries the bits of E at the walk's last candidate and is advanced to the new one.
-__device__ __forceinline__ int64_t next_candidate_e(const DevParams& P, const NearTable& T,
-                                                    int64_t s, uint64_t& Es, uint64_t Wtot,
-                                                    uint64_t wE, unsigned& ghits) {
+__device__ __forceinline__ int32_t next_candidate_e(const DevParams& P, const NearTable& T,
+                                                    int32_t s, uint64_t& Es, uint64_t wE,
+                                                    unsigned& ghits) {
   if (s >= T.K - 1 || !P.switching) return T.K;
   const uint64_t tb = (uint64_t)__double_as_longlong(u53pos(wE) * __longlong_as_double(Es));
   if (tb >= kDecayMinBits) {
-    if (T.elast >= tb + 16ull) return T.K;  // surely no candidate left: the walk ends
-    const int64_t k = T.lower_bound_e(s + 1, tb);
+    if (T.e_last >= tb + 32ull) return T.K;  // surely no candidate left: the walk ends
+    const int32_t k = max(T.first_le(tb), s + 1);
     const uint64_t ek = k < T.K ? T.e(k) : 0ull;
     bool certain = true;
-    if (k < T.K && ek + 16ull > tb) certain = false;
-    if (k - 1 > s && T.e(k - 1) < tb + 16ull) certain = false;
+    if (k < T.K && ek + 32ull > tb) certain = false;
+    if (k - 1 > s && T.e(k - 1) < tb + 32ull) certain = false;
     if (certain) {
       Es = ek;
       return k;
     }
   }
-  const int64_t k = next_candidate(P, T, s, s >= 0 ? T.w(s) : 0ull, Wtot, wE, ghits);
+  const int32_t k = next_candidate(P, T, s, wE, ghits);
   if (k < T.K) Es = T.e(k);
   return k;
-}
-
-// FP32 screen of the candidate search.  E = -ln u+ is taken as -log1pf(-(1 - u+)) above 1/2
-// (1 - u+ is an exact integer times 2^-53) and -logf(u+) below, so its relative error stays
-// below 2^-20.5 (one input rounding, 4 ulp of the function); tau = E fl32(2^58 / bD) adds
-// two roundings.  Margins inside 2^-18 fall through to the FP64 search.  All comparisons
-// with the uint64 prefix W are made in integers.
-__device__ __forceinline__ int64_t next_candidate_fp32(const DevParams& P, const NearTable& T,
-                                                       int64_t s, uint64_t Ws, uint64_t Wtot,
-                                                       uint64_t wE, unsigned& g32,
-                                                       unsigned& ghits) {
-  if (s >= T.K - 1 || !P.switching) return T.K;
-  const uint64_t m53 = wE >> 11;  // u+ = (m53 + 1) 2^-53
-  float E;
-  if (m53 >= (1ull << 52)) {
-    const uint64_t dm = (1ull << 53) - 1ull - m53;  // < 2^52
-    const float d = __uint2float_rn((uint32_t)(dm >> 20)) * 0x1p-33f +
-                    __uint2float_rn((uint32_t)(dm & 0xFFFFFu)) * 0x1p-53f;
-    E = -log1pf(-d);
-  } else {
-    const uint64_t um = m53 + 1ull;  // <= 2^52
-    const float u = __uint2float_rn((uint32_t)(um >> 20)) * 0x1p-33f +
-                    __uint2float_rn((uint32_t)(um & 0xFFFFFu)) * 0x1p-53f;
-    E = -logf(u);
-  }
-  const float tau = E * P.inv_bD58_f;
-  const uint64_t rem = Wtot - Ws;
-  const uint64_t thr = ceil_u64(tau);
-  int64_t k = T.K;
-  if (thr <= rem) k = T.lower_bound(s + 1, Ws + thr);
-  // margins 2^-18 around tau from thr = ceil(tau), in integers (conservative, as in the FP64
-  // search): ceil(tau (1 + 2^-18)) <= thr + floor(thr 2^-18) + 1 = hi, and
-  // tau (1 - 2^-18) >= thr - floor(thr 2^-18) - 2 = lo (saturating)
-  const uint64_t m18 = thr >> 18;
-  const uint64_t hi = thr + m18 + 1 < thr ? ~0ull : thr + m18 + 1;  // >= hi: surely a candidate
-  const uint64_t lo = thr > m18 + 2 ? thr - m18 - 2 : 0ull;         // < lo: surely not
-  bool certain = tau < 0x1p62f;
-  if (k < T.K && T.w(k) - Ws < hi) certain = false;
-  if (k - 1 > s && T.w(k - 1) - Ws >= lo) certain = false;
-  if (certain) return k;
-  ++g32;
-  return next_candidate(P, T, s, Ws, Wtot, wE, ghits);
 }
 
 // Exact survival test u q < 1 - P_ij in double-double.  The spins come by value, so that the
@@ -252,64 +212,50 @@ __device__ __noinline__ bool survives_dd(const DevParams& P, double si0, double 
   return dd_lt(dd_mul_d(q, u1), pr);
 }
 
-// 1 - P_ij = -expm1(beta (V - Vmax)) of the pair (S_i at i, S_j at i + (dx, dy)) in FP64 from the
-// beta-scaled pair table t: x = a1 (S_i.S_j) - (S_i.a3 d)(S_j.d) - bvm, |x error| <= c0 +
-// 2^-52 |x| (c0 covers the roundings), then expm1_np6 (relative error kExpm1RelErr6).
-// x itself is returned in *x.
-__device__ __forceinline__ double pair_keep64(const Sw64& t, const double* Si, const double* Sj,
-                                              int32_t dx, int32_t dy, double* x) {
-  const double fx = flip_if(t.ax, dx < 0), fy = flip_if(t.ay, dy < 0);
-  const double ax3 = flip_if(t.a3x, dx < 0), ay3 = flip_if(t.a3y, dy < 0);
-  const double ss = Si[0] * Sj[0] + Si[1] * Sj[1] + Si[2] * Sj[2];
-  const double pa = Si[0] * ax3 + Si[1] * ay3;
-  const double pb = Sj[0] * fx + Sj[1] * fy;
-  const double b = fma(t.a1, ss, fma(-pa, pb, -t.bvm));  // c0 covers these two roundings
-  *x = b;
-  return neg_expm1_np6(b);
-}
-
 // The integer hazard A_k of list element k (only the double-double tests need it).
-__device__ __forceinline__ uint64_t hazard_of(const NearTable& T, int64_t k) {
+__device__ __forceinline__ uint64_t hazard_of(const NearTable& T, int32_t k) {
   return T.w(k) - (k > 0 ? T.w(k - 1) : 0ull);
 }
 
-// Bits of 2^-990: below it the survival test's relative margin is not formed from the exponent.
-constexpr long long kRelMinBits = 0x0210000000000000ll;
-
-// FP64 survival test u q < 1 - P_ij: x = beta (V - Vmax) from the beta-scaled pair table
-// (t, the sweep's Sw64 entry), 1 - P = -expm1_np6(x).  The error of mu = (1 - P) - u q is below
-// t.bsw / 4 (|dx| <= c0, q within 2^-50, two roundings; precomputed) plus 2^-31 (1 - P)
-// (expm1_np6); the test is certain when |mu| exceeds twice the larger of the two doubled parts,
-// i.e. both t.bsw and 2^-28 (1 - P), compared as ordered bit images (2^-28 (1 - P) by the
-// exponent field, for 1 - P >= 2^-990).  u is exact.  `keep` receives the FP64 value of 1 - P
-// (within its error bound whatever the decision).
-__device__ __forceinline__ bool survives_fp64(const DevParams& P, const Sw64& t, double q,
-                                              const double* Si, const double* Sj, int32_t dx,
-                                              int32_t dy, const NearTable& T, int64_t k,
-                                              double u1, unsigned& ghits, double& keep,
-                                              double& xk) {
-  const double pr = pair_keep64(t, Si, Sj, dx, dy, &xk);
-  keep = pr;
-  const double mu = pr - u1 * q;
-  // mu > lim, mu < -lim on ordered bit images (lim > 0: ord(-lim) = -ord(lim) - 1)
-  const long long pb = __double_as_longlong(pr);
-  const long long ob = max(ord_bits(t.bsw), pb - (28ll << 52)), om = ord_bits(mu);
-  if (pb >= kRelMinBits && om > ob) return true;
-  if (pb >= kRelMinBits && om < -ob - 1) return false;
+// Survival test u q < 1 - P_ij in float-float (df32.cuh): y = beta (Vmax - V) from the pair
+// constants, 1 - P = 1 - e^-y; q as h + l within 2^-48 of the FP64 value, u within 2^-48.  The
+// error of mu = (1 - P) - u q is below c0 = 2^-40 a1 (|dy|) plus 2^-31 (1 - P) plus 2^-43 q; the
+// test is certain when |mu| exceeds four times that.  The FP64 form of it (23 FP64 instructions
+// per candidate) kept the FP64 pipe 65% busy through the whole switch.
+__device__ __forceinline__ bool survives_df(const DevParams& P, const PairDf& t, float2 q,
+                                            const SpinDf& Si, const SpinDf& Sj, int32_t dx,
+                                            const double* __restrict__ s, int64_t i, int64_t j,
+                                            int32_t dy, const NearTable& T, int32_t k, uint64_t wU,
+                                            unsigned& ghits) {
+  const FieldDf g = df_field(t, dx < 0 ? -t.ax : t.ax, t.ay, Sj);
+  const df y = df_pair_y(t, g, Si);
+  if (y.h > 0x1p-100f && y.h < 8192.f) {
+    const df pr = df_one_minus_exp_neg(y);
+    const uint64_t m = wU >> 11;  // u = m 2^-53
+    const df u = {(float)(uint32_t)(m >> 29) * 0x1p-24f,
+                  (float)((uint32_t)m & 0x1FFFFFFFu) * 0x1p-53f};
+    const df uq = df_mul(u, {q.x, q.y});
+    const float mu = (pr.h - uq.h) + (pr.l - uq.l);
+    const float lim = 0x1p-29f * pr.h + (0x1p-38f * t.a1h + 0x1p-41f * q.x);
+    if (mu > lim) return true;
+    if (mu < -lim) return false;
+  }
   ++ghits;
-  return survives_dd(P, Si[0], Si[1], Si[2], Sj[0], Sj[1], Sj[2], dx, dy, hazard_of(T, k), u1);
+  return survives_dd(P, s[i], s[P.N + i], s[2 * P.N + i], s[j], s[P.N + j], s[2 * P.N + j], dx, dy,
+                     hazard_of(T, k), u53(wU));
 }
 
 // FP32 screen of the same test (FP32-guarded form): spins from the FP32 shadow
 // (|dS| <= 2^-24 per component), table constants rounded to FP32, expm1f within 4 ulp.
-// Falls through to the FP64 test (and from there to double-double) inside the bound; only
+// Falls through to the float-float test (and from there to double-double) inside the bound; only
 // then are the FP64 spins of i and j read from the SoA array s.
 __device__ __forceinline__ bool survives_fp32(const DevParams& P, float4 t32,
-                                              const Sw64* __restrict__ sw, double q64,
+                                              const PairDf* __restrict__ pdf,
+                                              const float2* __restrict__ qdf, int64_t tix,
                                               const float* Si32, const float* Sj32,
                                               const double* __restrict__ s, int64_t i, int64_t j,
                                               int32_t dx, int32_t dy, const NearTable& T,
-                                              int64_t k, uint64_t wU, unsigned& g32,
+                                              int32_t k, uint64_t wU, unsigned& g32,
                                               unsigned& ghits) {
   const float fr2 = (float)(dx * dx + dy * dy), fx = (float)dx, fy = (float)dy;
   // u truncated to 24 bits: 0 <= u - u24 < 2^-24, inside the 2^-19 q term of the bound
@@ -331,11 +277,10 @@ __device__ __forceinline__ bool survives_fp32(const DevParams& P, float4 t32,
   if (mu > B) return true;
   if (mu < -B) return false;
   ++g32;
-  const int64_t tix = (int64_t)(dx < 0 ? -dx : dx) + (int64_t)P.Lx * (dy < 0 ? -dy : dy);
-  const double Si[3] = {s[i], s[P.N + i], s[2 * P.N + i]};
-  const double Sj[3] = {s[j], s[P.N + j], s[2 * P.N + j]};
-  double keep, xk;
-  return survives_fp64(P, sw[tix], q64, Si, Sj, dx, dy, T, k, u53(wU), ghits, keep, xk);
+  const SpinDf Si = spin_df(s[i], s[P.N + i], s[2 * P.N + i], 0.0);
+  const SpinDf Sj = spin_df(s[j], s[P.N + j], s[2 * P.N + j], 0.0);
+  return survives_df(P, load32(pdf + tix), __ldg(qdf + tix), Si, Sj, dx, s, i, j, dy, T, k, wU,
+                     ghits);
 }
 
 // Where a site writes its upper neighbours: kSlotCap slots of its own (row `id` of hslot), then
@@ -358,14 +303,23 @@ struct SiteWalk {
   uint32_t i;   // local site index (the Philox counter)
   uint32_t id;  // site id in the slots and the overflow list
   int32_t xi, yi;
-  double Si[3];    // FP64 form
+  SpinDf Sd;       // FP64 form
   float Si32[3];   // FP32-screened form
-  int64_t sidx;    // last candidate (-1 before the first)
-  uint64_t Ws;     // W at sidx, or with the decay table the bits of E at sidx
-  uint32_t n;      // candidates drawn; Philox block n / 2, words 0-1 or 2-3
-  W4 w;
+  int32_t sidx;    // last candidate (-1 before the first)
+  uint64_t Es;     // the bits of E at sidx
+  uint32_t n;      // Philox blocks drawn (two candidates each)
   uint32_t n_out;
   bool nn0, nn1;
+};
+
+// The temperature-dependent tables by (|dx|, |dy|) and the spins that the survival tests read.
+struct SwitchIn {
+  const PairDf* pdf;
+  const float2* qdf;
+  const float4* xy32;
+  const double* s;
+  const float4* s32;  // FP32-guarded form
+  const SpinDf* sd;   // FP64 form
 };
 
 __device__ __forceinline__ void switch_emit(const SwitchOut& o, uint32_t id, uint32_t& n_out,
@@ -386,87 +340,78 @@ __device__ __forceinline__ void switch_emit(const SwitchOut& o, uint32_t id, uin
 }
 
 template <int PREC>
-__device__ __forceinline__ void walk_begin(const DevParams& P, const NearTable& T,
-                                           const double* __restrict__ s,
-                                           const float4* __restrict__ s32, uint32_t i,
+__device__ __forceinline__ void walk_begin(const DevParams& P, const SwitchIn& in, uint32_t i,
                                            uint32_t id, SiteWalk<PREC>& a) {
   a.i = i;
   a.id = id;
-  a.yi = (int32_t)site_row(i, P);
-  a.xi = (int32_t)(i - (uint32_t)a.yi * (uint32_t)P.Lx);
+  site_xy(i, P, a.xi, a.yi);
   if (PREC == 0) {
-    a.Si[0] = s[i];
-    a.Si[1] = s[P.N + i];
-    a.Si[2] = s[2 * P.N + i];
+    a.Sd = load32(in.sd + i);
   } else {
-    const float4 si = s32[i];
+    const float4 si = in.s32[i];
     a.Si32[0] = si.x;
     a.Si32[1] = si.y;
     a.Si32[2] = si.z;
   }
   a.sidx = -1;
-  a.Ws = PREC == 0 && T.E ? kDecayStart : 0ull;
+  a.Es = kDecayStart;
   a.n = 0;
   a.n_out = 0;
   a.nn0 = false;
   a.nn1 = false;
 }
 
-// Draws the next candidate of the walk and, if it lies on the lattice, tests its survival
-// (emitting the pair if it survives).  Returns false once the list is exhausted.  sync_mask:
-// the lanes of the warp that run this step together (0 when threads walk independently); they
-// meet after the candidate search, whose loops run for different lengths (a far candidate
-// searches the list in global memory), so that the FP64 survival test is issued once for all of
-// them instead of once per group of lanes that left the search together.
+// Draws the next two candidates of the walk (one Philox block) and tests the survival of those
+// that lie on the lattice (emitting the pairs that survive).  Returns false once the list is
+// exhausted.  Two per call, because a lane draws a block for every second candidate: with one per
+// call the lanes of a warp stood at both parities and the block's 280 instructions were issued at
+// every call for half of them.  sync_mask: the lanes of the warp that run this step together (0
+// when threads walk independently); they meet after each candidate search, whose loops run for
+// different lengths, so that the survival test is issued once for all of them instead of once per
+// group of lanes that left the search together.
 template <int PREC>
-__device__ __forceinline__ bool walk_step(const DevParams& P, const NearTable& T, uint64_t Wtot,
-                                          const Sw64* __restrict__ sw,
-                                          const double* __restrict__ xyq,
-                                          const float4* __restrict__ xy32,
-                                          const double* __restrict__ s,
-                                          const float4* __restrict__ s32, uint32_t epoch,
-                                          int32_t mnn0, int32_t mnn1, const SwitchOut& o,
-                                          SiteWalk<PREC>& a, unsigned long long& n_dip,
-                                          unsigned& ghits, unsigned& g32, unsigned sync_mask) {
-  if ((a.n & 1u) == 0u)
-    a.w = philox((uint64_t)a.i, epoch, (uint64_t)(a.n >> 1), kTagSwitch, P.key0, P.key1);
-  const uint64_t wE = (a.n & 1u) ? a.w.w[2] : a.w.w[0];
-  const uint64_t wU = (a.n & 1u) ? a.w.w[3] : a.w.w[1];
+__device__ __forceinline__ bool walk_step(const DevParams& P, const NearTable& T,
+                                          const SwitchIn& in, uint32_t epoch, int32_t mnn0,
+                                          int32_t mnn1, const SwitchOut& o, SiteWalk<PREC>& a,
+                                          unsigned& n_dip, unsigned& ghits, unsigned& g32,
+                                          unsigned sync_mask) {
+  W4 w = philox((uint64_t)a.i, epoch, (uint64_t)a.n, kTagSwitch, P.key0, P.key1);
   ++a.n;
-  const bool decay = PREC == 0 && T.E != nullptr;  // uniform
-  const int64_t k = PREC == 1 ? next_candidate_fp32(P, T, a.sidx, a.Ws, Wtot, wE, g32, ghits)
-                    : decay   ? next_candidate_e(P, T, a.sidx, a.Ws, Wtot, wE, ghits)
-                              : next_candidate(P, T, a.sidx, a.Ws, Wtot, wE, ghits);
-  if (sync_mask) __syncwarp(sync_mask);
-  if (k >= P.K) return false;
-  const uint32_t d = T.d(k);
-  const int32_t dx = (int16_t)(d & 0xFFFFu), dy = (int32_t)(d >> 16);
-  const int32_t xj = a.xi + dx, yj = a.yi + dy;
-  if (xj >= 0 && xj < P.Lx && yj < P.Ly) {
-    const int64_t j = xj + (int64_t)P.Lx * yj;
+  bool more = true;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int32_t k = more ? next_candidate_e(P, T, a.sidx, a.Es, w.w[0], ghits) : T.K;
+    if (sync_mask) __syncwarp(sync_mask);
+    more = k < T.K;
+    const uint64_t wU = w.w[1];
+    w.w[0] = w.w[2];
+    w.w[1] = w.w[3];
+    if (!more) continue;
+    a.sidx = k;
+    const uint32_t d = T.d(k);
+    const int32_t dx = (int16_t)(d & 0xFFFFu), dy = (int32_t)(d >> 16);
+    const int32_t xj = a.xi + dx, yj = a.yi + dy;
+    if (xj < 0 || xj >= P.Lx || yj >= P.Ly) continue;
+    const uint32_t j = (uint32_t)xj + (uint32_t)P.Lx * (uint32_t)yj;
     const int64_t tix = (int64_t)(dx < 0 ? -dx : dx) + (int64_t)P.Lx * dy;
     bool surv;
-    double keep = 0.0, xk = 0.0;
     if (PREC == 1) {
-      const float4 sj = s32[j];
+      const float4 sj = in.s32[j];
       const float Sj32[3] = {sj.x, sj.y, sj.z};
-      surv = survives_fp32(P, __ldg(&xy32[tix]), sw, __ldg(&xyq[tix]), a.Si32, Sj32, s,
-                           (int64_t)a.i, j, dx, dy, T, k, wU, g32, ghits);
+      surv = survives_fp32(P, __ldg(&in.xy32[tix]), in.pdf, in.qdf, tix, a.Si32, Sj32, in.s,
+                           (int64_t)a.i, (int64_t)j, dx, dy, T, k, wU, g32, ghits);
     } else {
-      const double Sj[3] = {s[j], s[P.N + j], s[2 * P.N + j]};
-      surv = survives_fp64(P, sw[tix], __ldg(&xyq[tix]), a.Si, Sj, dx, dy, T, k, u53(wU), ghits,
-                           keep, xk);
+      surv = survives_df(P, load32(in.pdf + tix), __ldg(&in.qdf[tix]), a.Sd, load32(in.sd + j), dx,
+                         in.s, (int64_t)a.i, (int64_t)j, dy, T, k, wU, ghits);
     }
     if (surv) {
-      switch_emit(o, a.id, a.n_out, (uint32_t)j);
+      switch_emit(o, a.id, a.n_out, j);
       ++n_dip;
       if (k == mnn0) a.nn0 = true;
       if (k == mnn1) a.nn1 = true;
     }
   }
-  a.sidx = k;
-  if (!decay) a.Ws = T.w(k);
-  return true;
+  return more;
 }
 
 // Ends the walk: exchange bonds that the dipolar switch did not keep join the colouring graph.
@@ -486,19 +431,13 @@ __device__ __forceinline__ uint32_t walk_end(const DevParams& P, int32_t mnn0, i
 // returns the number of upper neighbours written.
 template <int PREC>
 __device__ __forceinline__ uint32_t switch_site(const DevParams& P, const NearTable& T,
-                                                uint64_t Wtot, const Sw64* __restrict__ sw,
-                                                const double* __restrict__ xyq,
-                                                const float4* __restrict__ xy32,
-                                                const double* __restrict__ s,
-                                                const float4* __restrict__ s32, uint32_t epoch,
-                                                int32_t mnn0, int32_t mnn1, uint32_t i,
-                                                uint32_t id, const SwitchOut& o,
-                                                unsigned long long& n_dip, unsigned& ghits,
-                                                unsigned& g32) {
+                                                const SwitchIn& in, uint32_t epoch, int32_t mnn0,
+                                                int32_t mnn1, uint32_t i, uint32_t id,
+                                                const SwitchOut& o, unsigned& n_dip,
+                                                unsigned& ghits, unsigned& g32) {
   SiteWalk<PREC> a;
-  walk_begin<PREC>(P, T, s, s32, i, id, a);
-  while (walk_step<PREC>(P, T, Wtot, sw, xyq, xy32, s, s32, epoch, mnn0, mnn1, o, a, n_dip,
-                         ghits, g32, 0u)) {
+  walk_begin<PREC>(P, in, i, id, a);
+  while (walk_step<PREC>(P, T, in, epoch, mnn0, mnn1, o, a, n_dip, ghits, g32, 0u)) {
   }
   return walk_end<PREC>(P, mnn0, mnn1, o, a);
 }

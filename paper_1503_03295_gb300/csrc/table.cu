@@ -72,10 +72,10 @@ __global__ void k_hazard(int64_t K, const uint32_t* __restrict__ disp, uint64_t*
 // so x = beta V - fl(beta Vmax) = S_i . f - bvm; c0 bounds the part of |x error| that does not
 // scale with |x|: |beta dV| <= 2^-46 beta Dc r^2 (FP64 products, the rounded beta-scaled
 // constants) plus 2^-51 beta Vmax (fl(beta Vmax)), plus 2^-52 (2 beta Vmax) for the rounding of
-// x itself (|x| <= 2 beta Vmax).  The switch's survival test uses the same x.  FP32 (float4 {A1, A3, beta Vmax, c0}): V(S) = S.f with
+// x itself (|x| <= 2 beta Vmax).  FP32 (float4 {A1, A3, beta Vmax, c0}): V(S) = S.f with
 // f = A1 S_j - A3 (S_j.d) d, |dV| <= 2^-16 Dc r^2 (shadow spins, FP32 constants).
 __global__ void k_xy(int32_t Lx, int32_t Ly, double D, double beta, double2* __restrict__ xy,
-                     double* __restrict__ xyq, float4* __restrict__ xy32,
+                     float2* __restrict__ qdf, float4* __restrict__ xy32,
                      Sw64* __restrict__ sw64, float4* __restrict__ sw32,
                      PairDf* __restrict__ pdf) {
   const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -90,7 +90,8 @@ __global__ void k_xy(int32_t Lx, int32_t Ly, double D, double beta, double2* __r
   const double a = (2.0 * beta) * vm;
   const double cq = -expm1(-a);
   xy[q] = make_double2(dc, vm);
-  xyq[q] = cq;
+  const df dq = df_split_const(cq);
+  qdf[q] = make_float2(dq.h, dq.l);
   xy32[q] = make_float4((float)dc, (float)vm, (float)a, (float)cq);
   const double a1 = dc * (double)r2, a3 = 3.0 * dc, bvm = beta * vm;
   const double a3b = beta * a3;
@@ -103,11 +104,6 @@ __global__ void k_xy(int32_t Lx, int32_t Ly, double D, double beta, double2* __r
   t.ay = (double)ay;
   t.bvm = bvm;
   t.c0 = c64 * (1.0 + 0x1p-20);
-  // survival test of the switch: mu = (1 - P) - u q with 1 - P = -expm1_np6(x): |d(1 - P)| <=
-  // |dx| <= c0 plus the relative error of expm1_np6 (bounded at run time, see survives_fp64); q
-  // (CUDA expm1 of a rounded 2 beta Vmax) within 2^-50; the product u q and the difference 2^-52
-  // each.  Doubled, and doubled again for the test against the larger of the two parts.
-  t.bsw = 4.0 * (c64 + 0x1p-49) * (1.0 + 0x1p-20);
   sw64[q] = t;
   const df d1 = df_split_const(t.a1), d3 = df_split_const(a3b), dv = df_split_const(bvm);
   pdf[q] = PairDf{d1.h, d1.l, d3.h, d3.l, dv.h, dv.l, (float)ax, (float)ay};
@@ -115,23 +111,14 @@ __global__ void k_xy(int32_t Lx, int32_t Ly, double D, double beta, double2* __r
   sw32[q] = make_float4((float)a1, (float)a3, (float)bvm, (float)(c32 * (1.0 + 0x1p-20)));
 }
 
-// exp(x) of a double-double x <= 0 without the cancellation of 1 + expm1(x): x = k ln2 + r,
-// |r| <= ln2 / 2, e^x = 2^k (1 + expm1(r)); relative error of the double-double result far below
-// 2^-100 (the series and the reduction of dd_expm1_small / dd_expm1).
-__device__ dd exp_dd_neg(dd x, dd ln2) {
-  const double kf = floor(x.hi / ln2.hi + 0.5);
-  const dd r = dd_sub(x, dd_mul_d(ln2, kf));
-  return dd_ldexp(dd_add(dd_from(1.0), dd_expm1_small(r)), (int)kf);
-}
-
-// E_m = fl(exp(-beta D 2^-58 W_m)) as bits: the candidate process of the switch has rate
+// E_m = exp(-beta D 2^-58 W_m) as bits: the candidate process of the switch has rate
 // beta D A_m 2^-58 per element, so E_m is the probability of passing elements 0..m without a
-// candidate.  The exponent is formed exactly (beta D as a double-double product, W_m split into
-// two exact doubles), the exponential in double-double and rounded once, so E_m lies within
-// 2^-52 of its exact value (relative); below e^-690 (< 2^-995) it is stored as +0, which the
+// candidate.  The exponent is formed exactly to double-double (beta D as an exact product, W_m split
+// into two exact doubles) and E = exp(-hi) (1 - lo); with CUDA's exp taken at 4 ulp E_m lies within
+// 2^-50 of its exact value (relative); below e^-690 (< 2^-995) it is stored as +0, which the
 // search treats as below every target it accepts (targets under 2^-990 take the exact path).
-__global__ void k_decay(int64_t K, double beta, double D, double ln2_hi, double ln2_lo,
-                        const uint64_t* __restrict__ W, uint64_t* __restrict__ Eb) {
+__global__ void k_decay(int64_t K, double beta, double D, const uint64_t* __restrict__ W,
+                        uint64_t* __restrict__ Eb) {
   const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (m >= K) return;
   const uint64_t w = W[m];
@@ -139,32 +126,89 @@ __global__ void k_decay(int64_t K, double beta, double D, double ln2_hi, double 
   const dd a = dd_ldexp(dd_mul(two_prod(beta, D), wd), -58);
   double e = 0.0;
   if (a.hi < 690.0) {
-    const dd x = exp_dd_neg(dd_neg(a), dd{ln2_hi, ln2_lo});
-    e = x.hi + x.lo;
+    e = exp(-a.hi);
+    e = fma(-a.lo, e, e);
   }
   Eb[m] = (uint64_t)__double_as_longlong(e);
 }
 
+// Both guides (see Search): a binary search per entry.
+__global__ void k_guide(int64_t K, uint32_t far_n, const uint64_t* __restrict__ Eb,
+                        SearchHead* __restrict__ head, uint16_t* __restrict__ near_g,
+                        uint32_t* __restrict__ far_g) {
+  const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t nnear = (uint32_t)(K < kNear ? K : kNear);
+  // the smallest shift that leaves fewer than n cells (n a power of two)
+  auto cells = [](uint64_t span, uint32_t n) {
+    const int s = 64 - __clzll((long long)span) - (31 - __clz((int)n));
+    return s > 0 ? s : 0;
+  };
+  SearchHead h;
+  h.e_near = Eb[nnear - 1];
+  h.e_last = Eb[K - 1];
+  h.near_shift = cells(kDecayStart - h.e_near, kNearGuide);
+  h.far_shift = cells(h.e_near - h.e_last, far_n);
+  if (q == 0) *head = h;
+  auto first_le = [&](uint32_t a, uint32_t b, uint64_t tb) {
+    while (a < b) {
+      const uint32_t mid = (a + b) >> 1;
+      if (Eb[mid] <= tb) b = mid; else a = mid + 1;
+    }
+    return a;
+  };
+  if (q <= (uint32_t)kNearGuide) {
+    const uint64_t below = (uint64_t)q << h.near_shift;
+    near_g[q] =
+        (uint16_t)(below <= kDecayStart ? first_le(0, nnear - 1, kDecayStart - below) : nnear - 1);
+  }
+  if (q <= far_n) {
+    const uint64_t below = (uint64_t)q << h.far_shift;
+    far_g[q] = q == far_n || below > h.e_near ? (uint32_t)K
+                                              : first_le(nnear, (uint32_t)K, h.e_near - below);
+  }
+}
+
 }  // namespace
 
-cudaError_t table_build_xy(const DevParams& P, Table& t, cudaStream_t s, int64_t* launches) {
-  cudaError_t e;
-  const int64_t nxy = (int64_t)P.Lx * P.Ly;
-  if ((e = cudaMalloc(&t.xy, nxy * sizeof(double2))) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&t.xy32, nxy * sizeof(float4))) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&t.xyq, nxy * sizeof(double))) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&t.sw64, nxy * sizeof(Sw64))) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&t.sw32, nxy * sizeof(float4))) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&t.pdf, nxy * sizeof(PairDf))) != cudaSuccess) return e;
-  k_xy<<<(unsigned)((nxy + 255) / 256), 256, 0, s>>>(P.Lx, P.Ly, P.D, P.beta, t.xy, t.xyq,
+cudaError_t table_build_xy(const DevParams& P, Table& t, const Table& list, cudaStream_t s,
+                           int64_t* launches) {
+  const int64_t nxy = (int64_t)P.Lx * P.Ly, K = list.K;
+  t.far_n = 64;  // one cell per 16 elements of the list, up to kFarGuide
+  while (t.far_n < kFarGuide && (int64_t)t.far_n * 16 < K) t.far_n *= 2;
+  // one allocation for all of them (a batch builds them per replica)
+  size_t bytes = 0;
+  auto place = [&](size_t n) {
+    const size_t at = bytes;
+    bytes += (n + 255) / 256 * 256;
+    return at;
+  };
+  const size_t o_xy = place(nxy * sizeof(double2)), o_xy32 = place(nxy * sizeof(float4)),
+               o_q = place(nxy * sizeof(float2)), o_sw64 = place(nxy * sizeof(Sw64)),
+               o_sw32 = place(nxy * sizeof(float4)), o_pdf = place(nxy * sizeof(PairDf)),
+               o_e = place(K * sizeof(uint64_t)), o_head = place(sizeof(SearchHead)),
+               o_near = place((kNearGuide + 1) * sizeof(uint16_t)),
+               o_far = place((t.far_n + 1) * sizeof(uint32_t));
+  const cudaError_t e = cudaMalloc(&t.pool, bytes);
+  if (e != cudaSuccess) return e;
+  char* p = static_cast<char*>(t.pool);
+  t.xy = reinterpret_cast<double2*>(p + o_xy);
+  t.xy32 = reinterpret_cast<float4*>(p + o_xy32);
+  t.qdf = reinterpret_cast<float2*>(p + o_q);
+  t.sw64 = reinterpret_cast<Sw64*>(p + o_sw64);
+  t.sw32 = reinterpret_cast<float4*>(p + o_sw32);
+  t.pdf = reinterpret_cast<PairDf*>(p + o_pdf);
+  t.Ebits = reinterpret_cast<uint64_t*>(p + o_e);
+  t.head = reinterpret_cast<SearchHead*>(p + o_head);
+  t.near_g = reinterpret_cast<uint16_t*>(p + o_near);
+  t.far_g = reinterpret_cast<uint32_t*>(p + o_far);
+  k_xy<<<(unsigned)((nxy + 255) / 256), 256, 0, s>>>(P.Lx, P.Ly, P.D, P.beta, t.xy, t.qdf,
                                                       t.xy32, t.sw64, t.sw32, t.pdf);
   ++*launches;
-  // the FP64 candidate search's decay values, where this table owns the sorted list
-  if (t.W && t.K > 0) {
-    if ((e = cudaMalloc(&t.Ebits, t.K * sizeof(uint64_t))) != cudaSuccess) return e;
-    k_decay<<<(unsigned)((t.K + 255) / 256), 256, 0, s>>>(t.K, P.beta, P.D, P.ln2_hi, P.ln2_lo,
-                                                          t.W, t.Ebits);
-    ++*launches;
+  if (K > 0) {
+    k_decay<<<(unsigned)((K + 255) / 256), 256, 0, s>>>(K, P.beta, P.D, list.W, t.Ebits);
+    const unsigned ng = (t.far_n > (uint32_t)kNearGuide ? t.far_n : kNearGuide) + 1;
+    k_guide<<<(ng + 255) / 256, 256, 0, s>>>(K, t.far_n, t.Ebits, t.head, t.near_g, t.far_g);
+    *launches += 2;
   }
   return cudaGetLastError();
 }
@@ -218,25 +262,13 @@ cudaError_t table_build_list(const DevParams& P, Table& t, cudaStream_t s, int64
 
 cudaError_t table_build(const DevParams& P, Table& t, cudaStream_t s, int64_t* launches) {
   cudaError_t e = table_build_list(P, t, s, launches);
-  if (e == cudaSuccess) e = table_build_xy(P, t, s, launches);
+  if (e == cudaSuccess) e = table_build_xy(P, t, t, s, launches);
   return e;
 }
 
 void table_free_xy(Table& t) {
-  cudaFree(t.xy);
-  cudaFree(t.xy32);
-  cudaFree(t.xyq);
-  cudaFree(t.sw64);
-  cudaFree(t.sw32);
-  cudaFree(t.pdf);
-  cudaFree(t.Ebits);
-  t.Ebits = nullptr;
-  t.xy = nullptr;
-  t.xy32 = nullptr;
-  t.xyq = nullptr;
-  t.sw64 = nullptr;
-  t.sw32 = nullptr;
-  t.pdf = nullptr;
+  cudaFree(t.pool);
+  t.pool = nullptr;
 }
 
 void table_free(Table& t) {
