@@ -231,11 +231,13 @@ typedef struct {
   int32_t sweep_blocks_per_sm; /* resident blocks per SM of the persistent sweep, >= 1 */
   int32_t kw_blocks_per_sm;    /* resident blocks per SM of the KW level kernel, >= 1 */
   int32_t use_graph;           /* 1: capture and replay graphs; 0: launch directly */
-  int32_t kw_schedule;         /* 0: all KW levels in one kernel, vertices bucketed by colour
-                                  and reduced largest colour first (order of Sec. 2.3.2 (2));
-                                  1: one kernel per level, each vertex recolours as soon as
-                                  its larger neighbours are done (2)'.  Same colours. */
-  int32_t kw_low;              /* first KW levels, while a group has at most kw_low_group vertices
+  int32_t kw_schedule;         /* 0: all KW levels in one kernel, each vertex recolouring as
+                                  soon as its larger neighbours are done (2)' while every
+                                  palette has at most 63 colours, else the vertices bucketed
+                                  by colour, largest first (order of Sec. 2.3.2 (2)); 1: one
+                                  kernel per level.  Same colours. */
+  int32_t kw_low;              /* where the dataflow kernel of schedule 0 does not run: the
+                                  first KW levels, while a group has at most kw_low_group vertices
                                   and g <= 64: 1: one block per group, internal edges staged
                                   in shared memory (rows when they do not fit); 2: one block
                                   per group, rows read at every level; 0: by the level

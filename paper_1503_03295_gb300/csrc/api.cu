@@ -194,7 +194,7 @@ cudaError_t grow(T*& ptr, uint64_t& cap, uint64_t need) {
   cudaFree(ptr);
   ptr = nullptr;
   cap = 0;
-  cudaError_t e = cudaMalloc(&ptr, ncap * sizeof(T));
+  cudaError_t e = cudaMalloc(&ptr, ncap * sizeof(T) + 32);  // rows are read by 32-byte sectors
   if (e == cudaSuccess) cap = ncap;
   return e;
 }

@@ -20,6 +20,7 @@
 #include "grid_dev.cuh"
 #include "kw_bcr.cuh"
 #include "kw_dev.cuh"
+#include "kw_flow.cuh"
 #include "sweep_dev.cuh"
 #include "switch_dev.cuh"
 
@@ -204,7 +205,9 @@ __global__ void __launch_bounds__(256) kb_rowsort(const BatchDev B) {
 
 // ---- step (2): colouring and classes ----------------------------------------------------
 
-__global__ void __launch_bounds__(256) kb_kw_init(const BatchDev B) {
+// Initial colours, in the words of the kernel that will run (flow: the dataflow kernel if every
+// palette allows it).
+__global__ void __launch_bounds__(256) kb_kw_init(const BatchDev B, int flow) {
   if (block_halted(B)) return;
   const int r = block_replica(B);
   const uint32_t base = B.site_start[r], N = B.site_start[r + 1] - base;
@@ -212,6 +215,10 @@ __global__ void __launch_bounds__(256) kb_kw_init(const BatchDev B) {
   if (i >= N) return;
   const RepPlan pl = B.plan[r];
   const uint32_t c = i - fdiv(i, pl.magic) * pl.g;
+  if (flow && B.ctl->gmax <= kFlowMaxPal) {
+    reinterpret_cast<uint32_t*>(B.word)[base + i] = c;
+    return;
+  }
   B.word[base + i] = pack(0, 0, c);
   B.col8[base + i] = (uint8_t)c;
   B.blk[base + i] = kNone;
@@ -361,7 +368,7 @@ __global__ void __launch_bounds__(256, 4) kb_kw_level(const BatchDev B, unsigned
 }
 
 // Final colours, and the colours in use per replica (bit sets).
-__global__ void __launch_bounds__(256) kb_kw_final(const BatchDev B) {
+__global__ void __launch_bounds__(256) kb_kw_final(const BatchDev B, int flow) {
   if (block_halted(B)) return;
   extern __shared__ uint32_t ubits[];
   const uint32_t nw = B.pal_cap / 32;
@@ -371,7 +378,9 @@ __global__ void __launch_bounds__(256) kb_kw_final(const BatchDev B) {
   const uint32_t base = B.site_start[r], N = B.site_start[r + 1] - base;
   const uint32_t i = (blockIdx.x - B.blk_start[r]) * kBatchBlock + threadIdx.x;
   if (i < N) {
-    const uint32_t c = (uint32_t)(B.word[base + i] & kColMask);
+    const uint32_t c = flow && B.ctl->gmax <= kFlowMaxPal
+                           ? reinterpret_cast<const uint32_t*>(B.word)[base + i] & 63u
+                           : (uint32_t)(B.word[base + i] & kColMask);
     B.colour[base + i] = c;
     if (c < B.pal_cap) atomicOr(&ubits[c >> 5], 1u << (c & 31));
   }
@@ -671,8 +680,35 @@ cudaError_t batch_colour(const BatchDev& B, const BatchLaunch& L, cudaStream_t s
   const size_t nw = B.pal_cap / 32;
   if ((e = cudaMemsetAsync(B.used, 0, (size_t)B.R * nw * sizeof(uint32_t), st)) != cudaSuccess)
     return e;
-  kb_kw_init<<<B.nblocks, kBatchBlock, 0, st>>>(B);
+  FlowShape shape;
+  const bool flow = L.flow && L.kw_schedule == 0 && L.levels < kFlowMaxLevels &&
+                    flow_shape(B.R, B.Ntot, &shape, &e);
+  if (L.flow && e != cudaSuccess) return e;
+  kb_kw_init<<<B.nblocks, kBatchBlock, 0, st>>>(B, flow ? 1 : 0);
   ++*L.launches;
+  if (flow) {
+    FlowView F{};
+    F.R = B.R;
+    F.site_start = B.site_start;
+    F.plan = B.plan;
+    F.row_ptr = B.row_ptr;
+    F.col = B.col;
+    F.word = reinterpret_cast<uint32_t*>(B.word);
+    F.lev_rounds = B.cnt->lev_rounds;
+    F.lev_stride = sizeof(DevCounters) / sizeof(unsigned);
+    F.bar = B.ctl->bar;
+    F.status = &B.ctl->status;
+    F.halt = &B.ctl->flag;
+    F.gmax = &B.ctl->gmax;
+    F.levels = L.levels;
+    F.cap = shape.cap;
+    F.min_tile = kFlowMinTile;
+    F.ns_limit = B.ns_limit;
+    F.vec = kFlowVecAll;
+    if ((e = flow_launch(F, shape, st)) != cudaSuccess) return e;
+    ++*L.launches;
+  }
+  const unsigned* skip = flow ? &B.ctl->gmax : nullptr;
   const uint32_t low_gmax = L.kw_low != 0 ? L.low_gmax : 0u;
   if (low_gmax) {
     KwLowView W{};
@@ -685,6 +721,7 @@ cudaError_t batch_colour(const BatchDev& B, const BatchLaunch& L, cudaStream_t s
     W.col8 = B.col8;
     W.cnt = B.cnt;
     W.halt = &B.ctl->flag;
+    W.flow = skip;
     W.gmax = low_gmax;
     W.gcap = low_gmax;
     W.ecap = L.low_ecap;
@@ -710,6 +747,7 @@ cudaError_t batch_colour(const BatchDev& B, const BatchLaunch& L, cudaStream_t s
     V.bar = B.ctl->bar;
     V.status = &B.ctl->status;
     V.halt = &B.ctl->flag;
+    V.flow = skip;
     V.pal = B.pal_cap;
     V.levels = L.levels;
     V.ns_limit = B.ns_limit;
@@ -730,7 +768,7 @@ cudaError_t batch_colour(const BatchDev& B, const BatchLaunch& L, cudaStream_t s
       ++*L.launches;
     }
   }
-  kb_kw_final<<<B.nblocks, kBatchBlock, nw * sizeof(uint32_t), st>>>(B);
+  kb_kw_final<<<B.nblocks, kBatchBlock, nw * sizeof(uint32_t), st>>>(B, flow ? 1 : 0);
   kb_colour_stats<<<1, 1024, 0, st>>>(B);
   kb_tile_hist<<<B.ntiles, 256, (size_t)B.pal_cap * sizeof(uint32_t), st>>>(B);
   *L.launches += 3;

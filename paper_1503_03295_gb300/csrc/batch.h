@@ -34,6 +34,9 @@ struct RepDesc {
   int32_t variant;     // colouring variant (reported t_R only)
 };
 
+// Palettes up to this size are coloured by the dataflow kernel (kw_flow.cuh).
+constexpr uint32_t kFlowMaxPal = 63;
+
 // Larger right-half neighbours listed per bucketed vertex of the KW colouring (records).
 constexpr int kKwItemList = 32;
 
@@ -122,6 +125,7 @@ struct BatchLaunch {
   uint32_t low_ecap;  // its staged-edge capacity per group
   int kw_grid;     // blocks of the persistent KW kernel(s)
   int sweep_grid;  // blocks of the persistent sweep kernel
+  int flow;        // schedule 0: palettes up to kFlowMaxPal by the dataflow kernel
   unsigned levels;  // KW level launches per colouring (>= every replica's M)
   uint64_t* scan_tmp;
   int64_t* launches;

@@ -144,6 +144,7 @@ cudaError_t alloc_palette(sco_batch* b, uint32_t pal) {
 void set_grids(sco_batch* b) {
   const int sms = num_sms();
   b->L.kw_schedule = b->tune.kw_schedule;
+  b->L.flow = 1;
   b->L.kw_low = b->tune.kw_low;
   b->L.low_gmax = (uint32_t)b->tune.kw_low_group;
   if (batch_low_setup(b->R, b->L.low_gmax, &b->low_occ, &b->low_ecap) != cudaSuccess) {
@@ -222,7 +223,7 @@ sco_status replan(sco_batch* b) {
     if (cap > 0xFFFFFFFFull) cap = 0xFFFFFFFFull;
     cudaFree(B.col);
     B.col = nullptr;
-    SCO_TRY(cudaMalloc(&B.col, cap * sizeof(uint32_t)));
+    SCO_TRY(cudaMalloc(&B.col, cap * sizeof(uint32_t) + 32));
     B.col_cap = cap;
   }
   if (h.flag & kReplanOvf) {
@@ -429,7 +430,7 @@ sco_status sco_batch_init(const sco_params* p, int32_t n, void* stream, sco_batc
   A(&B.ovf, 2 * (size_t)B.ovf_cap * sizeof(uint32_t));
   A(&B.row_ptr, (N + 1) * sizeof(uint32_t));
   B.col_cap = (unsigned long long)N * 24 + 1024;
-  A(&B.col, B.col_cap * sizeof(uint32_t));
+  A(&B.col, B.col_cap * sizeof(uint32_t) + 32);  // rows are read by 32-byte sectors
   A(&B.word, N * sizeof(unsigned long long));
   A(&B.col8, N);
   A(&B.blk, N * sizeof(uint32_t));

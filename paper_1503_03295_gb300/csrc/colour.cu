@@ -21,6 +21,7 @@
 
 #include "kw_bcr.cuh"
 #include "kw_dev.cuh"
+#include "kw_flow.cuh"
 #include "kw_low.cuh"
 
 namespace sco {
@@ -140,6 +141,28 @@ __global__ void __launch_bounds__(256, 4) k_kw_level(uint32_t N, uint32_t g, uns
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) rmax = max(rmax, __shfl_down_sync(0xffffffffu, rmax, o));
   if ((threadIdx.x & 31) == 0 && rmax) atomicMax(&cnt->lev_rounds[p & 31], rmax);
+}
+
+// Initial words of the dataflow kernel.
+__global__ void k_flow_init(uint32_t N, uint32_t g, uint32_t m32, uint32_t* __restrict__ word) {
+  const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v < N) word[v] = v - flow_div(v, g, m32) * g;
+}
+
+// Final colours of the dataflow kernel.
+__global__ void k_flow_final(uint32_t N, unsigned levels, uint32_t g, int variant,
+                             const uint32_t* __restrict__ word, uint32_t* __restrict__ colour,
+                             DevCounters* __restrict__ cnt) {
+  const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+  // (after a wait that gave up a vertex may keep a colour of an earlier level, below g as well)
+  if (v < N) colour[v] = word[v] & 63u;
+  if (v == 0) {
+    unsigned t = 0;
+    for (unsigned p = 1; p <= levels; ++p) t += cnt->lev_rounds[p & 31];
+    // plain BCR (2) spends exactly g rounds per level on the same colouring
+    cnt->kw_rounds = variant == 1 ? g * levels : t;
+    cnt->levels = levels;
+  }
 }
 
 __global__ void k_kw_final(int64_t N, unsigned levels, uint32_t g, int variant,
@@ -341,12 +364,39 @@ cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* 
   cudaError_t e = cudaMemsetAsync(cnt->lev_rounds, 0, sizeof(cnt->lev_rounds), st);
   if (e != cudaSuccess) return e;
   const unsigned nb = (unsigned)((N + 255) / 256);
-  k_kw_init<<<nb, 256, 0, st>>>(N, g, b.word, b.col8, b.blk);
-  ++*launches;
   unsigned long long magic = div_magic(g);
   uint32_t* site_start = reinterpret_cast<uint32_t*>(b.meta);
   RepPlan* plan = reinterpret_cast<RepPlan*>(b.meta + 2);
   k_kw_meta<<<1, 1, 0, st>>>((uint32_t)N, g, M, magic, site_start, plan);
+  ++*launches;
+  FlowShape shape;
+  if (g <= kFlowMaxPal && M < kFlowMaxLevels && flow_shape(1, N, &shape, &e)) {
+    if ((e = cudaMemsetAsync(cnt->bar, 0, sizeof(cnt->bar), st)) != cudaSuccess) return e;
+    FlowView F{};
+    F.R = 1;
+    F.site_start = site_start;
+    F.plan = plan;
+    F.row_ptr = row_ptr;
+    F.col = col;
+    F.word = reinterpret_cast<uint32_t*>(b.word);
+    F.lev_rounds = cnt->lev_rounds;
+    F.lev_stride = 0;
+    F.bar = cnt->bar;
+    F.status = &cnt->status;
+    F.levels = M;
+    F.cap = shape.cap;
+    F.min_tile = kFlowMinTile;
+    F.ns_limit = ns_limit;
+    F.vec = kFlowVecAll;
+    k_flow_init<<<nb, 256, 0, st>>>((uint32_t)N, g, g > 1 ? (uint32_t)(0x100000000ull / g) : 0xFFFFFFFFu,
+                                    F.word);
+    if ((e = flow_launch(F, shape, st)) != cudaSuccess) return e;
+    k_flow_final<<<nb, 256, 0, st>>>((uint32_t)N, M, g, variant, F.word, b.colour, cnt);
+    *launches += 3;
+    return cudaGetLastError();
+  }
+  if (e != cudaSuccess) return e;
+  k_kw_init<<<nb, 256, 0, st>>>(N, g, b.word, b.col8, b.blk);
   ++*launches;
   // levels 1..low: one block per group of g 2^low vertices
   const unsigned low = kw_low_levels(g, M, kLowMaxGroup);

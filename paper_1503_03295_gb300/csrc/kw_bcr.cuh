@@ -38,6 +38,7 @@ struct KwView {
   unsigned* bar;                // grid barrier words
   int* status;                  // sticky error word
   const int* halt;              // optional: nonzero on entry -> return at once
+  const unsigned* flow;         // optional: largest palette; up to kFlowMaxPal -> return at once
   unsigned pal;                 // >= every g, <= kBcrMaxPalette
   unsigned levels;              // >= every M, <= kBcrMaxLevels - 1
   unsigned long long ns_limit;  // bound of every barrier wait
@@ -300,7 +301,8 @@ __device__ __noinline__ bool kw_item_slow(uint32_t gv, uint32_t base, uint32_t c
 template <bool kBuckets>
 __global__ void __launch_bounds__(256, kBuckets ? kBcrBucketBlocks : 3) k_kw_bcr(const KwView V) {
   __shared__ int s_halt;
-  if (threadIdx.x == 0) s_halt = V.halt ? ld_status(V.halt) : 0;
+  if (threadIdx.x == 0)
+    s_halt = (V.halt && ld_status(V.halt)) || (V.flow && *V.flow <= kFlowMaxPal);
   __syncthreads();
   if (s_halt) return;
   extern __shared__ uint32_t sm[];

@@ -48,6 +48,7 @@ struct KwLowView {
   uint8_t* col8;                // colour (low byte), global vertex index
   DevCounters* cnt;             // R: lev_rounds
   const int* halt;              // optional: nonzero on entry -> return at once
+  const unsigned* flow;         // optional: largest palette; up to kFlowMaxPal -> return at once
   uint32_t gmax;                // group-size cap of kw_low_levels
   uint32_t gcap;                // >= every group size g 2^p0, <= gmax, even
   uint32_t ecap;                // internal edges staged per group (0: rows at every level)
@@ -144,7 +145,8 @@ __device__ __forceinline__ void low_for_nbrs(bool staged, uint32_t v, uint32_t b
 // lev_rounds[1..p0].
 __global__ void __launch_bounds__(kLowThreads, 4) k_kw_low(const KwLowView V) {
   __shared__ int s_halt;
-  if (threadIdx.x == 0) s_halt = V.halt ? ld_status(V.halt) : 0;
+  if (threadIdx.x == 0)
+    s_halt = (V.halt && ld_status(V.halt)) || (V.flow && *V.flow <= kFlowMaxPal);
   __syncthreads();
   if (s_halt) return;
   extern __shared__ uint4 lsm4[];

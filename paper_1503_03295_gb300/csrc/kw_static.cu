@@ -1,7 +1,7 @@
 // kw_static.cu -- Kuhn-Wattenhofer colouring of a caller's CSR graph that allocates nothing.
 //
-// Same colouring as sco_colour (one barrier-free dataflow kernel per level, see colour.cu),
-// for callers that cannot let a library allocate device memory.  Its working memory is one
+// Same colouring as sco_colour (palettes of at most 63 colours by the dataflow kernel of
+// kw_flow.cuh, larger ones by one barrier-free kernel per level), for callers that cannot let a library allocate device memory.  Its working memory is one
 // file-scope device array of fixed size: per-vertex words for up to
 // SCO_KW_STATIC_MAX_VERTICES vertices followed by a small control block.  Every call
 // shares that array; calls that overlap on the GPU race.
@@ -9,18 +9,17 @@
 #include <cstring>
 #include <mutex>
 
+#include "kw_flow.cuh"
 #include "sco.h"
 #include "sco_internal.h"
 
-namespace {
+namespace sco {
 
-using namespace sco;
+namespace {
 
 constexpr int64_t kMaxVertices = SCO_KW_STATIC_MAX_VERTICES;
 constexpr int kCtrlWords = 64;  // 512 bytes of control block after the vertex words
 constexpr int kMaxDevices = 64;
-constexpr int kStatusTimeout = 4;
-constexpr unsigned long long kColMask = 0xFFFFFFFFull;
 
 struct StaticCtrl {
   unsigned int max_degree;
@@ -31,40 +30,14 @@ struct StaticCtrl {
   unsigned int kw_rounds;
   unsigned int pad;
   unsigned int lev_rounds[32];
+  RepPlan plan;  // the dataflow kernel's view of the one lattice
+  unsigned int site_start[2];
+  unsigned int bar[2];
 };
 static_assert(sizeof(StaticCtrl) <= kCtrlWords * 8, "control block");
 
 // The scratch: kMaxVertices packed words, then the control block.  8 MiB + 512 B per device.
 static __device__ __align__(256) unsigned long long g_kw_scratch[kMaxVertices + kCtrlWords];
-
-__device__ __forceinline__ unsigned long long pack(unsigned p, unsigned r, unsigned c) {
-  return ((unsigned long long)p << 48) | ((unsigned long long)r << 32) | c;
-}
-__device__ __forceinline__ unsigned tag_of(unsigned long long w) { return (unsigned)(w >> 48); }
-__device__ __forceinline__ unsigned rnd_of(unsigned long long w) {
-  return (unsigned)(w >> 32) & 0xFFFFu;
-}
-__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ int ld_status(const int* p) {
-  int v;
-  asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ uint32_t fdiv(uint32_t u, unsigned long long M) {
-  return div_by_magic(u, M);  // M = 0 stands for g = 1
-}
 
 __global__ void k_st_degree(uint32_t n, const uint32_t* __restrict__ row_ptr,
                             StaticCtrl* __restrict__ ctrl) {
@@ -83,12 +56,20 @@ __global__ void k_st_setup(uint32_t n, StaticCtrl* __restrict__ ctrl) {
   ctrl->g = g;
   ctrl->levels = M;
   ctrl->magic = div_magic(g);
+  ctrl->plan = RepPlan{g, M, div_magic(g)};
+  ctrl->site_start[0] = 0;
+  ctrl->site_start[1] = n;
 }
 
 __global__ void k_st_init(uint32_t n, unsigned long long* __restrict__ word,
                           const StaticCtrl* __restrict__ ctrl) {
   const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v < n) word[v] = pack(0, 0, v % ctrl->g);
+}
+
+__global__ void k_st_flow_init(uint32_t n, uint32_t g, uint32_t m32, uint32_t* __restrict__ word) {
+  const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v < n) word[v] = v - flow_div(v, g, m32) * g;
 }
 
 __device__ __noinline__ unsigned st_mex_slow(uint32_t v, unsigned p, unsigned long long M,
@@ -111,8 +92,8 @@ __device__ __noinline__ unsigned st_mex_slow(uint32_t v, unsigned p, unsigned lo
   }
 }
 
-// One KW level (modified reduction (2)'); g, M and the divisor constant come from the
-// control block, and levels beyond M return at once.
+// One KW level (modified reduction (2)') of a palette too large for the dataflow kernel; g, M and
+// the divisor constant come from the control block.
 __global__ void __launch_bounds__(256) k_st_level(uint32_t n, unsigned p,
                                                   const uint32_t* __restrict__ row_ptr,
                                                   const uint32_t* __restrict__ col,
@@ -202,10 +183,12 @@ __global__ void __launch_bounds__(256) k_st_level(uint32_t n, unsigned p,
   if ((threadIdx.x & 31) == 0 && rmax) atomicMax(&ctrl->lev_rounds[p & 31], rmax);
 }
 
+// fword: the dataflow kernel's words (null: word)
 __global__ void k_st_final(uint32_t n, int variant, const unsigned long long* __restrict__ word,
-                           uint32_t* __restrict__ colour, StaticCtrl* __restrict__ ctrl) {
+                           const uint32_t* __restrict__ fword, uint32_t* __restrict__ colour,
+                           StaticCtrl* __restrict__ ctrl) {
   const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v < n) colour[v] = (uint32_t)(word[v] & kColMask);
+  if (v < n) colour[v] = fword ? fword[v] & 63u : (uint32_t)(word[v] & kColMask);
   if (v == 0) {
     unsigned t = 0;
     for (unsigned p = 1; p <= ctrl->levels; ++p) t += ctrl->lev_rounds[p & 31];
@@ -219,6 +202,10 @@ int g_blocks_per_sm[kMaxDevices] = {};
 int g_sms[kMaxDevices] = {};
 
 }  // namespace
+
+}  // namespace sco
+
+using namespace sco;
 
 extern "C" sco_status sco_kw_colour_static(const uint32_t* row_ptr, const uint32_t* col,
                                            int64_t n, int32_t variant, uint32_t* colour,
@@ -258,26 +245,54 @@ extern "C" sco_status sco_kw_colour_static(const uint32_t* row_ptr, const uint32
   const unsigned nb = (nn + 255) / 256;
   k_st_degree<<<nb, 256, 0, st>>>(nn, row_ptr, ctrl);
   k_st_setup<<<1, 1, 0, st>>>(nn, ctrl);
-  k_st_init<<<nb, 256, 0, st>>>(nn, word, ctrl);
-  if (cudaGetLastError() != cudaSuccess) return SCO_ECUDA;
-  unsigned pmax = 0;  // g >= 1 bounds the level count by ceil(log2 n)
-  while ((1ull << pmax) < (unsigned long long)n) ++pmax;
-  int64_t grid = (int64_t)g_blocks_per_sm[dev] * g_sms[dev];
-  const int64_t want = ((int64_t)nn / 2 + 255) / 256;
-  if (want < grid) grid = want > 0 ? want : 1;
-  unsigned long long ns_limit = 2000000000ull;
-  for (unsigned p = 1; p <= pmax; ++p) {
-    uint32_t a0 = nn;
-    unsigned a1 = p;
-    void* args[] = {(void*)&a0, (void*)&a1, (void*)&row_ptr, (void*)&col, (void*)&word,
-                    (void*)&ctrl, (void*)&ns_limit};
-    if (cudaLaunchCooperativeKernel((const void*)k_st_level, dim3((unsigned)grid), dim3(256), args,
-                                    0, st) != cudaSuccess)
-      return SCO_ECUDA;
-  }
-  k_st_final<<<nb, 256, 0, st>>>(nn, variant, word, colour, ctrl);
+  // Delta decides the kernel: small palettes run the dataflow kernel
   StaticCtrl h;
   std::memset(&h, 0, sizeof(h));
+  if (cudaMemcpyAsync(&h, ctrl, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+    return SCO_ECUDA;
+  if (cudaStreamSynchronize(st) != cudaSuccess) return SCO_ECUDA;
+  unsigned long long ns_limit = 2000000000ull;
+  FlowShape shape;
+  cudaError_t fe = cudaSuccess;
+  const bool flow = h.g <= kFlowMaxPal && h.levels < kFlowMaxLevels && flow_shape(1, nn, &shape, &fe);
+  if (fe != cudaSuccess) return SCO_ECUDA;
+  uint32_t* fword = flow ? reinterpret_cast<uint32_t*>(word) : nullptr;
+  if (flow) {
+    k_st_flow_init<<<nb, 256, 0, st>>>(
+        nn, h.g, h.g > 1 ? (uint32_t)(0x100000000ull / h.g) : 0xFFFFFFFFu, fword);
+    FlowView F{};
+    F.R = 1;
+    F.site_start = ctrl->site_start;
+    F.plan = &ctrl->plan;
+    F.row_ptr = row_ptr;
+    F.col = col;
+    F.word = fword;
+    F.lev_rounds = ctrl->lev_rounds;
+    F.bar = ctrl->bar;
+    F.status = &ctrl->status;
+    F.levels = h.levels;
+    F.cap = shape.cap;
+    F.min_tile = kFlowMinTile;
+    F.ns_limit = ns_limit;
+    F.vec = ((uintptr_t)col & 31u) == 0 ? kFlowVecInside : kFlowVecNone;
+    if (flow_launch(F, shape, st) != cudaSuccess) return SCO_ECUDA;
+  } else {
+    k_st_init<<<nb, 256, 0, st>>>(nn, word, ctrl);
+    if (cudaGetLastError() != cudaSuccess) return SCO_ECUDA;
+    int64_t grid = (int64_t)g_blocks_per_sm[dev] * g_sms[dev];
+    const int64_t want = ((int64_t)nn / 2 + 255) / 256;
+    if (want < grid) grid = want > 0 ? want : 1;
+    for (unsigned p = 1; p <= h.levels; ++p) {
+      uint32_t a0 = nn;
+      unsigned a1 = p;
+      void* args[] = {(void*)&a0, (void*)&a1, (void*)&row_ptr, (void*)&col, (void*)&word,
+                      (void*)&ctrl, (void*)&ns_limit};
+      if (cudaLaunchCooperativeKernel((const void*)k_st_level, dim3((unsigned)grid), dim3(256),
+                                      args, 0, st) != cudaSuccess)
+        return SCO_ECUDA;
+    }
+  }
+  k_st_final<<<nb, 256, 0, st>>>(nn, variant, word, fword, colour, ctrl);
   if (cudaMemcpyAsync(&h, ctrl, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess)
     return SCO_ECUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return SCO_ECUDA;
