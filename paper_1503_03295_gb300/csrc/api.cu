@@ -122,6 +122,7 @@ struct sco_ctx {
   uint32_t g = 1;
   uint64_t nnz = 0;
   bool dip_valid = false;  // cnt->max_degree_dip holds the dipolar Delta of the current graph
+  FullWork full;  // workspace of the full energy, once asked for
   int sticky = 0;
   unsigned long long ns_limit = 2000000000ull;  // bound of every device-side wait (2 s)
   // phase timing
@@ -322,6 +323,7 @@ void free_all(sco_ctx* c) {
   cudaFree(c->cb.imeta);
   cudaFree(c->cb.ilist);
   cudaFree(c->acc);
+  cudaFree(c->full.p);
   cudaFree(c->defer);
   cudaFree(c->prop);
   cudaFree(c->cnt);
@@ -466,7 +468,7 @@ sco_status sco_observables(sco_ctx* c, sco_obs* o, int32_t want_full) {
     c->dip_valid = true;
   }
   SCO_TRY(observables_run(c->P, c->s, c->row_ptr, c->col, c->tab.xy, c->graph_epoch >= 0, full,
-                          c->cnt, c->st, &c->launches));
+                          &c->full, c->cnt, c->st, &c->launches));
   sco_status st = read_counters(c);
   if (st != SCO_OK) return st;
   const DevCounters& h = *c->hcnt;
@@ -474,7 +476,7 @@ sco_status sco_observables(sco_ctx* c, sco_obs* o, int32_t want_full) {
   std::memset(o, 0, sizeof(*o));
   o->e_exchange = h.acc[4];
   o->e_switched = (c->graph_epoch >= 0 ? h.acc[5] : 0.0) + h.acc[4];
-  o->e_full = full ? h.acc[6] : NAN;
+  o->e_full = full ? h.acc[6] + h.acc[4] : NAN;
   o->mx = h.acc[0] / N;
   o->my = h.acc[1] / N;
   o->mz = h.acc[2] / N;

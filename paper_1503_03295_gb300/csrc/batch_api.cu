@@ -32,6 +32,7 @@ struct sco_batch {
   BatchDev B{};
   BatchLaunch L{};
   size_t scan_tmp_n = 0;  // elements the scan buffer serves
+  FullWork full;  // workspace of the full energy, once asked for
   DevCounters* hcnt = nullptr;  // pinned, R
   BatchCtl* hctl = nullptr;     // pinned
   int64_t t = 0;
@@ -109,6 +110,7 @@ void free_all(sco_batch* b) {
   cudaFree(B.dcnt);
   cudaFree(B.bcnt);
   cudaFree(b->L.scan_tmp);
+  cudaFree(b->full.p);
   for (auto& t : b->xy) table_free_xy(t);
   for (auto& t : b->lists) table_free(t);
   if (b->hcnt) cudaFreeHost(b->hcnt);
@@ -618,7 +620,8 @@ sco_status sco_batch_observables(sco_batch* b, int32_t r, sco_obs* o, int32_t wa
   const uint32_t base = b->site_start[r];
   const bool full = want_full && P.N <= 65536;
   SCO_TRY(observables_run(P, b->B.s + 3 * (size_t)base, b->B.row_ptr + base, b->B.col,
-                          b->xy[r].xy, b->have_graph, full, b->B.cnt + r, b->st, &b->launches));
+                          b->xy[r].xy, b->have_graph, full, &b->full, b->B.cnt + r, b->st,
+                          &b->launches));
   SCO_TRY(cudaMemcpyAsync(b->hcnt + r, b->B.cnt + r, sizeof(DevCounters), cudaMemcpyDeviceToHost,
                           b->st));
   sco_status s = read_ctl(b);
@@ -629,7 +632,7 @@ sco_status sco_batch_observables(sco_batch* b, int32_t r, sco_obs* o, int32_t wa
   const bool g = b->have_graph;
   o->e_exchange = h.acc[4];
   o->e_switched = (g ? h.acc[5] : 0.0) + h.acc[4];
-  o->e_full = full ? h.acc[6] : NAN;
+  o->e_full = full ? h.acc[6] + h.acc[4] : NAN;
   o->mx = h.acc[0] / N;
   o->my = h.acc[1] / N;
   o->mz = h.acc[2] / N;

@@ -109,9 +109,21 @@ cudaError_t spins_copies(int64_t N, const double* s, float4* s32, SpinDf* sd, cu
 // largest dipolar degree of the current graph into cnt->max_degree_dip
 cudaError_t dip_degree_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* col,
                            DevCounters* cnt, cudaStream_t st, int64_t* launches);
+// want_full: the dipolar part of the full energy, by transforms in *work (allocated here when first
+// needed or too small, kept by the caller) or, without it, by the direct sum
+struct FullWork {
+  void* p = nullptr;
+  size_t bytes = 0;
+};
 cudaError_t observables_run(const DevParams& P, const double* s, const uint32_t* row_ptr,
                             const uint32_t* col, const double2* xy, bool have_graph,
-                            bool want_full, DevCounters* cnt, cudaStream_t st, int64_t* launches);
+                            bool want_full, FullWork* work, DevCounters* cnt, cudaStream_t st,
+                            int64_t* launches);
+// ---- energy.cu ----
+bool full_energy_fft_ok(const DevParams& P);
+size_t full_energy_fft_bytes(const DevParams& P);
+cudaError_t full_energy_fft(const DevParams& P, const double* s, void* work, double* acc,
+                            cudaStream_t st, int64_t* launches);
 
 // ---- switch.cu ----
 constexpr int kSlotCap = 32;

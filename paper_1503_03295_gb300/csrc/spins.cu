@@ -125,7 +125,8 @@ __global__ void __launch_bounds__(256) k_pair_obs(DevParams P, const double* __r
   block_accumulate<1>(v, acc + 5);
 }
 
-// Full H of Eq. (6) by direct summation over all pairs (tiles of 256 j per block row).
+// Dipolar part of the full H of Eq. (6) by direct summation over all pairs (tiles of 256 j per block
+// row): lattices that the transforms of energy.cu do not take.
 __global__ void __launch_bounds__(256) k_full_energy(DevParams P, const double* __restrict__ s,
                                                      double* __restrict__ acc) {
   __shared__ double sj[3][256];
@@ -150,7 +151,6 @@ __global__ void __launch_bounds__(256) k_full_energy(DevParams P, const double* 
         const double bx = sj[0][k], by = sj[1][k], bz = sj[2][k];
         const double c = 1.0 / (r2 * r2 * sqrt(r2));
         e += pair_V(P.D * c, r2, ax, ay, az, bx, by, bz, (double)dx, (double)dy);
-        if (r2 == 1.0) e -= P.J * (ax * bx + ay * by + az * bz);
       }
     }
     __syncthreads();
@@ -199,7 +199,7 @@ cudaError_t dip_degree_run(const DevParams& P, const uint32_t* row_ptr, const ui
 
 cudaError_t observables_run(const DevParams& P, const double* s, const uint32_t* row_ptr,
                             const uint32_t* col, const double2* xy, bool have_graph,
-                            bool want_full, DevCounters* cnt, cudaStream_t st,
+                            bool want_full, FullWork* work, DevCounters* cnt, cudaStream_t st,
                             int64_t* launches) {
   cudaError_t e = cudaMemsetAsync(cnt->acc, 0, sizeof(cnt->acc), st);
   if (e != cudaSuccess) return e;
@@ -209,6 +209,20 @@ cudaError_t observables_run(const DevParams& P, const double* s, const uint32_t*
   if (have_graph) {
     k_pair_obs<<<nb, 256, 0, st>>>(P, s, row_ptr, col, xy, cnt->acc);
     ++*launches;
+  }
+  if (want_full && full_energy_fft_ok(P)) {
+    const size_t need = full_energy_fft_bytes(P);
+    if (work->bytes < need) {
+      if (work->p) {
+        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+        cudaFree(work->p);
+      }
+      work->p = nullptr;
+      work->bytes = 0;
+      if (cudaMalloc(&work->p, need) == cudaSuccess) work->bytes = need;
+      else cudaGetLastError();  // no room: the direct sum needs none
+    }
+    if (work->p) return full_energy_fft(P, s, work->p, cnt->acc + 6, st, launches);
   }
   if (want_full) {
     k_full_energy<<<(unsigned)((P.N + 255) / 256), 256, 0, st>>>(P, s, cnt->acc);
