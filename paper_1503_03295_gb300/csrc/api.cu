@@ -104,6 +104,7 @@ struct sco_ctx {
   float4* s32 = nullptr;    // FP32-guarded form: FP32 copy of the spins, one (x, y, z, 0) per site
   SpinDf* sd = nullptr;     // FP64 form: float-float copy of the spins
   SpinDf* propd = nullptr;  // FP64 form: the proposals of the step in float-float
+  float4* prop32 = nullptr;  // FP32-guarded form: the same in FP32
   double* s_epoch = nullptr;
   SwitchBufs sw{};
   uint32_t* row_ptr = nullptr;
@@ -112,7 +113,6 @@ struct sco_ctx {
   ColourBufs cb{};
   uint32_t cls_cap = 0;  // capacity of hist / off / cursor
   uint8_t* acc = nullptr;
-  uint32_t* defer = nullptr;  // N sites whose decision goes to the warp-parallel resolve
   double4_32a* prop = nullptr;  // N proposals {S', u} of the current MC step
   DevCounters* cnt = nullptr;   // device
   DevCounters* hcnt = nullptr;  // pinned mirror
@@ -253,9 +253,8 @@ sco_status do_colour(sco_ctx* c) {
     cudaFree(c->cb.cursor);
     cudaFree(c->cb.scan_tmp);
     cudaFree(c->cb.tile_cnt);
-    cudaFree(c->cb.dcnt);
     cudaFree(c->cb.bcnt);
-    c->cb.hist = c->cb.off = c->cb.cursor = c->cb.tile_cnt = c->cb.dcnt = c->cb.bcnt = nullptr;
+    c->cb.hist = c->cb.off = c->cb.cursor = c->cb.tile_cnt = c->cb.bcnt = nullptr;
     c->cb.scan_tmp = nullptr;
     const uint32_t cap = c->g + 64;
     const int64_t ntiles = (c->P.N + kClassTileSites - 1) / kClassTileSites;
@@ -265,7 +264,6 @@ sco_status do_colour(sco_ctx* c) {
     SCO_TRY(cudaMalloc(&c->cb.hist, (cap + 1) * sizeof(uint32_t)));
     SCO_TRY(cudaMalloc(&c->cb.off, (cap + 1) * sizeof(uint32_t)));
     SCO_TRY(cudaMalloc(&c->cb.cursor, (cap + 1) * sizeof(uint32_t)));
-    SCO_TRY(cudaMalloc(&c->cb.dcnt, (cap + 1) * sizeof(uint32_t)));
     SCO_TRY(cudaMalloc(&c->cb.bcnt, (size_t)32 * (cap + 1) * sizeof(uint32_t)));
     if (!c->cb.boff) SCO_TRY(cudaMalloc(&c->cb.boff, (size_t)kKwSplitBlocks * 64 * sizeof(uint32_t)));
     SCO_TRY(cudaMalloc(&c->cb.tile_cnt, tc * sizeof(uint32_t)));
@@ -295,6 +293,7 @@ void free_all(sco_ctx* c) {
   cudaFree(c->s32);
   cudaFree(c->sd);
   cudaFree(c->propd);
+  cudaFree(c->prop32);
   cudaFree(c->s_epoch);
   cudaFree(c->sw.hslot);
   cudaFree(c->sw.hcnt);
@@ -324,7 +323,6 @@ void free_all(sco_ctx* c) {
   cudaFree(c->cb.ilist);
   cudaFree(c->acc);
   cudaFree(c->full.p);
-  cudaFree(c->defer);
   cudaFree(c->prop);
   cudaFree(c->cnt);
   if (c->hcnt) cudaFreeHost(c->hcnt);
@@ -379,6 +377,7 @@ sco_status sco_init(const sco_params* p, void* stream, sco_ctx** out) {
     if (e == cudaSuccess) e = cudaMalloc(&c->propd, N * sizeof(SpinDf));
   } else if (e == cudaSuccess) {
     e = cudaMalloc(&c->s32, N * sizeof(float4));
+    if (e == cudaSuccess) e = cudaMalloc(&c->prop32, N * sizeof(float4));
   }
   if (e == cudaSuccess && p->n_sw > 1) e = cudaMalloc(&c->s_epoch, 3 * N * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->sw.hslot, N * kSlotCap * sizeof(uint32_t));
@@ -401,7 +400,6 @@ sco_status sco_init(const sco_params* p, void* stream, sco_ctx** out) {
   if (e == cudaSuccess) e = cudaMalloc(&c->cb.imeta, N * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&c->cb.ilist, kKwItemList * N * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&c->acc, N);
-  if (e == cudaSuccess) e = cudaMalloc(&c->defer, N * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&c->prop, N * sizeof(double4_32a));
   if (e == cudaSuccess) e = cudaMalloc(&c->cnt, sizeof(DevCounters));
   if (e == cudaSuccess) e = cudaMallocHost(&c->hcnt, sizeof(DevCounters));
@@ -451,9 +449,10 @@ sco_status sco_sweep(sco_ctx* c, int32_t n_mcs) {
     if (st != SCO_OK) return st;
     {
       PhaseTimer tm(c, kPhSweep);
-      SCO_TRY(sweep_run(c->P, c->tab, c->s, c->s32, c->sd, c->row_ptr, c->col, c->cb.perm,
-                        c->cb.off, c->g, (uint64_t)c->t, c->p.precision, c->acc, c->defer,
-                        c->cb.dcnt, c->prop, c->propd, c->cnt, c->st, &c->launches));
+      const SweepBufs b{c->s,       c->s32,  c->sd,    c->row_ptr, c->col, c->cb.perm,
+                        c->cb.off,  c->prop, c->propd, c->prop32,  c->acc};
+      SCO_TRY(sweep_run(c->P, c->tab, b, c->g, (uint64_t)c->t, c->p.precision, c->cnt, c->ns_limit,
+                        c->st, &c->launches));
     }
     c->t++;
   }

@@ -459,124 +459,12 @@ __global__ void __launch_bounds__(32) kb_tile_scatter(const BatchDev B) {
 __global__ void __launch_bounds__(256) kb_propose(const BatchDev B) {
   if (block_halted(B)) return;
   const int r = block_replica(B);
-  const RepDesc* d = B.desc + r;
   const uint32_t base = B.site_start[r], N = B.site_start[r + 1] - base;
   const uint32_t i = (blockIdx.x - B.blk_start[r]) * kBatchBlock + threadIdx.x;
   if (i >= N) return;
-  SiteCtx c;
-  c.i = i;
-  const bool ok = propose(d->P, c, B.ctl->step);
-  B.prop[base + i] = ok ? make_double4_32a(c.Sn[0], c.Sn[1], c.Sn[2], c.u)
-                        : make_double4_32a(0.0, 0.0, 1.0, -1.0);
-  if (B.propd) {
-    SpinDf p = spin_df(c.Sn[0], c.Sn[1], c.Sn[2], c.u);
-    if (!ok) p.u_h = -1.f;
-    B.propd[base + i] = p;
-  }
-}
-
-// Sites of class c (all replicas) one per thread; undecided ones go to the deferred list of
-// the colour; after a grid barrier one warp per deferred site settles it (FP64, then
-// double-double); a second barrier closes the colour.
-template <int PREC>
-__global__ void __launch_bounds__(128, PREC == 1 ? 6 : 5) kb_sweep(const BatchDev B) {
-  if (block_halted(B)) return;
-  extern __shared__ uint32_t wsm[];
-  const int R = B.R;
-  uint32_t* sbase = wsm;          // R + 1
-  uint32_t* sg1 = sbase + R + 1;  // R deferred by the FP32 screen
-  uint32_t* sg2 = sg1 + R;        // R sent on to double-double
-  for (int r = threadIdx.x; r <= R; r += blockDim.x) sbase[r] = B.site_start[r];
-  for (int r = threadIdx.x; r < R; r += blockDim.x) {
-    sg1[r] = 0;
-    sg2[r] = 0;
-  }
-  __syncthreads();
-  const uint32_t gmax = B.ctl->gmax;
-  const uint32_t nth = gridDim.x * blockDim.x;
-  const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  const uint32_t gwarp = gtid >> 5, nwarps = nth >> 5;
-  for (uint32_t c = 0; c < gmax; ++c) {
-    const uint32_t b = B.off[c], e = B.off[c + 1];
-    for (uint32_t idx = b + gtid; idx < e; idx += nth) {
-      const uint32_t gs = B.perm[idx];
-      const int r = find_le(sbase, R, gs);
-      const uint32_t base = sbase[r];
-      const RepDesc* d = B.desc + r;
-      const DevParams& P = d->P;
-      double* s = B.s + 3 * (size_t)base;
-      const uint32_t i = gs - base;
-      int dec;
-      if (PREC == 0) {
-        const SpinDf N = load32(B.propd + gs);
-        if (N.u_h < 0.f) {
-          B.acc[gs] = 0;
-          continue;
-        }
-        int32_t xi, yi;
-        site_xy(i, P, xi, yi);
-        dec = accept_df<1>(P, xi, yi, load32(B.sd + gs), N, d->pdf, B.sd + base, B.col,
-                           B.row_ptr[gs], B.row_ptr[gs + 1], i, 0);
-        if (dec != 2) {
-          if (dec == 1) {
-            const double4_32a v = B.prop[gs];
-            s[i] = v.x;
-            s[P.N + i] = v.y;
-            s[2 * P.N + i] = v.z;
-            B.sd[gs] = N;
-          }
-          B.acc[gs] = (uint8_t)dec;
-        }
-      } else {
-        float4* s32 = B.s32 + base;
-        SiteCtx x;
-        load_site(P, x, i, s);
-        if (!take_proposal(x, B.prop + base)) {
-          B.acc[gs] = 0;
-          continue;
-        }
-        dec = x.u != 0.0 ? accept_fp32(P, x, d->sw32, s32, B.row_ptr + base, B.col) : 1;
-        if (dec != 2) write_site(P, x, dec == 1, s, s32, B.acc + base);
-      }
-      if (dec == 2) {
-        B.defer[b + atomicAdd(&B.dcnt[c], 1u)] = gs;
-        if (PREC == 1) atomicAdd(&sg1[r], 1u);
-      }
-    }
-    if (!grid_sync(B.ctl->bar, &B.ctl->status, B.ns_limit)) break;
-    const uint32_t nd = ld_u32_gpu(&B.dcnt[c]);
-    if (nd == 0) continue;
-    for (uint32_t q = gwarp; q < nd; q += nwarps) {
-      const uint32_t gs = ld_u32_gpu(&B.defer[b + q]);
-      const int r = find_le(sbase, R, gs);
-      const uint32_t base = sbase[r];
-      const RepDesc* d = B.desc + r;
-      const DevParams& P = d->P;
-      const size_t so = 3 * (size_t)base;
-      double* s = B.s + so;
-      SiteCtx x;
-      load_site(P, x, gs - base, s);
-      take_proposal(x, B.prop + base);
-      int dec = accept_fp64_warp(P, x, d->sw64, s, B.row_ptr + base, B.col, lane);
-      if (dec == 2) {
-        if (lane == 0) atomicAdd(&sg2[r], 1u);
-        dec = accept_dd_warp(P, x, s, B.row_ptr + base, B.col, lane) ? 1 : 0;
-      }
-      if (lane == 0) {
-        write_site(P, x, dec == 1, s, PREC == 1 ? B.s32 + base : nullptr, B.acc + base);
-        if (PREC == 0 && dec == 1) B.sd[gs] = B.propd[gs];
-      }
-      __syncwarp();
-    }
-    if (!grid_sync(B.ctl->bar, &B.ctl->status, B.ns_limit)) break;
-  }
-  __syncthreads();
-  for (int r = threadIdx.x; r < R; r += blockDim.x) {
-    DevCounters* cr = B.cnt + r;
-    if (sg1[r]) atomicAdd(&cr->guard_fp32, (unsigned long long)sg1[r]);
-    if (sg2[r]) atomicAdd(&cr->guard_fp64, (unsigned long long)sg2[r]);
-  }
+  const uint32_t gs = base + i;
+  write_proposal(B.desc[r].P, B.ctl->step, i, B.prop + gs, B.propd ? B.propd + gs : nullptr,
+                 B.prop32 ? B.prop32 + gs : nullptr);
 }
 
 __global__ void kb_step_end(const BatchDev B) {
@@ -602,8 +490,6 @@ cudaError_t launch_coop(void (*k)(Args...), unsigned grid, unsigned block, size_
 size_t kw_smem(int R) { return (size_t)(3 * R + 2) * sizeof(uint32_t); }
 
 }  // namespace
-
-size_t batch_sweep_smem(int R) { return (size_t)(3 * R + 1) * sizeof(uint32_t); }
 
 int batch_kw_occupancy(int schedule, int R, unsigned pal) {
   int n = 0;
@@ -642,11 +528,11 @@ cudaError_t batch_low_setup(int R, uint32_t gcap, int* blocks_per_sm, uint32_t* 
 
 int batch_sweep_occupancy(int precision, int R) {
   int n = 0;
-  cudaError_t e = precision == 1
-                      ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kb_sweep<1>, 128,
-                                                                      batch_sweep_smem(R))
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kb_sweep<0>, 128,
-                                                                      batch_sweep_smem(R));
+  const cudaError_t e =
+      precision == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep<1, true, 3>,
+                                                                     kSweepThreads, sweep_smem(R))
+                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep<0, true, 2>,
+                                                                     kSweepThreads, sweep_smem(R));
   if (e != cudaSuccess || n < 1) n = 1;
   return n;
 }
@@ -781,17 +667,34 @@ cudaError_t batch_colour(const BatchDev& B, const BatchLaunch& L, cudaStream_t s
 }
 
 cudaError_t batch_sweep(const BatchDev& B, const BatchLaunch& L, cudaStream_t st) {
-  cudaError_t e;
-  if ((e = cudaMemsetAsync(B.dcnt, 0, (size_t)B.pal_cap * sizeof(uint32_t), st)) != cudaSuccess)
-    return e;
   kb_propose<<<B.nblocks, kBatchBlock, 0, st>>>(B);
-  ++*L.launches;
-  if (B.precision == 1)
-    e = launch_coop(kb_sweep<1>, (unsigned)L.sweep_grid, 128, batch_sweep_smem(B.R), st, B);
-  else
-    e = launch_coop(kb_sweep<0>, (unsigned)L.sweep_grid, 128, batch_sweep_smem(B.R), st, B);
-  ++*L.launches;
-  return e;
+  SweepView V{};
+  V.R = B.R;
+  V.site_start = B.site_start;
+  V.desc = B.desc;
+  V.s = B.s;
+  V.s32 = B.s32;
+  V.sd = B.sd;
+  V.row_ptr = B.row_ptr;
+  V.col = B.col;
+  V.perm = B.perm;
+  V.off = B.off;
+  V.prop = B.prop;
+  V.propd = B.propd;
+  V.prop32 = B.prop32;
+  V.acc = B.acc;
+  V.cnt = B.cnt;
+  V.gmax = &B.ctl->gmax;
+  V.bar = B.ctl->bar;
+  V.status = &B.ctl->status;
+  V.halt = &B.ctl->flag;
+  V.ns_limit = B.ns_limit;
+  *L.launches += 2;
+  return B.precision == 1
+             ? launch_coop(k_sweep<1, true, 3>, (unsigned)L.sweep_grid, kSweepThreads, sweep_smem(B.R),
+                           st, V)
+             : launch_coop(k_sweep<0, true, 2>, (unsigned)L.sweep_grid, kSweepThreads, sweep_smem(B.R),
+                           st, V);
 }
 
 cudaError_t batch_step_end(const BatchDev& B, const BatchLaunch& L, cudaStream_t st) {

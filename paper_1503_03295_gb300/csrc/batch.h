@@ -80,6 +80,7 @@ struct BatchDev {
   float4* s32;    // FP32-guarded form: FP32 copy of the spins, one (x, y, z, 0) per site
   SpinDf* sd;     // FP64 form: float-float copy
   SpinDf* propd;  // FP64 form: Ntot proposals in float-float
+  float4* prop32;  // FP32-guarded form: Ntot proposals in FP32
   uint8_t* acc;
   uint32_t* hslot;
   uint32_t* hcnt;
@@ -102,9 +103,7 @@ struct BatchDev {
   uint32_t* tile_cnt;  // pal_cap * ntiles + 1
   uint32_t* perm;      // Ntot, global sites sorted by (colour, global index)
   uint32_t* off;       // pal_cap + 1 class offsets
-  uint32_t* defer;     // Ntot
   double4_32a* prop;   // Ntot proposals {S', u} of the current MC step
-  uint32_t* dcnt;      // pal_cap
   uint32_t* bcnt;      // 32 x pal_cap KW bucket sizes per level
   unsigned long long* imask;  // Ntot per-level vertex records of the colouring kernel
   uint32_t* imeta;            // Ntot
@@ -140,6 +139,5 @@ int batch_kw_occupancy(int schedule, int R, unsigned pal);
 // kernel's shared-memory limit)
 cudaError_t batch_low_setup(int R, uint32_t gcap, int* blocks_per_sm, uint32_t* ecap);
 int batch_sweep_occupancy(int precision, int R);
-size_t batch_sweep_smem(int R);
 
 }  // namespace sco

@@ -84,6 +84,7 @@ void free_all(sco_batch* b) {
   cudaFree(B.s32);
   cudaFree(B.sd);
   cudaFree(B.propd);
+  cudaFree(B.prop32);
   cudaFree(B.acc);
   cudaFree(B.hslot);
   cudaFree(B.hcnt);
@@ -102,12 +103,10 @@ void free_all(sco_batch* b) {
   cudaFree(B.tile_cnt);
   cudaFree(B.perm);
   cudaFree(B.off);
-  cudaFree(B.defer);
   cudaFree(B.prop);
   cudaFree(B.imask);
   cudaFree(B.imeta);
   cudaFree(B.ilist);
-  cudaFree(B.dcnt);
   cudaFree(B.bcnt);
   cudaFree(b->L.scan_tmp);
   cudaFree(b->full.p);
@@ -124,14 +123,12 @@ cudaError_t alloc_palette(sco_batch* b, uint32_t pal) {
   cudaFree(B.used);
   cudaFree(B.tile_cnt);
   cudaFree(B.off);
-  cudaFree(B.dcnt);
   cudaFree(B.bcnt);
-  B.used = B.tile_cnt = B.off = B.dcnt = B.bcnt = nullptr;
+  B.used = B.tile_cnt = B.off = B.bcnt = nullptr;
   B.pal_cap = pal;
   cudaError_t e = cudaMalloc(&B.used, (size_t)b->R * (pal / 32) * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&B.tile_cnt, ((size_t)pal * B.ntiles + 1) * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&B.off, (pal + 1) * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&B.dcnt, pal * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&B.bcnt, (size_t)32 * pal * sizeof(uint32_t));
   const size_t need = std::max((size_t)B.Ntot + 1, (size_t)pal * B.ntiles + 1);
   if (e == cudaSuccess && need > b->scan_tmp_n) {
@@ -420,6 +417,7 @@ sco_status sco_batch_init(const sco_params* p, int32_t n, void* stream, sco_batc
     A(&B.propd, N * sizeof(SpinDf));
   } else {
     A(&B.s32, N * sizeof(float4));
+    A(&B.prop32, N * sizeof(float4));
   }
   A(&B.acc, N);
   A(&B.hslot, N * kSlotCap * sizeof(uint32_t));
@@ -438,7 +436,6 @@ sco_status sco_batch_init(const sco_params* p, int32_t n, void* stream, sco_batc
   A(&B.blk, N * sizeof(uint32_t));
   A(&B.colour, N * sizeof(uint32_t));
   A(&B.perm, N * sizeof(uint32_t));
-  A(&B.defer, N * sizeof(uint32_t));
   A(&B.prop, N * sizeof(double4_32a));
   A(&B.imask, N * sizeof(unsigned long long));
   A(&B.imeta, N * sizeof(uint32_t));

@@ -215,11 +215,59 @@ __host__ __device__ __forceinline__ df df_pair_y(const PairDf& t, const FieldDf&
   return df_fast(y.h, y.l);
 }
 
+// ---- the same pair term in plain FP32 (FP32-guarded form) --------------------------------
+// g = a1 S_b - a3 (S_b . d) d from FP32 spins and constants, y = bvm - S . g.  |error| <= kY32RelErr
+// a1 against the exact value of the FP64 spins: the spins' rounding (2^-25 per component) contributes
+// 12 2^-25 a1, the constants' and the 13 operations' below 40 2^-24 a1 (every intermediate is at most
+// 6 a1); measured 2^-20.6.
+constexpr float kY32RelErr = 0x1p-18f;
+__host__ __device__ __forceinline__ void f32_field(float a1, float a3, float fx, float fy, float bx,
+                                                   float by, float bz, float& gx, float& gy,
+                                                   float& gz) {
+  const float w = a3 * df_fma(bx, fx, df_fmul(by, fy));
+  gx = df_fma(a1, bx, -df_fmul(w, fx));
+  gy = df_fma(a1, by, -df_fmul(w, fy));
+  gz = a1 * bz;
+}
+__host__ __device__ __forceinline__ float f32_y(float bvm, float gx, float gy, float gz, float sx,
+                                                float sy, float sz) {
+  return df_fma(-sx, gx, df_fma(-sy, gy, df_fma(-sz, gz, bvm)));
+}
+// e^y = 2^k (1 + e0) for |y| < 8192, as df_exp_core (kNeg likewise); e0 by its series to r^8.
+template <bool kNeg>
+__host__ __device__ __forceinline__ float f32_exp_core(float y, int& k) {
+  const float t =
+      kNeg ? df_fma(y, kDfLog2e, 12582912.f) : df_fma(y, kDfLog2e, -0.1f) + 12582912.f;
+  const float kf = t - 12582912.f;
+  k = (int)df_bits(t) - 0x4B400000;
+  const float r = df_fma(-kf, kDfL2 + kDfL3, df_fma(-kf, kDfL1, y));
+  float w = df_fma(1.f / 40320.f, r, 1.f / 5040.f);
+  w = df_fma(w, r, 1.f / 720.f);
+  w = df_fma(w, r, 1.f / 120.f);
+  w = df_fma(w, r, 1.f / 24.f);
+  w = df_fma(w, r, 1.f / 6.f);
+  w = df_fma(w, r, 0.5f);
+  return df_fma(df_fmul(r, r), w, r);
+}
+// (e^y - 1) 2^-k for y >= 0, in (0, 1.42); relative error (given y) below kE32RelErr, measured
+// 2^-21.6 (y < 60)
+constexpr float kE32RelErr = 0x1p-20f;
+__host__ __device__ __forceinline__ float f32_expm1_scaled(float y, int& k) {
+  const float e = f32_exp_core<false>(y, k);
+  return (1.f - df_pow2_neg(k)) + e;
+}
+
 // p by a power of two into [1, 2) (p.h > 0 normal), the exponent added to e
 __device__ __forceinline__ void df_renorm(df& p, int& e) {
   const int b = __float_as_int(p.h), x = (b >> 23) - 127;
   p.h = __int_as_float(b - (x << 23));
   p.l *= __int_as_float((127 - x) << 23);
+  e += x;
+}
+
+__device__ __forceinline__ void f32_renorm(float& p, int& e) {
+  const int b = __float_as_int(p), x = (b >> 23) - 127;
+  p = __int_as_float(b - (x << 23));
   e += x;
 }
 

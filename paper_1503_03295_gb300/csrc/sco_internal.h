@@ -29,7 +29,7 @@ struct DevCounters {
   int ovf_full;                     // the switch wrote more half-edges than the overflow list holds
   double acc[8];                    // observable accumulators
   unsigned int lev_rounds[32];      // deepest dependency chain per KW level
-  unsigned int bar[2];              // grid barrier of the persistent colouring kernel
+  unsigned int bar[2];              // grid barrier of the persistent kernels
   unsigned int sw_next;             // next unclaimed site of the persistent switch kernel
 };
 
@@ -81,7 +81,7 @@ struct Table {
                              // (float-float)
   float4* xy32 = nullptr;    // by (|dx|, |dy|): FP32 copies {Dc, Vmax, 2 beta Vmax, q}
   Sw64* sw64 = nullptr;      // sweep, by (|dx|, |dy|): FP64 decision constants (see Sw64)
-  float4* sw32 = nullptr;    // the same in FP32 (with its own c0)
+  float4* sw32 = nullptr;    // FP32 sweep: {a1, a3, bvm, 0} of PairDf
   PairDf* pdf = nullptr;     // sweep, by (|dx|, |dy|): the FP64 form's pair constants in float-float
   void* pool = nullptr;      // the one allocation behind the temperature-dependent tables
   int32_t m_nn[2] = {-1, -1};
@@ -164,7 +164,6 @@ struct ColourBufs {
   uint32_t* hist;    // g + 1
   uint32_t* off;     // g + 1
   uint32_t* cursor;  // g
-  uint32_t* dcnt;    // g deferred sweep decisions per colour
   uint32_t* perm;    // N
   uint32_t* tile_cnt;  // (colour, tile, degree bin) counts (+1), scanned in place
   uint64_t* scan_tmp;
@@ -187,13 +186,24 @@ cudaError_t bucket_run(const DevParams& P, uint32_t g, const uint32_t* row_ptr, 
                        DevCounters* cnt, cudaStream_t st, int64_t* launches);
 
 // ---- sweep.cu ----
-// s32 (FP32-guarded form) or sd and propd (FP64 form): the working copies of the spins, and the
-// proposals of the step in float-float; the others may be null.
-cudaError_t sweep_run(const DevParams& P, const Table& t, double* s, float4* s32, SpinDf* sd,
-                      const uint32_t* row_ptr, const uint32_t* col, const uint32_t* perm,
-                      const uint32_t* off, uint32_t g, uint64_t step, int precision,
-                      uint8_t* acc, uint32_t* defer, uint32_t* dcnt, double4_32a* prop,
-                      SpinDf* propd, DevCounters* cnt, cudaStream_t st, int64_t* launches);
+// s32 and prop32 (FP32-guarded form) or sd and propd (FP64 form): the working copies of the spins and
+// the proposals of the step; the others are null.
+struct SweepBufs {
+  double* s;
+  float4* s32;
+  SpinDf* sd;
+  const uint32_t* row_ptr;
+  const uint32_t* col;
+  const uint32_t* perm;
+  const uint32_t* off;
+  double4_32a* prop;
+  SpinDf* propd;
+  float4* prop32;
+  uint8_t* acc;
+};
+cudaError_t sweep_run(const DevParams& P, const Table& t, const SweepBufs& b, uint32_t g,
+                      uint64_t step, int precision, DevCounters* cnt, unsigned long long ns_limit,
+                      cudaStream_t st, int64_t* launches);
 
 // ---- stats.cu ----
 // Graph diagnostics (see sco_get_graph_stats); copies 2 nb + 1 counts (survived, pairs, cross)

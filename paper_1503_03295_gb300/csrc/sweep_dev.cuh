@@ -15,6 +15,8 @@
 
 #include <cstdint>
 
+#include "batch.h"
+#include "grid_dev.cuh"
 #include "sco_internal.h"
 
 namespace sco {
@@ -32,7 +34,6 @@ struct SiteCtx {
 // products are renormalised by 2^kScale (exact) so that they never underflow.  The FP64 form's
 // first decision, accept_df, compares products of e^-x - 1 instead and takes no logarithm.
 constexpr int kScale64 = 600;
-constexpr int kScale32 = 60;
 
 // p by 2^600 on the exponent field when below 2^-600, counted in sc (a multiply would be issued
 // on every pair as a select); false for a subnormal or zero p (the decision then goes to the
@@ -181,88 +182,99 @@ __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t
   return 2;
 }
 
-// FP32 screen of the same decision: shadow spins (|dS| <= 2^-24 per component), FP32 table
-// constants, CUDA's single-precision expm1f / logf (<= 1 ulp; 4x margin: eps_f = 2^-21),
-// eps_r = 2^-23, and a compensated (Neumaier) sum of the V' - V terms.
-__device__ __forceinline__ int accept_fp32(const DevParams& P, const SiteCtx& c,
-                                           const float4* __restrict__ sw,
-                                           const float4* __restrict__ s32,
-                                           const uint32_t* __restrict__ row_ptr,
-                                           const uint32_t* __restrict__ col) {
-  if (c.u < 0x1p-100) return 2;
-  const float beta = P.beta_f;
-  const float ax = (float)c.S[0], ay = (float)c.S[1], az = (float)c.S[2];
-  const float nx = (float)c.Sn[0], ny = (float)c.Sn[1], nz = (float)c.Sn[2];
-  float sum = 0.f, comp = 0.f, sum_abs = 0.f, pz_o = 1.f, pz_n = 1.f, lin = 0.f, c0s = 0.f;
-  int sc_o = 0, sc_n = 0, n = 0;
-  const uint32_t e1 = row_ptr[c.i + 1];
-  for (uint32_t e = row_ptr[c.i]; e < e1; ++e) {
-    const uint32_t cj = col[e];
-    if (cj & kExchOnly) continue;
-    const int64_t j = cj;
-    const uint32_t yj = site_row((uint32_t)j, P);
-    const int32_t dx = (int32_t)((uint32_t)j - yj * (uint32_t)P.Lx) - c.xi;
-    const int32_t dy = (int32_t)yj - c.yi;
-    const float4 t =
-        __ldg(&sw[(int64_t)(dx < 0 ? -dx : dx) + (int64_t)P.Lx * (dy < 0 ? -dy : dy)]);
-    const float4 sj = s32[j];
-    const float bx = sj.x, by = sj.y, bz = sj.z;
-    const float fx = (float)dx, fy = (float)dy;
-    const float tp = t.y * (bx * fx + by * fy);
-    const float gx = t.x * bx - tp * fx;
-    const float gy = t.x * by - tp * fy;
-    const float gz = t.x * bz;
-    const float Vn = nx * gx + ny * gy + nz * gz;
-    const float Vo = ax * gx + ay * gy + az * gz;
-    const float xn = beta * Vn - t.z, xo = beta * Vo - t.z;
-    if (!(xn < 0.f) || !(xo < 0.f)) return 2;
-    const float zn = -expm1f(xn), zo = -expm1f(xo);
-    if (!(zn >= 0x1p-60f) || !(zo >= 0x1p-60f)) return 2;
-    // |dx| / z per pair (first order needs it small); FP32 reciprocal, 1.001 for its rounding
-    const float ln_ = (t.w + 0x1p-23f * -xn) * (1.001f * __frcp_rn(zn));
-    const float lo_ = (t.w + 0x1p-23f * -xo) * (1.001f * __frcp_rn(zo));
-    if (!(ln_ <= 0x1p-10f) || !(lo_ <= 0x1p-10f)) return 2;
-    lin += ln_ + lo_;
-    pz_n *= zn;
-    pz_o *= zo;
-    if (pz_n < 0x1p-60f) { pz_n *= 0x1p60f; ++sc_n; }
-    if (pz_o < 0x1p-60f) { pz_o *= 0x1p60f; ++sc_o; }
-    const float dv = Vn - Vo;
-    const float tsum = sum + dv;  // Neumaier compensated summation
-    comp += fabsf(sum) >= fabsf(dv) ? (sum - tsum) + dv : (dv - tsum) + sum;
-    sum = tsum;
-    sum_abs += fabsf(dv);
-    c0s += t.w;
+// The FP32-guarded form's screen: the same decision in plain FP32, from the FP32 spins and constants
+// (about 60 instructions per pair).  Bound as in accept_df, with kE32RelErr, c0 = kY32RelErr a1
+// (c0 / m < 2^((d >> 23) + 1 - 18), below 2^-6) and 2^-23 per product; it leaves about one site in
+// 10^4 to FP64.  N = {S', u}.
+template <int kG>
+__device__ __forceinline__ int accept_f32(const DevParams& P, int32_t xi, int32_t yi, float4 S,
+                                          float4 N, const float4* __restrict__ sw,
+                                          const float4* s32, const uint32_t* __restrict__ col,
+                                          uint32_t e0, uint32_t e1, uint32_t i, int sub) {
+  float pn = 1.f, po = 1.f;
+  int K = 0, n = 0, dmax = -0x40000000;
+  bool bad = false;
+  for (uint32_t e = e0 + sub; e < e1; e += kG) {
+    const uint32_t j = col[e];
+    if (j & kExchOnly) continue;
+    int32_t xj, yj;
+    site_xy(j, P, xj, yj);
+    const int32_t dx = xj - xi, dy = yj - yi;
+    const float4 b = s32[j];
+    const float4 t = __ldg(sw + (abs(dx) + (int64_t)P.Lx * abs(dy)));  // {a1, a3, bvm, 0}
+    float gx, gy, gz;
+    f32_field(t.x, t.y, (float)dx, (float)dy, b.x, b.y, b.z, gx, gy, gz);
+    const float yn = f32_y(t.z, gx, gy, gz, N.x, N.y, N.z);
+    const float yo = f32_y(t.z, gx, gy, gz, S.x, S.y, S.z);
+    if (!(fminf(yn, yo) > 0x1p-100f && fmaxf(yn, yo) < 8192.f)) {
+      bad = true;
+      continue;
+    }
+    int kn, ko;
+    const float mn = f32_expm1_scaled(yn, kn), mo = f32_expm1_scaled(yo, ko);
+    dmax = max(dmax, __float_as_int(t.x) - __float_as_int(fminf(mn, mo)));
+    pn *= mn;
+    po *= mo;
+    f32_renorm(pn, kn);
+    f32_renorm(po, ko);
+    K += ko - kn;
     ++n;
   }
-  float tex = 0.f, bex = 0.f;
+  if (kG > 1) {
+#pragma unroll
+    for (int o = kG / 2; o > 0; o >>= 1) {
+      pn *= __shfl_down_sync(0xffffffffu, pn, o, kG);
+      po *= __shfl_down_sync(0xffffffffu, po, o, kG);
+      K += __shfl_down_sync(0xffffffffu, K, o, kG);
+      n += __shfl_down_sync(0xffffffffu, n, o, kG);
+      dmax = max(dmax, __shfl_down_sync(0xffffffffu, dmax, o, kG));
+      bad |= __shfl_down_sync(0xffffffffu, (int)bad, o, kG) != 0;
+    }
+  }
+  if (sub != 0) return 0;
+  if (N.w == 0.f) return 1;  // u = 0 accepts outright
+  if (bad) return 2;
+  float bound = 0x1p-20f + (float)n * (2.f * kE32RelErr + 0x1p-22f);
+  if (n > 0) {
+    const int x = (dmax >> 23) + 1 - 18;
+    if (x > -6) return 2;
+    bound += 2.84f * (float)n * __int_as_float((max(x, -100) + 127) << 23);
+  }
+  float X = N.w * po;
   if (P.J != 0.0) {
-    float h0 = 0.f, h1 = 0.f, h2 = 0.f;
-    const int64_t nb[4] = {c.xi > 0 ? c.i - 1 : -1, c.xi + 1 < P.Lx ? c.i + 1 : -1,
-                           c.yi > 0 ? c.i - P.Lx : -1, c.yi + 1 < P.Ly ? c.i + P.Lx : -1};
+    float hx = 0.f, hy = 0.f, hz = 0.f;
+    const int32_t nb[4] = {xi > 0 ? -1 : 0, xi + 1 < P.Lx ? 1 : 0, yi > 0 ? -P.Lx : 0,
+                           yi + 1 < P.Ly ? P.Lx : 0};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      if (nb[q] < 0) continue;
-      const float4 sq = s32[nb[q]];
-      h0 += sq.x;
-      h1 += sq.y;
-      h2 += sq.z;
+      if (nb[q] == 0) continue;
+      const float4 b = s32[(int32_t)i + nb[q]];
+      hx += b.x;
+      hy += b.y;
+      hz += b.z;
     }
-    const float bj = P.bJ_f;
-    tex = -bj * ((nx - ax) * h0 + (ny - ay) * h1 + (nz - az) * h2);
-    bex = 0x1p-14f * fabsf(bj);
+    const float w = -P.bJ_f * ((N.x - S.x) * hx + (N.y - S.y) * hy + (N.z - S.z) * hz);
+    const float aj = fabsf(P.bJ_f);
+    if (!(aj < 512.f)) return 2;
+    int k;
+    const float e = w < 0.f ? f32_exp_core<true>(w, k) : f32_exp_core<false>(w, k);
+    X *= 1.f + e;
+    K += k;
+    // |w error|: 24 terms below 8 beta J in all, each off by less than 2^-21 relative
+    bound += kE32RelErr + 0x1p-17f * aj;
   }
-  const float lo = logf(pz_o), ln = logf(pz_n);
-  const float scale = (float)((sc_n - sc_o) * kScale32) * 0.693147182f;
-  const float lu = logf((float)c.u);
-  const float bdv = beta * (sum + comp);
-  const float mu = lu + ((bdv + tex) + ((lo - ln) + scale));
-  const float B = 2.0f * (2.0f * c0s * 1.001f + (float)(n + 2) * 0x1p-23f * beta * sum_abs +
-                          lin * 1.001f + n * (0x1p-19f + 0x1p-22f) +
-                          0x1p-21f * (fabsf(lo) + fabsf(ln)) + 0x1p-20f * fabsf(lu) + 0x1p-23f +
-                          bex + 0x1p-21f * (fabsf(scale) + fabsf(tex) + fabsf(bdv) + fabsf(mu)));
-  if (mu < -B) return 1;
-  if (mu > B) return 0;
+  bound *= 2.f;
+  if (!(bound < 0.25f)) return 2;
+  int kx = 0, kn = 0;
+  f32_renorm(X, kx);
+  f32_renorm(pn, kn);
+  K += kx - kn;
+  if (K >= 2) return 0;   // X 2^K >= 4 > 2 pn
+  if (K <= -2) return 1;  // X 2^K < 1/2 pn
+  const float D = X * (K == 0 ? 1.f : (K > 0 ? 2.f : 0.5f)) - pn;
+  const float lim = bound * pn;
+  if (D < -lim) return 1;
+  if (D > lim) return 0;
   return 2;
 }
 
@@ -271,15 +283,24 @@ __device__ __forceinline__ int accept_fp32(const DevParams& P, const SiteCtx& c,
 // The square root and the spin are computed once, after the attempts (whose count differs
 // between the lanes of a warp).
 __device__ __forceinline__ bool propose(const DevParams& P, SiteCtx& c, uint64_t step) {
-  double a1 = 0.0, a2 = 0.0, s = 0.0;
-  uint64_t wu = 0;
+  double a1, a2, s;
+  W4 w;
   bool ok = false;
   for (uint64_t a = 0; a < 64 && !ok; ++a) {
-    const W4 w = philox((uint64_t)c.i, step, a, kTagPropose, P.key0, P.key1);
-    ok = marsaglia_point(w.w[0], w.w[1], a1, a2, s);
-    wu = w.w[2];
+    w = philox((uint64_t)c.i, step, a, kTagPropose, P.key0, P.key1);
+    // 0 < s < 1 from the leading 24 bits of each word in FP32 (s off by less than 2^-20) unless it
+    // is within 2^-18 of either end: the lanes of a warp go through as many attempts as the
+    // unluckiest needs, and each cost three FP64 instructions (305 us for 5.3 million sites)
+    const float f1 = (float)((int)(w.w[0] >> 40) - (1 << 23)) * 0x1p-23f;
+    const float f2 = (float)((int)(w.w[1] >> 40) - (1 << 23)) * 0x1p-23f;
+    const float f = f1 * f1 + f2 * f2;
+    ok = f < 1.f;
+    if (fabsf(f - 0.5f) > 0.5f - 0x1p-18f && f < 1.f + 0x1p-18f)
+      ok = marsaglia_point(w.w[0], w.w[1], a1, a2, s);
   }
   if (!ok) return false;
+  marsaglia_point(w.w[0], w.w[1], a1, a2, s);
+  const uint64_t wu = w.w[2];
   marsaglia_spin(a1, a2, s, c.Sn[0], c.Sn[1], c.Sn[2]);
   c.u = u53(wu);
   return true;
@@ -305,18 +326,6 @@ __device__ __forceinline__ void load_site(const DevParams& P, SiteCtx& c, uint32
   c.S[0] = s[i];
   c.S[1] = s[P.N + i];
   c.S[2] = s[2 * P.N + i];
-}
-
-__device__ __forceinline__ void write_site(const DevParams& P, const SiteCtx& c, bool ok,
-                                           double* __restrict__ s, float4* __restrict__ s32,
-                                           uint8_t* __restrict__ acc) {
-  if (ok) {
-    s[c.i] = c.Sn[0];
-    s[P.N + c.i] = c.Sn[1];
-    s[2 * P.N + c.i] = c.Sn[2];
-    if (s32) s32[c.i] = make_float4((float)c.Sn[0], (float)c.Sn[1], (float)c.Sn[2], 0.f);
-  }
-  acc[c.i] = ok ? 1 : 0;
 }
 
 __device__ __forceinline__ double warp_sum_d(double v) {
@@ -466,6 +475,245 @@ __device__ bool accept_dd_warp(const DevParams& P, const SiteCtx& c,
   }
   const dd lu = dd_log(dd_from(c.u), ln2);
   return dd_lt(dd_add(lu, sum), dd_from(0.0));
+}
+
+
+// ---- the sweep of a whole MC step, one lattice or a batch ----------------------------------
+// One persistent cooperative kernel walks the colours in ascending order, one grid barrier apart
+// (a launch per colour took 6 to 7 us for a small class, most of it launch and drain).  The trailing
+// colours that hold at most kTailSites sites each are left to block 0, one __syncthreads apart.
+constexpr int kSweepThreads = 512;
+constexpr uint32_t kTailSites = 64;
+
+struct SweepView {
+  int R;                       // lattices
+  const uint32_t* site_start;  // R + 1 (batch)
+  const RepDesc* desc;         // R (batch)
+  DevParams P;                 // one lattice: its parameters and tables
+  const PairDf* pdf;
+  const float4* sw32;
+  const Sw64* sw;
+  double* s;
+  float4* s32;
+  SpinDf* sd;
+  const uint32_t* row_ptr;
+  const uint32_t* col;
+  const uint32_t* perm;        // sites by colour, global indices
+  const uint32_t* off;         // class starts, g + 1
+  const double4_32a* prop;     // proposals {S', u} by global site, FP64
+  const SpinDf* propd;         // and in float-float (FP64 form)
+  const float4* prop32;        // or FP32 (FP32-guarded form)
+  uint8_t* acc;
+  DevCounters* cnt;            // R
+  uint32_t g;                  // colours
+  const unsigned* gmax;        // or on the device (batch)
+  unsigned* bar;
+  int* status;
+  const int* halt;             // optional: nonzero on entry -> return at once
+  unsigned long long ns_limit;
+};
+
+// One site's decision in FP64 then double-double by a whole warp, for the sites that the first
+// decision leaves open: a function of its own, so that its registers stay out of the sweep.
+__device__ __noinline__ bool settle_site(const DevParams& P, uint32_t i,
+                                         const Sw64* __restrict__ sw, const double* s,
+                                         const uint32_t* __restrict__ row_ptr,
+                                         const uint32_t* __restrict__ col,
+                                         const double4_32a* __restrict__ prop, int lane,
+                                         unsigned& ndd) {
+  SiteCtx c;
+  load_site(P, c, i, s);
+  take_proposal(c, prop);
+  int d = accept_fp64_warp(P, c, sw, s, row_ptr, col, lane);
+  if (d == 2) {
+    ++ndd;
+    d = accept_dd_warp(P, c, s, row_ptr, col, lane) ? 1 : 0;
+  }
+  return d == 1;
+}
+
+// The n sites perm[b ..], kG lanes per site, warps w, w + nw, ...; undecided sites are settled at once
+// by their warp.  sbase: site bases in shared memory (batch); sg: counters of screened-out and
+// double-double decisions (batch: per lattice, one lattice: none) beside n32 and ndd.
+template <int kPrec, bool kBatch, int kG>
+__device__ __forceinline__ void sweep_class(const SweepView& V, const uint32_t* sbase, uint32_t* sg,
+                                            uint32_t b, uint32_t n, uint32_t w, uint32_t nw,
+                                            unsigned& n32, unsigned& ndd) {
+  constexpr uint32_t kSites = 32 / kG;
+  const int lane = threadIdx.x & 31, sub = lane % kG;
+  for (uint32_t q = w * kSites; q < n; q += nw * kSites) {
+    const uint32_t idx = q + lane / kG;
+    uint32_t gs = 0, base = 0, e0 = 0, e1 = 0;
+    int r = 0;
+    if (idx < n) {
+      gs = V.perm[b + idx];
+      if (kBatch) {
+        r = find_le(sbase, V.R, gs);
+        base = sbase[r];
+      }
+    }
+    const RepDesc* dr = kBatch ? V.desc + r : nullptr;
+    const DevParams& P = kBatch ? dr->P : V.P;
+    const uint32_t i = gs - base;
+    int32_t xi, yi;
+    site_xy(i, P, xi, yi);
+    SpinDf Nd;
+    float4 N4;
+    bool move;
+    int d;
+    if (kPrec == 0) {
+      SpinDf S;
+      Nd.u_h = -1.f;
+      if (idx < n) Nd = load32(V.propd + gs);
+      move = Nd.u_h >= 0.f;
+      if (move) {
+        e0 = V.row_ptr[gs];
+        e1 = V.row_ptr[gs + 1];
+        S = load32(V.sd + gs);
+      }
+      d = accept_df<kG>(P, xi, yi, S, Nd, kBatch ? dr->pdf : V.pdf, V.sd + base, V.col, e0, e1, i,
+                        sub);
+    } else {
+      float4 S;
+      N4.w = -1.f;
+      if (idx < n) N4 = V.prop32[gs];
+      move = N4.w >= 0.f;
+      if (move) {
+        e0 = V.row_ptr[gs];
+        e1 = V.row_ptr[gs + 1];
+        S = V.s32[gs];
+      }
+      d = accept_f32<kG>(P, xi, yi, S, N4, kBatch ? dr->sw32 : V.sw32, V.s32 + base, V.col, e0, e1,
+                         i, sub);
+    }
+    const bool mine = sub == 0 && idx < n;
+    if (!mine || !move) d = 0;
+    for (unsigned open = __ballot_sync(0xffffffffu, d == 2); open != 0; open &= open - 1) {
+      const int src = __ffs(open) - 1;
+      const uint32_t gi = __shfl_sync(0xffffffffu, gs, src);
+      uint32_t bi = 0;
+      int ri = 0;
+      if (kBatch) {
+        ri = find_le(sbase, V.R, gi);
+        bi = sbase[ri];
+      }
+      const RepDesc* di = kBatch ? V.desc + ri : nullptr;
+      unsigned dd = 0;
+      const bool ok = settle_site(kBatch ? di->P : V.P, gi - bi, kBatch ? di->sw64 : V.sw,
+                                  V.s + 3 * (size_t)bi, V.row_ptr + bi, V.col, V.prop + bi, lane, dd);
+      if (lane == src) {
+        d = ok ? 1 : 0;
+        if (kBatch) {
+          if (kPrec == 1) atomicAdd(&sg[2 * ri], 1u);
+          if (dd) atomicAdd(&sg[2 * ri + 1], dd);
+        } else {
+          n32 += kPrec == 1 ? 1u : 0u;
+          ndd += dd;
+        }
+      }
+    }
+    if (mine) {
+      if (d == 1) {
+        const double4_32a v = V.prop[gs];
+        double* s = V.s + 3 * (size_t)base;
+        s[i] = v.x;
+        s[P.N + i] = v.y;
+        s[2 * P.N + i] = v.z;
+        if (kPrec == 0) V.sd[gs] = Nd;
+        else V.s32[gs] = make_float4(N4.x, N4.y, N4.z, 0.f);
+      }
+      V.acc[gs] = d == 1 ? 1 : 0;
+    }
+  }
+}
+
+// Lanes per site: 2 while the class gives every second lane a site (one lane per site took 2.37 ms
+// per step at L = 2304 in the FP64 form, two 2.20, four 2.28), 8 and 32 below, where the class would
+// leave lanes idle and a row's serial chain sets the time.
+template <int kPrec, bool kBatch>
+__device__ __forceinline__ void sweep_tiers(const SweepView& V, const uint32_t* sbase, uint32_t* sg,
+                                            uint32_t b, uint32_t n, uint32_t w, uint32_t nw,
+                                            unsigned& n32, unsigned& ndd) {
+  const uint32_t nth = nw * 32;
+  if (n >= nth / 2) sweep_class<kPrec, kBatch, 2>(V, sbase, sg, b, n, w, nw, n32, ndd);
+  else if (n >= nth / 32) sweep_class<kPrec, kBatch, 8>(V, sbase, sg, b, n, w, nw, n32, ndd);
+  else sweep_class<kPrec, kBatch, 32>(V, sbase, sg, b, n, w, nw, n32, ndd);
+}
+
+inline size_t sweep_smem(int R) { return (size_t)(3 * R + 1) * sizeof(uint32_t); }
+
+template <int kPrec, bool kBatch, int kBlocks>
+__global__ void __launch_bounds__(kSweepThreads, kBlocks) k_sweep(const __grid_constant__ SweepView V) {
+  __shared__ int s_halt;
+  __shared__ unsigned s_tail;
+  if (threadIdx.x == 0) {
+    s_halt = V.halt ? ld_status(V.halt) : 0;
+    s_tail = 0;
+  }
+  __syncthreads();
+  if (s_halt) return;
+  extern __shared__ uint32_t wsm[];
+  uint32_t* sbase = wsm;         // R + 1 (batch)
+  uint32_t* sg = wsm + V.R + 1;  // 2 R (batch)
+  if (kBatch) {
+    for (int r = threadIdx.x; r <= V.R; r += blockDim.x) sbase[r] = V.site_start[r];
+    for (int r = threadIdx.x; r < 2 * V.R; r += blockDim.x) sg[r] = 0;
+  }
+  const uint32_t g = V.gmax ? *V.gmax : V.g;
+  for (uint32_t c = threadIdx.x; c < g; c += blockDim.x)
+    if (V.off[c + 1] - V.off[c] > kTailSites) atomicMax(&s_tail, c + 1);
+  __syncthreads();
+  const uint32_t tail = s_tail;  // colours from here on are small
+  const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  unsigned n32 = 0, ndd = 0;
+  bool ok = true;
+  uint32_t b = V.off[0];
+  for (uint32_t c = 0; c < tail && ok; ++c) {
+    const uint32_t e = V.off[c + 1];
+    if (e > b) {
+      sweep_tiers<kPrec, kBatch>(V, sbase, sg, b, e - b, w, (gridDim.x * blockDim.x) >> 5, n32, ndd);
+      if (gridDim.x > 1) ok = grid_sync(V.bar, V.status, V.ns_limit);
+      else __syncthreads();
+    }
+    b = e;
+  }
+  if (blockIdx.x == 0 && ok) {
+    for (uint32_t c = tail; c < g; ++c) {
+      const uint32_t e = V.off[c + 1];
+      if (e > b) {
+        sweep_tiers<kPrec, kBatch>(V, sbase, sg, b, e - b, w, kSweepThreads / 32, n32, ndd);
+        __syncthreads();
+      }
+      b = e;
+    }
+  }
+  if (kBatch) {
+    __syncthreads();
+    for (int r = threadIdx.x; r < V.R; r += blockDim.x) {
+      if (sg[2 * r]) atomicAdd(&V.cnt[r].guard_fp32, (unsigned long long)sg[2 * r]);
+      if (sg[2 * r + 1]) atomicAdd(&V.cnt[r].guard_fp64, (unsigned long long)sg[2 * r + 1]);
+    }
+  } else {
+    if (n32) atomicAdd(&V.cnt->guard_fp32, (unsigned long long)n32);
+    if (ndd) atomicAdd(&V.cnt->guard_fp64, (unsigned long long)ndd);
+  }
+}
+
+// A site's proposal for MC step `step` in the forms the sweep reads (see take_proposal).
+__device__ __forceinline__ void write_proposal(const DevParams& P, uint64_t step, uint32_t i,
+                                               double4_32a* prop, SpinDf* propd, float4* prop32) {
+  SiteCtx c;
+  c.i = i;
+  const bool ok = propose(P, c, step);
+  *prop = ok ? make_double4_32a(c.Sn[0], c.Sn[1], c.Sn[2], c.u)
+             : make_double4_32a(0.0, 0.0, 1.0, -1.0);
+  if (propd) {
+    SpinDf d = spin_df(c.Sn[0], c.Sn[1], c.Sn[2], c.u);
+    if (!ok) d.u_h = -1.f;
+    *propd = d;
+  }
+  if (prop32)
+    *prop32 = make_float4((float)c.Sn[0], (float)c.Sn[1], (float)c.Sn[2], ok ? (float)c.u : -1.f);
 }
 
 }  // namespace

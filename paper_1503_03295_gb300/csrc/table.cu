@@ -72,8 +72,7 @@ __global__ void k_hazard(int64_t K, const uint32_t* __restrict__ disp, uint64_t*
 // so x = beta V - fl(beta Vmax) = S_i . f - bvm; c0 bounds the part of |x error| that does not
 // scale with |x|: |beta dV| <= 2^-46 beta Dc r^2 (FP64 products, the rounded beta-scaled
 // constants) plus 2^-51 beta Vmax (fl(beta Vmax)), plus 2^-52 (2 beta Vmax) for the rounding of
-// x itself (|x| <= 2 beta Vmax).  FP32 (float4 {A1, A3, beta Vmax, c0}): V(S) = S.f with
-// f = A1 S_j - A3 (S_j.d) d, |dV| <= 2^-16 Dc r^2 (shadow spins, FP32 constants).
+// x itself (|x| <= 2 beta Vmax).
 __global__ void k_xy(int32_t Lx, int32_t Ly, double D, double beta, double2* __restrict__ xy,
                      float2* __restrict__ qdf, float4* __restrict__ xy32,
                      Sw64* __restrict__ sw64, float4* __restrict__ sw32,
@@ -107,8 +106,7 @@ __global__ void k_xy(int32_t Lx, int32_t Ly, double D, double beta, double2* __r
   sw64[q] = t;
   const df d1 = df_split_const(t.a1), d3 = df_split_const(a3b), dv = df_split_const(bvm);
   pdf[q] = PairDf{d1.h, d1.l, d3.h, d3.l, dv.h, dv.l, (float)ax, (float)ay};
-  const double c32 = beta * (0x1p-16 * dc * (double)r2) + 0x1p-21 * bvm;
-  sw32[q] = make_float4((float)a1, (float)a3, (float)bvm, (float)(c32 * (1.0 + 0x1p-20)));
+  sw32[q] = make_float4((float)t.a1, (float)a3b, (float)bvm, 0.f);
 }
 
 // E_m = exp(-beta D 2^-58 W_m) as bits: the candidate process of the switch has rate

@@ -18,7 +18,7 @@ int main() {
   std::mt19937_64 g(7);
   std::uniform_real_distribution<double> U(0, 1);
   std::normal_distribution<double> G(0, 1);
-  L em = 0, ep = 0, ey = 0;
+  L em = 0, ep = 0, ey = 0, fm = 0, fy = 0;
   for (long i = 0; i < 3000000; ++i) {
     const double y0 = i % 4 == 0 ? U(g) * 0.42 : i % 4 == 1 ? U(g) * 20
                     : i % 4 == 2 ? std::exp(-U(g) * 60) : std::exp(U(g) * 9);
@@ -30,6 +30,12 @@ int main() {
     // given y: y itself to 2^-42 of its size (ln 2 in three parts)
     const L x = k == 0 ? expm1l(Y) : expl(Y - k * logl(2.0L)) - ldexpl(1, -k);
     em = fmaxl(em, fabsl((L)m.h + m.l - x) - Y * 0x1p-42L > 0 ? fabsl(((L)m.h + m.l - x) / x) : 0);
+    {
+      int kf;
+      const float m32 = f32_expm1_scaled(h, kf);
+      const L H = h, x32 = kf == 0 ? expm1l(H) : expl(H - kf * logl(2.0L)) - ldexpl(1, -kf);
+      if (h < 60.f) fm = fmaxl(fm, fabsl((m32 - x32) / x32));
+    }
     ep = fmaxl(ep, fabsl(((L)p.h + p.l + expm1l(-Y)) / expm1l(-Y)));
   }
   for (long i = 0; i < 1000000; ++i) {
@@ -59,9 +65,15 @@ int main() {
     const L ss = (L)S[0][0] * S[1][0] + (L)S[0][1] * S[1][1] + (L)S[0][2] * S[1][2];
     const L pa = (L)S[0][0] * dx + (L)S[0][1] * dy, pb = (L)S[1][0] * dx + (L)S[1][1] * dy;
     const L V = (L)c * ((L)r2 * ss - 3 * pa * pb);
+    float gx, gy, gz;
+    f32_field((float)a1, (float)a3, t.ax, t.ay, (float)S[1][0], (float)S[1][1], (float)S[1][2], gx, gy,
+              gz);
+    const float y32 = f32_y((float)bvm, gx, gy, gz, (float)S[0][0], (float)S[0][1], (float)S[0][2]);
+    fy = fmaxl(fy, fabsl((L)y32 - (L)beta * ((L)A * 0x1p-59L - V)) / (L)a1);
     ey = fmaxl(ey, fabsl((L)y.h + y.l - (L)beta * ((L)A * 0x1p-59L - V)) / (L)a1);
   }
-  std::printf("%.3f %.3f %.3f\n", (double)log2l(em), (double)log2l(ep), (double)log2l(ey));
+  std::printf("%.3f %.3f %.3f %.3f %.3f\n", (double)log2l(em), (double)log2l(ep), (double)log2l(ey),
+              (double)log2l(fm), (double)log2l(fy));
 }
 """
 
@@ -76,7 +88,10 @@ def test_bounds(tmp_path):
     src.write_text(SRC)
     subprocess.run([nvcc, "-std=c++17", "-O2", "-Xcompiler", "-ffp-contract=off", "-I", _build.CSRC,
                     "-o", str(exe), str(src)], check=True, capture_output=True)
-    em, ep, ey = map(float, subprocess.run([str(exe)], capture_output=True, check=True,
-                                           text=True).stdout.split())
+    em, ep, ey, fm, fy = map(float, subprocess.run([str(exe)], capture_output=True, check=True,
+                                                   text=True).stdout.split())
     # 2^-31: kDfExpRelErr (relative, e^y - 1 and 1 - e^-y); 2^-40: kYRelErr (of a1)
     assert em <= -31.0 and ep <= -31.0 and ey <= -40.0, (em, ep, ey)
+    # the plain FP32 terms: 2^-20 kE32RelErr, 2^-18 kY32RelErr
+    assert fm <= -20.0 and fy <= -18.0, (fm, fy)
+    print(em, ep, ey, fm, fy)

@@ -1,5 +1,6 @@
-"""The FP64 form's float-float sweep against the oracle where its dispatch changes: lanes per site
-by class size, pairs and exchange factors outside its range (settled in FP64 / double-double)."""
+"""The sweeps of both precisions against the oracle where their dispatch changes: lanes per site by
+class size, the trailing colours left to one block, one block for a small lattice, pairs and exchange
+factors outside the range of the first decision (settled in FP64 / double-double)."""
 import numpy as np
 import pytest
 
@@ -19,11 +20,17 @@ pytestmark = pytest.mark.gpu
     (31, 17, 0.4, -0.5, 1.0, 3),      # antiferromagnetic exchange
     (16, 16, 3.0, 0.0, 1e-9, 2),      # pair constants near 1e-9
     (1, 37, 0.3, 0.0, 1.0, 3),        # a chain (Lx = 1)
+    (45, 45, 0.5, 1.0, 0.1, 3), (46, 45, 0.5, 1.0, 0.1, 3),  # one block of the sweep, and more
 ])
 def test_sweep_matches_oracle(Lx, Ly, T, J, D, n):
-    g = sco.Lattice(sco.make_params(Lx, Ly, T=T, J=J, D=D, seed=11))
     o = O.Chain(O.make_params(Lx, Ly, T=T, J=J, D=D, seed=11))
-    g.sweep(n)
     o.sweep(n)
-    assert np.array_equal(g.accepts(), o.accepts())
-    assert np.array_equal(g.spins(), o.spins())
+    for prec in (sco.FP64, sco.FP32_GUARDED):
+        p = sco.make_params(Lx, Ly, T=T, J=J, D=D, seed=11, precision=prec)
+        g = sco.Lattice(p)
+        g.sweep(n)
+        assert np.array_equal(g.accepts(), o.accepts()), prec
+        assert np.array_equal(g.spins(), o.spins()), prec
+        with sco.Batch([p, sco.make_params(16, T=0.5, precision=prec)]) as b:
+            b.run(n)
+            assert np.array_equal(b.spins(0), o.spins()), prec
