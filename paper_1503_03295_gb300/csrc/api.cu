@@ -236,7 +236,7 @@ sco_status do_switch(sco_ctx* c, uint32_t epoch, const double* src, const float4
   c->nnz = c->hcnt->nnz;
   SCO_TRY(grow(c->col, c->col_cap, c->nnz > 0 ? c->nnz : 1));
   // rows are left unsorted (their order changes no result); getters sort their copies
-  SCO_TRY(csr_fill(c->P, c->sw, c->row_ptr, c->col, c->hcnt->ovf_n > 0, false, c->cnt, c->st,
+  SCO_TRY(csr_fill(c->P, c->sw, c->row_ptr, c->col, c->hcnt->ovf_n > 0, c->cnt, c->st,
                    &c->launches));
   c->dip_valid = false;
   c->g = c->hcnt->max_degree + 1;
@@ -532,7 +532,7 @@ sco_status sco_get_graph(sco_ctx* c, uint32_t* row_ptr, uint32_t* col, uint32_t*
     // the device rows are unsorted: copy, sort every row by neighbour index, then read back
     uint32_t* tmp = nullptr;
     SCO_TRY(cudaMalloc(&tmp, c->nnz * sizeof(uint32_t)));
-    cudaError_t e = csr_sorted_copy(c->P, c->row_ptr, c->col, tmp, c->nnz, c->cnt, c->st,
+    cudaError_t e = csr_sorted_copy(c->P, c->row_ptr, c->col, 0u, tmp, c->nnz, c->cnt, c->st,
                                     &c->launches);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(col, tmp, c->nnz * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->st);

@@ -616,6 +616,8 @@ sco_status sco_batch_observables(sco_batch* b, int32_t r, sco_obs* o, int32_t wa
   const DevParams& P = b->P[r];
   const uint32_t base = b->site_start[r];
   const bool full = want_full && P.N <= 65536;
+  if (b->have_graph)
+    SCO_TRY(dip_degree_run(P, b->B.row_ptr + base, b->B.col, b->B.cnt + r, b->st, &b->launches));
   SCO_TRY(observables_run(P, b->B.s + 3 * (size_t)base, b->B.row_ptr + base, b->B.col,
                           b->xy[r].xy, b->have_graph, full, &b->full, b->B.cnt + r, b->st,
                           &b->launches));
@@ -696,9 +698,19 @@ sco_status sco_batch_get_graph(sco_batch* b, int32_t r, uint32_t* row_ptr, uint3
   const uint32_t e0 = rp[0];
   if (row_ptr)
     for (size_t i = 0; i <= N; ++i) row_ptr[i] = rp[i] - e0;
-  if (col && rp[N] > e0)
-    SCO_TRY(cudaMemcpyAsync(col, b->B.col + e0, (size_t)(rp[N] - e0) * sizeof(uint32_t),
-                            cudaMemcpyDeviceToHost, b->st));
+  if (col && rp[N] > e0) {
+    // the device rows are unsorted: copy, sort every row by neighbour index, then read back
+    const size_t nnz = rp[N] - e0;
+    uint32_t* tmp = nullptr;
+    SCO_TRY(cudaMalloc(&tmp, nnz * sizeof(uint32_t)));
+    cudaError_t e = csr_sorted_copy(b->P[r], b->B.row_ptr + base, b->B.col, e0, tmp, nnz,
+                                    b->B.cnt + r, b->st, &b->launches);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(col, tmp, nnz * sizeof(uint32_t), cudaMemcpyDeviceToHost, b->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
+    cudaFree(tmp);
+    SCO_TRY(e);
+  }
   if (colour)
     SCO_TRY(cudaMemcpyAsync(colour, b->B.colour + base, N * sizeof(uint32_t),
                             cudaMemcpyDeviceToHost, b->st));

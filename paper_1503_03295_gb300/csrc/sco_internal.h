@@ -143,16 +143,15 @@ cudaError_t switch_run(const DevParams& P, const Table& t, const double* s, cons
                        cudaStream_t st, int64_t* launches);
 cudaError_t csr_scan(const DevParams& P, SwitchBufs& b, uint32_t* row_ptr, DevCounters* cnt,
                      cudaStream_t st, int64_t* launches);
-// sort_rows: sort every row by neighbour index and record the largest dipolar degree; else a row
-// holds its lower neighbours in the order of their atomic slots, then its upper ones in switching
-// order (no result depends on the order inside a row).
+// A row holds its lower neighbours in the order of their atomic slots, then its upper ones in
+// switching order (no result depends on the order inside a row).
 cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, const uint32_t* row_ptr,
-                     uint32_t* col, bool has_overflow, bool sort_rows, DevCounters* cnt,
-                     cudaStream_t st, int64_t* launches);
-// out = col with every row sorted by neighbour index (the documented layout of the getters);
-// also records the largest dipolar degree in cnt.
+                     uint32_t* col, bool has_overflow, DevCounters* cnt, cudaStream_t st,
+                     int64_t* launches);
+// out = col[first ..] with every row sorted by neighbour index (the documented layout of the
+// getters), row_ptr[0] = first; also records the largest dipolar degree in cnt.
 cudaError_t csr_sorted_copy(const DevParams& P, const uint32_t* row_ptr, const uint32_t* col,
-                            uint32_t* out, uint64_t nnz, DevCounters* cnt, cudaStream_t st,
+                            uint32_t first, uint32_t* out, uint64_t nnz, DevCounters* cnt, cudaStream_t st,
                             int64_t* launches);
 
 // ---- colour.cu ----

@@ -95,25 +95,30 @@ __global__ void __launch_bounds__(256) k_site_obs(DevParams P, const double* __r
 }
 
 // Pseudointeraction energy H' of Eq. (4) over surviving dipolar pairs (each once, i < j):
-// Vbar = V - beta^-1 log(1 - exp(beta (V - Vmax))).  acc[5].
+// Vbar = V - beta^-1 log(1 - exp(beta (V - Vmax))).  acc[5].  kG lanes per site: a term is a chain of
+// about 150 FP64 instructions, so a small lattice takes as long as the longest row of a lane
+// (L = 16: 154 us with one lane per site, 31 us with 32).
+template <int kG>
 __global__ void __launch_bounds__(256) k_pair_obs(DevParams P, const double* __restrict__ s,
                                                   const uint32_t* __restrict__ row_ptr,
                                                   const uint32_t* __restrict__ col,
                                                   const double2* __restrict__ xy,
                                                   double* __restrict__ acc) {
   double v[1] = {0.0};
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < P.N;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t yi = (int32_t)site_row((uint32_t)i, P);
-    const int32_t xi = (int32_t)((uint32_t)i - (uint32_t)yi * (uint32_t)P.Lx);
+  const int sub = threadIdx.x % kG;
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kG; i < P.N;
+       i += (int64_t)gridDim.x * blockDim.x / kG) {
+    int32_t xi, yi;
+    site_xy((uint32_t)i, P, xi, yi);
     const double ax = s[i], ay = s[P.N + i], az = s[2 * P.N + i];
-    for (uint32_t e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
+    for (uint32_t e = row_ptr[i] + sub; e < row_ptr[i + 1]; e += kG) {
       const uint32_t c = col[e];
       if (c & kExchOnly) continue;
       const int64_t j = c;
       if (j <= i) continue;
-      const uint32_t yj = site_row((uint32_t)j, P);
-      const int32_t dx = (int32_t)((uint32_t)j - yj * (uint32_t)P.Lx) - xi, dy = (int32_t)yj - yi;
+      int32_t xj, yj;
+      site_xy(c, P, xj, yj);
+      const int32_t dx = xj - xi, dy = yj - yi;
       const double2 t = xy[(int64_t)(dx < 0 ? -dx : dx) + (int64_t)P.Lx * (dy < 0 ? -dy : dy)];
       const double V = pair_V(t.x, (double)dx * dx + (double)dy * dy, ax, ay, az, s[j],
                               s[P.N + j], s[2 * P.N + j], (double)dx, (double)dy);
@@ -207,7 +212,11 @@ cudaError_t observables_run(const DevParams& P, const double* s, const uint32_t*
   k_site_obs<<<nb, 256, 0, st>>>(P, s, cnt->acc);
   ++*launches;
   if (have_graph) {
-    k_pair_obs<<<nb, 256, 0, st>>>(P, s, row_ptr, col, xy, cnt->acc);
+    // lanes per site: as many as leave the grid's threads a site each
+    const int64_t threads = (int64_t)nb * 256;
+    if (P.N * 32 <= threads) k_pair_obs<32><<<nb, 256, 0, st>>>(P, s, row_ptr, col, xy, cnt->acc);
+    else if (P.N * 8 <= threads) k_pair_obs<8><<<nb, 256, 0, st>>>(P, s, row_ptr, col, xy, cnt->acc);
+    else k_pair_obs<1><<<nb, 256, 0, st>>>(P, s, row_ptr, col, xy, cnt->acc);
     ++*launches;
   }
   if (want_full && full_energy_fft_ok(P)) {

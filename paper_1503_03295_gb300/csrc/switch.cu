@@ -9,9 +9,7 @@ namespace sco {
 
 namespace {
 
-// Persistent: each warp claims 32 sites at a time from a global counter, and a lane whose walk
-// ends takes up the next claimed site at once, so that the lanes of a warp stay busy although
-// the number of candidates differs from site to site (Poisson, mean about 14 at T = 0.6D).
+// Persistent: the warps claim the lattice's sites from a global counter (switch_range).
 // Bound by instruction issue (57% busy, 21 of 32 lanes active) and the latency of the neighbours'
 // records.  Four blocks per SM (64 registers; three and five measured 0.3 and 0.25 ms slower at
 // L = 2304).  With the guided search, the float-float survival test and two candidates per step the
@@ -27,46 +25,10 @@ __global__ void __launch_bounds__(256, 4) k_switch(const __grid_constant__ DevPa
   const NearTable T = near_table(S, sh);
   __syncthreads();
   const SwitchOut o{b.hslot, b.indeg, b.ovf, b.ovf_cap, &cnt->ovf_n, &cnt->ovf_full};
-  const uint32_t N = (uint32_t)P.N;
-  const unsigned lane = threadIdx.x & 31u;
-  const unsigned below = (1u << lane) - 1u;
-  unsigned n_half = 0, n_dip = 0, ghits = 0, g32 = 0;
-  SiteWalk<PREC> a;
-  bool active = false, drained = false;  // drained, pool and pool_n are warp-uniform
-  uint32_t pool = 0, pool_n = 0;
-  for (;;) {
-    unsigned need = __ballot_sync(0xffffffffu, !active);
-    while (need != 0u && !drained) {
-      if (pool_n == 0u) {
-        uint32_t base = 0;
-        if (lane == 0) base = atomicAdd(&cnt->sw_next, 32u);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (base >= N) {
-          drained = true;
-          break;
-        }
-        pool = base;
-        pool_n = min(32u, N - base);
-      }
-      const uint32_t take = min((uint32_t)__popc(need), pool_n);
-      const uint32_t rank = (uint32_t)__popc(need & below);
-      if (!active && rank < take) {
-        walk_begin<PREC>(P, in, pool + rank, pool + rank, a);
-        active = true;
-      }
-      pool += take;
-      pool_n -= take;
-      need = __ballot_sync(0xffffffffu, !active);
-    }
-    const unsigned act = __ballot_sync(0xffffffffu, active);
-    if (act == 0u) break;
-    if (active && !walk_step<PREC>(P, T, in, epoch, mnn0, mnn1, o, a, n_dip, ghits, g32, act)) {
-      const uint32_t n_out = walk_end<PREC>(P, mnn0, mnn1, o, a);
-      b.hcnt[a.i] = n_out;
-      n_half += n_out;
-      active = false;
-    }
-  }
+  unsigned n_dip = 0, ghits = 0, g32 = 0;
+  const unsigned n_half =
+      switch_range<PREC, true>(P, T, in, epoch, mnn0, mnn1, &cnt->sw_next, (uint32_t)P.N, 0u, b.hcnt, o,
+                         n_dip, ghits, g32);
   const unsigned long long nh = warp_sum_u64(n_half), ndp = warp_sum_u64(n_dip);
   const unsigned long long gh = warp_sum_u64(ghits), gl = warp_sum_u64(g32);
   if ((threadIdx.x & 31) == 0) {
@@ -141,11 +103,11 @@ __global__ void k_fill_ovf(unsigned long long n, const uint32_t* __restrict__ ov
   col[lo] = i | (jv & kExchOnly);
 }
 
-__global__ void k_rowsort(int64_t N, const uint32_t* __restrict__ row_ptr,
+__global__ void k_rowsort(int64_t N, const uint32_t* __restrict__ row_ptr, uint32_t first,
                           uint32_t* __restrict__ col, DevCounters* __restrict__ cnt) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   unsigned nd = 0;
-  if (i < N) nd = sort_row(col + row_ptr[i], row_ptr[i + 1] - row_ptr[i]);
+  if (i < N) nd = sort_row(col + (row_ptr[i] - first), row_ptr[i + 1] - row_ptr[i]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) nd = max(nd, __shfl_down_sync(0xffffffffu, nd, o));
   if ((threadIdx.x & 31) == 0 && nd) atomicMax(&cnt->max_degree_dip, nd);
@@ -191,8 +153,8 @@ cudaError_t csr_scan(const DevParams& P, SwitchBufs& b, uint32_t* row_ptr, DevCo
 }
 
 cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, const uint32_t* row_ptr,
-                     uint32_t* col, bool has_overflow, bool sort_rows, DevCounters* cnt,
-                     cudaStream_t st, int64_t* launches) {
+                     uint32_t* col, bool has_overflow, DevCounters* cnt, cudaStream_t st,
+                     int64_t* launches) {
   cudaError_t e = cudaMemsetAsync(b.lcur, 0, P.N * sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
   const unsigned nb = (unsigned)((P.N + 255) / 256);
@@ -212,19 +174,16 @@ cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, const uint32_t* ro
       ++*launches;
     }
   }
-  if (sort_rows) {
-    k_rowsort<<<nb, 256, 0, st>>>(P.N, row_ptr, col, cnt);
-    ++*launches;
-  }
   return cudaGetLastError();
 }
 
 cudaError_t csr_sorted_copy(const DevParams& P, const uint32_t* row_ptr, const uint32_t* col,
-                            uint32_t* out, uint64_t nnz, DevCounters* cnt, cudaStream_t st,
-                            int64_t* launches) {
-  cudaError_t e = cudaMemcpyAsync(out, col, nnz * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
+                            uint32_t first, uint32_t* out, uint64_t nnz, DevCounters* cnt,
+                            cudaStream_t st, int64_t* launches) {
+  cudaError_t e =
+      cudaMemcpyAsync(out, col + first, nnz * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) return e;
-  k_rowsort<<<(unsigned)((P.N + 255) / 256), 256, 0, st>>>(P.N, row_ptr, out, cnt);
+  k_rowsort<<<(unsigned)((P.N + 255) / 256), 256, 0, st>>>(P.N, row_ptr, first, out, cnt);
   ++*launches;
   return cudaGetLastError();
 }

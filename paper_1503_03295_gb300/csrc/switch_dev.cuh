@@ -365,23 +365,18 @@ __device__ __forceinline__ void walk_begin(const DevParams& P, const SwitchIn& i
 // that lie on the lattice (emitting the pairs that survive).  Returns false once the list is
 // exhausted.  Two per call, because a lane draws a block for every second candidate: with one per
 // call the lanes of a warp stood at both parities and the block's 280 instructions were issued at
-// every call for half of them.  sync_mask: the lanes of the warp that run this step together (0
-// when threads walk independently); they meet after each candidate search, whose loops run for
-// different lengths, so that the survival test is issued once for all of them instead of once per
-// group of lanes that left the search together.
+// every call for half of them.
 template <int PREC>
 __device__ __forceinline__ bool walk_step(const DevParams& P, const NearTable& T,
                                           const SwitchIn& in, uint32_t epoch, int32_t mnn0,
                                           int32_t mnn1, const SwitchOut& o, SiteWalk<PREC>& a,
-                                          unsigned& n_dip, unsigned& ghits, unsigned& g32,
-                                          unsigned sync_mask) {
+                                          unsigned& n_dip, unsigned& ghits, unsigned& g32) {
   W4 w = philox((uint64_t)a.i, epoch, (uint64_t)a.n, kTagSwitch, P.key0, P.key1);
   ++a.n;
   bool more = true;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int32_t k = more ? next_candidate_e(P, T, a.sidx, a.Es, w.w[0], ghits) : T.K;
-    if (sync_mask) __syncwarp(sync_mask);
     more = k < T.K;
     const uint64_t wU = w.w[1];
     w.w[0] = w.w[2];
@@ -427,19 +422,78 @@ __device__ __forceinline__ uint32_t walk_end(const DevParams& P, int32_t mnn0, i
   return a.n_out;
 }
 
-// Switches the half-plane pairs of site i (local index, slot id `id`) at this epoch in one go;
-// returns the number of upper neighbours written.
-template <int PREC>
-__device__ __forceinline__ uint32_t switch_site(const DevParams& P, const NearTable& T,
-                                                const SwitchIn& in, uint32_t epoch, int32_t mnn0,
-                                                int32_t mnn1, uint32_t i, uint32_t id,
-                                                const SwitchOut& o, unsigned& n_dip,
-                                                unsigned& ghits, unsigned& g32) {
+// Switches the half-plane pairs of the sites below `end` that the calling warp claims, 32 at a time,
+// from *next (local indices; site i writes slots id0 + i).  kRefill: a lane whose walk ends takes up
+// the next claimed site at once, so that the lanes of a warp stay busy although the number of
+// candidates differs from site to site (Poisson, mean about 14 at T = 0.6D); else the warp claims
+// again once all its lanes are done.  One lattice (parameters in constant memory) is faster with it
+// (switch phase at L = 2304 2.96 against 3.14 ms), the batch, whose parameters are read from shared
+// memory at every step, without (64 replicas 2.45 against 3.10 ms).  Returns upper neighbours written.
+template <int PREC, bool kRefill>
+__device__ __forceinline__ unsigned switch_range(const DevParams& P, const NearTable& T,
+                                                 const SwitchIn& in, uint32_t epoch, int32_t mnn0,
+                                                 int32_t mnn1, unsigned* next, uint32_t end,
+                                                 uint32_t id0, uint32_t* __restrict__ hcnt,
+                                                 const SwitchOut& o, unsigned& n_dip,
+                                                 unsigned& ghits, unsigned& g32) {
+  const unsigned lane = threadIdx.x & 31u;
+  unsigned n_half = 0;
   SiteWalk<PREC> a;
-  walk_begin<PREC>(P, in, i, id, a);
-  while (walk_step<PREC>(P, T, in, epoch, mnn0, mnn1, o, a, n_dip, ghits, g32, 0u)) {
+  if (!kRefill) {
+    for (;;) {
+      uint32_t base = 0;
+      if (lane == 0) base = atomicAdd(next, 32u);
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (base >= end) return n_half;
+      const uint32_t i = base + lane;
+      if (i < end) {
+        walk_begin<PREC>(P, in, i, id0 + i, a);
+        while (walk_step<PREC>(P, T, in, epoch, mnn0, mnn1, o, a, n_dip, ghits, g32)) {
+        }
+        const uint32_t n_out = walk_end<PREC>(P, mnn0, mnn1, o, a);
+        hcnt[a.id] = n_out;
+        n_half += n_out;
+      }
+      __syncwarp();
+    }
   }
-  return walk_end<PREC>(P, mnn0, mnn1, o, a);
+  const unsigned below = (1u << lane) - 1u;
+  bool active = false, drained = false;  // drained, pool and pool_n are warp-uniform
+  uint32_t pool = 0, pool_n = 0;
+  for (;;) {
+    unsigned need = __ballot_sync(0xffffffffu, !active);
+    while (need != 0u && !drained) {
+      if (pool_n == 0u) {
+        uint32_t base = 0;
+        if (lane == 0) base = atomicAdd(next, 32u);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (base >= end) {
+          drained = true;
+          break;
+        }
+        pool = base;
+        pool_n = min(32u, end - base);
+      }
+      const uint32_t take = min((uint32_t)__popc(need), pool_n);
+      const uint32_t rank = (uint32_t)__popc(need & below);
+      if (!active && rank < take) {
+        walk_begin<PREC>(P, in, pool + rank, id0 + pool + rank, a);
+        active = true;
+      }
+      pool += take;
+      pool_n -= take;
+      need = __ballot_sync(0xffffffffu, !active);
+    }
+    const unsigned act = __ballot_sync(0xffffffffu, active);
+    if (act == 0u) break;
+    if (active && !walk_step<PREC>(P, T, in, epoch, mnn0, mnn1, o, a, n_dip, ghits, g32)) {
+      const uint32_t n_out = walk_end<PREC>(P, mnn0, mnn1, o, a);
+      hcnt[a.id] = n_out;
+      n_half += n_out;
+      active = false;
+    }
+  }
+  return n_half;
 }
 
 // Compare-exchange on the neighbour index (the exchange flag travels with its entry).

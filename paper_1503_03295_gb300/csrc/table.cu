@@ -130,12 +130,16 @@ __global__ void k_decay(int64_t K, double beta, double D, const uint64_t* __rest
   Eb[m] = (uint64_t)__double_as_longlong(e);
 }
 
-// Both guides (see Search): a binary search per entry.
+// Both guides (see Search).  The cells' bounds fall with the cell number as E does with the element,
+// so element m is the first at or below the bounds of the cells in (cell of E_(m-1), cell of E_m]:
+// each element writes its own, and one thread past the list the rest (a binary search per cell took
+// 20 us for a list of 32,000).
 __global__ void k_guide(int64_t K, uint32_t far_n, const uint64_t* __restrict__ Eb,
                         SearchHead* __restrict__ head, uint16_t* __restrict__ near_g,
                         uint32_t* __restrict__ far_g) {
-  const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t nnear = (uint32_t)(K < kNear ? K : kNear);
+  const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (m > K) return;
+  const int64_t nnear = K < kNear ? K : kNear;
   // the smallest shift that leaves fewer than n cells (n a power of two)
   auto cells = [](uint64_t span, uint32_t n) {
     const int s = 64 - __clzll((long long)span) - (31 - __clz((int)n));
@@ -146,23 +150,17 @@ __global__ void k_guide(int64_t K, uint32_t far_n, const uint64_t* __restrict__ 
   h.e_last = Eb[K - 1];
   h.near_shift = cells(kDecayStart - h.e_near, kNearGuide);
   h.far_shift = cells(h.e_near - h.e_last, far_n);
-  if (q == 0) *head = h;
-  auto first_le = [&](uint32_t a, uint32_t b, uint64_t tb) {
-    while (a < b) {
-      const uint32_t mid = (a + b) >> 1;
-      if (Eb[mid] <= tb) b = mid; else a = mid + 1;
-    }
-    return a;
-  };
-  if (q <= (uint32_t)kNearGuide) {
-    const uint64_t below = (uint64_t)q << h.near_shift;
-    near_g[q] =
-        (uint16_t)(below <= kDecayStart ? first_le(0, nnear - 1, kDecayStart - below) : nnear - 1);
+  if (m == 0) *head = h;
+  if (m < nnear) {
+    int64_t q = m > 0 ? (int64_t)((kDecayStart - Eb[m - 1]) >> h.near_shift) + 1 : 0;
+    const int64_t q1 =
+        m == nnear - 1 ? kNearGuide : (int64_t)((kDecayStart - Eb[m]) >> h.near_shift);
+    for (; q <= q1; ++q) near_g[q] = (uint16_t)m;
   }
-  if (q <= far_n) {
-    const uint64_t below = (uint64_t)q << h.far_shift;
-    far_g[q] = q == far_n || below > h.e_near ? (uint32_t)K
-                                              : first_le(nnear, (uint32_t)K, h.e_near - below);
+  if (m >= nnear) {
+    int64_t q = m > nnear ? (int64_t)((h.e_near - Eb[m - 1]) >> h.far_shift) + 1 : 0;
+    const int64_t q1 = m == K ? far_n : (int64_t)((h.e_near - Eb[m]) >> h.far_shift);
+    for (; q <= q1; ++q) far_g[q] = (uint32_t)m;
   }
 }
 
@@ -204,8 +202,8 @@ cudaError_t table_build_xy(const DevParams& P, Table& t, const Table& list, cuda
   ++*launches;
   if (K > 0) {
     k_decay<<<(unsigned)((K + 255) / 256), 256, 0, s>>>(K, P.beta, P.D, list.W, t.Ebits);
-    const unsigned ng = (t.far_n > (uint32_t)kNearGuide ? t.far_n : kNearGuide) + 1;
-    k_guide<<<(ng + 255) / 256, 256, 0, s>>>(K, t.far_n, t.Ebits, t.head, t.near_g, t.far_g);
+    k_guide<<<(unsigned)((K + 1 + 255) / 256), 256, 0, s>>>(K, t.far_n, t.Ebits, t.head, t.near_g,
+                                                            t.far_g);
     *launches += 2;
   }
   return cudaGetLastError();
