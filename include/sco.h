@@ -233,7 +233,7 @@ typedef struct {
   int32_t use_graph;           /* 1: capture and replay graphs; 0: launch directly */
   int32_t kw_schedule;         /* 0: all KW levels in one kernel, each vertex recolouring as
                                   soon as its larger neighbours are done (2)' while every
-                                  palette has at most 63 colours, else the vertices bucketed
+                                  palette has at most 255 colours, else the vertices bucketed
                                   by colour, largest first (order of Sec. 2.3.2 (2)); 1: one
                                   kernel per level.  Same colours. */
   int32_t kw_low;              /* where the dataflow kernel of schedule 0 does not run: the

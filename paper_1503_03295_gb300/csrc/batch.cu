@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(256) kb_kw_final(const BatchDev B, int flow) {
   const uint32_t i = (blockIdx.x - B.blk_start[r]) * kBatchBlock + threadIdx.x;
   if (i < N) {
     const uint32_t c = flow && B.ctl->gmax <= kFlowMaxPal
-                           ? reinterpret_cast<const uint32_t*>(B.word)[base + i] & 63u
+                           ? reinterpret_cast<const uint32_t*>(B.word)[base + i] & 0xFFu
                            : (uint32_t)(B.word[base + i] & kColMask);
     B.colour[base + i] = c;
     if (c < B.pal_cap) atomicOr(&ubits[c >> 5], 1u << (c & 31));

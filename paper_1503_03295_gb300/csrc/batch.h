@@ -34,8 +34,11 @@ struct RepDesc {
   int32_t variant;     // colouring variant (reported t_R only)
 };
 
-// Palettes up to this size are coloured by the dataflow kernel (kw_flow.cuh).
-constexpr uint32_t kFlowMaxPal = 63;
+// Palettes up to this size are coloured by the dataflow kernel (kw_flow.cuh): a colour has a byte of
+// a word in shared memory.  Against the kernels by rounds and buckets, per colouring: L = 1024,
+// palette 77 29.2 -> 2.8 ms; L = 512, 118 27.5 -> 9.7; L = 1024, 136 89.5 -> 13.2; L = 256, 170
+// 35.9 -> 23.4 (chains of 1500 rounds).
+constexpr uint32_t kFlowMaxPal = 255;
 
 // Larger right-half neighbours listed per bucketed vertex of the KW colouring (records).
 constexpr int kKwItemList = 32;

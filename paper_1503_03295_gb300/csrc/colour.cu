@@ -155,7 +155,7 @@ __global__ void k_flow_final(uint32_t N, unsigned levels, uint32_t g, int varian
                              DevCounters* __restrict__ cnt) {
   const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
   // (after a wait that gave up a vertex may keep a colour of an earlier level, below g as well)
-  if (v < N) colour[v] = word[v] & 63u;
+  if (v < N) colour[v] = word[v] & 0xFFu;
   if (v == 0) {
     unsigned t = 0;
     for (unsigned p = 1; p <= levels; ++p) t += cnt->lev_rounds[p & 31];

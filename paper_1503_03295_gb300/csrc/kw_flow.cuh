@@ -17,7 +17,7 @@
 // lists until every lane has recoloured: nothing waits for a barrier, and a step of the chain is
 // one poll of a short list.  No cycle of waits can form: a vertex only waits for larger previous
 // colours, every warp takes its vertices in descending order, and all blocks are resident
-// (cooperative launch).  Palettes of at most 63 colours; one lattice or a batch of them.
+// (cooperative launch).  Palettes of at most 255 colours; one lattice or a batch of them.
 #pragma once
 
 #include <algorithm>
@@ -95,7 +95,7 @@ __device__ __forceinline__ uint32_t flow_slots(uint32_t N, uint32_t g, unsigned 
   return (uint32_t)(full * half + (rem > half ? rem - half : 0ull));
 }
 
-// u / g for g <= 63: one 32-bit multiply, corrected (see site_xy)
+// u / g: one 32-bit multiply, corrected (see site_xy)
 __device__ __forceinline__ uint32_t flow_div(uint32_t u, uint32_t g, uint32_t m32) {
   uint32_t q = __umulhi(u, m32);
   if (u - q * g >= g) ++q;
@@ -105,11 +105,12 @@ __device__ __forceinline__ uint32_t flow_magic(uint32_t g) {
   return g > 1 ? (uint32_t)(0x100000000ull / g) : 0xFFFFFFFFu;
 }
 
-// Sort key of a vertex: previous colour, largest first, then the number of eight-entry sectors of its
-// row (so that the lanes of a warp read about the same number of them); kFlowKeys: no vertex.
-__device__ __forceinline__ uint32_t flow_key(uint32_t c, uint32_t b, uint32_t e) {
+// Sort key of a vertex: previous colour, largest first, then (palettes up to 64) the number of
+// eight-entry sectors of its row, so that the lanes of a warp read about the same number of them;
+// kFlowKeys: no vertex.
+__device__ __forceinline__ uint32_t flow_key(uint32_t c, uint32_t b, uint32_t e, uint32_t pal) {
   const uint32_t ns = ((e + 7) >> 3) - (b >> 3);
-  return 4 * (63u - c) + (ns < 3 ? 0u : min(ns - 2, 3u));
+  return pal > 64 ? 255u - c : 4 * (63u - c) + (ns < 3 ? 0u : min(ns - 2, 3u));
 }
 // Lanes of the warp that hold the same key (all lanes call it).
 __device__ __forceinline__ unsigned flow_peers(uint32_t key) {
@@ -123,9 +124,9 @@ __device__ __forceinline__ unsigned flow_peers(uint32_t key) {
 }
 
 // Word of a vertex in shared memory: round << 8 | colour once it is done, before that 2^31 | previous
-// colour << 24 | kFlowNone.  A done right-half neighbour is a larger one (a smaller one waits for
+// colour << 16 | kFlowNone.  A done right-half neighbour is a larger one (a smaller one waits for
 // this vertex), so only open ones are compared.  flow_bit(kFlowNone) is no colour.
-constexpr uint32_t kFlowNone = 64u;
+constexpr uint32_t kFlowNone = 255u;
 
 // 1 << c for c < 32, else 0 (shl clamps)
 __device__ __forceinline__ uint32_t flow_bit(uint32_t c) {
@@ -166,6 +167,7 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
                            : V.vec == kFlowVecInside ? V.row_ptr[V.site_start[1]]
                                                      : 0u;
   const uint32_t m0 = flow_magic(pl0.g);
+  const uint32_t pal = V.gmax ? *V.gmax : pl0.g;
   bool ok = true;
   for (unsigned p = 1; p <= V.levels && ok; ++p) {
     __syncthreads();
@@ -232,8 +234,8 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
         const uint32_t q = q0 + a * T + tid;
-        const uint32_t key = q < n ? flow_key(c[a] & 63u, rb[a], re[a]) : kFlowKeys;
-        if (q < n) st[q] = 0x80000000u | ((c[a] & 63u) << 24) | (key << 8) | kFlowNone;
+        const uint32_t key = q < n ? flow_key(c[a] & 0xFFu, rb[a], re[a], pal) : kFlowKeys;
+        if (q < n) st[q] = 0x80000000u | ((c[a] & 0xFFu) << 16) | (key << 8) | kFlowNone;
         if (q0 + a * T >= n) break;  // uniform
         const unsigned peers = flow_peers(key);
         if (q < n && (peers & below) == 0) atomicAdd(&cur[key], (uint32_t)__popc(peers));
@@ -271,7 +273,7 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
       at = __shfl_sync(0xffffffffu, at, __ffs(peers) - 1);
       if (q < n) {
         ord[at + __popc(peers & below)] = (uint16_t)q;
-        st[q] = w & 0xFF0000FFu;
+        st[q] = w & 0xFFFF00FFu;
       }
     }
     __syncthreads();
@@ -284,7 +286,7 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
       uint32_t mlo = 0;  // colours below 32 taken
       int m = 0;         // the largest round << 8 (and bits below)
       int r = 0;
-      auto add = [&](uint32_t w) { mlo |= flow_bit(w & 0x7Fu); };
+      auto add = [&](uint32_t w) { mlo |= flow_bit(w & 0xFFu); };
       if (open) {
         loc = ord[t0 + lane];
         uint32_t k;
@@ -293,7 +295,7 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
         gv = base + (s0 + loc - rp[r]) + (k + 1) * half;
         b = V.row_ptr[gv];
         e = V.row_ptr[gv + 1];
-        c = (st[loc] >> 24) & 63u;
+        c = (st[loc] >> 16) & 0xFFu;
         lo = 2 * k * half;
         // the block's part of the right half: vertices [fa, fa + len), words from la on
         const uint32_t h0 = k * half + rp[r], g0 = max(h0, s0), g1 = min(h0 + half, s0 + n);
@@ -301,7 +303,7 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
         len = g1 - g0;
         la = g0 - s0;
       }
-      const uint32_t lthr = 0x80000000u | (c << 24) | 0xFFFFFFu;  // open and larger: words above it
+      const uint32_t lthr = 0x80000000u | (c << 16) | 0xFFFFu;  // open and larger: words above it
       const uint32_t done_at = p << 27;                           // done: global words from it on
       const uint32_t* own = st + la;
       const uint32_t none = V.cap - la;  // word cap: no colour
@@ -362,9 +364,9 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
           for (uint32_t a = 0; a < kFlowLook; ++a) {
             const uint32_t y = w[a];
             const bool left = u[a] - lo < half, done = y >= done_at;
-            go = go && f < fcnt && (left || done || (y & 63u) <= c);
+            go = go && f < fcnt && (left || done || (y & 0xFFu) <= c);
             if (go) {
-              if (left || done) add(y & 63u);
+              if (left || done) add(y);
               if (!left && done) m = max(m, (int)(y & 0x7FFFFFFu));
               ++f;
               moved = true;
@@ -389,16 +391,17 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
         }
         if (open && q0 >= e && k == cnt && f == fcnt) {
           uint32_t cn = (uint32_t)__ffs((int)~mlo) - 1;
-          if (mlo == 0xFFFFFFFFu) {  // rare: the colours from 32 on, from the row again
-            uint32_t mhi = 0;
+          for (uint32_t taken = mlo, c0 = 32; taken == 0xFFFFFFFFu; c0 += 32) {
+            // rare: colours c0 .. c0 + 31, from the row again
+            taken = 0;
             for (uint32_t q = b; q < e; ++q) {
               const uint32_t u = V.col[q] & kIndexMask;
               if (u - lo >= 2 * half) continue;
               const bool mine = u - fa < len, left = u - lo < half;
               const uint32_t y = mine ? flow_lds(own + (u - fa)) : flow_ld(&V.word[base + u]);
-              if (left || (mine ? (int)y >= 0 : y >= done_at)) mhi |= flow_bit((y & 0x7Fu) - 32u);
+              if (left || (mine ? (int)y >= 0 : y >= done_at)) taken |= flow_bit((y & 0xFFu) - c0);
             }
-            cn = 31u + (uint32_t)__ffs((int)~mhi);
+            cn = c0 - 1 + (uint32_t)__ffs((int)~taken);
           }
           const uint32_t rd = (uint32_t)(m >> 8) + 1;
           *reinterpret_cast<volatile uint32_t*>(st + loc) = (rd << 8) | cn;

@@ -1,8 +1,8 @@
 // kw_static.cu -- Kuhn-Wattenhofer colouring of a caller's CSR graph that allocates nothing.
 //
-// Same colouring as sco_colour (palettes of at most 63 colours by the dataflow kernel of
-// kw_flow.cuh, larger ones by one barrier-free kernel per level), for callers that cannot let a library allocate device memory.  Its working memory is one
-// file-scope device array of fixed size: per-vertex words for up to
+// Same colouring as sco_colour (palettes of at most 255 colours by the dataflow kernel of
+// kw_flow.cuh, larger ones by one barrier-free kernel per level), for callers that cannot let a
+// library allocate device memory.  Its working memory is one file-scope device array of fixed size: per-vertex words for up to
 // SCO_KW_STATIC_MAX_VERTICES vertices followed by a small control block.  Every call
 // shares that array; calls that overlap on the GPU race.
 #include <cstdint>
@@ -188,7 +188,7 @@ __global__ void k_st_final(uint32_t n, int variant, const unsigned long long* __
                            const uint32_t* __restrict__ fword, uint32_t* __restrict__ colour,
                            StaticCtrl* __restrict__ ctrl) {
   const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v < n) colour[v] = fword ? fword[v] & 63u : (uint32_t)(word[v] & kColMask);
+  if (v < n) colour[v] = fword ? fword[v] & 0xFFu : (uint32_t)(word[v] & kColMask);
   if (v == 0) {
     unsigned t = 0;
     for (unsigned p = 1; p <= ctrl->levels; ++p) t += ctrl->lev_rounds[p & 31];

@@ -26,8 +26,8 @@ def _compare(g, o):
     (64, 33, 0.5, 0.0),      # just above
     (301, 299, 0.6, 0.0), (700, 301, 0.9, 1.0),
     (1024, 700, 0.3, 0.0),   # larger blocks, mean degree 30: lists read in parts
-    (40, 40, 0.1, 0.0),      # palette above 63, few vertices
-    (1100, 1000, 0.14, 0.0),  # palette above 63, many vertices
+    (40, 40, 0.1, 0.0), (301, 200, 0.1, 0.0),  # palettes of 65 to 255: colours above 31 looked up again
+    (40, 40, 0.006, 0.0), (200, 150, 0.011, 0.0),  # palettes above 255: the other kernels
 ])
 def test_colouring_matches_oracle(Lx, Ly, T, J):
     D = 1.0 if J == 0.0 else 0.1
@@ -56,9 +56,9 @@ def test_static_rows_at_any_alignment(offset):
     assert np.array_equal(out.cpu().numpy().view(np.uint32), lat.colours())
 
 
-@pytest.mark.parametrize("cold", [0.5, 0.1])  # 0.1: one replica's palette above 63
+@pytest.mark.parametrize("cold", [0.5, 0.1, 0.006])  # one replica's palette above 64, above 255
 def test_batch_matches_single_lattices(cold):
-    ps = [sco.make_params(40, T=cold, seed=1), sco.make_params(3, 2, T=0.5, seed=2),
+    ps = [sco.make_params(36, T=cold, seed=1), sco.make_params(3, 2, T=0.5, seed=2),
           sco.make_params(90, 70, T=0.7, seed=3), sco.make_params(64, T=1e12, seed=4)]
     with sco.Batch(ps) as b:
         b.run(2)
