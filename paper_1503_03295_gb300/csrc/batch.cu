@@ -521,9 +521,9 @@ cudaError_t batch_low_setup(int R, uint32_t gcap, int* blocks_per_sm, uint32_t* 
 int batch_sweep_occupancy(int precision, int R) {
   int n = 0;
   const cudaError_t e =
-      precision == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep<1, true, 3>,
+      precision == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep<1, true, true, 3>,
                                                                      kSweepThreads, sweep_smem(R))
-                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep<0, true, 2>,
+                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep<0, true, true, 2>,
                                                                      kSweepThreads, sweep_smem(R));
   if (e != cudaSuccess || n < 1) n = 1;
   return n;
@@ -685,10 +685,10 @@ cudaError_t batch_sweep(const BatchDev& B, const BatchLaunch& L, cudaStream_t st
   V.ns_limit = B.ns_limit;
   *L.launches += 2;
   return B.precision == 1
-             ? launch_coop(k_sweep<1, true, 3>, (unsigned)L.sweep_grid, kSweepThreads, sweep_smem(B.R),
-                           st, V)
-             : launch_coop(k_sweep<0, true, 2>, (unsigned)L.sweep_grid, kSweepThreads, sweep_smem(B.R),
-                           st, V);
+             ? launch_coop(k_sweep<1, true, true, 3>, (unsigned)L.sweep_grid, kSweepThreads,
+                           sweep_smem(B.R), st, V)
+             : launch_coop(k_sweep<0, true, true, 2>, (unsigned)L.sweep_grid, kSweepThreads,
+                           sweep_smem(B.R), st, V);
 }
 
 cudaError_t batch_step_end(const BatchDev& B, const BatchLaunch& L, cudaStream_t st) {

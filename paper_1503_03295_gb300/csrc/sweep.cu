@@ -10,14 +10,24 @@ namespace sco {
 
 namespace {
 
+// In the order of perm (see take_proposal).
 __global__ void __launch_bounds__(256) k_propose(const DevParams P, uint64_t step,
+                                                 const uint32_t* __restrict__ perm,
                                                  double4_32a* __restrict__ prop,
                                                  SpinDf* __restrict__ propd,
                                                  float4* __restrict__ prop32) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= P.N) return;
-  write_proposal(P, step, (uint32_t)i, prop + i, propd ? propd + i : nullptr,
+  write_proposal(P, step, perm[i], prop + i, propd ? propd + i : nullptr,
                  prop32 ? prop32 + i : nullptr);
+}
+
+template <bool kExch>
+const void* sweep_kernel(int precision, int per) {
+  return precision == 1 ? (per > 1 ? (const void*)k_sweep<1, false, kExch, 3>
+                                   : (const void*)k_sweep<1, false, kExch, 1>)
+                        : (per > 1 ? (const void*)k_sweep<0, false, kExch, 2>
+                                   : (const void*)k_sweep<0, false, kExch, 1>);
 }
 
 }  // namespace
@@ -25,7 +35,8 @@ __global__ void __launch_bounds__(256) k_propose(const DevParams P, uint64_t ste
 cudaError_t sweep_run(const DevParams& P, const Table& t, const SweepBufs& b, uint32_t g,
                       uint64_t step, int precision, DevCounters* cnt, unsigned long long ns_limit,
                       cudaStream_t st, int64_t* launches) {
-  k_propose<<<(unsigned)((P.N + 255) / 256), 256, 0, st>>>(P, step, b.prop, b.propd, b.prop32);
+  k_propose<<<(unsigned)((P.N + 255) / 256), 256, 0, st>>>(P, step, b.perm, b.prop, b.propd,
+                                                             b.prop32);
   // Two blocks per SM (64 registers; three at 42 in FP32: 1.59 ms per step at L = 2304 against 1.66)
   // on a large lattice; below kSweepWide sites per SM one block per
   // SM at 128 registers and without spills (L = 256: 0.130 ms per step against 0.163, L = 1024:
@@ -59,10 +70,8 @@ cudaError_t sweep_run(const DevParams& P, const Table& t, const SweepBufs& b, ui
   V.ns_limit = ns_limit;
   void* args[] = {(void*)&V};
   *launches += 2;
-  const void* k = precision == 1 ? (per > 1 ? (const void*)k_sweep<1, false, 3>
-                                            : (const void*)k_sweep<1, false, 1>)
-                                 : (per > 1 ? (const void*)k_sweep<0, false, 2>
-                                             : (const void*)k_sweep<0, false, 1>);
+  const void* k = P.J != 0.0 ? sweep_kernel<true>(precision, per) : sweep_kernel<false>(precision, per);
+  if (grid == 1) return cudaLaunchKernel(k, dim3(1), dim3(kSweepThreads), args, sweep_smem(1), st);
   return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kSweepThreads), args, sweep_smem(1), st);
 }
 

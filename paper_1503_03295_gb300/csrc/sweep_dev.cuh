@@ -80,7 +80,13 @@ __device__ __forceinline__ bool renorm600(double& p, int& sc) {
 // 2^-43 per factor, the exchange factor its argument's error and kDfExpRelErr.
 constexpr float kDfExpRelErr = 0x1p-31f;  // measured 2^-31.8 (y < 60), 20 M points
 
-template <int kG>
+// Index step from site (xi, yi) to its exchange neighbour q (0 to 3: left, right, down, up); 0: none.
+__device__ __forceinline__ int32_t exch_step(const DevParams& P, int32_t xi, int32_t yi, int q) {
+  if (q < 2) return q == 0 ? (xi > 0 ? -1 : 0) : (xi + 1 < P.Lx ? 1 : 0);
+  return q == 2 ? (yi > 0 ? -P.Lx : 0) : (yi + 1 < P.Ly ? P.Lx : 0);
+}
+
+template <int kG, bool kExch>
 __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t yi,
                                          const SpinDf& S, const SpinDf& N,
                                          const PairDf* __restrict__ pdf, const SpinDf* sd,
@@ -89,8 +95,26 @@ __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t
   df pn = {1.f, 0.f}, po = {1.f, 0.f};
   int K = 0, n = 0, dmax = -0x40000000;  // K: exponent of prod E_o / prod E_n beside po / pn
   bool bad = false;
+  uint32_t jn = e0 + sub < e1 ? col[e0 + sub] : 0u;  // the entry one iteration ahead
+  df ws = {0.f, 0.f};  // (S' - S) . (sum of the neighbours' spins), this lane's part
+  if (kExch && P.J != 0.0 && sub < 4) {
+    df hx = {0.f, 0.f}, hy = hx, hz = hx;
+#pragma unroll
+    for (int q = 0; q < 4; q += kG < 4 ? kG : 4) {
+      const int32_t k = exch_step(P, xi, yi, q + sub);
+      if (k == 0) continue;
+      const SpinDf b = load32(sd + (int32_t)i + k);
+      hx = df_add(hx, {b.hx, b.lx});
+      hy = df_add(hy, {b.hy, b.ly});
+      hz = df_add(hz, {b.hz, b.lz});
+    }
+    ws = df_mul(df_sub({N.hx, N.lx}, {S.hx, S.lx}), hx);
+    ws = df_add(ws, df_mul(df_sub({N.hy, N.ly}, {S.hy, S.ly}), hy));
+    ws = df_add(ws, df_mul(df_sub({N.hz, N.lz}, {S.hz, S.lz}), hz));
+  }
   for (uint32_t e = e0 + sub; e < e1; e += kG) {
-    const uint32_t j = col[e];
+    const uint32_t j = jn;
+    if (e + kG < e1) jn = col[e + kG];
     if (j & kExchOnly) continue;
     int32_t xj, yj;
     site_xy(j, P, xj, yj);
@@ -128,6 +152,14 @@ __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t
       dmax = max(dmax, __shfl_down_sync(0xffffffffu, dmax, o, kG));
       bad |= __shfl_down_sync(0xffffffffu, (int)bad, o, kG) != 0;
     }
+    if (kExch) {  // (whole warps: the lattices of a batch differ in J)
+#pragma unroll
+      for (int o = kG < 4 ? kG / 2 : 2; o > 0; o >>= 1) {
+        const df q = {__shfl_down_sync(0xffffffffu, ws.h, o, kG),
+                      __shfl_down_sync(0xffffffffu, ws.l, o, kG)};
+        ws = df_add(ws, q);
+      }
+    }
   }
   if (sub != 0) return 0;
   if (N.u_h == 0.f && N.u_l == 0.f) return 1;  // u = 0 accepts outright
@@ -139,23 +171,9 @@ __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t
     bound += 2.84f * (float)n * __int_as_float((max(x, -100) + 127) << 23);
   }
   df X = df_mul({N.u_h, N.u_l}, po);
-  if (P.J != 0.0) {
-    // e^tex, tex = -beta J (S' - S) . (sum of the neighbours' spins)
-    df hx = {0.f, 0.f}, hy = hx, hz = hx;
-    const int32_t nb[4] = {xi > 0 ? -1 : 0, xi + 1 < P.Lx ? 1 : 0, yi > 0 ? -P.Lx : 0,
-                           yi + 1 < P.Ly ? P.Lx : 0};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (nb[q] == 0) continue;
-      const SpinDf b = load32(sd + (int32_t)i + nb[q]);
-      hx = df_add(hx, {b.hx, b.lx});
-      hy = df_add(hy, {b.hy, b.ly});
-      hz = df_add(hz, {b.hz, b.lz});
-    }
-    df w = df_mul(df_sub({N.hx, N.lx}, {S.hx, S.lx}), hx);
-    w = df_add(w, df_mul(df_sub({N.hy, N.ly}, {S.hy, S.ly}), hy));
-    w = df_add(w, df_mul(df_sub({N.hz, N.lz}, {S.hz, S.lz}), hz));
-    w = df_mul(w, {-P.bJ_h, -P.bJ_l});
+  if (kExch && P.J != 0.0) {
+    // e^tex, tex = -beta J w
+    df w = df_mul(ws, {-P.bJ_h, -P.bJ_l});
     w = df_fast(w.h, w.l);
     const float aj = fabsf(P.bJ_h);
     // |w error| <= 2^-40 beta J 4 (float-float sums of 12 terms below 2 each, scaled)
@@ -186,7 +204,7 @@ __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t
 // (about 60 instructions per pair).  Bound as in accept_df, with kE32RelErr, c0 = kY32RelErr a1
 // (c0 / m < 2^((d >> 23) + 1 - 18), below 2^-6) and 2^-23 per product; it leaves about one site in
 // 10^4 to FP64.  N = {S', u}.
-template <int kG>
+template <int kG, bool kExch>
 __device__ __forceinline__ int accept_f32(const DevParams& P, int32_t xi, int32_t yi, float4 S,
                                           float4 N, const float4* __restrict__ sw,
                                           const float4* s32, const uint32_t* __restrict__ col,
@@ -194,8 +212,24 @@ __device__ __forceinline__ int accept_f32(const DevParams& P, int32_t xi, int32_
   float pn = 1.f, po = 1.f;
   int K = 0, n = 0, dmax = -0x40000000;
   bool bad = false;
+  uint32_t jn = e0 + sub < e1 ? col[e0 + sub] : 0u;  // the entry one iteration ahead
+  float ws = 0.f;  // (S' - S) . (sum of the neighbours' spins), this lane's part
+  if (kExch && P.J != 0.0 && sub < 4) {
+    float hx = 0.f, hy = 0.f, hz = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; q += kG < 4 ? kG : 4) {
+      const int32_t k = exch_step(P, xi, yi, q + sub);
+      if (k == 0) continue;
+      const float4 b = s32[(int32_t)i + k];
+      hx += b.x;
+      hy += b.y;
+      hz += b.z;
+    }
+    ws = (N.x - S.x) * hx + (N.y - S.y) * hy + (N.z - S.z) * hz;
+  }
   for (uint32_t e = e0 + sub; e < e1; e += kG) {
-    const uint32_t j = col[e];
+    const uint32_t j = jn;
+    if (e + kG < e1) jn = col[e + kG];
     if (j & kExchOnly) continue;
     int32_t xj, yj;
     site_xy(j, P, xj, yj);
@@ -230,6 +264,10 @@ __device__ __forceinline__ int accept_f32(const DevParams& P, int32_t xi, int32_
       dmax = max(dmax, __shfl_down_sync(0xffffffffu, dmax, o, kG));
       bad |= __shfl_down_sync(0xffffffffu, (int)bad, o, kG) != 0;
     }
+    if (kExch) {  // (whole warps: the lattices of a batch differ in J)
+#pragma unroll
+      for (int o = kG < 4 ? kG / 2 : 2; o > 0; o >>= 1) ws += __shfl_down_sync(0xffffffffu, ws, o, kG);
+    }
   }
   if (sub != 0) return 0;
   if (N.w == 0.f) return 1;  // u = 0 accepts outright
@@ -241,19 +279,8 @@ __device__ __forceinline__ int accept_f32(const DevParams& P, int32_t xi, int32_
     bound += 2.84f * (float)n * __int_as_float((max(x, -100) + 127) << 23);
   }
   float X = N.w * po;
-  if (P.J != 0.0) {
-    float hx = 0.f, hy = 0.f, hz = 0.f;
-    const int32_t nb[4] = {xi > 0 ? -1 : 0, xi + 1 < P.Lx ? 1 : 0, yi > 0 ? -P.Lx : 0,
-                           yi + 1 < P.Ly ? P.Lx : 0};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (nb[q] == 0) continue;
-      const float4 b = s32[(int32_t)i + nb[q]];
-      hx += b.x;
-      hy += b.y;
-      hz += b.z;
-    }
-    const float w = -P.bJ_f * ((N.x - S.x) * hx + (N.y - S.y) * hy + (N.z - S.z) * hz);
+  if (kExch && P.J != 0.0) {
+    const float w = -P.bJ_f * ws;
     const float aj = fabsf(P.bJ_f);
     if (!(aj < 512.f)) return 2;
     int k;
@@ -306,11 +333,13 @@ __device__ __forceinline__ bool propose(const DevParams& P, SiteCtx& c, uint64_t
   return true;
 }
 
-// Proposals are drawn for every site of a lattice by k_propose before the colour classes of a
-// step run (they depend only on (seed, site, step)), one double4 {S'x, S'y, S'z, u} per site;
-// u = -1 marks a site whose 64 attempts were all rejected (no move).
-__device__ __forceinline__ bool take_proposal(SiteCtx& c, const double4_32a* __restrict__ prop) {
-  const double4_32a q = prop[c.i];
+// Proposals are drawn for every site before the colour classes of a step run (they depend only on
+// (seed, site, step)), one double4 {S'x, S'y, S'z, u} per site; u = -1 marks a site whose 64 attempts
+// were all rejected (no move).  One lattice keeps them in the order of perm, so that a class reads
+// its own as one stream (by site, each class touched nearly every 64-byte pair of sectors of the
+// records); a batch by global site.
+__device__ __forceinline__ bool take_proposal(SiteCtx& c, const double4_32a* prop) {
+  const double4_32a q = *prop;
   c.Sn[0] = q.x;
   c.Sn[1] = q.y;
   c.Sn[2] = q.z;
@@ -500,7 +529,7 @@ struct SweepView {
   const uint32_t* col;
   const uint32_t* perm;        // sites by colour, global indices
   const uint32_t* off;         // class starts, g + 1
-  const double4_32a* prop;     // proposals {S', u} by global site, FP64
+  const double4_32a* prop;     // proposals {S', u}, FP64 (see take_proposal)
   const SpinDf* propd;         // and in float-float (FP64 form)
   const float4* prop32;        // or FP32 (FP32-guarded form)
   uint8_t* acc;
@@ -519,8 +548,7 @@ __device__ __noinline__ bool settle_site(const DevParams& P, uint32_t i,
                                          const Sw64* __restrict__ sw, const double* s,
                                          const uint32_t* __restrict__ row_ptr,
                                          const uint32_t* __restrict__ col,
-                                         const double4_32a* __restrict__ prop, int lane,
-                                         unsigned& ndd) {
+                                         const double4_32a* prop, int lane, unsigned& ndd) {
   SiteCtx c;
   load_site(P, c, i, s);
   take_proposal(c, prop);
@@ -535,7 +563,7 @@ __device__ __noinline__ bool settle_site(const DevParams& P, uint32_t i,
 // The n sites perm[b ..], kG lanes per site, warps w, w + nw, ...; undecided sites are settled at once
 // by their warp.  sbase: site bases in shared memory (batch); sg: counters of screened-out and
 // double-double decisions (batch: per lattice, one lattice: none) beside n32 and ndd.
-template <int kPrec, bool kBatch, int kG>
+template <int kPrec, bool kBatch, bool kExch, int kG>
 __device__ __forceinline__ void sweep_class(const SweepView& V, const uint32_t* sbase, uint32_t* sg,
                                             uint32_t b, uint32_t n, uint32_t w, uint32_t nw,
                                             unsigned& n32, unsigned& ndd) {
@@ -564,27 +592,29 @@ __device__ __forceinline__ void sweep_class(const SweepView& V, const uint32_t* 
     if (kPrec == 0) {
       SpinDf S;
       Nd.u_h = -1.f;
-      if (idx < n) Nd = load32(V.propd + gs);
-      move = Nd.u_h >= 0.f;
-      if (move) {
+      if (idx < n) {
+        Nd = load32(V.propd + (kBatch ? gs : b + idx));
         e0 = V.row_ptr[gs];
         e1 = V.row_ptr[gs + 1];
         S = load32(V.sd + gs);
       }
-      d = accept_df<kG>(P, xi, yi, S, Nd, kBatch ? dr->pdf : V.pdf, V.sd + base, V.col, e0, e1, i,
-                        sub);
+      move = Nd.u_h >= 0.f;
+      if (!move) e1 = e0;
+      d = accept_df<kG, kExch>(P, xi, yi, S, Nd, kBatch ? dr->pdf : V.pdf, V.sd + base, V.col, e0, e1, i,
+                               sub);
     } else {
       float4 S;
       N4.w = -1.f;
-      if (idx < n) N4 = V.prop32[gs];
-      move = N4.w >= 0.f;
-      if (move) {
+      if (idx < n) {
+        N4 = V.prop32[kBatch ? gs : b + idx];
         e0 = V.row_ptr[gs];
         e1 = V.row_ptr[gs + 1];
         S = V.s32[gs];
       }
-      d = accept_f32<kG>(P, xi, yi, S, N4, kBatch ? dr->sw32 : V.sw32, V.s32 + base, V.col, e0, e1,
-                         i, sub);
+      move = N4.w >= 0.f;
+      if (!move) e1 = e0;
+      d = accept_f32<kG, kExch>(P, xi, yi, S, N4, kBatch ? dr->sw32 : V.sw32, V.s32 + base, V.col, e0,
+                                e1, i, sub);
     }
     const bool mine = sub == 0 && idx < n;
     if (!mine || !move) d = 0;
@@ -600,7 +630,8 @@ __device__ __forceinline__ void sweep_class(const SweepView& V, const uint32_t* 
       const RepDesc* di = kBatch ? V.desc + ri : nullptr;
       unsigned dd = 0;
       const bool ok = settle_site(kBatch ? di->P : V.P, gi - bi, kBatch ? di->sw64 : V.sw,
-                                  V.s + 3 * (size_t)bi, V.row_ptr + bi, V.col, V.prop + bi, lane, dd);
+                                  V.s + 3 * (size_t)bi, V.row_ptr + bi, V.col,
+                                  V.prop + (kBatch ? gi : b + q + src / kG), lane, dd);
       if (lane == src) {
         d = ok ? 1 : 0;
         if (kBatch) {
@@ -614,7 +645,7 @@ __device__ __forceinline__ void sweep_class(const SweepView& V, const uint32_t* 
     }
     if (mine) {
       if (d == 1) {
-        const double4_32a v = V.prop[gs];
+        const double4_32a v = V.prop[kBatch ? gs : b + idx];
         double* s = V.s + 3 * (size_t)base;
         s[i] = v.x;
         s[P.N + i] = v.y;
@@ -630,19 +661,22 @@ __device__ __forceinline__ void sweep_class(const SweepView& V, const uint32_t* 
 // Lanes per site: 2 while the class gives every second lane a site (one lane per site took 2.37 ms
 // per step at L = 2304 in the FP64 form, two 2.20, four 2.28), 8 and 32 below, where the class would
 // leave lanes idle and a row's serial chain sets the time.
-template <int kPrec, bool kBatch>
+__device__ __forceinline__ uint32_t sweep_lanes(uint32_t n, uint32_t nw) {
+  return n >= nw * 16 ? 2 : n >= nw ? 8 : 32;
+}
+template <int kPrec, bool kBatch, bool kExch>
 __device__ __forceinline__ void sweep_tiers(const SweepView& V, const uint32_t* sbase, uint32_t* sg,
                                             uint32_t b, uint32_t n, uint32_t w, uint32_t nw,
                                             unsigned& n32, unsigned& ndd) {
-  const uint32_t nth = nw * 32;
-  if (n >= nth / 2) sweep_class<kPrec, kBatch, 2>(V, sbase, sg, b, n, w, nw, n32, ndd);
-  else if (n >= nth / 32) sweep_class<kPrec, kBatch, 8>(V, sbase, sg, b, n, w, nw, n32, ndd);
-  else sweep_class<kPrec, kBatch, 32>(V, sbase, sg, b, n, w, nw, n32, ndd);
+  const uint32_t k = sweep_lanes(n, nw);
+  if (k == 2) sweep_class<kPrec, kBatch, kExch, 2>(V, sbase, sg, b, n, w, nw, n32, ndd);
+  else if (k == 8) sweep_class<kPrec, kBatch, kExch, 8>(V, sbase, sg, b, n, w, nw, n32, ndd);
+  else sweep_class<kPrec, kBatch, kExch, 32>(V, sbase, sg, b, n, w, nw, n32, ndd);
 }
 
 inline size_t sweep_smem(int R) { return (size_t)(3 * R + 1) * sizeof(uint32_t); }
 
-template <int kPrec, bool kBatch, int kBlocks>
+template <int kPrec, bool kBatch, bool kExch, int kBlocks>
 __global__ void __launch_bounds__(kSweepThreads, kBlocks) k_sweep(const __grid_constant__ SweepView V) {
   __shared__ int s_halt;
   __shared__ unsigned s_tail;
@@ -660,6 +694,10 @@ __global__ void __launch_bounds__(kSweepThreads, kBlocks) k_sweep(const __grid_c
     for (int r = threadIdx.x; r < 2 * V.R; r += blockDim.x) sg[r] = 0;
   }
   const uint32_t g = V.gmax ? *V.gmax : V.g;
+  // class starts in shared memory: the barrier drops what L1 holds
+  constexpr uint32_t kOffs = 256;
+  __shared__ uint32_t soff[kOffs + 1];
+  for (uint32_t c = threadIdx.x; c <= min(g, kOffs); c += blockDim.x) soff[c] = V.off[c];
   for (uint32_t c = threadIdx.x; c < g; c += blockDim.x)
     if (V.off[c + 1] - V.off[c] > kTailSites) atomicMax(&s_tail, c + 1);
   __syncthreads();
@@ -667,11 +705,12 @@ __global__ void __launch_bounds__(kSweepThreads, kBlocks) k_sweep(const __grid_c
   const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   unsigned n32 = 0, ndd = 0;
   bool ok = true;
-  uint32_t b = V.off[0];
+  uint32_t b = soff[0];
   for (uint32_t c = 0; c < tail && ok; ++c) {
-    const uint32_t e = V.off[c + 1];
+    const uint32_t e = c + 1 <= kOffs ? soff[c + 1] : V.off[c + 1];
     if (e > b) {
-      sweep_tiers<kPrec, kBatch>(V, sbase, sg, b, e - b, w, (gridDim.x * blockDim.x) >> 5, n32, ndd);
+      sweep_tiers<kPrec, kBatch, kExch>(V, sbase, sg, b, e - b, w, (gridDim.x * blockDim.x) >> 5, n32,
+                                        ndd);
       if (gridDim.x > 1) ok = grid_sync(V.bar, V.status, V.ns_limit);
       else __syncthreads();
     }
@@ -679,9 +718,9 @@ __global__ void __launch_bounds__(kSweepThreads, kBlocks) k_sweep(const __grid_c
   }
   if (blockIdx.x == 0 && ok) {
     for (uint32_t c = tail; c < g; ++c) {
-      const uint32_t e = V.off[c + 1];
+      const uint32_t e = c + 1 <= kOffs ? soff[c + 1] : V.off[c + 1];
       if (e > b) {
-        sweep_tiers<kPrec, kBatch>(V, sbase, sg, b, e - b, w, kSweepThreads / 32, n32, ndd);
+        sweep_tiers<kPrec, kBatch, kExch>(V, sbase, sg, b, e - b, w, kSweepThreads / 32, n32, ndd);
         __syncthreads();
       }
       b = e;
