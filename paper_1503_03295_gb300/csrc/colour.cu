@@ -143,10 +143,18 @@ __global__ void __launch_bounds__(256, 4) k_kw_level(uint32_t N, uint32_t g, uns
   if ((threadIdx.x & 31) == 0 && rmax) atomicMax(&cnt->lev_rounds[p & 31], rmax);
 }
 
-// Initial words of the dataflow kernel.
-__global__ void k_flow_init(uint32_t N, uint32_t g, uint32_t m32, uint32_t* __restrict__ word) {
+// Initial words of the dataflow kernel, its one-lattice view and its counters.
+__global__ void k_flow_init(uint32_t N, RepPlan pl, uint32_t m32, uint32_t* __restrict__ word,
+                            uint32_t* __restrict__ site_start, RepPlan* __restrict__ plan,
+                            DevCounters* __restrict__ cnt) {
   const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v < N) word[v] = v - flow_div(v, g, m32) * g;
+  if (v < N) word[v] = v - flow_div(v, pl.g, m32) * pl.g;
+  if (v < 32) cnt->lev_rounds[v] = 0;
+  if (v < 2) {
+    cnt->bar[v] = 0;
+    site_start[v] = v * N;
+  }
+  if (v == 0) *plan = pl;
 }
 
 // Final colours of the dataflow kernel.
@@ -252,7 +260,8 @@ __global__ void __launch_bounds__(32) k_tile_scatter(uint32_t N, uint32_t g, uin
                                                      const uint32_t* __restrict__ row_ptr,
                                                      const uint32_t* __restrict__ base,
                                                      uint32_t* __restrict__ perm,
-                                                     uint32_t* __restrict__ off) {
+                                                     uint32_t* __restrict__ off,
+                                                     DevCounters* __restrict__ cnt) {
   extern __shared__ uint32_t run[];
   const int lane = threadIdx.x;
   const uint32_t nk = g * dk;
@@ -274,8 +283,16 @@ __global__ void __launch_bounds__(32) k_tile_scatter(uint32_t N, uint32_t g, uin
     __syncwarp();
   }
   if (blockIdx.x == 0) {
-    for (uint32_t c = lane; c < g; c += 32) off[c] = base[(size_t)c * ntiles * dk];
-    if (lane == 0) off[g] = N;
+    unsigned used = 0;
+    for (uint32_t c = lane; c < g; c += 32) {
+      off[c] = base[(size_t)c * ntiles * dk];
+      used += base[(size_t)(c + 1) * ntiles * dk] > off[c];
+    }
+    used = __reduce_add_sync(0xffffffffu, used);
+    if (lane == 0) {
+      off[g] = N;
+      cnt->n_colours = used;
+    }
   }
 }
 
@@ -290,7 +307,8 @@ __global__ void __launch_bounds__(512) k_tile_sort(uint32_t N, uint32_t g, uint3
                                                       const uint32_t* __restrict__ row_ptr,
                                                       const uint32_t* __restrict__ base,
                                                       uint32_t* __restrict__ perm,
-                                                      uint32_t* __restrict__ off) {
+                                                      uint32_t* __restrict__ off,
+                                                  DevCounters* __restrict__ cnt) {
   extern __shared__ uint32_t run[];  // per key: its start minus the sorted position of its first site
   __shared__ uint32_t a[kClassTile];
   const uint32_t v0 = blockIdx.x * kClassTile;
@@ -324,18 +342,17 @@ __global__ void __launch_bounds__(512) k_tile_sort(uint32_t N, uint32_t g, uint3
   for (uint32_t q = threadIdx.x; q < n; q += blockDim.x)
     perm[run[a[q] >> 11] + q] = v0 + (a[q] & 2047u);
   if (blockIdx.x == 0) {
-    for (uint32_t c = threadIdx.x; c < g; c += blockDim.x) off[c] = base[(size_t)c * ntiles * dk];
-    if (threadIdx.x == 0) off[g] = N;
+    unsigned used = 0;
+    for (uint32_t c0 = 0; c0 < g; c0 += blockDim.x) {
+      const uint32_t c = c0 + threadIdx.x;
+      if (c < g) off[c] = base[(size_t)c * ntiles * dk];
+      used += __syncthreads_count(c < g && base[(size_t)(c + 1) * ntiles * dk] > off[c]);
+    }
+    if (threadIdx.x == 0) {
+      off[g] = N;
+      cnt->n_colours = used;
+    }
   }
-}
-
-__global__ void k_nonempty_off(uint32_t g, const uint32_t* __restrict__ off,
-                               DevCounters* __restrict__ cnt) {
-  unsigned n = 0;
-  for (uint32_t c = threadIdx.x; c < g; c += blockDim.x) n += off[c + 1] > off[c];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) n += __shfl_down_sync(0xffffffffu, n, o);
-  if ((threadIdx.x & 31) == 0 && n) atomicAdd(&cnt->n_colours, n);
 }
 
 // Fallback for palettes too large for shared memory: sites keep ascending order inside a
@@ -412,17 +429,13 @@ cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* 
   const int64_t G = (N + g - 1) / g;
   unsigned M = 0;  // levels (N < 2^30 keeps every index below 2^32)
   while (((int64_t)1 << M) < G) ++M;
-  cudaError_t e = cudaMemsetAsync(cnt->lev_rounds, 0, sizeof(cnt->lev_rounds), st);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   const unsigned nb = (unsigned)((N + 255) / 256);
   unsigned long long magic = div_magic(g);
   uint32_t* site_start = reinterpret_cast<uint32_t*>(b.meta);
   RepPlan* plan = reinterpret_cast<RepPlan*>(b.meta + 2);
-  k_kw_meta<<<1, 1, 0, st>>>((uint32_t)N, g, M, magic, site_start, plan);
-  ++*launches;
   FlowShape shape;
   if (g <= kFlowMaxPal && M < kFlowMaxLevels && flow_shape(1, N, &shape, &e)) {
-    if ((e = cudaMemsetAsync(cnt->bar, 0, sizeof(cnt->bar), st)) != cudaSuccess) return e;
     FlowView F{};
     F.R = 1;
     F.site_start = site_start;
@@ -439,16 +452,19 @@ cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* 
     F.min_tile = kFlowMinTile;
     F.ns_limit = ns_limit;
     F.vec = kFlowVecAll;
-    k_flow_init<<<nb, 256, 0, st>>>((uint32_t)N, g, g > 1 ? (uint32_t)(0x100000000ull / g) : 0xFFFFFFFFu,
-                                    F.word);
+    k_flow_init<<<nb, 256, 0, st>>>((uint32_t)N, RepPlan{g, M, magic},
+                                    g > 1 ? (uint32_t)(0x100000000ull / g) : 0xFFFFFFFFu, F.word,
+                                    site_start, plan, cnt);
     if ((e = flow_launch(F, shape, st)) != cudaSuccess) return e;
     k_flow_final<<<nb, 256, 0, st>>>((uint32_t)N, M, g, variant, F.word, b.colour, cnt);
     *launches += 3;
     return cudaGetLastError();
   }
+  if (e == cudaSuccess) e = cudaMemsetAsync(cnt->lev_rounds, 0, sizeof(cnt->lev_rounds), st);
   if (e != cudaSuccess) return e;
+  k_kw_meta<<<1, 1, 0, st>>>((uint32_t)N, g, M, magic, site_start, plan);
   k_kw_init<<<nb, 256, 0, st>>>(N, g, b.word, b.col8, b.blk);
-  ++*launches;
+  *launches += 2;
   // levels 1..low: one block per group of g 2^low vertices
   const unsigned low = kw_low_levels(g, M, kLowMaxGroup);
   if (low > 0) {
@@ -603,8 +619,7 @@ cudaError_t bucket_run(const DevParams& P, uint32_t g, const uint32_t* row_ptr, 
   const int64_t N = P.N;
   const uint32_t ntiles = (uint32_t)((N + kClassTile - 1) / kClassTile);
   if (g <= kMaxStablePalette) {
-    cudaError_t e = cudaMemsetAsync(&cnt->n_colours, 0, sizeof(unsigned), st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     const uint32_t dk = deg_bins(g);
     const size_t sh = (size_t)g * dk * sizeof(uint32_t);
     k_tile_hist<<<ntiles, 256, sh, st>>>((uint32_t)N, g, dk, ntiles, b.colour, row_ptr,
@@ -620,13 +635,11 @@ cudaError_t bucket_run(const DevParams& P, uint32_t g, const uint32_t* row_ptr, 
                                     (int)sh)) != cudaSuccess)
         return e;
       k_tile_sort<<<ntiles, 512, sh, st>>>((uint32_t)N, g, dk, ntiles, b.colour, row_ptr,
-                                           b.tile_cnt, b.perm, b.off);
+                                           b.tile_cnt, b.perm, b.off, cnt);
     } else {
       k_tile_scatter<<<ntiles, 32, sh, st>>>((uint32_t)N, g, dk, ntiles, b.colour, row_ptr,
-                                             b.tile_cnt, b.perm, b.off);
+                                             b.tile_cnt, b.perm, b.off, cnt);
     }
-    ++*launches;
-    k_nonempty_off<<<1, 1024, 0, st>>>(g, b.off, cnt);
     ++*launches;
     return cudaGetLastError();
   }

@@ -485,9 +485,10 @@ inline bool flow_shape(int R, int64_t sites, FlowShape* sh, cudaError_t* err) {
 }
 inline cudaError_t flow_launch(const FlowView& F, const FlowShape& sh, cudaStream_t st) {
   void* args[] = {(void*)&F};
-  return cudaLaunchCooperativeKernel(
-      sh.threads == 512 ? (const void*)k_kw_flow<512> : (const void*)k_kw_flow<1024>,
-      dim3(sh.grid), dim3(sh.threads), args, kw_flow_smem(F.R, sh.cap, sh.threads), st);
+  const void* k = sh.threads == 512 ? (const void*)k_kw_flow<512> : (const void*)k_kw_flow<1024>;
+  const size_t smem = kw_flow_smem(F.R, sh.cap, sh.threads);
+  if (sh.grid == 1) return cudaLaunchKernel(k, dim3(1), dim3(sh.threads), args, smem, st);
+  return cudaLaunchCooperativeKernel(k, dim3(sh.grid), dim3(sh.threads), args, smem, st);
 }
 
 }  // namespace

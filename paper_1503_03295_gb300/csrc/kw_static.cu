@@ -2,9 +2,9 @@
 //
 // Same colouring as sco_colour (palettes of at most 255 colours by the dataflow kernel of
 // kw_flow.cuh, larger ones by one barrier-free kernel per level), for callers that cannot let a
-// library allocate device memory.  Its working memory is one file-scope device array of fixed size: per-vertex words for up to
-// SCO_KW_STATIC_MAX_VERTICES vertices followed by a small control block.  Every call
-// shares that array; calls that overlap on the GPU race.
+// library allocate device memory.  Its working memory is one file-scope device array of fixed
+// size: per-vertex words for up to SCO_KW_STATIC_MAX_VERTICES vertices followed by a small control
+// block.  Every call shares that array; calls that overlap on the GPU race.
 #include <cstdint>
 #include <cstring>
 #include <mutex>

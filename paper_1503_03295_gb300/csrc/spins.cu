@@ -1,5 +1,6 @@
 // spins.cu -- initial spins and the observables of the SCO chain.
 #include <cmath>
+#include <algorithm>
 #include <cstdint>
 
 #include "sco_internal.h"
@@ -209,13 +210,16 @@ cudaError_t observables_run(const DevParams& P, const double* s, const uint32_t*
   cudaError_t e = cudaMemsetAsync(cnt->acc, 0, sizeof(cnt->acc), st);
   if (e != cudaSuccess) return e;
   const int nb = 4 * num_sms();
-  k_site_obs<<<nb, 256, 0, st>>>(P, s, cnt->acc);
+  // (a small lattice's blocks are bound by their atomic sums: 14 us of an L = 16 step at 4 per SM)
+  k_site_obs<<<(unsigned)std::min<int64_t>(nb, (P.N + 255) / 256), 256, 0, st>>>(P, s, cnt->acc);
   ++*launches;
   if (have_graph) {
     // lanes per site: as many as leave the grid's threads a site each
     const int64_t threads = (int64_t)nb * 256;
-    if (P.N * 32 <= threads) k_pair_obs<32><<<nb, 256, 0, st>>>(P, s, row_ptr, col, xy, cnt->acc);
-    else if (P.N * 8 <= threads) k_pair_obs<8><<<nb, 256, 0, st>>>(P, s, row_ptr, col, xy, cnt->acc);
+    if (P.N * 32 <= threads)
+      k_pair_obs<32><<<(unsigned)((P.N + 7) / 8), 256, 0, st>>>(P, s, row_ptr, col, xy, cnt->acc);
+    else if (P.N * 8 <= threads)
+      k_pair_obs<8><<<(unsigned)((P.N + 31) / 32), 256, 0, st>>>(P, s, row_ptr, col, xy, cnt->acc);
     else k_pair_obs<1><<<nb, 256, 0, st>>>(P, s, row_ptr, col, xy, cnt->acc);
     ++*launches;
   }
