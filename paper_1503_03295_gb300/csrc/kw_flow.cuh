@@ -112,17 +112,6 @@ __device__ __forceinline__ uint32_t flow_key(uint32_t c, uint32_t b, uint32_t e,
   const uint32_t ns = ((e + 7) >> 3) - (b >> 3);
   return pal > 64 ? 255u - c : 4 * (63u - c) + (ns < 3 ? 0u : min(ns - 2, 3u));
 }
-// Lanes of the warp that hold the same key (all lanes call it).
-__device__ __forceinline__ unsigned flow_peers(uint32_t key) {
-  unsigned m = 0xffffffffu;
-#pragma unroll
-  for (int b = 0; b < 9; ++b) {
-    const unsigned v = __ballot_sync(0xffffffffu, (key >> b) & 1u);
-    m &= (key >> b) & 1u ? v : ~v;
-  }
-  return m;
-}
-
 // Word of a vertex in shared memory: round << 8 | colour once it is done, before that 2^31 | previous
 // colour << 16 | kFlowNone.  A done right-half neighbour is a larger one (a smaller one waits for
 // this vertex), so only open ones are compared.  flow_bit(kFlowNone) is no colour.
@@ -159,7 +148,6 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
   uint16_t* list = ord + V.cap + (threadIdx.x & ~31u) * kFlowList + (threadIdx.x & 31u);
   const uint32_t tid = threadIdx.x;
   const int lane = (int)(tid & 31);
-  const unsigned below = (1u << lane) - 1u;
   for (int r = tid; r <= R; r += T) sbase[r] = V.site_start[r];
   if (tid == 0) st[V.cap] = kFlowNone;
   const RepPlan pl0 = V.plan[0];
@@ -237,8 +225,7 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
         const uint32_t key = q < n ? flow_key(c[a] & 0xFFu, rb[a], re[a], pal) : kFlowKeys;
         if (q < n) st[q] = 0x80000000u | ((c[a] & 0xFFu) << 16) | (key << 8) | kFlowNone;
         if (q0 + a * T >= n) break;  // uniform
-        const unsigned peers = flow_peers(key);
-        if (q < n && (peers & below) == 0) atomicAdd(&cur[key], (uint32_t)__popc(peers));
+        if (q < n) atomicAdd(&cur[key], 1u);
       }
     }
     __syncthreads();
@@ -267,12 +254,8 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
       const uint32_t q = q0 + tid;
       const uint32_t w = q < n ? st[q] : 0u;
       const uint32_t key = q < n ? (w >> 8) & 0xFFu : kFlowKeys;
-      const unsigned peers = flow_peers(key);
-      uint32_t at = 0;
-      if (q < n && (peers & below) == 0) at = atomicAdd(&cur[key], (uint32_t)__popc(peers));
-      at = __shfl_sync(0xffffffffu, at, __ffs(peers) - 1);
       if (q < n) {
-        ord[at + __popc(peers & below)] = (uint16_t)q;
+        ord[atomicAdd(&cur[key], 1u)] = (uint16_t)q;
         st[q] = w & 0xFFFF00FFu;
       }
     }
