@@ -236,8 +236,8 @@ sco_status do_switch(sco_ctx* c, uint32_t epoch, const double* src, const float4
   c->nnz = c->hcnt->nnz;
   SCO_TRY(grow(c->col, c->col_cap, c->nnz > 0 ? c->nnz : 1));
   // rows are left unsorted (their order changes no result); getters sort their copies
-  SCO_TRY(csr_fill(c->P, c->sw, c->row_ptr, c->col, c->hcnt->ovf_n > 0, c->cnt, c->st,
-                   &c->launches));
+  SCO_TRY(csr_fill(c->P, c->sw, c->hcnt->max_degree + 1, c->row_ptr, c->col, c->hcnt->ovf_n > 0,
+                   c->cnt, c->st, &c->launches));
   c->dip_valid = false;
   c->g = c->hcnt->max_degree + 1;
   c->graph_epoch = epoch;
@@ -270,7 +270,7 @@ sco_status do_colour(sco_ctx* c) {
     SCO_TRY(cudaMalloc(&c->cb.scan_tmp, scan_tmp_bytes(tc > cap + 1 ? tc : cap + 1)));
     c->cls_cap = cap;
   }
-  SCO_TRY(kw_run(c->P, c->row_ptr, c->col, c->g, c->p.colour_variant, c->cb, c->cnt,
+  SCO_TRY(kw_run(c->P, c->row_ptr, c->col, c->sw.lcur, c->g, c->p.colour_variant, c->cb, c->cnt,
                  c->ns_limit, c->st, &c->launches));
   SCO_TRY(bucket_run(c->P, c->g, c->row_ptr, c->cb, c->cnt, c->st, &c->launches));
   c->colour_valid = true;
@@ -300,7 +300,6 @@ void free_all(sco_ctx* c) {
   cudaFree(c->sw.indeg);
   cudaFree(c->sw.deg);
   cudaFree(c->sw.lcur);
-  cudaFree(c->sw.ocur);
   cudaFree(c->sw.ovf);
   cudaFree(c->sw.scan_tmp);
   cudaFree(c->row_ptr);
@@ -385,7 +384,6 @@ sco_status sco_init(const sco_params* p, void* stream, sco_ctx** out) {
   if (e == cudaSuccess) e = cudaMalloc(&c->sw.indeg, N * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&c->sw.deg, (N + 1) * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&c->sw.lcur, N * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&c->sw.ocur, N * sizeof(uint32_t));
   c->sw.ovf_cap = (uint32_t)(N > 65536 ? N : 65536);
   if (e == cudaSuccess) e = cudaMalloc(&c->sw.ovf, 2 * (size_t)c->sw.ovf_cap * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&c->sw.scan_tmp, scan_tmp_bytes(N + 1));

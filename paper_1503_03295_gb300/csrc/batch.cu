@@ -140,7 +140,8 @@ __global__ void __launch_bounds__(1024) kb_plan(const BatchDev B) {
     const unsigned long long G = ((unsigned long long)N + g - 1) / g;
     unsigned M = 0;
     while ((1ull << M) < G) ++M;
-    B.plan[r] = RepPlan{g, M, div_magic(g)};
+    B.plan[r] = RepPlan{g, (uint16_t)M, (uint16_t)near_levels(g, (uint32_t)B.desc[r].P.Lx),
+                        div_magic(g)};
     B.cnt[r].g = g;
     B.cnt[r].levels = M;
     B.cnt[r].nnz = (unsigned long long)(B.row_ptr[base + N] - B.row_ptr[base]);
@@ -171,12 +172,12 @@ __global__ void __launch_bounds__(256) kb_fill(const BatchDev B) {
   if (i >= N) return;
   const uint32_t gs = base + i;
   const uint32_t n = min(B.hcnt[gs], (uint32_t)kSlotCap);
-  const uint32_t up = B.row_ptr[gs] + B.indeg[gs];
+  const RowFill F = row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx);
+  const uint32_t end = near_end(F, i);
   for (uint32_t q = 0; q < n; ++q) {
-    const uint32_t jv = B.hslot[(size_t)gs * kSlotCap + q];
-    const uint32_t jg = base + (jv & kIndexMask);
-    B.col[up + q] = jv;
-    B.col[B.row_ptr[jg] + atomicAdd(&B.lcur[jg], 1u)] = i | (jv & kExchOnly);
+    const uint32_t jv = B.hslot[(size_t)gs * kSlotCap + q], j = jv & kIndexMask;
+    B.col[row_place(F, j < end, B.row_ptr, B.lcur, gs)] = jv;
+    B.col[row_place(F, j < end, B.row_ptr, B.lcur, base + j)] = i | (jv & kExchOnly);
   }
 }
 
@@ -186,12 +187,13 @@ __global__ void __launch_bounds__(256) kb_fill_ovf(const BatchDev B) {
   if (n > B.ovf_cap) n = B.ovf_cap;
   for (unsigned long long q = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; q < n;
        q += (unsigned long long)gridDim.x * blockDim.x) {
-    const uint32_t gs = B.ovf[2 * q], jv = B.ovf[2 * q + 1];
+    const uint32_t gs = B.ovf[2 * q], jv = B.ovf[2 * q + 1], j = jv & kIndexMask;
     const int r = find_le(B.site_start, B.R, gs);
     const uint32_t base = B.site_start[r];
-    const uint32_t jg = base + (jv & kIndexMask);
-    B.col[B.row_ptr[gs] + B.indeg[gs] + kSlotCap + atomicAdd(&B.ocur[gs], 1u)] = jv;
-    B.col[B.row_ptr[jg] + atomicAdd(&B.lcur[jg], 1u)] = (gs - base) | (jv & kExchOnly);
+    const RowFill F = row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx);
+    const bool near = j < near_end(F, gs - base);
+    B.col[row_place(F, near, B.row_ptr, B.lcur, gs)] = jv;
+    B.col[row_place(F, near, B.row_ptr, B.lcur, base + j)] = (gs - base) | (jv & kExchOnly);
   }
 }
 
@@ -536,8 +538,6 @@ cudaError_t batch_switch(const BatchDev& B, const BatchLaunch& L, cudaStream_t s
     return e;
   if ((e = cudaMemsetAsync(B.lcur, 0, (size_t)B.Ntot * sizeof(uint32_t), st)) != cudaSuccess)
     return e;
-  if ((e = cudaMemsetAsync(B.ocur, 0, (size_t)B.Ntot * sizeof(uint32_t), st)) != cudaSuccess)
-    return e;
   // up to 8 blocks' worth of sites each while the grid stays two waves of four blocks per SM
   const uint32_t per = std::max(1u, std::min(8u, B.nblocks / (8u * (uint32_t)num_sms())));
   const unsigned nsw = (B.nblocks + per - 1) / per;
@@ -573,6 +573,7 @@ cudaError_t batch_colour(const BatchDev& B, const BatchLaunch& L, cudaStream_t s
     F.plan = B.plan;
     F.row_ptr = B.row_ptr;
     F.col = B.col;
+    F.rows = B.lcur;
     F.word = reinterpret_cast<uint32_t*>(B.word);
     F.lev_rounds = B.cnt->lev_rounds;
     F.lev_stride = sizeof(DevCounters) / sizeof(unsigned);

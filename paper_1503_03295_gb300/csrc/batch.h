@@ -34,19 +34,14 @@ struct RepDesc {
   int32_t variant;     // colouring variant (reported t_R only)
 };
 
-// Palettes up to this size are coloured by the dataflow kernel (kw_flow.cuh): a colour has a byte of
-// a word in shared memory.  Against the kernels by rounds and buckets, per colouring: L = 1024,
-// palette 77 29.2 -> 2.8 ms; L = 512, 118 27.5 -> 9.7; L = 1024, 136 89.5 -> 13.2; L = 256, 170
-// 35.9 -> 23.4 (chains of 1500 rounds).
-constexpr uint32_t kFlowMaxPal = 255;
-
 // Larger right-half neighbours listed per bucketed vertex of the KW colouring (records).
 constexpr int kKwItemList = 32;
 
 // Per-step plan of replica r, written on the device once the graph is known.
 struct RepPlan {
   uint32_t g;       // Delta + 1
-  uint32_t levels;  // KW levels M
+  uint16_t levels;  // KW levels M
+  uint16_t near;    // levels whose groups the near parts of the rows cover (near_levels; 0: none)
   unsigned long long magic;  // div_magic(g)
 };
 
@@ -89,8 +84,7 @@ struct BatchDev {
   uint32_t* hcnt;
   uint32_t* indeg;
   uint32_t* deg;  // Ntot + 1 (deg[Ntot] stays 0)
-  uint32_t* lcur;
-  uint32_t* ocur;
+  uint32_t* lcur;  // row cursors, then what the rows hold (see RowFill)
   uint32_t* ovf;
   uint32_t ovf_cap;
   uint32_t* row_ptr;  // Ntot + 1

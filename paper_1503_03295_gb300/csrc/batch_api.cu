@@ -91,7 +91,6 @@ void free_all(sco_batch* b) {
   cudaFree(B.indeg);
   cudaFree(B.deg);
   cudaFree(B.lcur);
-  cudaFree(B.ocur);
   cudaFree(B.ovf);
   cudaFree(B.row_ptr);
   cudaFree(B.col);
@@ -425,7 +424,6 @@ sco_status sco_batch_init(const sco_params* p, int32_t n, void* stream, sco_batc
   A(&B.indeg, N * sizeof(uint32_t));
   A(&B.deg, (N + 1) * sizeof(uint32_t));
   A(&B.lcur, N * sizeof(uint32_t));
-  A(&B.ocur, N * sizeof(uint32_t));
   B.ovf_cap = (uint32_t)std::max<size_t>(N, 65536);
   A(&B.ovf, 2 * (size_t)B.ovf_cap * sizeof(uint32_t));
   A(&B.row_ptr, (N + 1) * sizeof(uint32_t));

@@ -378,7 +378,7 @@ __global__ void k_kw_meta(uint32_t N, uint32_t g, unsigned levels, unsigned long
                           uint32_t* site_start, RepPlan* plan) {
   site_start[0] = 0;
   site_start[1] = N;
-  plan[0] = RepPlan{g, levels, magic};
+  plan[0] = RepPlan{g, (uint16_t)levels, 0, magic};
 }
 
 // Blocks per SM and staged-edge capacity of the block-local level kernel for groups of gcap
@@ -423,7 +423,7 @@ constexpr int kRecWBlocks = 6;
 constexpr uint64_t kRecWarpRows = 12;
 
 cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* col,
-                   uint32_t g, int variant, ColourBufs& b, DevCounters* cnt,
+                   const uint32_t* rows, uint32_t g, int variant, ColourBufs& b, DevCounters* cnt,
                    unsigned long long ns_limit, cudaStream_t st, int64_t* launches) {
   const int64_t N = P.N;
   const int64_t G = (N + g - 1) / g;
@@ -442,6 +442,7 @@ cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* 
     F.plan = plan;
     F.row_ptr = row_ptr;
     F.col = col;
+    F.rows = rows;
     F.word = reinterpret_cast<uint32_t*>(b.word);
     F.lev_rounds = cnt->lev_rounds;
     F.lev_stride = 0;
@@ -452,7 +453,7 @@ cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* 
     F.min_tile = kFlowMinTile;
     F.ns_limit = ns_limit;
     F.vec = kFlowVecAll;
-    k_flow_init<<<nb, 256, 0, st>>>((uint32_t)N, RepPlan{g, M, magic},
+    k_flow_init<<<nb, 256, 0, st>>>((uint32_t)N, RepPlan{g, (uint16_t)M, (uint16_t)near_levels(g, (uint32_t)P.Lx), magic},
                                     g > 1 ? (uint32_t)(0x100000000ull / g) : 0xFFFFFFFFu, F.word,
                                     site_start, plan, cnt);
     if ((e = flow_launch(F, shape, st)) != cudaSuccess) return e;

@@ -43,9 +43,10 @@ constexpr int kFlowChunk = 8;          // row entries read together (a multiple 
 struct FlowView {
   int R;                       // lattices (1 for a single lattice)
   const uint32_t* site_start;  // R + 1 first vertex of each lattice
-  const RepPlan* plan;         // R: g, levels, magic
+  const RepPlan* plan;         // R: g, levels, near, magic
   const uint32_t* row_ptr;     // global entry offsets; col entries lattice-local
   const uint32_t* col;
+  const uint32_t* rows;        // near entries of a row in the high half (see RowFill; null: no plan has near)
   // global vertex index: level << 27 | round << 8 | colour, the level and round of the last
   // recolouring; level 0 and the initial colour on entry
   uint32_t* word;
@@ -195,6 +196,11 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
     }
     own = min(own, V.cap);
     const uint32_t s0 = min(total, blockIdx.x * own), n = min(own, total - s0);
+    // first entry of vertex gv's row that the level looks at (near_levels)
+    auto row_begin = [&](uint32_t gv, int r) {
+      const uint32_t near = R == 1 ? pl0.near : V.plan[r].near;
+      return p <= near ? V.row_ptr[gv + 1] - (V.rows[gv] >> 16) : V.row_ptr[gv];
+    };
     // lattice, group and offsets of a slot
     auto locate = [&](uint32_t slot, int& r, uint32_t& k, uint32_t& half) {
       r = R == 1 ? 0 : find_le(rp, R, slot);
@@ -215,7 +221,7 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
           locate(s0 + q, r, k, half);
           const uint32_t gv = sbase[r] + (s0 + q - rp[r]) + (k + 1) * half;
           c[a] = flow_ld(&V.word[gv]);
-          rb[a] = V.row_ptr[gv];
+          rb[a] = row_begin(gv, r);
           re[a] = V.row_ptr[gv + 1];
         }
       }
@@ -276,7 +282,7 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
         locate(s0 + loc, r, k, half);
         base = sbase[r];
         gv = base + (s0 + loc - rp[r]) + (k + 1) * half;
-        b = V.row_ptr[gv];
+        b = row_begin(gv, r);
         e = V.row_ptr[gv + 1];
         c = (st[loc] >> 16) & 0xFFu;
         lo = 2 * k * half;

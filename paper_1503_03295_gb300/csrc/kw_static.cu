@@ -56,7 +56,7 @@ __global__ void k_st_setup(uint32_t n, StaticCtrl* __restrict__ ctrl) {
   ctrl->g = g;
   ctrl->levels = M;
   ctrl->magic = div_magic(g);
-  ctrl->plan = RepPlan{g, M, div_magic(g)};
+  ctrl->plan = RepPlan{g, (uint16_t)M, 0, div_magic(g)};
   ctrl->site_start[0] = 0;
   ctrl->site_start[1] = n;
 }

@@ -127,13 +127,43 @@ cudaError_t full_energy_fft(const DevParams& P, const double* s, void* work, dou
 
 // ---- switch.cu ----
 constexpr int kSlotCap = 32;
+
+// Palettes up to this size are coloured by the dataflow kernel (kw_flow.cuh): a colour has a byte of
+// a word in shared memory.  Against the kernels by rounds and buckets, per colouring: L = 1024,
+// palette 77 29.2 -> 2.8 ms; L = 512, 118 27.5 -> 9.7; L = 1024, 136 89.5 -> 13.2; L = 256, 170
+// 35.9 -> 23.4 (chains of 1500 rounds).
+constexpr uint32_t kFlowMaxPal = 255;
+
+// The colouring's level p only looks at neighbours in the same group of g 2^p consecutive sites, for
+// the low levels about a sixth of a row, but every row is read at every level.  So the fill
+// puts the neighbours in the same group at level near_levels (two lattice rows at most) at the end
+// of the row, and the levels up to that one read that end alone.  Sectors read over all levels, by
+// the rows that a group spans, against whole rows: 0.56 rows 0.894, 1.1 0.849, 2.25 0.847, 4.5
+// 0.870, 9 0.902 (L = 256, T = 0.6 D); 1.4 0.826, 2.9 0.834, 5.8 0.866 (L = 512, T = 0.4 D).
+// Per colouring, without and with: L = 2304 3.96 -> 3.77 ms, L = 1024 T = 0.4 D 1.21 -> 1.15; groups of
+// up to one row 3.81 and 1.16, four rows 3.78 and 1.15.
+__host__ __device__ inline unsigned near_levels(uint32_t g, uint32_t Lx) {
+  unsigned p = 0;
+  if (g <= kFlowMaxPal)
+    while ((g << (p + 1)) <= 2 * Lx) ++p;
+  return p;
+}
+// Where the fill puts the neighbours of a lattice: cur counts a row's far (low 16 bits) and near
+// entries, which stay below 2^16 for palettes of the dataflow kernel; larger ones have no near part
+// and count in 32 bits.
+struct RowFill {
+  uint32_t group, mask;  // sites per group (0: no near part), far count in a cursor
+};
+__host__ __device__ inline RowFill row_fill(uint32_t g, uint32_t Lx) {
+  const unsigned p = near_levels(g, Lx);
+  return p ? RowFill{g << p, 0xFFFFu} : RowFill{0, 0xFFFFFFFFu};
+}
 struct SwitchBufs {
   uint32_t* hslot;  // N * kSlotCap upper neighbours (j | flag) per site
   uint32_t* hcnt;   // N half-degree per site
-  uint32_t* indeg;  // N lower-neighbour count per site (also the fill cursor base)
+  uint32_t* indeg;  // N lower-neighbour count per site
   uint32_t* deg;    // N + 1
-  uint32_t* lcur;   // N lower fill cursor
-  uint32_t* ocur;   // N overflow fill cursor
+  uint32_t* lcur;   // N row cursors, then what the rows hold (see RowFill)
   uint32_t* ovf;    // 2 * ovf_cap (i, j | flag)
   uint32_t ovf_cap;
   uint64_t* scan_tmp;
@@ -143,9 +173,9 @@ cudaError_t switch_run(const DevParams& P, const Table& t, const double* s, cons
                        cudaStream_t st, int64_t* launches);
 cudaError_t csr_scan(const DevParams& P, SwitchBufs& b, uint32_t* row_ptr, DevCounters* cnt,
                      cudaStream_t st, int64_t* launches);
-// A row holds its lower neighbours in the order of their atomic slots, then its upper ones in
-// switching order (no result depends on the order inside a row).
-cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, const uint32_t* row_ptr,
+// A row holds its far neighbours from its start and its near ones from its end, each in the order of
+// their atomic slots (no result depends on the order inside a row).
+cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, uint32_t g, const uint32_t* row_ptr,
                      uint32_t* col, bool has_overflow, DevCounters* cnt, cudaStream_t st,
                      int64_t* launches);
 // out = col[first ..] with every row sorted by neighbour index (the documented layout of the
@@ -177,8 +207,9 @@ struct ColourBufs {
 constexpr int kKwSplitBlocks = 2048;
 constexpr uint32_t kMaxStablePalette = 12288;  // palettes up to this size get stable classes
 constexpr int64_t kClassTileSites = 2048;
-// ns_limit: bound of every device-side wait of the colouring kernels (SCO_ETIMEOUT after it)
-cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* col,
+// rows: the cursors that csr_fill left; ns_limit: bound of every device-side wait of the colouring
+// kernels (SCO_ETIMEOUT after it)
+cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* col, const uint32_t* rows,
                    uint32_t g, int variant, ColourBufs& b, DevCounters* cnt,
                    unsigned long long ns_limit, cudaStream_t st, int64_t* launches);
 cudaError_t bucket_run(const DevParams& P, uint32_t g, const uint32_t* row_ptr, ColourBufs& b,

@@ -57,50 +57,59 @@ __global__ void k_degree(int64_t N, const uint32_t* __restrict__ hcnt,
     atomicMax(&cnt->max_degree, m);
 }
 
-// Row i holds its lower neighbours (j < i, scattered here by the sites j) followed by its
-// upper neighbours (written by site i from its slots).  Rows are sorted afterwards.
-__global__ void k_fill(int64_t N, const uint32_t* __restrict__ hslot,
-                       const uint32_t* __restrict__ hcnt, const uint32_t* __restrict__ indeg,
-                       const uint32_t* __restrict__ row_ptr, uint32_t* __restrict__ lcur,
-                       uint32_t* __restrict__ col) {
+// Every surviving half-edge (i, j) goes into rows i and j (see RowFill): a thread per site, eight
+// half-edges at a time, whose slot and row-pointer loads, atomics and stores are each issued
+// together (the atomics' returns were the chain).
+__global__ void k_fill(int64_t N, RowFill F, const uint32_t* __restrict__ hslot,
+                       const uint32_t* __restrict__ hcnt, const uint32_t* __restrict__ row_ptr,
+                       uint32_t* __restrict__ cur, uint32_t* __restrict__ col) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
   const uint32_t n = min(hcnt[i], (uint32_t)kSlotCap);
-  const uint32_t up = row_ptr[i] + indeg[i];
-  // eight half-edges at a time: their slot and row-pointer loads, then their atomics, then their
-  // stores, each group issued together (the atomics' returns were the chain)
+  const uint32_t end = near_end(F, (uint32_t)i);
   constexpr uint32_t kB = 8;
   for (uint32_t q0 = 0; q0 < n; q0 += kB) {
-    uint32_t jv[kB], base[kB], lo[kB];
+    uint32_t jv[kB], base[kB], at[kB];
+    uint32_t nn = 0;
 #pragma unroll
     for (uint32_t a = 0; a < kB; ++a)
-      jv[a] = q0 + a < n ? hslot[i * (int64_t)kSlotCap + q0 + a] : 0u;
+      jv[a] = q0 + a < n ? hslot[i * (int64_t)kSlotCap + q0 + a] : kIndexMask;
 #pragma unroll
-    for (uint32_t a = 0; a < kB; ++a) base[a] = q0 + a < n ? row_ptr[jv[a] & kIndexMask] : 0u;
+    for (uint32_t a = 0; a < kB; ++a) {
+      const uint32_t j = jv[a] & kIndexMask;
+      const bool on = q0 + a < n, near = on && j < end;
+      base[a] = on ? row_ptr[near ? j + 1 : j] : 0u;
+      nn += near ? 1u : 0u;
+    }
+    uint32_t own = atomicAdd(&cur[i], (min(n - q0, kB) - nn) | (nn << 16));
 #pragma unroll
-    for (uint32_t a = 0; a < kB; ++a)
-      lo[a] = q0 + a < n ? base[a] + atomicAdd(&lcur[jv[a] & kIndexMask], 1u) : 0u;
+    for (uint32_t a = 0; a < kB; ++a) {
+      const uint32_t j = jv[a] & kIndexMask;
+      at[a] = q0 + a < n ? atomicAdd(&cur[j], j < end ? 0x10000u : 1u) : 0u;
+    }
+    const uint32_t b = row_ptr[i], e = row_ptr[i + 1];
 #pragma unroll
     for (uint32_t a = 0; a < kB; ++a) {
       if (q0 + a >= n) continue;
-      col[up + q0 + a] = jv[a];
-      col[lo[a]] = (uint32_t)i | (jv[a] & kExchOnly);
+      const bool near = (jv[a] & kIndexMask) < end;
+      col[near ? e - 1 - (own >> 16) : b + (own & F.mask)] = jv[a];
+      own += near ? 0x10000u : 1u;
+      col[near ? base[a] - 1 - (at[a] >> 16) : base[a] + (at[a] & F.mask)] =
+          (uint32_t)i | (jv[a] & kExchOnly);
     }
   }
 }
 
-__global__ void k_fill_ovf(unsigned long long n, const uint32_t* __restrict__ ovf,
-                           const uint32_t* __restrict__ indeg,
-                           const uint32_t* __restrict__ row_ptr, uint32_t* __restrict__ lcur,
-                           uint32_t* __restrict__ ocur, uint32_t* __restrict__ col) {
+__global__ void k_fill_ovf(unsigned long long n, RowFill F, const uint32_t* __restrict__ ovf,
+                           const uint32_t* __restrict__ row_ptr, uint32_t* __restrict__ cur,
+                           uint32_t* __restrict__ col) {
   const unsigned long long q = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
   if (q >= n) return;
   const uint32_t i = ovf[2 * q], jv = ovf[2 * q + 1];
   const uint32_t j = jv & kIndexMask;
-  const uint32_t up = row_ptr[i] + indeg[i] + kSlotCap + atomicAdd(&ocur[i], 1u);
-  const uint32_t lo = row_ptr[j] + atomicAdd(&lcur[j], 1u);
-  col[up] = jv;
-  col[lo] = i | (jv & kExchOnly);
+  const bool near = j < near_end(F, i);
+  col[row_place(F, near, row_ptr, cur, i)] = jv;
+  col[row_place(F, near, row_ptr, cur, j)] = i | (jv & kExchOnly);
 }
 
 __global__ void k_rowsort(int64_t N, const uint32_t* __restrict__ row_ptr, uint32_t first,
@@ -152,13 +161,14 @@ cudaError_t csr_scan(const DevParams& P, SwitchBufs& b, uint32_t* row_ptr, DevCo
                        reinterpret_cast<uint64_t*>(&cnt->nnz), st, launches);
 }
 
-cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, const uint32_t* row_ptr,
+cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, uint32_t g, const uint32_t* row_ptr,
                      uint32_t* col, bool has_overflow, DevCounters* cnt, cudaStream_t st,
                      int64_t* launches) {
   cudaError_t e = cudaMemsetAsync(b.lcur, 0, P.N * sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
   const unsigned nb = (unsigned)((P.N + 255) / 256);
-  k_fill<<<nb, 256, 0, st>>>(P.N, b.hslot, b.hcnt, b.indeg, row_ptr, b.lcur, col);
+  const RowFill F = row_fill(g, (uint32_t)P.Lx);
+  k_fill<<<nb, 256, 0, st>>>(P.N, F, b.hslot, b.hcnt, row_ptr, b.lcur, col);
   ++*launches;
   if (has_overflow) {
     unsigned long long n = 0;
@@ -166,11 +176,8 @@ cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, const uint32_t* ro
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e;
     if (n > b.ovf_cap) n = b.ovf_cap;
-    e = cudaMemsetAsync(b.ocur, 0, P.N * sizeof(uint32_t), st);
-    if (e != cudaSuccess) return e;
     if (n > 0) {
-      k_fill_ovf<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, b.ovf, b.indeg, row_ptr, b.lcur,
-                                                              b.ocur, col);
+      k_fill_ovf<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, F, b.ovf, row_ptr, b.lcur, col);
       ++*launches;
     }
   }

@@ -550,5 +550,19 @@ __device__ __forceinline__ unsigned sort_row(uint32_t* __restrict__ r, uint32_t 
   return nd;
 }
 
+// End of site i's group (see RowFill): neighbours below it from above i, and from below i those i is
+// one of for, are near.
+__device__ __forceinline__ uint32_t near_end(const RowFill& F, uint32_t i) {
+  return F.group ? (i / F.group + 1) * F.group : 0u;
+}
+// The next place in site i's row.
+__device__ __forceinline__ uint32_t row_place(const RowFill& F, bool near,
+                                              const uint32_t* __restrict__ row_ptr,
+                                              uint32_t* __restrict__ cur, uint32_t i) {
+  const uint32_t base = row_ptr[near ? i + 1 : i];
+  const uint32_t at = atomicAdd(&cur[i], near ? 0x10000u : 1u);
+  return near ? base - 1 - (at >> 16) : base + (at & F.mask);
+}
+
 }  // namespace
 }  // namespace sco

@@ -27,6 +27,8 @@ def _compare(g, o):
     (301, 299, 0.6, 0.0), (700, 301, 0.9, 1.0),
     (1024, 700, 0.3, 0.0),   # larger blocks, mean degree 30: lists read in parts
     (40, 40, 0.1, 0.0), (301, 200, 0.1, 0.0),  # palettes of 65 to 255: colours above 31 looked up again
+    # near parts of the rows: none (one column), of a few levels, of every level
+    (1, 700, 0.2, 0.0), (7, 900, 0.4, 0.0), (900, 2, 0.3, 0.0),
     (40, 40, 0.006, 0.0), (200, 150, 0.011, 0.0),  # palettes above 255: the other kernels
 ])
 def test_colouring_matches_oracle(Lx, Ly, T, J):
