@@ -37,7 +37,7 @@ constexpr unsigned kFlowMaxLevels = 32;
 // mean degree 23, from 1.36 to 1.23 ms per colouring, but does not fit beside the words of a large
 // lattice's blocks), and neighbours outside the block looked up together.
 __host__ __device__ constexpr int flow_list(int threads) { return threads == 512 ? 40 : 24; }
-__host__ __device__ constexpr int flow_look(int threads) { return threads == 512 ? 8 : 4; }
+__host__ __device__ constexpr int flow_look(int threads) { return threads == 512 ? 8 : 6; }
 constexpr int kFlowChunk = 8;          // row entries read together (a multiple of 8)
 
 struct FlowView {
