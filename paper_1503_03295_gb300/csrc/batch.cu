@@ -171,14 +171,8 @@ __global__ void __launch_bounds__(256) kb_fill(const BatchDev B) {
   const uint32_t i = (blockIdx.x - B.blk_start[r]) * kBatchBlock + threadIdx.x;
   if (i >= N) return;
   const uint32_t gs = base + i;
-  const uint32_t n = min(B.hcnt[gs], (uint32_t)kSlotCap);
-  const RowFill F = row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx);
-  const uint32_t end = near_end(F, i);
-  for (uint32_t q = 0; q < n; ++q) {
-    const uint32_t jv = B.hslot[(size_t)gs * kSlotCap + q], j = jv & kIndexMask;
-    B.col[row_place(F, j < end, B.row_ptr, B.lcur, gs)] = jv;
-    B.col[row_place(F, j < end, B.row_ptr, B.lcur, base + j)] = i | (jv & kExchOnly);
-  }
+  fill_rows(row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx), i, B.hslot + (size_t)gs * kSlotCap,
+            B.hcnt[gs], B.row_ptr + base, B.lcur + base, B.col);
 }
 
 __global__ void __launch_bounds__(256) kb_fill_ovf(const BatchDev B) {

@@ -57,47 +57,11 @@ __global__ void k_degree(int64_t N, const uint32_t* __restrict__ hcnt,
     atomicMax(&cnt->max_degree, m);
 }
 
-// Every surviving half-edge (i, j) goes into rows i and j (see RowFill): a thread per site, eight
-// half-edges at a time, whose slot and row-pointer loads, atomics and stores are each issued
-// together (the atomics' returns were the chain).
 __global__ void k_fill(int64_t N, RowFill F, const uint32_t* __restrict__ hslot,
                        const uint32_t* __restrict__ hcnt, const uint32_t* __restrict__ row_ptr,
                        uint32_t* __restrict__ cur, uint32_t* __restrict__ col) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  const uint32_t n = min(hcnt[i], (uint32_t)kSlotCap);
-  const uint32_t end = near_end(F, (uint32_t)i);
-  constexpr uint32_t kB = 8;
-  for (uint32_t q0 = 0; q0 < n; q0 += kB) {
-    uint32_t jv[kB], base[kB], at[kB];
-    uint32_t nn = 0;
-#pragma unroll
-    for (uint32_t a = 0; a < kB; ++a)
-      jv[a] = q0 + a < n ? hslot[i * (int64_t)kSlotCap + q0 + a] : kIndexMask;
-#pragma unroll
-    for (uint32_t a = 0; a < kB; ++a) {
-      const uint32_t j = jv[a] & kIndexMask;
-      const bool on = q0 + a < n, near = on && j < end;
-      base[a] = on ? row_ptr[near ? j + 1 : j] : 0u;
-      nn += near ? 1u : 0u;
-    }
-    uint32_t own = atomicAdd(&cur[i], (min(n - q0, kB) - nn) | (nn << 16));
-#pragma unroll
-    for (uint32_t a = 0; a < kB; ++a) {
-      const uint32_t j = jv[a] & kIndexMask;
-      at[a] = q0 + a < n ? atomicAdd(&cur[j], j < end ? 0x10000u : 1u) : 0u;
-    }
-    const uint32_t b = row_ptr[i], e = row_ptr[i + 1];
-#pragma unroll
-    for (uint32_t a = 0; a < kB; ++a) {
-      if (q0 + a >= n) continue;
-      const bool near = (jv[a] & kIndexMask) < end;
-      col[near ? e - 1 - (own >> 16) : b + (own & F.mask)] = jv[a];
-      own += near ? 0x10000u : 1u;
-      col[near ? base[a] - 1 - (at[a] >> 16) : base[a] + (at[a] & F.mask)] =
-          (uint32_t)i | (jv[a] & kExchOnly);
-    }
-  }
+  if (i < N) fill_rows(F, (uint32_t)i, hslot + i * (int64_t)kSlotCap, hcnt[i], row_ptr, cur, col);
 }
 
 __global__ void k_fill_ovf(unsigned long long n, RowFill F, const uint32_t* __restrict__ ovf,

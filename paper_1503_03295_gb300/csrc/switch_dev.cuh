@@ -564,5 +564,45 @@ __device__ __forceinline__ uint32_t row_place(const RowFill& F, bool near,
   return near ? base - 1 - (at >> 16) : base + (at & F.mask);
 }
 
+// Every surviving half-edge (i, j) of site i's slots goes into rows i and j (see RowFill; indices and
+// arrays of one lattice): eight half-edges at a time, whose slot and row-pointer loads, atomics and
+// stores are each issued together (the atomics' returns were the chain).
+__device__ __forceinline__ void fill_rows(const RowFill& F, uint32_t i,
+                                          const uint32_t* __restrict__ slot, uint32_t hcnt,
+                                          const uint32_t* __restrict__ row_ptr,
+                                          uint32_t* __restrict__ cur, uint32_t* __restrict__ col) {
+  const uint32_t n = min(hcnt, (uint32_t)kSlotCap);
+  const uint32_t end = near_end(F, i);
+  constexpr uint32_t kB = 8;
+  for (uint32_t q0 = 0; q0 < n; q0 += kB) {
+    uint32_t jv[kB], base[kB], at[kB];
+    uint32_t nn = 0;
+#pragma unroll
+    for (uint32_t a = 0; a < kB; ++a) jv[a] = q0 + a < n ? slot[q0 + a] : kIndexMask;
+#pragma unroll
+    for (uint32_t a = 0; a < kB; ++a) {
+      const uint32_t j = jv[a] & kIndexMask;
+      const bool on = q0 + a < n, near = on && j < end;
+      base[a] = on ? row_ptr[near ? j + 1 : j] : 0u;
+      nn += near ? 1u : 0u;
+    }
+    uint32_t own = atomicAdd(&cur[i], (min(n - q0, kB) - nn) | (nn << 16));
+#pragma unroll
+    for (uint32_t a = 0; a < kB; ++a) {
+      const uint32_t j = jv[a] & kIndexMask;
+      at[a] = q0 + a < n ? atomicAdd(&cur[j], j < end ? 0x10000u : 1u) : 0u;
+    }
+    const uint32_t b = row_ptr[i], e = row_ptr[i + 1];
+#pragma unroll
+    for (uint32_t a = 0; a < kB; ++a) {
+      if (q0 + a >= n) continue;
+      const bool near = (jv[a] & kIndexMask) < end;
+      col[near ? e - 1 - (own >> 16) : b + (own & F.mask)] = jv[a];
+      own += near ? 0x10000u : 1u;
+      col[near ? base[a] - 1 - (at[a] >> 16) : base[a] + (at[a] & F.mask)] = i | (jv[a] & kExchOnly);
+    }
+  }
+}
+
 }  // namespace
 }  // namespace sco
