@@ -514,15 +514,12 @@ cudaError_t batch_low_setup(int R, uint32_t gcap, int* blocks_per_sm, uint32_t* 
   return cudaSuccess;
 }
 
-int batch_sweep_occupancy(int precision, int R) {
+int batch_sweep_occupancy(int precision, int R, uint32_t sites) {
   int n = 0;
-  const cudaError_t e =
-      precision == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep<1, true, true, 3>,
-                                                                     kSweepThreads, sweep_smem(R))
-                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep<0, true, true, 2>,
-                                                                     kSweepThreads, sweep_smem(R));
-  if (e != cudaSuccess || n < 1) n = 1;
-  return n;
+  const int per = sweep_blocks(sites, precision);
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &n, sweep_kernel<true, true>(precision, per), kSweepThreads, sweep_smem(R));
+  return e != cudaSuccess || n < 1 ? 1 : std::min(n, per);
 }
 
 cudaError_t batch_switch(const BatchDev& B, const BatchLaunch& L, cudaStream_t st) {
@@ -679,11 +676,11 @@ cudaError_t batch_sweep(const BatchDev& B, const BatchLaunch& L, cudaStream_t st
   V.halt = &B.ctl->flag;
   V.ns_limit = B.ns_limit;
   *L.launches += 2;
-  return B.precision == 1
-             ? launch_coop(k_sweep<1, true, true, 3>, (unsigned)L.sweep_grid, kSweepThreads,
-                           sweep_smem(B.R), st, V)
-             : launch_coop(k_sweep<0, true, true, 2>, (unsigned)L.sweep_grid, kSweepThreads,
-                           sweep_smem(B.R), st, V);
+  void* args[] = {(void*)&V};
+  const unsigned most = (B.Ntot + (uint32_t)kSweepSites - 1) / (uint32_t)kSweepSites;
+  return cudaLaunchCooperativeKernel(
+      sweep_kernel<true, true>(B.precision, sweep_blocks(B.Ntot, B.precision)),
+      dim3(std::min((unsigned)L.sweep_grid, most)), dim3(kSweepThreads), args, sweep_smem(B.R), st);
 }
 
 cudaError_t batch_step_end(const BatchDev& B, const BatchLaunch& L, cudaStream_t st) {

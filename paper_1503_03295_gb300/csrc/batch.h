@@ -135,6 +135,6 @@ int batch_kw_occupancy(int schedule, int R, unsigned pal);
 // blocks per SM of the block-local level kernel and its staged-edge capacity (sets the
 // kernel's shared-memory limit)
 cudaError_t batch_low_setup(int R, uint32_t gcap, int* blocks_per_sm, uint32_t* ecap);
-int batch_sweep_occupancy(int precision, int R);
+int batch_sweep_occupancy(int precision, int R, uint32_t sites);
 
 }  // namespace sco

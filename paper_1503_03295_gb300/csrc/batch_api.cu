@@ -464,7 +464,7 @@ sco_status sco_batch_init(const sco_params* p, int32_t n, void* stream, sco_batc
   b->tune.kw_low = 1;
   b->tune.kw_low_group = 2048;
   b->kw_occ = batch_kw_occupancy(0, n, B.pal_cap);
-  b->sweep_occ = batch_sweep_occupancy(B.precision, n);
+  b->sweep_occ = batch_sweep_occupancy(B.precision, n, B.Ntot);
   b->tune.steps_per_graph = 4;
   b->tune.sweep_blocks_per_sm = b->sweep_occ;
   b->tune.kw_blocks_per_sm = std::min(4, b->kw_occ);

@@ -22,14 +22,6 @@ __global__ void __launch_bounds__(256) k_propose(const DevParams P, uint64_t ste
                  prop32 ? prop32 + i : nullptr);
 }
 
-template <bool kExch>
-const void* sweep_kernel(int precision, int per) {
-  return precision == 1 ? (per > 1 ? (const void*)k_sweep<1, false, kExch, 3>
-                                   : (const void*)k_sweep<1, false, kExch, 1>)
-                        : (per > 1 ? (const void*)k_sweep<0, false, kExch, 2>
-                                   : (const void*)k_sweep<0, false, kExch, 1>);
-}
-
 }  // namespace
 
 cudaError_t sweep_run(const DevParams& P, const Table& t, const SweepBufs& b, uint32_t g,
@@ -37,13 +29,7 @@ cudaError_t sweep_run(const DevParams& P, const Table& t, const SweepBufs& b, ui
                       cudaStream_t st, int64_t* launches) {
   k_propose<<<(unsigned)((P.N + 255) / 256), 256, 0, st>>>(P, step, b.perm, b.prop, b.propd,
                                                              b.prop32);
-  // Two blocks per SM (64 registers; three at 42 in FP32: 1.59 ms per step at L = 2304 against 1.66)
-  // on a large lattice; below kSweepWide sites per SM one block per
-  // SM at 128 registers and without spills (L = 256: 0.130 ms per step against 0.163, L = 1024:
-  // 0.642 against 0.594), a block per kSweepSites sites, so that its barriers have few blocks to wait
-  // for, and up to kSweepOne sites a single one.
-  constexpr int64_t kSweepWide = 2048, kSweepSites = 256, kSweepOne = 2048;
-  const int per = P.N < kSweepWide * num_sms() ? 1 : precision == 1 ? 3 : 2;
+  const int per = sweep_blocks(P.N, precision);
   const int64_t want = P.N <= kSweepOne ? 1 : (P.N + kSweepSites - 1) / kSweepSites;
   const unsigned grid = (unsigned)std::min<int64_t>(per * num_sms(), want);
   SweepView V{};
@@ -70,7 +56,8 @@ cudaError_t sweep_run(const DevParams& P, const Table& t, const SweepBufs& b, ui
   V.ns_limit = ns_limit;
   void* args[] = {(void*)&V};
   *launches += 2;
-  const void* k = P.J != 0.0 ? sweep_kernel<true>(precision, per) : sweep_kernel<false>(precision, per);
+  const void* k = P.J != 0.0 ? sweep_kernel<false, true>(precision, per)
+                              : sweep_kernel<false, false>(precision, per);
   if (grid == 1) return cudaLaunchKernel(k, dim3(1), dim3(kSweepThreads), args, sweep_smem(1), st);
   return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kSweepThreads), args, sweep_smem(1), st);
 }

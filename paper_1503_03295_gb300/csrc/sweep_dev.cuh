@@ -738,6 +738,24 @@ __global__ void __launch_bounds__(kSweepThreads, kBlocks) k_sweep(const __grid_c
   }
 }
 
+// Resident blocks per SM for `sites` sites: two (64 registers; three at 42 in FP32: 1.59 ms per step
+// at L = 2304 against 1.66) on a large lattice or batch; below kSweepWide sites per SM one, at 128
+// registers and without spills (L = 256: 0.130 ms per step against 0.163, L = 1024: 0.642 against
+// 0.594; 10 lattices of L = 128, FP32, with the
+// proposals: 95 us against 111), a block per kSweepSites sites, so that its
+// barriers have few blocks to wait for, and up to kSweepOne sites a single one.
+constexpr int64_t kSweepWide = 2048, kSweepSites = 256, kSweepOne = 2048;
+inline int sweep_blocks(int64_t sites, int precision) {
+  return sites < kSweepWide * num_sms() ? 1 : precision == 1 ? 3 : 2;
+}
+template <bool kBatch, bool kExch>
+const void* sweep_kernel(int precision, int per) {
+  return precision == 1 ? (per > 1 ? (const void*)k_sweep<1, kBatch, kExch, 3>
+                                   : (const void*)k_sweep<1, kBatch, kExch, 1>)
+                        : (per > 1 ? (const void*)k_sweep<0, kBatch, kExch, 2>
+                                   : (const void*)k_sweep<0, kBatch, kExch, 1>);
+}
+
 // A site's proposal for MC step `step` in the forms the sweep reads (see take_proposal).
 __device__ __forceinline__ void write_proposal(const DevParams& P, uint64_t step, uint32_t i,
                                                double4_32a* prop, SpinDf* propd, float4* prop32) {
