@@ -553,7 +553,7 @@ cudaError_t batch_colour(const BatchDev& B, const BatchLaunch& L, cudaStream_t s
     return e;
   FlowShape shape;
   const bool flow = L.flow && L.kw_schedule == 0 && L.levels < kFlowMaxLevels &&
-                    flow_shape(B.R, B.Ntot, &shape, &e);
+                    flow_shape(B.R, B.Ntot, 0, &shape, &e);
   if (L.flow && e != cudaSuccess) return e;
   kb_kw_init<<<B.nblocks, kBatchBlock, 0, st>>>(B, flow ? 1 : 0);
   ++*L.launches;
@@ -574,7 +574,7 @@ cudaError_t batch_colour(const BatchDev& B, const BatchLaunch& L, cudaStream_t s
     F.gmax = &B.ctl->gmax;
     F.levels = L.levels;
     F.cap = shape.cap;
-    F.min_tile = kFlowMinTile;
+    F.min_tile = shape.min_tile;
     F.ns_limit = B.ns_limit;
     F.vec = kFlowVecAll;
     if ((e = flow_launch(F, shape, st)) != cudaSuccess) return e;

@@ -435,7 +435,7 @@ cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* 
   uint32_t* site_start = reinterpret_cast<uint32_t*>(b.meta);
   RepPlan* plan = reinterpret_cast<RepPlan*>(b.meta + 2);
   FlowShape shape;
-  if (g <= kFlowMaxPal && M < kFlowMaxLevels && flow_shape(1, N, &shape, &e)) {
+  if (g <= kFlowMaxPal && M < kFlowMaxLevels && flow_shape(1, N, g, &shape, &e)) {
     FlowView F{};
     F.R = 1;
     F.site_start = site_start;
@@ -450,7 +450,7 @@ cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* 
     F.status = &cnt->status;
     F.levels = M;
     F.cap = shape.cap;
-    F.min_tile = kFlowMinTile;
+    F.min_tile = shape.min_tile;
     F.ns_limit = ns_limit;
     F.vec = kFlowVecAll;
     k_flow_init<<<nb, 256, 0, st>>>((uint32_t)N, RepPlan{g, (uint16_t)M, (uint16_t)near_levels(g, (uint32_t)P.Lx), magic},

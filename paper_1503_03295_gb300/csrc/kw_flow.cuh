@@ -435,14 +435,18 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
 struct FlowShape {
   int threads;
   unsigned grid;
-  uint32_t cap;
+  uint32_t cap, min_tile;
 };
 // A block owns at least kFlowMinTile vertices: fewer blocks on a small lattice, whose vertices then
-// wait for fewer other blocks (L = 256: 0.45 ms per colouring with 1024, 0.46 with 512, 0.63 with
-// 2048, 0.97 with 4096).  Blocks of up to kFlowSmall vertices run 512 threads (L = 256: 0.45 ms
+// wait for fewer other blocks (L = 256, palette 37: 350 us per colouring with 1024, 358 with 768, 375
+// with 512); kFlowThinTile for palettes up to kFlowThin, whose short rows wait for few (exchange
+// lattices, palettes of 12 to 17, with 1024, 512 and 256: L = 52 141, 125 and 118 us, L = 128 193, 171
+// and 167, L = 256 228, 207 and 205), but a single block up to twice that (L = 24 77 us against
+// 84 with two).  A batch, whose palettes are on the device, has 1024.  Blocks of up to kFlowSmall vertices run 512 threads (L = 256: 0.45 ms
 // against 0.53 with 1024), larger ones 1024 (L = 2304: 4.05 ms against 4.77).
-constexpr uint32_t kFlowMinTile = 1024, kFlowSmall = 4096;
-inline bool flow_shape(int R, int64_t sites, FlowShape* sh, cudaError_t* err) {
+constexpr uint32_t kFlowMinTile = 1024, kFlowThinTile = 256, kFlowThin = 24, kFlowSmall = 4096;
+// g: the palette (0: not known)
+inline bool flow_shape(int R, int64_t sites, uint32_t g, FlowShape* sh, cudaError_t* err) {
   static std::atomic<int> smem_of[64];  // per device, once its kernels' limit is raised
   int dev = 0;
   *err = cudaGetDevice(&dev);
@@ -470,8 +474,11 @@ inline bool flow_shape(int R, int64_t sites, FlowShape* sh, cudaError_t* err) {
   }
   const size_t s_smem = (size_t)smem_of[dev].load();
   const int64_t right = (sites + 1) / 2;  // right-half vertices of a level at most
+  sh->min_tile = g == 0 || g > kFlowThin    ? kFlowMinTile
+                 : right <= 2 * kFlowThinTile ? 2 * kFlowThinTile
+                                              : kFlowThinTile;
   sh->grid = (unsigned)std::max<int64_t>(
-      1, std::min<int64_t>(num_sms(), (right + kFlowMinTile - 1) / kFlowMinTile));
+      1, std::min<int64_t>(num_sms(), (right + sh->min_tile - 1) / sh->min_tile));
   const int64_t own = (right + sh->grid - 1) / sh->grid;
   sh->threads = own <= kFlowSmall ? 512 : 1024;
   const size_t fixed = kw_flow_smem(R, 0, sh->threads);

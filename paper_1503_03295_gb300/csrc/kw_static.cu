@@ -254,7 +254,7 @@ extern "C" sco_status sco_kw_colour_static(const uint32_t* row_ptr, const uint32
   unsigned long long ns_limit = 2000000000ull;
   FlowShape shape;
   cudaError_t fe = cudaSuccess;
-  const bool flow = h.g <= kFlowMaxPal && h.levels < kFlowMaxLevels && flow_shape(1, nn, &shape, &fe);
+  const bool flow = h.g <= kFlowMaxPal && h.levels < kFlowMaxLevels && flow_shape(1, nn, h.g, &shape, &fe);
   if (fe != cudaSuccess) return SCO_ECUDA;
   uint32_t* fword = flow ? reinterpret_cast<uint32_t*>(word) : nullptr;
   if (flow) {
@@ -272,7 +272,7 @@ extern "C" sco_status sco_kw_colour_static(const uint32_t* row_ptr, const uint32
     F.status = &ctrl->status;
     F.levels = h.levels;
     F.cap = shape.cap;
-    F.min_tile = kFlowMinTile;
+    F.min_tile = shape.min_tile;
     F.ns_limit = ns_limit;
     F.vec = ((uintptr_t)col & 31u) == 0 ? kFlowVecInside : kFlowVecNone;
     if (flow_launch(F, shape, st) != cudaSuccess) return SCO_ECUDA;

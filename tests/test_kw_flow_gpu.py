@@ -24,6 +24,7 @@ def _compare(g, o):
     (45, 46, 1e12, 0.0),     # no pairs: palette 1, 2070 vertices, 12 levels
     (64, 32, 0.5, 0.0),      # 2048 vertices: one block of 1024 right-half ones
     (64, 33, 0.5, 0.0),      # just above
+    (32, 32, 0.85, 1.0), (33, 32, 0.85, 1.0),  # palettes up to 24: one block of 512, several of 256
     (301, 299, 0.6, 0.0), (700, 301, 0.9, 1.0),
     (1024, 700, 0.3, 0.0),   # larger blocks, mean degree 30: lists read in parts
     (40, 40, 0.1, 0.0), (301, 200, 0.1, 0.0),  # palettes of 65 to 255: colours above 31 looked up again
