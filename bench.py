@@ -179,13 +179,9 @@ class ClockSampler:
 
 
 FP64_NOMINAL_GFLOPS = 1250.0  # GB300 FP64 (vector and tensor), nominal: context only
-# FP64 sweep kernels, per pair of the switched graph and per spin update, from one ncu capture
-# of the current kernels on a smaller lattice at T = 0.6 D (DRAM bytes and executed FP64
-# thread-instructions scale with the updates and pairs, not with L): see the named profile
-SWEEP64_EXECUTED_FP64_PER_PAIR = 28.0  # k_propose + k_sweep + k_resolve, thread-instructions
-SWEEP64_DRAM_BYTES_PER_UPDATE = 2352.0  # dram__bytes_read.sum + dram__bytes_write.sum
-SWEEP64_TRAFFIC_T = 0.6
-SWEEP64_EXECUTED_SOURCE = "profiles/k_sweep_fp64_L1024_T0.6.md"
+# lattices up to about this size are coloured by the kernel that reads every level's rows; larger
+# ones take the first levels block by block
+DATAFLOW_MAX_SITES = 10_000_000
 
 
 def fp64_peak(local):
@@ -213,9 +209,9 @@ def algorithmic_bytes(k, M, p0, cache=False):
     """Bytes per spin update that each phase must move at least once, k the mean degree, M the
     KW levels and p0 the block-local ones: switch + CSR 40 + 16k; colouring + classes: the
     first p0 levels read the rows once and write the colours (4 + 4k + 9), every later level
-    half the rows and colours (4 + 2k), classes 12; sweep 60 + 8k.  With the FP64 form's pair
-    cache (cache=True) the switch also writes a 16-byte record per kept pair and the fill a
-    4-byte id per CSR entry (+12k), and the sweep reads per pair endpoint the id and one
+    half the rows and colours (4 + 2k), classes 12; sweep 60 + 8k.  cache=True: the plan of a form
+    that keeps the switch's value of every pair for the sweep, a 16-byte record per kept pair and
+    a 4-byte id per CSR entry (+12k), of which the sweep reads per pair endpoint the id and one
     16-byte record half and writes 16 bytes for one of the two endpoints (+28k)."""
     colour = (4 + 4 * k + 9 if p0 else 0) + (M - p0) * (4 + 2 * k) + 12
     if cache:
@@ -227,11 +223,10 @@ def algorithmic_flops(k, cand):
     """FP64 operations per spin update of the FP64 form, planning figures: 51 per switching
     candidate (the pair energy 30, one expm1 20, and one multiply for the candidate search on
     the table of decay values, which takes the place of a logarithm) and, per pair endpoint of
-    the sweep, two pair energies (20) and the pseudointeraction term of the proposed spin (50, a
-    log1mexp counted as two transcendentals): the old spin's term is read from the pair cache,
-    which the switch filled, so 70 (120 without the cache); the colouring has none.  The kernels
-    issue fewer (about 23 per candidate, 28.0 per pair endpoint: see
-    SWEEP64_EXECUTED_FP64_PER_PAIR), so these fractions measure work done against the plan."""
+    the sweep, two pair energies (20) and one pseudointeraction term (50, a log1mexp counted as
+    two transcendentals), 70; the colouring has none.  The kernels decide in float-float on the
+    FP32 units and use the FP64 ones only for what that leaves open, so the rate of these
+    operations can pass the FP64 peak."""
     return {"switch": 51.0 * cand, "colour": 0.0, "sweep": 70.0 * k}
 
 
@@ -243,9 +238,8 @@ def phase_ms(ph):
 
 def rooflines(per_step, N, k, M, p0, cand, hbm, how, fp64_gflops=None):
     """HBM roofline of every phase and, for the FP64 form (fp64_gflops: the measured FP64
-    peak; its bytes include the pair cache), the FP64-ALU roofline against the planning
-    operation counts."""
-    ab = algorithmic_bytes(k, M, p0, cache=bool(fp64_gflops))
+    peak), the rate of the planned FP64 operations beside that peak."""
+    ab = algorithmic_bytes(k, M, p0)
     af = algorithmic_flops(k, cand)
     out = {}
     for ph, ms in per_step.items():
@@ -253,7 +247,7 @@ def rooflines(per_step, N, k, M, p0, cand, hbm, how, fp64_gflops=None):
         r = {"hbm_achieved_GBs": gbs, "hbm_frac": gbs / hbm, "algorithmic_bytes_per_update": ab[ph]}
         if fp64_gflops and af[ph] > 0:
             gf = af[ph] * N / (ms / 1e3) / 1e9
-            r.update({"fp64_achieved_GFLOPs": gf, "fp64_frac": gf / fp64_gflops,
+            r.update({"fp64_plan_GFLOPs": gf, "fp64_plan_vs_fp64_peak": gf / fp64_gflops,
                       "algorithmic_fp64_ops_per_update": af[ph]})
         out[ph] = r
     return out
@@ -419,8 +413,7 @@ def run_long(args, rank, world, dev, stream):
 def run_nsw100(args, rank, world, dev, stream):
     """The paper's schedule on the benchmark lattice: switch and colour every n_sw = 100 MC
     steps (Sec. 3.1), FP64.  Eq. (8)'s t_ave = t_switch / 100 + t_color / 100 + t_MC, from the
-    phase times of K steps (K / 100 switches); the graph of each epoch carries the pair cache
-    from one step to the next."""
+    phase times of K steps (K / 100 switches)."""
     import paper_1503_03295_gb300 as sco
 
     K = args.nsw100_steps
@@ -740,40 +733,14 @@ def main():
     hbm, how = peaks()
     fpk = res["fp64_peak"]
     per_step = phase_ms(f64["phases"])
-    p0 = low_levels(g, levels)
+    p0 = low_levels(g, levels) if N > DATAFLOW_MAX_SITES else 0
     roof = rooflines(per_step, N, k, levels, p0, cand, hbm, how, fpk["gflops"])
-    # the dominant kernel: k_sweep of the sweep phase is the longest kernel of the step in the
-    # ncu launch list; the colour phase, about as long in all, is spread over the block-local
-    # kernel and three launches per grid-wide level
-    dom = "sweep" if "sweep" in per_step else max(per_step, key=per_step.get)
-    if roof[dom].get("fp64_achieved_GFLOPs"):
-        primary = {"bound": "alu", "kernel": dom, "achieved": roof[dom]["fp64_achieved_GFLOPs"],
-                   "peak": fpk["gflops"], "unit": "GFLOP/s",
-                   "frac": roof[dom]["fp64_frac"], "traffic": None,
-                   "peak_source": "measured in this run: sco_probe_fp64, independent FP64 FMA "
-                                  "chains filling every SM (2 flops per FMA), SM clock %s MHz" % (
-                                      fpk["clocks"]["sm_mhz"],),
-                   "algorithmic_fp64_ops_per_update": roof[dom]["algorithmic_fp64_ops_per_update"]}
-        if dom == "sweep" and SWEEP64_EXECUTED_FP64_PER_PAIR:
-            # the same phase against the FP64 instructions its kernels execute (ncu count of a
-            # class launch per pair of the switched graph), at the measured FMA issue rate
-            ex = SWEEP64_EXECUTED_FP64_PER_PAIR * k
-            rate = ex * N / (per_step["sweep"] / 1e3)
-            primary["executed"] = {
-                "fp64_lane_inst_per_update": ex, "achieved_inst_per_s": rate,
-                "peak_inst_per_s": fpk["dfma_per_s"], "frac": rate / fpk["dfma_per_s"],
-                "source": SWEEP64_EXECUTED_SOURCE}
-            if abs(args.T - SWEEP64_TRAFFIC_T) < 1e-9 and SWEEP64_DRAM_BYTES_PER_UPDATE:
-                primary["traffic"] = SWEEP64_DRAM_BYTES_PER_UPDATE * N
-                primary["traffic_unit"] = ("DRAM bytes per step of the sweep phase: ncu bytes "
-                                           "per spin update of the same kernels on a smaller "
-                                           "lattice at this T, times N")
-                primary["traffic_source"] = SWEEP64_EXECUTED_SOURCE
-    else:
-        primary = {"bound": "hbm", "kernel": dom, "achieved": roof[dom]["hbm_achieved_GBs"],
-                   "peak": hbm, "unit": "GB/s", "frac": roof[dom]["hbm_frac"], "traffic": None,
-                   "peak_source": how,
-                   "algorithmic_bytes_per_update": roof[dom]["algorithmic_bytes_per_update"]}
+    # the dominant phase: on the benchmark lattice the colouring, one kernel for nearly all of it
+    dom = max(per_step, key=per_step.get)
+    primary = {"bound": "hbm", "kernel": dom, "achieved": roof[dom]["hbm_achieved_GBs"],
+               "peak": hbm, "unit": "GB/s", "frac": roof[dom]["hbm_frac"], "traffic": None,
+               "peak_source": how,
+               "algorithmic_bytes_per_update": roof[dom]["algorithmic_bytes_per_update"]}
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K,
         "warmup": args.warmup, "ms_per_step": f64["ms"] / K, "higher_is_better": True,

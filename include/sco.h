@@ -296,10 +296,9 @@ sco_status sco_batch_set_temperature(sco_batch* b, int32_t r, double T);
  * colouring, neighbour waits); drops the captured graphs.  Synchronises. */
 sco_status sco_batch_set_wait_limit(sco_batch* b, uint64_t ns);
 
-/* Self-test of the library's own elementary function: the branch-free expm1 for x <= 0.35 used
- * by the FP64 decisions of the switch (argument reduction by ln 2, a degree-8
- * polynomial on |r| <= 0.35, -1 below x = -40), stated relative error bound 2^-42, which those
- * decisions carry in their error bounds.  Evaluates it at n >= 17 points of [-50, 0.35] (16
+/* Self-test of the library's own elementary function: the branch-free expm1 for x <= 0.35
+ * (argument reduction by ln 2, a degree-8 polynomial on |r| <= 0.35, -1 below x = -40), stated
+ * relative error bound 2^-42.  Evaluates it at n >= 17 points of [-50, 0.35] (16
  * fixed points, then Philox-jittered evenly spaced ones from `seed`) and returns the largest
  * relative error against the library's double-double expm1 (max_rel_err) and against CUDA's
  * expm1 (max_rel_diff_cuda, may be NULL).  Synchronous; uses the current device.  There is no
@@ -307,8 +306,9 @@ sco_status sco_batch_set_wait_limit(sco_batch* b, uint64_t ns);
 sco_status sco_selftest_expm1(int64_t n, uint64_t seed, double* max_rel_err,
                               double* max_rel_diff_cuda);
 
-/* The same for either degree of the polynomial: degree 8 (the one above, used by the switch)
- * or degree 6 (used by the sweep decisions, stated relative error bound 2^-31).  Any other
+/* The same for either degree of the polynomial: degree 8 (the one above) or degree 6 (used by the
+ * sweep's FP64 decision of the sites that its first one leaves open, stated relative error bound
+ * 2^-31).  Any other
  * degree: SCO_EINVAL. */
 sco_status sco_selftest_expm1_deg(int64_t n, uint64_t seed, int32_t degree, double* max_rel_err,
                                   double* max_rel_diff_cuda);
@@ -337,7 +337,8 @@ sco_status sco_probe_fp64(int64_t iters, double out[3]);
 sco_status sco_sync(sco_ctx* c);
 
 /* Bound (ns) of every device-side wait of this context's kernels (the grid barriers and
- * neighbour waits of the colouring, Sec. 2.3.3); default 2 s, at most 1 h.  A wait that runs
+ * neighbour waits of the colouring, Sec. 2.3.3, and the grid barriers between the colours of a
+ * sweep); default 2 s, at most 1 h.  A wait that runs
  * past it gives up, the kernel returns, and SCO_ETIMEOUT becomes the context's sticky
  * status: sco_sync and every later call return it, and the context does no further work (it
  * must be destroyed).  Limits below 1 ms are checked on every spin of a wait.  Used by tests

@@ -4,12 +4,12 @@
 // no host round trip and can be captured in one CUDA graph.
 //
 // Per step: (A) switch + CSR of every replica (Sec. 2.1), (2) Kuhn-Wattenhofer colouring of
-// every replica's graph (Sec. 2.3.3) and global colour classes (sites of all replicas sorted
-// by (colour, global index)), (3) one persistent cooperative kernel that walks the colours
-// in ascending order; class c of the batch is the union of every replica's class c, and a
-// grid barrier separates colours.  Each site takes exactly the decisions of a single-lattice
-// run (same per-site code, same random streams), so replica r is bit-identical to a
-// single-lattice run with its parameters.
+// every replica's graph (Sec. 2.3.3; every level in one kernel while no palette is above
+// kFlowMaxPal) and global colour classes (sites of all replicas sorted by (colour, global index)),
+// (3) one persistent cooperative kernel that walks the colours in ascending order; class c of the
+// batch is the union of every replica's class c, and a grid barrier separates colours.  Each site
+// takes exactly the decisions of a single-lattice run (same per-site code, same random streams), so
+// replica r is bit-identical to a single-lattice run with its parameters.
 //
 // Buffers that can overflow (CSR entries, overflow half-edges, palette) are checked on the
 // device; a step that would overflow sets a replan flag before touching the spins, every

@@ -12,10 +12,12 @@
 // (colour < g) are exactly the left half and the right-half neighbours with a larger
 // previous colour, all of them final.  The result therefore does not depend on the order
 // in which ready vertices are processed, and the synchronous round of a vertex is one more
-// than the largest round among those larger neighbours.  Each level runs as one persistent
-// cooperative kernel in which every thread recolours its own vertices once their larger
-// neighbours are done: no grid-wide barrier between rounds,
-// same colours as the synchronous rounds, and t_R recovered from the per-vertex rounds.
+// than the largest round among those larger neighbours.  So a vertex recolours as soon as its larger
+// neighbours are done, with the colours of the synchronous rounds, and t_R is recovered from the
+// per-vertex rounds.  Palettes of at most kFlowMaxPal colours whose right halves fit the blocks'
+// shared memory (about 10 million sites) run every level in one kernel (kw_flow.cuh); the others
+// take the first levels group by group (kw_low.cuh), then buckets of equal previous colour
+// (kw_bcr.cuh, from 2^20 sites) or one persistent kernel per level (k_kw_level).
 #include <algorithm>
 #include <cstdint>
 
@@ -453,7 +455,8 @@ cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* 
     F.min_tile = shape.min_tile;
     F.ns_limit = ns_limit;
     F.vec = kFlowVecAll;
-    k_flow_init<<<nb, 256, 0, st>>>((uint32_t)N, RepPlan{g, (uint16_t)M, (uint16_t)near_levels(g, (uint32_t)P.Lx), magic},
+    const uint16_t near = (uint16_t)near_levels(g, (uint32_t)P.Lx);
+    k_flow_init<<<nb, 256, 0, st>>>((uint32_t)N, RepPlan{g, (uint16_t)M, near, magic},
                                     g > 1 ? (uint32_t)(0x100000000ull / g) : 0xFFFFFFFFu, F.word,
                                     site_start, plan, cnt);
     if ((e = flow_launch(F, shape, st)) != cudaSuccess) return e;

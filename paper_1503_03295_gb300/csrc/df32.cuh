@@ -219,7 +219,7 @@ __host__ __device__ __forceinline__ df df_pair_y(const PairDf& t, const FieldDf&
 // g = a1 S_b - a3 (S_b . d) d from FP32 spins and constants, y = bvm - S . g.  |error| <= kY32RelErr
 // a1 against the exact value of the FP64 spins: the spins' rounding (2^-25 per component) contributes
 // 12 2^-25 a1, the constants' and the 13 operations' below 40 2^-24 a1 (every intermediate is at most
-// 6 a1); measured 2^-20.6.
+// 6 a1); measured 2^-20.0.
 constexpr float kY32RelErr = 0x1p-18f;
 __host__ __device__ __forceinline__ void f32_field(float a1, float a3, float fx, float fy, float bx,
                                                    float by, float bz, float& gx, float& gy,
@@ -250,7 +250,7 @@ __host__ __device__ __forceinline__ float f32_exp_core(float y, int& k) {
   return df_fma(df_fmul(r, r), w, r);
 }
 // (e^y - 1) 2^-k for y >= 0, in (0, 1.42); relative error (given y) below kE32RelErr, measured
-// 2^-21.6 (y < 60)
+// 2^-23.2 (y < 60)
 constexpr float kE32RelErr = 0x1p-20f;
 __host__ __device__ __forceinline__ float f32_expm1_scaled(float y, int& k) {
   const float e = f32_exp_core<false>(y, k);

@@ -30,9 +30,6 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 
 // Grid-wide barrier of a cooperative launch (all blocks resident).  bar[0] is an arrival
 // counter: block 0 adds 2^31 - (blocks - 1) and every other block 1, so the top bit flips

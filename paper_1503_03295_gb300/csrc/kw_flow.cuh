@@ -18,6 +18,12 @@
 // one poll of a short list.  No cycle of waits can form: a vertex only waits for larger previous
 // colours, every warp takes its vertices in descending order, and all blocks are resident
 // (cooperative launch).  Palettes of at most 255 colours; one lattice or a batch of them.
+//
+// Per colouring, by rounds and buckets (kw_low.cuh, kw_bcr.cuh, k_kw_level) and here: L = 2304, T =
+// 0.6 D 6.63 -> 3.67 ms, L = 1024, T = 0.4 D 3.47 -> 1.13, 1000 x 1337, T = 0.8 D 2.57 -> 0.94, L =
+// 256 1.74 -> 0.35, a static graph of 400,000 vertices 2.50 -> 0.42.  At L = 1500 it issues on 58% of
+// the cycles with 22 of 32 lanes active, the ALU pipe 53% busy, DRAM 9%; the waits are for rows and
+// words in L2 (4.0 warps per issue) and at the ends of the levels (2.3).
 #pragma once
 
 #include <algorithm>
@@ -310,7 +316,8 @@ __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowV
             // entries of [b, e) among the chunk's
             uint32_t in = e - q0 < kFlowChunk ? (1u << (e - q0)) - 1u : (1u << kFlowChunk) - 1u;
             if (q0 < b) in &= ~((1u << (b - q0)) - 1u);
-            if (q0 + kFlowChunk <= vec_end) {  // whole sectors: a load of 32 rows takes 32 passes through L1 at any width
+            // whole sectors: a load of 32 rows takes 32 passes through L1 at any width
+            if (q0 + kFlowChunk <= vec_end) {
 #pragma unroll
               for (int a = 0; a < kFlowChunk; a += 8) {
                 struct __align__(32) Eight { uint32_t v[8]; } t = {};
@@ -442,8 +449,9 @@ struct FlowShape {
 // with 512); kFlowThinTile for palettes up to kFlowThin, whose short rows wait for few (exchange
 // lattices, palettes of 12 to 17, with 1024, 512 and 256: L = 52 141, 125 and 118 us, L = 128 193, 171
 // and 167, L = 256 228, 207 and 205), but a single block up to twice that (L = 24 77 us against
-// 84 with two).  A batch, whose palettes are on the device, has 1024.  Blocks of up to kFlowSmall vertices run 512 threads (L = 256: 0.45 ms
-// against 0.53 with 1024), larger ones 1024 (L = 2304: 4.05 ms against 4.77).
+// 84 with two).  A batch, whose palettes are on the device, has 1024.  Blocks of up to kFlowSmall
+// vertices run 512 threads (L = 256: 0.45 ms against 0.53 with 1024), larger ones 1024 (1000 x 1337:
+// 0.94 ms against 1.01; L = 2304: 4.05 against 4.77).
 constexpr uint32_t kFlowMinTile = 1024, kFlowThinTile = 256, kFlowThin = 24, kFlowSmall = 4096;
 // g: the palette (0: not known)
 inline bool flow_shape(int R, int64_t sites, uint32_t g, FlowShape* sh, cudaError_t* err) {

@@ -24,7 +24,6 @@ struct DevParams {
   int64_t K;        // half-plane displacement count
   double J, D, beta, bD;  // beta = fl(1/T), bD = fl(beta * D)
   double inv_bD58;        // fl(2^58 / bD): exponential draw -> hazard prefix units
-  float inv_bD58_f;       // its FP32 rounding
   float beta_f;           // fl32(beta), for the FP32 screens (no FP64 operation there)
   float bJ_f;             // fl32(fl(beta J))
   float bJ_h, bJ_l;       // fl(beta J) in float-float
@@ -187,13 +186,10 @@ __device__ __forceinline__ double pair_V(double Dc, double r2, double ax, double
 // clamped at -1000 so that 2^k stays normal).  Relative error below
 // 2^-43: interpolation 2^-43.2; Horner <= gamma_16 p(|r|) / p(r) <= 23 u; r off by at most
 // |k| |ln2 - fl(ln2)| <= 58 x 2.3e-17; for k <= -1 the 2^k expm1(r) part (<= 0.42 2^k) carries
-// these while |expm1(x)| >= 0.29.  Stated as kExpm1RelErr = 2^-42; the FP64 decisions carry it
-// in their error bounds.
-constexpr double kExpm1RelErr = 0x1p-42;
+// these while |expm1(x)| >= 0.29.  Stated as 2^-42 (self-test only).
 // The same with p of degree 6 (expm1_poly6, interpolation error < 2.9e-10): relative error below
-// 2^-31.6 by the same argument; stated as kExpm1RelErr6 = 2^-31.  For the sweep decisions, whose
-// bound adds these errors relatively (the switch's survival margin is absolute and keeps the
-// accurate one: next to the thinning bound of a far pair it must stay small).
+// 2^-31.6 by the same argument; stated as kExpm1RelErr6 = 2^-31.  For the sweep's FP64 decision of
+// the sites that the float-float (or FP32) one leaves open, whose bound adds these errors relatively.
 constexpr double kExpm1RelErr6 = 0x1p-31;
 template <int kDeg>
 __device__ __forceinline__ double expm1_np_deg(double x) {
@@ -260,7 +256,6 @@ struct __align__(64) Sw64 {
   double bvm;       // fl(beta Vmax)
   double c0;        // bound on |error of x| not scaling with |x|, plus 2^-52 (2 beta Vmax)
 };
-
 // x with its sign flipped when neg (bit operation, no FP64 instruction)
 __device__ __forceinline__ double flip_if(double x, bool neg) {
   return __longlong_as_double(__double_as_longlong(x) ^ ((long long)neg << 63));
@@ -274,12 +269,7 @@ __device__ __forceinline__ bool neg_strict(double x) {
 __device__ __forceinline__ unsigned long long pos_bits(double x) {
   return (unsigned long long)__double_as_longlong(x);
 }
-// a signed integer ordered like the value of a (non-NaN) double: ord(a) < ord(b) iff a < b
-// (the two zeros map to 0 and -1; no FP64 instruction)
-__device__ __forceinline__ long long ord_bits(double x) {
-  const long long b = __double_as_longlong(x);
-  return b >= 0 ? b : (long long)(0x8000000000000000ull - (unsigned long long)b) - 1;
-}
+
 // biased exponent field of a double >= 0 (x >= 2^(e - 1023) for normal x; 0 for zero and
 // subnormals, which then read as tiny)
 __device__ __forceinline__ int exp_field(double x) {

@@ -1,6 +1,6 @@
 // selftest.cu -- device self-test of the library's own elementary functions, expm1 (the degree-8
-// expm1_np of the FP64 switch, the degree-6 expm1_np6 of the FP64 sweep decisions) on points of
-// [-50, 0.35] and log_np (the FP64 candidate search of the switch) on points of (0, 1]: relative
+// expm1_np, the degree-6 expm1_np6 of the sweep's FP64 decision) on points of [-50, 0.35] and log_np
+// (the candidate search where the decay table is not certain) on points of (0, 1]: relative
 // error against the double-double versions and difference from CUDA's.
 #include <cstdint>
 #include <cstring>

@@ -10,11 +10,12 @@ namespace sco {
 namespace {
 
 // Persistent: the warps claim the lattice's sites from a global counter (switch_range).
-// Bound by instruction issue (57% busy, 21 of 32 lanes active) and the latency of the neighbours'
+// Bound by instruction issue (58% busy, 24 of 32 lanes active) and the latency of the neighbours'
 // records.  Four blocks per SM (64 registers; three and five measured 0.3 and 0.25 ms slower at
 // L = 2304).  With the guided search, the float-float survival test and two candidates per step the
-// FP64 form's switch phase takes 3.09 ms at L = 2304, T = 0.6 D (5.68 before), the FP32-screened
-// one 2.75 (5.87).
+// FP64 form's switch phase takes 2.92 ms at L = 2304, T = 0.6 D (6.25 before), the FP32-screened
+// one 2.60 (5.87).  Searching both candidates before testing either took 3.13 (spills), with
+// prefetches of their records 3.74.
 template <int PREC>
 __global__ void __launch_bounds__(256, 4) k_switch(const __grid_constant__ DevParams P,
                                                    const __grid_constant__ Search S,
