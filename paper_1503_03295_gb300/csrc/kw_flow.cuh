@@ -20,8 +20,8 @@
 // (cooperative launch).  Palettes of at most 255 colours; one lattice or a batch of them.
 //
 // Per colouring, by rounds and buckets (kw_low.cuh, kw_bcr.cuh, k_kw_level) and here: L = 2304, T =
-// 0.6 D 6.63 -> 3.67 ms, L = 1024, T = 0.4 D 3.47 -> 1.13, 1000 x 1337, T = 0.8 D 2.57 -> 0.94, L =
-// 256 1.74 -> 0.35, a static graph of 400,000 vertices 2.50 -> 0.42.  At L = 1500 it issues on 58% of
+// 0.6 D 6.63 -> 3.60 ms, L = 1024, T = 0.4 D 3.47 -> 1.10, 1000 x 1337, T = 0.8 D 2.57 -> 0.92, L =
+// 256 1.74 -> 0.34, a static graph of 400,000 vertices 2.47 -> 0.44.  At L = 1500 it issues on 58% of
 // the cycles with 22 of 32 lanes active, the ALU pipe 53% busy, DRAM 9%; the waits are for rows and
 // words in L2 (4.0 warps per issue) and at the ends of the levels (2.3).
 #pragma once
