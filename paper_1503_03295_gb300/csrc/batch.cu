@@ -215,9 +215,10 @@ __global__ void __launch_bounds__(256) kb_kw_init(const BatchDev B, int flow) {
 // One KW level for every replica.  The right-half slots of all replicas at level p are
 // numbered consecutively (a block-local scan of the per-replica counts); thread t owns
 // slots t + k * nthreads and recolours their vertices as in the single-lattice kernel.
+// flow: as in KwView (the dataflow kernel's 32-bit words are not this kernel's).
 __global__ void __launch_bounds__(256, 4) kb_kw_level(const BatchDev B, unsigned p,
-                                                    uint32_t low_gmax) {
-  if (block_halted(B)) return;
+                                                    uint32_t low_gmax, const unsigned* flow) {
+  if (block_halted(B) || (flow && *flow <= kFlowMaxPal)) return;
   extern __shared__ uint32_t ksm[];
   const int R = B.R;
   uint32_t* rp = ksm;               // R + 1 slot prefix at level p
@@ -635,7 +636,7 @@ cudaError_t batch_colour(const BatchDev& B, const BatchLaunch& L, cudaStream_t s
   } else {
     for (unsigned p = 1; p <= L.levels; ++p) {
       if ((e = launch_coop(kb_kw_level, (unsigned)L.kw_grid, 256, kw_smem(B.R), st, B, p,
-                           low_gmax)) != cudaSuccess)
+                           low_gmax, skip)) != cudaSuccess)
         return e;
       ++*L.launches;
     }
