@@ -139,7 +139,8 @@ template <int kT, int kOwn>
 __global__ void __launch_bounds__(kT, 1) k_kw_flow(const __grid_constant__ FlowView V) {
   __shared__ int s_halt;
   if (threadIdx.x == 0)
-    s_halt = (V.halt && ld_status(V.halt)) || (V.gmax && *V.gmax > kFlowMaxPal);
+    s_halt = (V.halt && ld_status(V.halt)) || ld_status(V.status) ||
+             (V.gmax && *V.gmax > kFlowMaxPal);
   __syncthreads();
   if (s_halt) return;
   constexpr uint32_t T = kT, kFlowList = flow_list(kT), kFlowLook = flow_look(kT);

@@ -684,7 +684,8 @@ __global__ void __launch_bounds__(kSweepThreads, kBlocks) k_sweep(const __grid_c
   __shared__ int s_halt;
   __shared__ unsigned s_tail;
   if (threadIdx.x == 0) {
-    s_halt = V.halt ? ld_status(V.halt) : 0;
+    // an error before this step (a colouring whose wait ran out): the classes may not be there
+    s_halt = (V.halt && ld_status(V.halt)) || ld_status(V.status);
     s_tail = 0;
   }
   __syncthreads();

@@ -10,8 +10,8 @@ pytestmark = pytest.mark.gpu
 
 
 def test_small_palettes_after_a_palette_above_2048():
-    # 2116 sites at T = 1e-7 D: every pair survives, palette 2116; then T = 0.5 D, palette below 64
-    ps = [sco.make_params(46, T=1e-7, seed=1), sco.make_params(40, T=0.7, seed=2)]
+    # 2116 sites at T = 1e-6 D: nearly every pair survives; then T = 0.5 D, palette below 64
+    ps = [sco.make_params(46, T=1e-6, seed=1), sco.make_params(40, T=0.7, seed=2)]
     lats = [sco.Lattice(p) for p in ps]
     with sco.Batch(ps) as b:
         b.run(1)
