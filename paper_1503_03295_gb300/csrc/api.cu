@@ -712,7 +712,6 @@ sco_status sco_set_temperature(sco_ctx* c, double T) {
   c->p = q;
   c->P = make_dev_params(q);
   // the temperature-dependent tables (pair energies scaled by beta, candidate probabilities)
-  table_free_xy(c->tab);
   SCO_TRY(table_build_xy(c->P, c->tab, c->tab, c->st, &c->launches));
   SCO_TRY(cudaStreamSynchronize(c->st));
   // the graph belongs to the old temperature: the next MC step switches again, same epoch

@@ -751,7 +751,6 @@ sco_status sco_batch_set_temperature(sco_batch* b, int32_t r, double T) {
   drop_graphs(b);
   b->p[r] = q;
   b->P[r] = make_dev_params(q);
-  table_free_xy(b->xy[r]);
   SCO_TRY(table_build_xy(b->P[r], b->xy[r], b->lists[b->list_of[r]], b->st, &b->launches));
   set_tables(b, r);
   const RepDesc& d = b->desc[r];

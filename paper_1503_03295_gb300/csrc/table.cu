@@ -184,8 +184,12 @@ cudaError_t table_build_xy(const DevParams& P, Table& t, const Table& list, cuda
                o_e = place(K * sizeof(uint64_t)), o_head = place(sizeof(SearchHead)),
                o_near = place((kNearGuide + 1) * sizeof(uint16_t)),
                o_far = place((t.far_n + 1) * sizeof(uint32_t));
-  const cudaError_t e = cudaMalloc(&t.pool, bytes);
-  if (e != cudaSuccess) return e;
+  if (t.pool_bytes < bytes) {
+    table_free_xy(t);
+    const cudaError_t e = cudaMalloc(&t.pool, bytes);
+    if (e != cudaSuccess) return e;
+    t.pool_bytes = bytes;
+  }
   char* p = static_cast<char*>(t.pool);
   t.xy = reinterpret_cast<double2*>(p + o_xy);
   t.xy32 = reinterpret_cast<float4*>(p + o_xy32);
@@ -265,6 +269,17 @@ cudaError_t table_build(const DevParams& P, Table& t, cudaStream_t s, int64_t* l
 void table_free_xy(Table& t) {
   cudaFree(t.pool);
   t.pool = nullptr;
+  t.pool_bytes = 0;
+  t.xy = nullptr;
+  t.qdf = nullptr;
+  t.xy32 = nullptr;
+  t.sw64 = nullptr;
+  t.sw32 = nullptr;
+  t.pdf = nullptr;
+  t.Ebits = nullptr;
+  t.head = nullptr;
+  t.near_g = nullptr;
+  t.far_g = nullptr;
 }
 
 void table_free(Table& t) {
