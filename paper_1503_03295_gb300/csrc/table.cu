@@ -133,34 +133,53 @@ __global__ void k_decay(int64_t K, double beta, double D, const uint64_t* __rest
 // Both guides (see Search).  The cells' bounds fall with the cell number as E does with the element,
 // so element m is the first at or below the bounds of the cells in (cell of E_(m-1), cell of E_m]:
 // each element writes its own, and one thread past the list the rest (a binary search per cell took
-// 20 us for a list of 32,000).
+// 20 us for a list of 32,000).  E is rounded: where neighbours differ by less than its error (beta D
+// below about 1e-11) an entry may lie a few units above the one before it, or above the top of its
+// guide.  The cells are therefore clamped to the guide; which of two such entries a cell then names is
+// settled by the search's own margin of 32 units.
+__host__ __device__ inline uint64_t guide_cell(uint64_t top, uint64_t e, int shift, uint64_t n) {
+  if (e >= top) return 0;
+  const uint64_t q = (top - e) >> shift;
+  return q < n ? q : n;
+}
+// the smallest shift that leaves fewer than n cells (n a power of two) from top down to bottom
+__host__ __device__ inline int guide_shift(uint64_t top, uint64_t bottom, uint64_t n) {
+  if (top <= bottom) return 0;
+#ifdef __CUDA_ARCH__
+  const int s = __clzll((long long)n) - __clzll((long long)(top - bottom)) + 1;
+#else
+  const int s = __builtin_clzll(n) - __builtin_clzll(top - bottom) + 1;
+#endif
+  return s > 0 ? s : 0;
+}
+struct GuideRange {
+  int64_t first, last;  // cells that an element writes (none: last < first)
+};
+// element m of the part [m0, m1) of the list, whose last one writes every remaining cell
+__host__ __device__ inline GuideRange guide_range(const uint64_t* E, int64_t m, int64_t m0, int64_t m1,
+                                                  uint64_t top, int shift, uint64_t n) {
+  return {m > m0 ? (int64_t)guide_cell(top, E[m - 1], shift, n) + 1 : 0,
+          m == m1 - 1 ? (int64_t)n : (int64_t)guide_cell(top, E[m], shift, n)};
+}
 __global__ void k_guide(int64_t K, uint32_t far_n, const uint64_t* __restrict__ Eb,
                         SearchHead* __restrict__ head, uint16_t* __restrict__ near_g,
                         uint32_t* __restrict__ far_g) {
   const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (m > K) return;
   const int64_t nnear = K < kNear ? K : kNear;
-  // the smallest shift that leaves fewer than n cells (n a power of two)
-  auto cells = [](uint64_t span, uint32_t n) {
-    const int s = 64 - __clzll((long long)span) - (31 - __clz((int)n));
-    return s > 0 ? s : 0;
-  };
   SearchHead h;
   h.e_near = Eb[nnear - 1];
   h.e_last = Eb[K - 1];
-  h.near_shift = cells(kDecayStart - h.e_near, kNearGuide);
-  h.far_shift = cells(h.e_near - h.e_last, far_n);
+  h.near_shift = guide_shift(kDecayStart, h.e_near, kNearGuide);
+  h.far_shift = guide_shift(h.e_near, h.e_last, far_n);
   if (m == 0) *head = h;
   if (m < nnear) {
-    int64_t q = m > 0 ? (int64_t)((kDecayStart - Eb[m - 1]) >> h.near_shift) + 1 : 0;
-    const int64_t q1 =
-        m == nnear - 1 ? kNearGuide : (int64_t)((kDecayStart - Eb[m]) >> h.near_shift);
-    for (; q <= q1; ++q) near_g[q] = (uint16_t)m;
+    const GuideRange r = guide_range(Eb, m, 0, nnear, kDecayStart, h.near_shift, kNearGuide);
+    for (int64_t q = r.first; q <= r.last; ++q) near_g[q] = (uint16_t)m;
   }
   if (m >= nnear) {
-    int64_t q = m > nnear ? (int64_t)((h.e_near - Eb[m - 1]) >> h.far_shift) + 1 : 0;
-    const int64_t q1 = m == K ? far_n : (int64_t)((h.e_near - Eb[m]) >> h.far_shift);
-    for (; q <= q1; ++q) far_g[q] = (uint32_t)m;
+    const GuideRange r = guide_range(Eb, m, nnear, K + 1, h.e_near, h.far_shift, far_n);
+    for (int64_t q = r.first; q <= r.last; ++q) far_g[q] = (uint32_t)m;
   }
 }
 
