@@ -183,10 +183,24 @@ __host__ __device__ __forceinline__ df df_one_minus_exp_neg(df y) {
   return {mh, ((ch - mh) - eh) + (cl - el)};
 }
 
-// A spin record from FP64 components (u: the acceptance uniform of a proposal, else 0).
-__host__ __device__ __forceinline__ SpinDf spin_df(double x, double y, double z, double u) {
+// The record of a proposal: a spin of length 1 and its acceptance uniform.
+__host__ __device__ __forceinline__ SpinDf proposal_df(double x, double y, double z, double u) {
   const df a = df_split(x), b = df_split(y), c = df_split(z), w = df_split(u);
   return {a.h, b.h, c.h, w.h, a.l, b.l, c.l, w.l};
+}
+// The record of a spin, which may be one that a caller set.  The error bounds below are for |S| <= 1;
+// up to kUnitMax per component (|S|^2 <= 3.01) the errors of the pair terms grow threefold, within the
+// factors that the decisions hold in hand.  Beyond (infinite or not a number among them) the components
+// are NaN, and every decision that reads them is left to FP64 and double-double.
+constexpr double kUnitMax = 1.0 + 0x1p-10;
+__host__ __device__ __forceinline__ bool spin_in_bounds(double x, double y, double z) {
+  return x >= -kUnitMax && x <= kUnitMax && y >= -kUnitMax && y <= kUnitMax && z >= -kUnitMax &&
+         z <= kUnitMax;
+}
+__host__ __device__ __forceinline__ SpinDf spin_df(double x, double y, double z, double u) {
+  if (spin_in_bounds(x, y, z)) return proposal_df(x, y, z, u);
+  const float nan = df_from_bits(0x7FC00000u);
+  return {nan, nan, nan, 0.f, nan, nan, nan, 0.f};
 }
 
 // The beta-scaled field of spin b (at displacement (sx |dx|, sy |dy|), t its pair constants) on the

@@ -28,12 +28,19 @@ __global__ void k_init(DevParams P, double* __restrict__ s, float4* __restrict__
   if (sd) sd[i] = spin_df(x, y, z, 0.0);
 }
 
+// The FP32 copy of a spin; NaN out of bounds, as in the float-float one (see spin_df).
+__device__ __forceinline__ float4 spin_f32(double x, double y, double z) {
+  if (spin_in_bounds(x, y, z)) return make_float4((float)x, (float)y, (float)z, 0.f);
+  const float nan = __int_as_float(0x7FC00000);
+  return make_float4(nan, nan, nan, 0.f);
+}
+
 __global__ void k_copies(int64_t n, const double* __restrict__ s, float4* __restrict__ s32,
                          SpinDf* __restrict__ sd) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double x = s[i], y = s[n + i], z = s[2 * n + i];
-  if (s32) s32[i] = make_float4((float)x, (float)y, (float)z, 0.f);
+  if (s32) s32[i] = spin_f32(x, y, z);
   if (sd) sd[i] = spin_df(x, y, z, 0.0);
 }
 

@@ -123,7 +123,8 @@ __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t
     const PairDf t = load32(pdf + (abs(dx) + (int64_t)P.Lx * abs(dy)));
     const FieldDf g = df_field(t, dx < 0 ? -t.ax : t.ax, dy < 0 ? -t.ay : t.ay, b);
     const df yn = df_pair_y(t, g, N), yo = df_pair_y(t, g, S);
-    if (!(fminf(yn.h, yo.h) > 0x1p-100f && fmaxf(yn.h, yo.h) < 8192.f)) {
+    // (the sum, not the maximum, which passes over a NaN)
+    if (!(fminf(yn.h, yo.h) > 0x1p-100f && yn.h + yo.h < 8192.f)) {
       bad = true;
       continue;
     }
@@ -177,7 +178,7 @@ __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t
     w = df_fast(w.h, w.l);
     const float aj = fabsf(P.bJ_h);
     // |w error| <= 2^-40 beta J 4 (float-float sums of 12 terms below 2 each, scaled)
-    if (!(aj < 512.f)) return 2;
+    if (!(aj < 512.f && fabsf(w.h) < 8192.f)) return 2;  // (out of range, or a NaN spin)
     int k;
     const df e = w.h < 0.f ? df_exp_core<true>(w, k) : df_exp_core<false>(w, k);
     X = df_mul(X, df_add({1.f, 0.f}, e));
@@ -240,7 +241,7 @@ __device__ __forceinline__ int accept_f32(const DevParams& P, int32_t xi, int32_
     f32_field(t.x, t.y, (float)dx, (float)dy, b.x, b.y, b.z, gx, gy, gz);
     const float yn = f32_y(t.z, gx, gy, gz, N.x, N.y, N.z);
     const float yo = f32_y(t.z, gx, gy, gz, S.x, S.y, S.z);
-    if (!(fminf(yn, yo) > 0x1p-100f && fmaxf(yn, yo) < 8192.f)) {
+    if (!(fminf(yn, yo) > 0x1p-100f && yn + yo < 8192.f)) {
       bad = true;
       continue;
     }
@@ -282,7 +283,7 @@ __device__ __forceinline__ int accept_f32(const DevParams& P, int32_t xi, int32_
   if (kExch && P.J != 0.0) {
     const float w = -P.bJ_f * ws;
     const float aj = fabsf(P.bJ_f);
-    if (!(aj < 512.f)) return 2;
+    if (!(aj < 512.f && fabsf(w) < 8192.f)) return 2;
     int k;
     const float e = w < 0.f ? f32_exp_core<true>(w, k) : f32_exp_core<false>(w, k);
     X *= 1.f + e;
@@ -769,7 +770,7 @@ __device__ __forceinline__ void write_proposal(const DevParams& P, uint64_t step
   *prop = ok ? make_double4_32a(c.Sn[0], c.Sn[1], c.Sn[2], c.u)
              : make_double4_32a(0.0, 0.0, 1.0, -1.0);
   if (propd) {
-    SpinDf d = spin_df(c.Sn[0], c.Sn[1], c.Sn[2], c.u);
+    SpinDf d = proposal_df(c.Sn[0], c.Sn[1], c.Sn[2], c.u);
     if (!ok) d.u_h = -1.f;
     *propd = d;
   }
