@@ -221,6 +221,10 @@ __host__ __device__ __forceinline__ FieldDf df_field(const PairDf& t, float fx, 
 // y = bvm - S . g, normalised.  |error| <= kYRelErr a1 against the exact beta (Vmax - V) of the
 // FP64 spins (48-bit inputs, unnormalised sums; measured below 2^-42 a1), for |y| < 8192.
 constexpr float kYRelErr = 0x1p-40f;
+// and for y above kYMin: a1 >= y / 12 then (|S|^2 <= 3.01), so that a3 = 3 a1 / r^2, r < 2^15.6, is above
+// 2^-94 and its low part, 2^-24 of it, well above the smallest FP32 number, 2^-149 (below, far pairs'
+// errors reach past kYRelErr a1).
+constexpr float kYMin = 0x1p-60f;
 __host__ __device__ __forceinline__ df df_pair_y(const PairDf& t, const FieldDf& g,
                                                  const SpinDf& s) {
   df y = df_sub({t.bvmh, t.bvml}, df_mul(g.x, {s.hx, s.lx}));

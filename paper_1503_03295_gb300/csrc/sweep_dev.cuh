@@ -124,7 +124,7 @@ __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t
     const FieldDf g = df_field(t, dx < 0 ? -t.ax : t.ax, dy < 0 ? -t.ay : t.ay, b);
     const df yn = df_pair_y(t, g, N), yo = df_pair_y(t, g, S);
     // (the sum, not the maximum, which passes over a NaN)
-    if (!(fminf(yn.h, yo.h) > 0x1p-100f && yn.h + yo.h < 8192.f)) {
+    if (!(fminf(yn.h, yo.h) > kYMin && yn.h + yo.h < 8192.f)) {
       bad = true;
       continue;
     }
@@ -241,7 +241,7 @@ __device__ __forceinline__ int accept_f32(const DevParams& P, int32_t xi, int32_
     f32_field(t.x, t.y, (float)dx, (float)dy, b.x, b.y, b.z, gx, gy, gz);
     const float yn = f32_y(t.z, gx, gy, gz, N.x, N.y, N.z);
     const float yo = f32_y(t.z, gx, gy, gz, S.x, S.y, S.z);
-    if (!(fminf(yn, yo) > 0x1p-100f && yn + yo < 8192.f)) {
+    if (!(fminf(yn, yo) > kYMin && yn + yo < 8192.f)) {
       bad = true;
       continue;
     }

@@ -229,7 +229,7 @@ __device__ __forceinline__ bool survives_df(const DevParams& P, const PairDf& t,
                                             unsigned& ghits) {
   const FieldDf g = df_field(t, dx < 0 ? -t.ax : t.ax, t.ay, Sj);
   const df y = df_pair_y(t, g, Si);
-  if (y.h > 0x1p-100f && y.h < 8192.f) {
+  if (y.h > kYMin && y.h < 8192.f) {
     const df pr = df_one_minus_exp_neg(y);
     const uint64_t m = wU >> 11;  // u = m 2^-53
     const df u = {(float)(uint32_t)(m >> 29) * 0x1p-24f,

@@ -45,3 +45,50 @@ int main() {
 }
 """)
     assert out == ["0"]
+
+
+def test_weak_pairs(tmp_path):
+    # y = beta (Vmax - V) of pairs so weak that FP32 runs out of exponents: within kYRelErr a1 (FP32: kY32RelErr
+    # a1) wherever it is above kYMin
+    out = run(tmp_path, r"""
+#include <cmath>
+#include <cstdio>
+#include <random>
+#include "df32.cuh"
+using namespace sco;
+typedef long double L;
+int main() {
+  std::mt19937_64 g(11);
+  std::uniform_real_distribution<double> U(0, 1);
+  std::normal_distribution<double> G(0, 1);
+  L ey = 0, fy = 0;
+  long n = 0;
+  for (long i = 0; i < 2000000; ++i) {
+    const int dx = (int)std::exp(U(g) * 10.39), dy = (int)std::exp(U(g) * 10.39);
+    const double r2 = (double)dx * dx + (double)dy * dy, c = 1 / (r2 * r2 * std::sqrt(r2));
+    const double beta = std::exp2(-U(g) * 90), a1 = beta * (c * r2), a3 = beta * (3 * c);
+    const double A = (double)(unsigned long long)(0x1p60 / (r2 * std::sqrt(r2)) * (1 + 0x1p-50)) + 1;
+    const double bvm = beta * (A * 0x1p-59);
+    double S[2][3];
+    for (auto& s : S) {
+      for (double& x : s) x = G(g);
+      const double m = std::sqrt(s[0] * s[0] + s[1] * s[1] + s[2] * s[2]);
+      for (double& x : s) x /= m;
+    }
+    const df d1 = df_split_const(a1), d3 = df_split_const(a3), dv = df_split_const(bvm);
+    const PairDf t = {d1.h, d1.l, d3.h, d3.l, dv.h, dv.l, (float)dx, (float)dy};
+    const SpinDf a = spin_df(S[0][0], S[0][1], S[0][2], 0), b = spin_df(S[1][0], S[1][1], S[1][2], 0);
+    const df y = df_pair_y(t, df_field(t, t.ax, t.ay, b), a);
+    const L ss = (L)S[0][0] * S[1][0] + (L)S[0][1] * S[1][1] + (L)S[0][2] * S[1][2];
+    const L pa = (L)S[0][0] * dx + (L)S[0][1] * dy, pb = (L)S[1][0] * dx + (L)S[1][1] * dy;
+    const L Y = (L)beta * ((L)A * 0x1p-59L - (L)c * ((L)r2 * ss - 3 * pa * pb));
+    float gx, gy, gz;
+    f32_field((float)a1, (float)a3, t.ax, t.ay, (float)S[1][0], (float)S[1][1], (float)S[1][2], gx, gy, gz);
+    const float y32 = f32_y((float)bvm, gx, gy, gz, (float)S[0][0], (float)S[0][1], (float)S[0][2]);
+    if (y.h > kYMin) ey = fmaxl(ey, fabsl((L)y.h + y.l - Y) / (L)a1), ++n;
+    if (y32 > kYMin) fy = fmaxl(fy, fabsl((L)y32 - Y) / (L)a1);
+  }
+  std::printf("%d %d %d\n", ey <= kYRelErr, fy <= kY32RelErr, n > 100000);
+}
+""")
+    assert out == ["1", "1", "1"], out
