@@ -158,6 +158,25 @@ __host__ __device__ __forceinline__ df df_exp_core(df y, int& k) {
   return {eh, (p.h - (eh - r.h)) + (r.l + p.l)};
 }
 
+// y by a multiple of 8192 ln 2 into the range of df_exp_core (a little across 0 at most), the multiple's
+// power of two in k, for |y| < kFoldMax: q below 2^8 and L1, L2 of 10 bits, so both products and the first
+// difference are exact; the rest is off by less than 2^-43 |y|.
+constexpr float kFoldMax = 0x1p20f, kDfFoldInv = 1.f / 5678.26170f;
+__host__ __device__ __forceinline__ df df_fold(df y, int& k) {
+  const int q = (int)(y.h * kDfFoldInv);
+  const float kf = (float)q * 8192.f;
+  k = q * 8192;
+  const df s = df_two_sum(df_fma(-kf, kDfL1, y.h), -df_fmul(kf, kDfL2));
+  return df_fast(s.h, s.l + df_fma(-kf, kDfL3, y.l));
+}
+// the same in plain FP32, off by less than 2^-23 |y|
+__host__ __device__ __forceinline__ float f32_fold(float y, int& k) {
+  const int q = (int)(y * kDfFoldInv);
+  const float kf = (float)q * 8192.f;
+  k = q * 8192;
+  return df_fma(-kf, kDfL2 + kDfL3, df_fma(-kf, kDfL1, y));
+}
+
 // 2^-k for k >= 0 (0 above 126)
 __host__ __device__ __forceinline__ float df_pow2_neg(int k) {
   return k > 126 ? 0.f : df_from_bits((uint32_t)(127 - k) << 23);

@@ -94,10 +94,9 @@ __device__ __forceinline__ int32_t exch_step(const DevParams& P, int32_t xi, int
 // 2.6 with all of them).
 constexpr int kByMantissa = 3;
 __device__ __forceinline__ int decide_far(int K, float bound) {
+  if (bound < 0.25f) return K >= 2 ? 0 : K <= -2 ? 1 : kByMantissa;
   const float m = bound * 1.4427f;  // in factors of two
-  if ((float)(K - 1) > m) return 0;
-  if ((float)(K + 1) < -m) return 1;
-  return bound < 0.25f ? kByMantissa : 2;
+  return (float)(K - 1) > m ? 0 : (float)(K + 1) < -m ? 1 : 2;
 }
 
 template <int kG, bool kExch>
@@ -192,11 +191,14 @@ __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t
     w = df_fast(w.h, w.l);
     const float aj = fabsf(P.bJ_h);
     // |w error| <= 2^-40 beta J 4 (float-float sums of 12 terms below 2 each, scaled)
-    if (!(aj < 512.f && fabsf(w.h) < 8192.f)) return 2;  // (out of range, or a NaN spin)
-    int k;
+    int k, k0 = 0;
+    if (!(fabsf(w.h) < 8192.f)) {
+      if (!(fabsf(w.h) < kFoldMax)) return 2;  // (or a NaN spin)
+      w = df_fold(w, k0);
+    }
     const df e = w.h < 0.f ? df_exp_core<true>(w, k) : df_exp_core<false>(w, k);
     X = df_mul(X, df_add({1.f, 0.f}, e));
-    K += k;
+    K += k + k0;
     bound += 0x1p-31f + 0x1p-38f * aj;
   }
   bound *= 2.f;
@@ -294,13 +296,16 @@ __device__ __forceinline__ int accept_f32(const DevParams& P, int32_t xi, int32_
   }
   float X = N.w * po;
   if (kExch && P.J != 0.0) {
-    const float w = -P.bJ_f * ws;
+    float w = -P.bJ_f * ws;
     const float aj = fabsf(P.bJ_f);
-    if (!(aj < 512.f && fabsf(w) < 8192.f)) return 2;
-    int k;
+    int k, k0 = 0;
+    if (!(fabsf(w) < 8192.f)) {
+      if (!(fabsf(w) < kFoldMax)) return 2;
+      w = f32_fold(w, k0);
+    }
     const float e = w < 0.f ? f32_exp_core<true>(w, k) : f32_exp_core<false>(w, k);
     X *= 1.f + e;
-    K += k;
+    K += k + k0;
     // |w error|: 24 terms below 8 beta J in all, each off by less than 2^-21 relative
     bound += kE32RelErr + 0x1p-17f * aj;
   }

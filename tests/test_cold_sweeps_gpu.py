@@ -11,6 +11,18 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("Lx,Ly,T,J,D", [(40, 33, 0.02, 0.0, 1.0), (64, 20, 0.005, 0.0, 1.0), (33, 30, 0.002, 0.0, 1.0)])
 def test_errors_that_add_up_beside_wide_margins(Lx, Ly, T, J, D):
+    _compare(Lx, Ly, T, J, D)
+
+
+@pytest.mark.parametrize("Lx,Ly,T,J,D", [
+    (40, 33, 0.0015, 1.0, 0.1), (40, 33, 0.0015, -1.0, 0.01),  # beta J = 667
+    (31, 30, 1e-4, 1.0, 0.0), (31, 30, 2e-5, -1.0, 1e-3),      # 1e4, 5e4
+])
+def test_strong_exchange(Lx, Ly, T, J, D):
+    _compare(Lx, Ly, T, J, D)
+
+
+def _compare(Lx, Ly, T, J, D):
     n = 3
     o = O.Chain(O.make_params(Lx, Ly, T=T, J=J, D=D, seed=11))
     o.sweep(n)

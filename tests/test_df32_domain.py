@@ -92,3 +92,34 @@ int main() {
 }
 """)
     assert out == ["1", "1", "1"], out
+
+
+def test_folds(tmp_path):
+    # an exponent of up to 2^20 as k ln 2 + y' with y' in the exponential's range
+    out = run(tmp_path, r"""
+#include <cmath>
+#include <cstdio>
+#include <random>
+#include "df32.cuh"
+using namespace sco;
+typedef long double L;
+int main() {
+  std::mt19937_64 g(3);
+  std::uniform_real_distribution<double> U(0, 1);
+  L e = 0, f = 0;
+  int bad = 0;
+  for (long i = 0; i < 2000000; ++i) {
+    const double y0 = (i & 1 ? -1 : 1) * std::exp2(13 + 7 * U(g)) * 0.999999;
+    const float h = (float)y0, l = (float)(y0 - h);
+    int k, kf;
+    const df y = df_fold({h, l}, k);
+    const float y32 = f32_fold(h, kf);
+    e = fmaxl(e, fabsl((L)y.h + y.l + k * logl(2.0L) - ((L)h + l)) / fabsl((L)h));
+    f = fmaxl(f, fabsl((L)y32 + kf * logl(2.0L) - (L)h) / fabsl((L)h));
+    const float s = i & 1 ? -1.f : 1.f;
+    bad += !(s * y.h > -0.1f && s * y.h < 5679.f && s * y32 > -0.1f && s * y32 < 5679.f) || k % 8192 != 0 || kf != k;
+  }
+  std::printf("%d %d %d\n", e <= 0x1p-43L, f <= 0x1p-23L, bad);
+}
+""")
+    assert out == ["1", "1", "0"], out
