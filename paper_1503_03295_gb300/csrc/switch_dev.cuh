@@ -228,8 +228,11 @@ __device__ __forceinline__ bool survives_df(const DevParams& P, const PairDf& t,
                                             int32_t dy, const NearTable& T, int32_t k, uint64_t wU,
                                             unsigned& ghits) {
   const FieldDf g = df_field(t, dx < 0 ? -t.ax : t.ax, t.ay, Sj);
-  const df y = df_pair_y(t, g, Si);
-  if (y.h > kYMin && y.h < 8192.f) {
+  df y = df_pair_y(t, g, Si);
+  if (y.h > kYMin) {
+    // e^-y is below 2^-144 from 100 on, where a1 2^-38 still bounds the error (y beyond the range of the
+    // exponential went to double-double: every such candidate below about T = D / 2048)
+    if (y.h > 100.f) y = {100.f, 0.f};
     const df pr = df_one_minus_exp_neg(y);
     const uint64_t m = wU >> 11;  // u = m 2^-53
     const df u = {(float)(uint32_t)(m >> 29) * 0x1p-24f,

@@ -1,0 +1,26 @@
+"""The switch at temperatures where beta (Vmax - V) leaves the exponential's range: the survival test
+needs no double-double there, and the graph is the oracle's."""
+import numpy as np
+import pytest
+
+import oracle as O
+import paper_1503_03295_gb300 as sco
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T", [1e-3, 4e-4, 1e-4, 1e-5, 1e-6])
+def test_strong_pairs(T):
+    o = O.Chain(O.make_params(20, 17, T=T, seed=11))
+    o.switch()
+    ro, co = o.graph()
+    for prec in (sco.FP64, sco.FP32_GUARDED):
+        p = sco.make_params(20, 17, T=T, seed=11, precision=prec)
+        g = sco.Lattice(p)
+        g.switch()
+        rg, cg = g.graph()
+        assert np.array_equal(rg.astype(np.int64), ro) and np.array_equal(cg, co)
+        assert g.observables()["guard_hits_fp64"] <= 5
+        with sco.Batch([p, sco.make_params(16, T=0.5, precision=prec)]) as b:
+            b.run(1)
+            assert np.array_equal(b.graph(0)[1], co)
