@@ -160,10 +160,11 @@ __host__ __device__ __forceinline__ df df_exp_core(df y, int& k) {
 
 // y by a multiple of 8192 ln 2 into the range of df_exp_core (a little across 0 at most), the multiple's
 // power of two in k, for |y| < kFoldMax: q below 2^8 and L1, L2 of 10 bits, so both products and the first
-// difference are exact; the rest is off by less than 2^-43 |y|.
+// difference are exact; the rest is off by less than 2^-43 |y|.  keep: what at least remains of a
+// larger y (with 128, df_expm1_scaled's 2^-k stays 0).
 constexpr float kFoldMax = 0x1p20f, kDfFoldInv = 1.f / 5678.26170f;
-__host__ __device__ __forceinline__ df df_fold(df y, int& k) {
-  const int q = (int)(y.h * kDfFoldInv);
+__host__ __device__ __forceinline__ df df_fold(df y, int& k, float keep = 0.f) {
+  const int q = (int)((y.h - keep) * kDfFoldInv);
   const float kf = (float)q * 8192.f;
   k = q * 8192;
   const df s = df_two_sum(df_fma(-kf, kDfL1, y.h), -df_fmul(kf, kDfL2));

@@ -76,7 +76,7 @@ __device__ __forceinline__ bool renorm600(double& p, int& sc) {
 // (df_expm1_scaled given y), and dy / (1 - e^-y) <= 1.42 c0 / m with |dy| <= c0 = kYRelErr a1, where
 // c0 / m < 2^((d >> 23) + 1 - 40) for d the largest difference of the FP32 bit images of a1 and m
 // (a difference of 2^23 is a factor of two, off by at most 2^0.09); it has to stay below 2^-9, or
-// the site is left undecided (y <= 0 in float-float, or y >= 8192, likewise).  The products add
+// the site is left undecided (y below kYMin or above kFoldMax likewise).  The products add
 // 2^-43 per factor, the exchange factor its argument's error and kDfExpRelErr.
 constexpr float kDfExpRelErr = 0x1p-31f;  // measured 2^-31.8 (y < 60), 20 M points
 
@@ -135,13 +135,20 @@ __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t
     const SpinDf b = load32(sd + j);
     const PairDf t = load32(pdf + (abs(dx) + (int64_t)P.Lx * abs(dy)));
     const FieldDf g = df_field(t, dx < 0 ? -t.ax : t.ax, dy < 0 ? -t.ay : t.ay, b);
-    const df yn = df_pair_y(t, g, N), yo = df_pair_y(t, g, S);
+    df yn = df_pair_y(t, g, N), yo = df_pair_y(t, g, S);
     // (the sum, not the maximum, which passes over a NaN)
-    if (!(fminf(yn.h, yo.h) > kYMin && yn.h + yo.h < 8192.f)) {
-      bad = true;
-      continue;
-    }
     int kn, ko;
+    if (!(fminf(yn.h, yo.h) > kYMin && yn.h + yo.h < 8192.f)) {
+      // T from D / 2048 down to 4e-6 D; the exponents of a site add up to less than 105 beta D (the sum of
+      // r^-3 is 9.04, y <= 8 beta D r^-3)
+      if (!(fminf(yn.h, yo.h) > kYMin && yn.h + yo.h < kFoldMax) || P.bD > 0x1p24) {
+        bad = true;
+        continue;
+      }
+      yn = df_fold(yn, kn, 128.f);
+      yo = df_fold(yo, ko, 128.f);
+      K += ko - kn;
+    }
     const df mn = df_expm1_scaled(yn, kn), mo = df_expm1_scaled(yo, ko);
     dmax = max(dmax, __float_as_int(t.a1h) - __float_as_int(fminf(mn.h, mo.h)));
     pn = df_mul(pn, mn);

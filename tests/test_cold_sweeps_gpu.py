@@ -22,7 +22,13 @@ def test_strong_exchange(Lx, Ly, T, J, D):
     _compare(Lx, Ly, T, J, D)
 
 
-def _compare(Lx, Ly, T, J, D):
+@pytest.mark.parametrize("Lx,Ly,T,J,D", [(20, 17, 4e-4, 0.0, 1.0), (20, 17, 2e-5, 0.0, 1.0), (17, 12, 2e-5, 1.0, 0.1)])
+def test_strong_pairs(Lx, Ly, T, J, D):
+    # beta (Vmax - V) up to 2e5: the FP64 form (the FP32-guarded one leaves these sites to FP64)
+    _compare(Lx, Ly, T, J, D, guarded=False)
+
+
+def _compare(Lx, Ly, T, J, D, guarded=True):
     n = 3
     o = O.Chain(O.make_params(Lx, Ly, T=T, J=J, D=D, seed=11))
     o.sweep(n)
@@ -33,6 +39,8 @@ def _compare(Lx, Ly, T, J, D):
         assert np.array_equal(g.accepts(), o.accepts()), prec
         assert np.array_equal(g.spins(), o.spins()), prec
         ob = g.observables()
+        if not guarded and prec == sco.FP32_GUARDED:
+            continue
         assert ob["guard_hits_fp32"] + ob["guard_hits_fp64"] < g.N * n // 5, ob
         with sco.Batch([p, sco.make_params(16, T=0.5, precision=prec)]) as b:
             b.run(n)

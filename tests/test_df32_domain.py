@@ -114,6 +114,14 @@ int main() {
     int k, kf;
     const df y = df_fold({h, l}, k);
     const float y32 = f32_fold(h, kf);
+    if (h > 0) {  // as the pair terms use it
+      int kk, ke;
+      const df r = df_fold({h, l}, kk, 128.f);
+      e = fmaxl(e, fabsl((L)r.h + r.l + kk * logl(2.0L) - ((L)h + l)) / fabsl((L)h));
+      const df m = df_expm1_scaled(r, ke);
+      const L x = expl((L)h + l - (kk + ke) * logl(2.0L));  // (e^y - 1) 2^-k
+      bad += !(fabsl((L)m.h + m.l - x) <= (0x1p-31L + 0x1p-42L * h) * x) || ke < 127;
+    }
     e = fmaxl(e, fabsl((L)y.h + y.l + k * logl(2.0L) - ((L)h + l)) / fabsl((L)h));
     f = fmaxl(f, fabsl((L)y32 + kf * logl(2.0L) - (L)h) / fabsl((L)h));
     const float s = i & 1 ? -1.f : 1.f;
