@@ -59,6 +59,7 @@ DevParams make_dev_params(const sco_params& p) {
   P.beta = 1.0 / p.T;
   P.bD = P.beta * p.D;
   P.inv_bD58 = P.bD > 0.0 ? 0x1p58 / P.bD : 0.0;
+  P.inv_bD58_f = (float)P.inv_bD58;
   P.beta_f = (float)P.beta;
   P.bJ_f = (float)(P.beta * P.J);
   P.bJ_h = P.bJ_f;

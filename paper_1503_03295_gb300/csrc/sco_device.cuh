@@ -24,6 +24,7 @@ struct DevParams {
   int64_t K;        // half-plane displacement count
   double J, D, beta, bD;  // beta = fl(1/T), bD = fl(beta * D)
   double inv_bD58;        // fl(2^58 / bD): exponential draw -> hazard prefix units
+  float inv_bD58_f;       // fl32(inv_bD58)
   float beta_f;           // fl32(beta), for the FP32 screens (no FP64 operation there)
   float bJ_f;             // fl32(fl(beta J))
   float bJ_h, bJ_l;       // fl(beta J) in float-float

@@ -46,9 +46,16 @@ struct NearTable {
   __device__ __forceinline__ uint64_t e(int32_t k) const {
     return k < nnear ? sE[k] : __ldg(&E[k]);
   }
-  // first k in [lo, K) with W[k] >= target, K if none
+  // first k in [lo, K) with W[k] >= target, K if none.  Used where the walk's hazards are large, so that
+  // the next candidate is mostly lo itself or near it: the bracket doubles from there (a binary search
+  // of the whole list read it 15 times and more in global memory)
   __device__ __forceinline__ int32_t lower_bound(int32_t lo, uint64_t target) const {
-    uint32_t a = (uint32_t)lo, b = (uint32_t)K;
+    uint32_t a = (uint32_t)lo, b = a, step = 1;
+    while (b < (uint32_t)K && __ldg(&W[b]) < target) {
+      a = b + 1;
+      b = a + step < (uint32_t)K ? a + step : (uint32_t)K;
+      step *= 2;
+    }
     while (a < b) {
       const uint32_t mid = (a + b) >> 1;
       if (__ldg(&W[mid]) >= target) b = mid; else a = mid + 1;
@@ -160,6 +167,49 @@ __device__ __noinline__ int32_t next_candidate(const DevParams& P, const NearTab
   return next_candidate_dd(P, T, s, Ws, up);
 }
 
+// ceil(x) as above for a float.
+__device__ __forceinline__ uint64_t ceil_u64f(float x) {
+  const uint32_t b = __float_as_uint(x);
+  if (b == 0u || (b >> 31)) return 0ull;
+  const int ex = (int)((b >> 23) & 0xFFu) - 150;  // x = mant * 2^ex
+  const uint64_t mant = (uint64_t)((b & 0x7FFFFFu) | 0x800000u);
+  if (ex >= 0) return ex >= 40 ? ~0ull : mant << ex;
+  if (ex <= -25) return 1ull;  // 0 < x < 1
+  const uint64_t q = mant >> (-ex);
+  return q + ((q << (-ex)) != mant ? 1ull : 0ull);
+}
+
+// FP32 screen of that search (FP32-guarded form): E = -ln u+ as -log1pf(-(1 - u+)) above 1/2 (1 - u+ is
+// an integer times 2^-53) and -logf(u+) below, relative error below 2^-20.5 (one input rounding, 4 ulp
+// of the function); tau = E fl32(2^58 / bD) adds two roundings.  Margins inside 2^-18 fall through to
+// the FP64 search.  Comparisons with W are made in integers.  Without it the FP32 form's switch at T =
+// 0.02 D (L = 64) took 0.696 ms, with it 0.630 (T =
+// 0.001 D: 3.01 and 2.54).
+__device__ __noinline__ int32_t next_candidate_f32(const DevParams& P, const NearTable T, int32_t s,
+                                                   uint64_t wE, unsigned& g32, unsigned& ghits) {
+  const uint64_t Ws = s >= 0 ? T.w(s) : 0ull;
+  const uint64_t m53 = wE >> 11;  // u+ = (m53 + 1) 2^-53
+  const bool high = m53 >= (1ull << 52);
+  const uint64_t m = high ? (1ull << 53) - 1ull - m53 : m53 + 1ull;  // <= 2^52
+  const float v = __uint2float_rn((uint32_t)(m >> 20)) * 0x1p-33f +
+                  __uint2float_rn((uint32_t)(m & 0xFFFFFu)) * 0x1p-53f;
+  const float tau = -(high ? log1pf(-v) : logf(v)) * P.inv_bD58_f;
+  const uint64_t rem = T.w(T.K - 1) - Ws;
+  const uint64_t thr = ceil_u64f(tau);
+  int32_t k = T.K;
+  if (thr <= rem) k = T.lower_bound(s + 1, Ws + thr);
+  // as in next_candidate, with 2^-18
+  const uint64_t m18 = thr >> 18;
+  const uint64_t hi = thr + m18 + 1 < thr ? ~0ull : thr + m18 + 1;
+  const uint64_t lo = thr > m18 + 2 ? thr - m18 - 2 : 0ull;
+  bool certain = tau < 0x1p62f;
+  if (k < T.K && T.w(k) - Ws < hi) certain = false;
+  if (k - 1 > s && T.w(k - 1) - Ws >= lo) certain = false;
+  if (certain) return k;
+  ++g32;
+  return next_candidate(P, T, s, wE, ghits);
+}
+
 // Targets below 2^-990 take the search with a logarithm (the decay table's values there are not
 // normal).
 constexpr uint64_t kDecayMinBits = 0x0210000000000000ull;
@@ -172,9 +222,10 @@ constexpr uint64_t kDecayMinBits = 0x0210000000000000ull;
 // candidate is certain when E_k's bits lie at least 32 below the target's and E_(k-1)'s at least
 // 32 above; otherwise (or for a target below 2^-990) the search with the logarithm decides.
 // Es carries the bits of E at the walk's last candidate and is advanced to the new one.
+template <int PREC>
 __device__ __forceinline__ int32_t next_candidate_e(const DevParams& P, const NearTable& T,
                                                     int32_t s, uint64_t& Es, uint64_t wE,
-                                                    unsigned& ghits) {
+                                                    unsigned& g32, unsigned& ghits) {
   if (s >= T.K - 1 || !P.switching) return T.K;
   const uint64_t tb = (uint64_t)__double_as_longlong(u53pos(wE) * __longlong_as_double(Es));
   if (tb >= kDecayMinBits) {
@@ -189,7 +240,8 @@ __device__ __forceinline__ int32_t next_candidate_e(const DevParams& P, const Ne
       return k;
     }
   }
-  const int32_t k = next_candidate(P, T, s, wE, ghits);
+  const int32_t k = PREC == 1 ? next_candidate_f32(P, T, s, wE, g32, ghits)
+                              : next_candidate(P, T, s, wE, ghits);
   if (k < T.K) Es = T.e(k);
   return k;
 }
@@ -379,7 +431,7 @@ __device__ __forceinline__ bool walk_step(const DevParams& P, const NearTable& T
   bool more = true;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const int32_t k = more ? next_candidate_e(P, T, a.sidx, a.Es, w.w[0], ghits) : T.K;
+    const int32_t k = more ? next_candidate_e<PREC>(P, T, a.sidx, a.Es, w.w[0], g32, ghits) : T.K;
     more = k < T.K;
     const uint64_t wU = w.w[1];
     w.w[0] = w.w[2];
