@@ -119,11 +119,16 @@ __global__ void __launch_bounds__(256) k_pair_obs(DevParams P, const double* __r
     int32_t xi, yi;
     site_xy((uint32_t)i, P, xi, yi);
     const double ax = s[i], ay = s[P.N + i], az = s[2 * P.N + i];
-    for (uint32_t e = row_ptr[i] + sub; e < row_ptr[i + 1]; e += kG) {
+    // each lane goes to its next pair before the term, which so has all lanes: smaller neighbours and
+    // bonds lie among the larger ones (skipped inside the loop, L = 1024 took 4.96 ms against 3.24)
+    const uint32_t e1 = row_ptr[i + 1];
+    auto pair = [&](uint32_t e) {
+      while (e < e1 && ((col[e] & kExchOnly) || (int64_t)col[e] <= i)) e += kG;
+      return e;
+    };
+    for (uint32_t e = pair(row_ptr[i] + sub); e < e1; e = pair(e + kG)) {
       const uint32_t c = col[e];
-      if (c & kExchOnly) continue;
       const int64_t j = c;
-      if (j <= i) continue;
       int32_t xj, yj;
       site_xy(c, P, xj, yj);
       const int32_t dx = xj - xi, dy = yj - yi;

@@ -68,9 +68,14 @@ __global__ void __launch_bounds__(256) k_edge_stats(const DevParams P, const uin
        i += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t yi = site_row((uint32_t)i, P), xi = (uint32_t)i - yi * (uint32_t)P.Lx;
     const uint32_t ci = cell_of(xi, yi, P, cx, cy);
-    for (uint32_t e = row_ptr[i], e1 = row_ptr[i + 1]; e < e1; ++e) {
+    // to the next pair first, as in k_pair_obs
+    const uint32_t e1 = row_ptr[i + 1];
+    auto pair = [&](uint32_t e) {
+      while (e < e1 && ((col[e] & kExchOnly) || (int64_t)col[e] <= i)) ++e;
+      return e;
+    };
+    for (uint32_t e = pair(row_ptr[i]); e < e1; e = pair(e + 1)) {
       const uint32_t cj = col[e];
-      if ((cj & kExchOnly) || (int64_t)cj <= i) continue;
       const uint32_t yj = site_row(cj, P), xj = cj - yj * (uint32_t)P.Lx;
       const int64_t dx = (int64_t)xj - xi, dy = (int64_t)yj - yi;
       atomicAdd(&h[shell_bin(dx * dx + dy * dy, nb)], 1u);
