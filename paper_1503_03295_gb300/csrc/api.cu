@@ -123,6 +123,7 @@ struct sco_ctx {
   uint64_t nnz = 0;
   bool dip_valid = false;  // cnt->max_degree_dip holds the dipolar Delta of the current graph
   FullWork full;  // workspace of the full energy, once asked for
+  SortWork sorted;  // and of the sorted rows
   int sticky = 0;
   unsigned long long ns_limit = 2000000000ull;  // bound of every device-side wait (2 s)
   // phase timing
@@ -322,6 +323,7 @@ void free_all(sco_ctx* c) {
   cudaFree(c->cb.ilist);
   cudaFree(c->acc);
   cudaFree(c->full.p);
+  c->sorted.release();
   cudaFree(c->prop);
   cudaFree(c->cnt);
   if (c->hcnt) cudaFreeHost(c->hcnt);
@@ -527,15 +529,13 @@ sco_status sco_get_graph(sco_ctx* c, uint32_t* row_ptr, uint32_t* col, uint32_t*
     SCO_TRY(cudaMemcpyAsync(row_ptr, c->row_ptr, (c->P.N + 1) * sizeof(uint32_t),
                             cudaMemcpyDeviceToHost, c->st));
   if (col && c->nnz) {
-    // the device rows are unsorted: copy, sort every row by neighbour index, then read back
-    uint32_t* tmp = nullptr;
-    SCO_TRY(cudaMalloc(&tmp, c->nnz * sizeof(uint32_t)));
-    cudaError_t e = csr_sorted_copy(c->P, c->row_ptr, c->col, 0u, tmp, c->nnz, c->cnt, c->st,
+    // the device rows are unsorted: a copy with every row sorted by neighbour index, then read back
+    cudaError_t e = csr_sorted_copy(c->P, c->row_ptr, c->col, 0u, c->nnz, c->sorted, c->cnt, c->st,
                                     &c->launches);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(col, tmp, c->nnz * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->st);
+      e = cudaMemcpyAsync(col, c->sorted.p, c->nnz * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
-    cudaFree(tmp);
+    if (c->sorted.cap > kSortKeep + kSortKeep / 4) c->sorted.release();
     SCO_TRY(e);
     c->dip_valid = true;
   }

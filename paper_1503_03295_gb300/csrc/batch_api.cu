@@ -33,6 +33,7 @@ struct sco_batch {
   BatchLaunch L{};
   size_t scan_tmp_n = 0;  // elements the scan buffer serves
   FullWork full;  // workspace of the full energy, once asked for
+  SortWork sorted;  // and of the sorted rows
   DevCounters* hcnt = nullptr;  // pinned, R
   BatchCtl* hctl = nullptr;     // pinned
   int64_t t = 0;
@@ -109,6 +110,7 @@ void free_all(sco_batch* b) {
   cudaFree(B.bcnt);
   cudaFree(b->L.scan_tmp);
   cudaFree(b->full.p);
+  b->sorted.release();
   for (auto& t : b->xy) table_free_xy(t);
   for (auto& t : b->lists) table_free(t);
   if (b->hcnt) cudaFreeHost(b->hcnt);
@@ -697,16 +699,14 @@ sco_status sco_batch_get_graph(sco_batch* b, int32_t r, uint32_t* row_ptr, uint3
   if (row_ptr)
     for (size_t i = 0; i <= N; ++i) row_ptr[i] = rp[i] - e0;
   if (col && rp[N] > e0) {
-    // the device rows are unsorted: copy, sort every row by neighbour index, then read back
+    // the device rows are unsorted: a copy with every row sorted by neighbour index, then read back
     const size_t nnz = rp[N] - e0;
-    uint32_t* tmp = nullptr;
-    SCO_TRY(cudaMalloc(&tmp, nnz * sizeof(uint32_t)));
-    cudaError_t e = csr_sorted_copy(b->P[r], b->B.row_ptr + base, b->B.col, e0, tmp, nnz,
+    cudaError_t e = csr_sorted_copy(b->P[r], b->B.row_ptr + base, b->B.col, e0, nnz, b->sorted,
                                     b->B.cnt + r, b->st, &b->launches);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(col, tmp, nnz * sizeof(uint32_t), cudaMemcpyDeviceToHost, b->st);
+      e = cudaMemcpyAsync(col, b->sorted.p, nnz * sizeof(uint32_t), cudaMemcpyDeviceToHost, b->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
-    cudaFree(tmp);
+    if (b->sorted.cap > kSortKeep + kSortKeep / 4) b->sorted.release();
     SCO_TRY(e);
   }
   if (colour)

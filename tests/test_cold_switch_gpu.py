@@ -24,3 +24,17 @@ def test_strong_pairs(T):
         with sco.Batch([p, sco.make_params(16, T=0.5, precision=prec)]) as b:
             b.run(1)
             assert np.array_equal(b.graph(0)[1], co)
+
+
+@pytest.mark.parametrize("Lx,Ly,T", [(1, 1, 0.5), (6, 6, 1e-6), (33, 1, 1e-9), (8, 8, 1e-9), (13, 5, 1e-9), (70, 60, 0.05),
+                                     (46, 45, 1e-6)])
+def test_rows_of_any_length_come_sorted(Lx, Ly, T):
+    # rows around 32 and 64 entries, and of 2000; twice, as the copy's workspace is kept
+    lat = sco.Lattice(sco.make_params(Lx, Ly, T=T, J=1.0, seed=2))
+    o = O.Chain(O.make_params(Lx, Ly, T=T, J=1.0, seed=2))
+    lat.switch()
+    o.switch()
+    ro, co = o.graph()
+    for _ in range(2):
+        rg, cg = lat.graph()
+        assert np.array_equal(rg.astype(np.int64), ro) and np.array_equal(cg, co)
