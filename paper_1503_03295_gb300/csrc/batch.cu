@@ -171,8 +171,9 @@ __global__ void __launch_bounds__(256) kb_fill(const BatchDev B) {
   const uint32_t i = (blockIdx.x - B.blk_start[r]) * kBatchBlock + threadIdx.x;
   if (i >= N) return;
   const uint32_t gs = base + i;
-  fill_rows(row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx), i, B.hslot + (size_t)gs * kSlotCap,
-            B.hcnt[gs], B.row_ptr + base, B.lcur + base, B.col);
+  fill_rows(row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx, B.desc[r].P.N), i,
+            B.hslot + (size_t)gs * kSlotCap, B.hcnt[gs], B.indeg + base, B.row_ptr + base,
+            B.lcur + base, B.col);
 }
 
 __global__ void __launch_bounds__(256) kb_fill_ovf(const BatchDev B) {
@@ -181,13 +182,12 @@ __global__ void __launch_bounds__(256) kb_fill_ovf(const BatchDev B) {
   if (n > B.ovf_cap) n = B.ovf_cap;
   for (unsigned long long q = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; q < n;
        q += (unsigned long long)gridDim.x * blockDim.x) {
-    const uint32_t gs = B.ovf[2 * q], jv = B.ovf[2 * q + 1], j = jv & kIndexMask;
+    const uint32_t gs = B.ovf[2 * q];
     const int r = find_le(B.site_start, B.R, gs);
     const uint32_t base = B.site_start[r];
-    const RowFill F = row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx);
-    const bool near = j < near_end(F, gs - base);
-    B.col[row_place(F, near, B.row_ptr, B.lcur, gs)] = jv;
-    B.col[row_place(F, near, B.row_ptr, B.lcur, base + j)] = (gs - base) | (jv & kExchOnly);
+    const RowFill F = row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx, B.desc[r].P.N);
+    fill_overflow(F, gs - base, B.ovf[2 * q + 1], B.row_ptr + base, B.indeg + base, B.hcnt + base,
+                  B.lcur + base, B.col);
   }
 }
 

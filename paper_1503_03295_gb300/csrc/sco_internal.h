@@ -154,16 +154,25 @@ __host__ __device__ inline unsigned near_levels(uint32_t g, uint32_t Lx) {
 // Where the fill puts the neighbours of a lattice: cur counts a row's far (low 16 bits) and near
 // entries, which stay below 2^16 for palettes of the dataflow kernel; larger ones have no near part
 // and count in 32 bits.
+// On larger lattices (kSplitSites), rows of palettes beyond the dataflow kernel hold the smaller
+// neighbours first, then the larger ones in the order of their slots, by distance: the lanes of a warp,
+// at neighbouring sites, then look at the words of neighbouring sites at a time.  The cursors count the
+// smaller neighbours only.  Per colouring in this order and all by atomic order: L = 300, palette 300 517
+// and 552 ms, L = 256 804 and 890, L = 200 461 and 472, L = 128 274 and 271, L = 64 (palette 421) 1717 and
+// 1331 (there the spread makes neighbouring lanes wait for different vertices).
+constexpr int64_t kSplitSites = 1 << 15;
 struct RowFill {
   uint32_t group, mask;  // sites per group (0: no near part), far count in a cursor
+  bool split;            // smaller neighbours, then larger ones
 };
-__host__ __device__ inline RowFill row_fill(uint32_t g, uint32_t Lx) {
+__host__ __device__ inline RowFill row_fill(uint32_t g, uint32_t Lx, int64_t N) {
   const unsigned p = near_levels(g, Lx);
-  return p ? RowFill{g << p, 0xFFFFu} : RowFill{0, 0xFFFFFFFFu};
+  return p ? RowFill{g << p, 0xFFFFu, false}
+           : RowFill{0, 0xFFFFFFFFu, g > kFlowMaxPal && N >= kSplitSites};
 }
 struct SwitchBufs {
   uint32_t* hslot;  // N * kSlotCap upper neighbours (j | flag) per site
-  uint32_t* hcnt;   // N half-degree per site
+  uint32_t* hcnt;   // N half-degree per site (the fill counts the overflow half-edges down)
   uint32_t* indeg;  // N lower-neighbour count per site
   uint32_t* deg;    // N + 1
   uint32_t* lcur;   // N row cursors, then what the rows hold (see RowFill)

@@ -60,22 +60,20 @@ __global__ void k_degree(int64_t N, const uint32_t* __restrict__ hcnt,
 }
 
 __global__ void k_fill(int64_t N, RowFill F, const uint32_t* __restrict__ hslot,
-                       const uint32_t* __restrict__ hcnt, const uint32_t* __restrict__ row_ptr,
-                       uint32_t* __restrict__ cur, uint32_t* __restrict__ col) {
+                       const uint32_t* __restrict__ hcnt, const uint32_t* __restrict__ indeg,
+                       const uint32_t* __restrict__ row_ptr, uint32_t* __restrict__ cur,
+                       uint32_t* __restrict__ col) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < N) fill_rows(F, (uint32_t)i, hslot + i * (int64_t)kSlotCap, hcnt[i], row_ptr, cur, col);
+  if (i < N)
+    fill_rows(F, (uint32_t)i, hslot + i * (int64_t)kSlotCap, hcnt[i], indeg, row_ptr, cur, col);
 }
 
 __global__ void k_fill_ovf(unsigned long long n, RowFill F, const uint32_t* __restrict__ ovf,
-                           const uint32_t* __restrict__ row_ptr, uint32_t* __restrict__ cur,
-                           uint32_t* __restrict__ col) {
+                           const uint32_t* __restrict__ row_ptr,
+                           const uint32_t* __restrict__ indeg, uint32_t* hcnt,
+                           uint32_t* __restrict__ cur, uint32_t* __restrict__ col) {
   const unsigned long long q = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
-  if (q >= n) return;
-  const uint32_t i = ovf[2 * q], jv = ovf[2 * q + 1];
-  const uint32_t j = jv & kIndexMask;
-  const bool near = j < near_end(F, i);
-  col[row_place(F, near, row_ptr, cur, i)] = jv;
-  col[row_place(F, near, row_ptr, cur, j)] = i | (jv & kExchOnly);
+  if (q < n) fill_overflow(F, ovf[2 * q], ovf[2 * q + 1], row_ptr, indeg, hcnt, cur, col);
 }
 
 // Rows sorted by neighbour index (distinct inside a row) into `out`, a warp per row: an entry's place is
@@ -159,8 +157,8 @@ cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, uint32_t g, const 
   cudaError_t e = cudaMemsetAsync(b.lcur, 0, P.N * sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
   const unsigned nb = (unsigned)((P.N + 255) / 256);
-  const RowFill F = row_fill(g, (uint32_t)P.Lx);
-  k_fill<<<nb, 256, 0, st>>>(P.N, F, b.hslot, b.hcnt, row_ptr, b.lcur, col);
+  const RowFill F = row_fill(g, (uint32_t)P.Lx, P.N);
+  k_fill<<<nb, 256, 0, st>>>(P.N, F, b.hslot, b.hcnt, b.indeg, row_ptr, b.lcur, col);
   ++*launches;
   if (has_overflow) {
     unsigned long long n = 0;
@@ -169,7 +167,8 @@ cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, uint32_t g, const 
     if (e != cudaSuccess) return e;
     if (n > b.ovf_cap) n = b.ovf_cap;
     if (n > 0) {
-      k_fill_ovf<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, F, b.ovf, row_ptr, b.lcur, col);
+      k_fill_ovf<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, F, b.ovf, row_ptr, b.indeg, b.hcnt,
+                                                                b.lcur, col);
       ++*launches;
     }
   }

@@ -564,12 +564,26 @@ __device__ __forceinline__ uint32_t row_place(const RowFill& F, bool near,
   const uint32_t at = atomicAdd(&cur[i], near ? 0x10000u : 1u);
   return near ? base - 1 - (at >> 16) : base + (at & F.mask);
 }
+// The places of the overflow half-edge i -> jv in rows i and j.
+__device__ __forceinline__ void fill_overflow(const RowFill& F, uint32_t i, uint32_t jv,
+                                              const uint32_t* __restrict__ row_ptr,
+                                              const uint32_t* __restrict__ indeg, uint32_t* hcnt,
+                                              uint32_t* __restrict__ cur, uint32_t* __restrict__ col) {
+  const uint32_t j = jv & kIndexMask;
+  const bool near = j < near_end(F, i);
+  // (a split row's larger neighbours beyond the slots: places hcnt - 1 down to kSlotCap of that part)
+  const uint32_t at = F.split ? row_ptr[i] + indeg[i] + atomicSub(&hcnt[i], 1u) - 1u
+                              : row_place(F, near, row_ptr, cur, i);
+  col[at] = jv;
+  col[row_place(F, near, row_ptr, cur, j)] = i | (jv & kExchOnly);
+}
 
 // Every surviving half-edge (i, j) of site i's slots goes into rows i and j (see RowFill; indices and
 // arrays of one lattice): eight half-edges at a time, whose slot and row-pointer loads, atomics and
 // stores are each issued together (the atomics' returns were the chain).
 __device__ __forceinline__ void fill_rows(const RowFill& F, uint32_t i,
                                           const uint32_t* __restrict__ slot, uint32_t hcnt,
+                                          const uint32_t* __restrict__ indeg,
                                           const uint32_t* __restrict__ row_ptr,
                                           uint32_t* __restrict__ cur, uint32_t* __restrict__ col) {
   const uint32_t n = min(hcnt, (uint32_t)kSlotCap);
@@ -587,7 +601,8 @@ __device__ __forceinline__ void fill_rows(const RowFill& F, uint32_t i,
       base[a] = on ? row_ptr[near ? j + 1 : j] : 0u;
       nn += near ? 1u : 0u;
     }
-    uint32_t own = atomicAdd(&cur[i], (min(n - q0, kB) - nn) | (nn << 16));
+    uint32_t own = F.split ? indeg[i] + q0
+                           : atomicAdd(&cur[i], (min(n - q0, kB) - nn) | (nn << 16));
 #pragma unroll
     for (uint32_t a = 0; a < kB; ++a) {
       const uint32_t j = jv[a] & kIndexMask;

@@ -38,3 +38,19 @@ def test_rows_of_any_length_come_sorted(Lx, Ly, T):
     for _ in range(2):
         rg, cg = lat.graph()
         assert np.array_equal(rg.astype(np.int64), ro) and np.array_equal(cg, co)
+
+
+@pytest.mark.parametrize("Lx,Ly", [(183, 180), (181, 180)])  # 32,940 and 32,580 sites: both row orders
+def test_rows_of_palettes_above_255(Lx, Ly):
+    p = sco.make_params(Lx, Ly, T=0.0105, seed=3)
+    o = O.Chain(O.make_params(Lx, Ly, T=0.0105, seed=3))
+    o.colour()
+    ro, co = o.graph()
+    lat = sco.Lattice(p)
+    lat.colour()
+    assert lat.sizes()[3] > 255
+    with sco.Batch([p, sco.make_params(16, T=0.5)]) as b:
+        b.run(1)
+        for rg, cg, c in (*[(*lat.graph(), lat.colours())], *[(*b.graph(0), b.colours(0))]):
+            assert np.array_equal(rg.astype(np.int64), ro) and np.array_equal(cg, co)
+            assert np.array_equal(c.astype(np.int32), o.colours())
