@@ -1,10 +1,10 @@
 // kw_static.cu -- Kuhn-Wattenhofer colouring of a caller's CSR graph that allocates nothing.
 //
 // Same colouring as sco_colour (palettes of at most 255 colours by the dataflow kernel of
-// kw_flow.cuh, larger ones by one barrier-free kernel per level), for callers that cannot let a
-// library allocate device memory.  Its working memory is one file-scope device array of fixed
-// size: per-vertex words for up to SCO_KW_STATIC_MAX_VERTICES vertices followed by a small control
-// block.  Every call shares that array; calls that overlap on the GPU race.
+// kw_flow.cuh, larger ones and sparse scattered graphs by one barrier-free kernel per level), for
+// callers that cannot let a library allocate device memory.  Its working memory is one file-scope
+// device array of fixed size: per-vertex words for up to SCO_KW_STATIC_MAX_VERTICES vertices followed
+// by a small control block.  Every call shares that array; calls that overlap on the GPU race.
 #include <cstdint>
 #include <cstring>
 #include <mutex>
@@ -28,7 +28,8 @@ struct StaticCtrl {
   int status;
   unsigned long long magic;  // multiplier of g (div_magic)
   unsigned int kw_rounds;
-  unsigned int pad;
+  unsigned int seen, far;    // sampled entries, and those that join distant vertices
+  unsigned int entries;
   unsigned int lev_rounds[32];
   RepPlan plan;  // the dataflow kernel's view of the one lattice
   unsigned int site_start[2];
@@ -39,10 +40,27 @@ static_assert(sizeof(StaticCtrl) <= kCtrlWords * 8, "control block");
 // The scratch: kMaxVertices packed words, then the control block.  8 MiB + 512 B per device.
 static __device__ __align__(256) unsigned long long g_kw_scratch[kMaxVertices + kCtrlWords];
 
+// The larger graphs' first entries of about 256 rows say whether neighbours lie near one another (see
+// scattered_static).
+constexpr uint32_t kScatterMin = 1u << 14, kSampledRows = 256, kSampledEntries = 4;
+
 __global__ void k_st_degree(uint32_t n, const uint32_t* __restrict__ row_ptr,
-                            StaticCtrl* __restrict__ ctrl) {
+                            const uint32_t* __restrict__ col, StaticCtrl* __restrict__ ctrl) {
   const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned d = v < n ? row_ptr[v + 1] - row_ptr[v] : 0u;
+  if (v == 0) ctrl->entries = row_ptr[n] - row_ptr[0];
+  if (n >= kScatterMin && d > 0 && v % (n / kSampledRows) == 0) {
+    const uint32_t m = min(d, kSampledEntries), b = row_ptr[v];
+    uint32_t u[kSampledEntries];
+#pragma unroll
+    for (uint32_t q = 0; q < kSampledEntries; ++q) u[q] = q < m ? col[b + q] & kIndexMask : v;
+    unsigned far = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < kSampledEntries; ++q)
+      far += (u[q] > v ? u[q] - v : v - u[q]) > n / 64 ? 1u : 0u;
+    atomicAdd(&ctrl->seen, m);
+    if (far) atomicAdd(&ctrl->far, far);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) d = max(d, __shfl_down_sync(0xffffffffu, d, o));
   if ((threadIdx.x & 31) == 0 && d) atomicMax(&ctrl->max_degree, d);
@@ -92,7 +110,20 @@ __device__ __noinline__ unsigned st_mex_slow(uint32_t v, unsigned p, unsigned lo
   }
 }
 
-// One KW level (modified reduction (2)') of a palette too large for the dataflow kernel; g, M and
+// Sparse graphs whose neighbours lie anywhere are coloured level by level as well: hardly a vertex finds
+// its neighbours in its block then, the chains are short, and the dataflow kernel's sort and barrier per
+// level are not repaid.  Neighbours further apart than n / 64 make up most of the sampled entries.  Dataflow
+// kernel and level kernels, in us: a shuffled path, n = 30,000 161 and 156, 100,000 190 and 174, 1,000,000
+// 514 and 349 (in order 477 and 521); a shuffled square grid, n = 100,000 189 and 205, 200,000 241 and 218,
+// 1,000,000 536 and 404 (in order 526 and 759); six random matchings, n = 1,000,000 551 and 466; its
+// 8-neighbour grid, shuffled, 554 and 561; random graphs of mean degree 1 and 2, n = 200,000 221 and 196,
+// 221 and 220; 3 and 4, n = 400,000 280 and 268, 281 and 287; 5 and 6, n = 1,000,000 513 and 497, 529 and 550.
+inline bool scattered_static(const StaticCtrl& c, uint32_t n) {
+  if (n < kScatterMin || c.seen == 0 || 2 * c.far <= c.seen) return false;
+  return c.g <= 3 || (n >= (1u << 17) && (c.g <= 7 || c.entries < (double)n * n / 187000.0));
+}
+
+// One KW level (modified reduction (2)') of a graph that the dataflow kernel does not take; g, M and
 // the divisor constant come from the control block.
 __global__ void __launch_bounds__(256) k_st_level(uint32_t n, unsigned p,
                                                   const uint32_t* __restrict__ row_ptr,
@@ -243,9 +274,9 @@ extern "C" sco_status sco_kw_colour_static(const uint32_t* row_ptr, const uint32
   const uint32_t nn = (uint32_t)n;
   if (cudaMemsetAsync(ctrl, 0, sizeof(StaticCtrl), st) != cudaSuccess) return SCO_ECUDA;
   const unsigned nb = (nn + 255) / 256;
-  k_st_degree<<<nb, 256, 0, st>>>(nn, row_ptr, ctrl);
+  k_st_degree<<<nb, 256, 0, st>>>(nn, row_ptr, col, ctrl);
   k_st_setup<<<1, 1, 0, st>>>(nn, ctrl);
-  // Delta decides the kernel: small palettes run the dataflow kernel
+  // Delta and the sample decide the kernel: small palettes mostly run the dataflow kernel
   StaticCtrl h;
   std::memset(&h, 0, sizeof(h));
   if (cudaMemcpyAsync(&h, ctrl, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess)
@@ -254,7 +285,8 @@ extern "C" sco_status sco_kw_colour_static(const uint32_t* row_ptr, const uint32
   unsigned long long ns_limit = 2000000000ull;
   FlowShape shape;
   cudaError_t fe = cudaSuccess;
-  const bool flow = h.g <= kFlowMaxPal && h.levels < kFlowMaxLevels && flow_shape(1, nn, h.g, &shape, &fe);
+  const bool flow = h.g <= kFlowMaxPal && h.levels < kFlowMaxLevels && !scattered_static(h, nn) &&
+                    flow_shape(1, nn, h.g, &shape, &fe);
   if (fe != cudaSuccess) return SCO_ECUDA;
   uint32_t* fword = flow ? reinterpret_cast<uint32_t*>(word) : nullptr;
   if (flow) {
