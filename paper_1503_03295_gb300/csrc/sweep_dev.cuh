@@ -78,7 +78,7 @@ __device__ __forceinline__ bool renorm600(double& p, int& sc) {
 // (a difference of 2^23 is a factor of two, off by at most 2^0.09); it has to stay below 2^-9, or
 // the site is left undecided (y below kYMin or above kFoldMax likewise).  The products add
 // 2^-43 per factor, the exchange factor its argument's error and kDfExpRelErr.
-constexpr float kDfExpRelErr = 0x1p-31f;  // measured 2^-31.8 (y < 60), 20 M points
+constexpr float kDfExpRelErr = 0x1p-31f;  // largest seen 2^-31.6 (y < 8192)
 
 // Index step from site (xi, yi) to its exchange neighbour q (0 to 3: left, right, down, up); 0: none.
 __device__ __forceinline__ int32_t exch_step(const DevParams& P, int32_t xi, int32_t yi, int q) {
