@@ -634,9 +634,10 @@ cudaError_t bucket_run(const DevParams& P, uint32_t g, const uint32_t* row_ptr, 
     if (e != cudaSuccess) return e;
     if (ntiles <= (uint32_t)(2 * num_sms())) {
       // (beside 8 KB of static shared memory)
+      // (the same value from every thread and lattice: a smaller one would fail another's launch)
       if (sh > 40 * 1024 &&
           (e = cudaFuncSetAttribute(k_tile_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sh)) != cudaSuccess)
+                                    (int)(kMaxStablePalette * sizeof(uint32_t)))) != cudaSuccess)
         return e;
       k_tile_sort<<<ntiles, 512, sh, st>>>((uint32_t)N, g, dk, ntiles, b.colour, row_ptr,
                                            b.tile_cnt, b.perm, b.off, cnt);
