@@ -140,8 +140,9 @@ __global__ void __launch_bounds__(1024) kb_plan(const BatchDev B) {
     const unsigned long long G = ((unsigned long long)N + g - 1) / g;
     unsigned M = 0;
     while ((1ull << M) < G) ++M;
-    B.plan[r] = RepPlan{g, (uint16_t)M, (uint16_t)near_levels(g, (uint32_t)B.desc[r].P.Lx),
-                        div_magic(g)};
+    B.plan[r] =
+        RepPlan{g, (uint16_t)M,
+                (uint16_t)near_levels(g, (uint32_t)B.desc[r].P.Lx, kFlowMaxPal), div_magic(g)};
     B.cnt[r].g = g;
     B.cnt[r].levels = M;
     B.cnt[r].nnz = (unsigned long long)(B.row_ptr[base + N] - B.row_ptr[base]);
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(256) kb_fill(const BatchDev B) {
   const uint32_t i = (blockIdx.x - B.blk_start[r]) * kBatchBlock + threadIdx.x;
   if (i >= N) return;
   const uint32_t gs = base + i;
-  fill_rows(row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx, B.desc[r].P.N), i,
+  fill_rows(row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx, B.desc[r].P.N, kFlowMaxPal), i,
             B.hslot + (size_t)gs * kSlotCap, B.hcnt[gs], B.indeg + base, B.row_ptr + base,
             B.lcur + base, B.col);
 }
@@ -185,7 +186,8 @@ __global__ void __launch_bounds__(256) kb_fill_ovf(const BatchDev B) {
     const uint32_t gs = B.ovf[2 * q];
     const int r = find_le(B.site_start, B.R, gs);
     const uint32_t base = B.site_start[r];
-    const RowFill F = row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx, B.desc[r].P.N);
+    const RowFill F =
+        row_fill(B.plan[r].g, (uint32_t)B.desc[r].P.Lx, B.desc[r].P.N, kFlowMaxPal);
     fill_overflow(F, gs - base, B.ovf[2 * q + 1], B.row_ptr + base, B.indeg + base, B.hcnt + base,
                   B.lcur + base, B.col);
   }

@@ -14,7 +14,7 @@
 // in which ready vertices are processed, and the synchronous round of a vertex is one more
 // than the largest round among those larger neighbours.  So a vertex recolours as soon as its larger
 // neighbours are done, with the colours of the synchronous rounds, and t_R is recovered from the
-// per-vertex rounds.  Palettes of at most kFlowMaxPal colours whose right halves fit the blocks'
+// per-vertex rounds.  Palettes of at most flow_max_pal colours whose right halves fit the blocks'
 // shared memory (about 10 million sites) run every level in one kernel (kw_flow.cuh); the others
 // take the first levels group by group (kw_low.cuh), then buckets of equal previous colour
 // (kw_bcr.cuh, from 2^20 sites) or one persistent kernel per level (k_kw_level).
@@ -437,7 +437,7 @@ cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* 
   uint32_t* site_start = reinterpret_cast<uint32_t*>(b.meta);
   RepPlan* plan = reinterpret_cast<RepPlan*>(b.meta + 2);
   FlowShape shape;
-  if (g <= kFlowMaxPal && M < kFlowMaxLevels && flow_shape(1, N, g, &shape, &e)) {
+  if (g <= flow_max_pal(N) && M < kFlowMaxLevels && flow_shape(1, N, g, &shape, &e)) {
     FlowView F{};
     F.R = 1;
     F.site_start = site_start;
@@ -455,7 +455,7 @@ cudaError_t kw_run(const DevParams& P, const uint32_t* row_ptr, const uint32_t* 
     F.min_tile = shape.min_tile;
     F.ns_limit = ns_limit;
     F.vec = kFlowVecAll;
-    const uint16_t near = (uint16_t)near_levels(g, (uint32_t)P.Lx);
+    const uint16_t near = (uint16_t)near_levels(g, (uint32_t)P.Lx, flow_max_pal(N));
     k_flow_init<<<nb, 256, 0, st>>>((uint32_t)N, RepPlan{g, (uint16_t)M, near, magic},
                                     g > 1 ? (uint32_t)(0x100000000ull / g) : 0xFFFFFFFFu, F.word,
                                     site_start, plan, cnt);

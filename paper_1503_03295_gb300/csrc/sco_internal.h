@@ -131,11 +131,20 @@ cudaError_t full_energy_fft(const DevParams& P, const double* s, void* work, dou
 // ---- switch.cu ----
 constexpr int kSlotCap = 32;
 
-// Palettes up to this size are coloured by the dataflow kernel (kw_flow.cuh): a colour has a byte of
-// a word in shared memory.  Against the kernels by rounds and buckets, per colouring: L = 1024,
-// palette 77 29.2 -> 2.8 ms; L = 512, 118 27.5 -> 9.7; L = 1024, 136 89.5 -> 13.2; L = 256, 170
-// 35.9 -> 23.4 (chains of 1500 rounds).
+// Palettes up to this size can be coloured by the dataflow kernel (kw_flow.cuh): a colour has a byte of
+// a word in shared memory.  A batch takes it up to there, a lattice up to flow_max_pal.
 constexpr uint32_t kFlowMaxPal = 255;
+// With rows of hundreds of entries, read in parts of a list, and chains of hundreds of hops the dataflow
+// kernel loses to one kernel per level.  Per colouring, ms, dataflow kernel and kernel per level:
+//   L = 64, palette 236: 30.2, 30.1; 202: 19.1, 22.0;  L = 80, 222: 29.7, 29.0;  L = 100, 215: 38.4, 33.7;
+//   203: 26.6, 28.0;  L = 128, 223: 50.6, 40.9; 207: 37.4, 37.6;  L = 160, 240: 68.3, 46.8; 210: 41.0, 36.4;
+//   195: 35.0, 37.6;  L = 200, 243: 94.1, 63.6; 209: 56.4, 49.1; 199: 33.1, 41.5;  L = 256, 248: 87.4, 74.9;
+//   224: 60.7, 63.5;  L = 400, 247: 106, 91; 225: 78.9, 78.7;  L = 512, 243: 126, 109; 234: 98.5, 97.8;  L =
+//   700, 246: 135, 126; 233: 114, 122;  L = 1000, 248: 155, 168;  L = 1100 (buckets from 2^20 sites), 248:
+//   178, 327.
+__host__ __device__ inline uint32_t flow_max_pal(int64_t N) {
+  return N < 4608 || N > 800000 ? kFlowMaxPal : N < 50000 ? 208 : 224;
+}
 
 // The colouring's level p only looks at neighbours in the same group of g 2^p consecutive sites, for
 // the low levels about a sixth of a row, but every row is read at every level.  So the fill
@@ -145,9 +154,10 @@ constexpr uint32_t kFlowMaxPal = 255;
 // 0.870, 9 0.902 (L = 256, T = 0.6 D); 1.4 0.826, 2.9 0.834, 5.8 0.866 (L = 512, T = 0.4 D).
 // Per colouring, without and with: L = 2304 3.96 -> 3.77 ms, L = 1024 T = 0.4 D 1.21 -> 1.15; groups of
 // up to one row 3.81 and 1.16, four rows 3.78 and 1.15.
-__host__ __device__ inline unsigned near_levels(uint32_t g, uint32_t Lx) {
+// max_pal: the largest palette that the dataflow kernel will take.
+__host__ __device__ inline unsigned near_levels(uint32_t g, uint32_t Lx, uint32_t max_pal) {
   unsigned p = 0;
-  if (g <= kFlowMaxPal)
+  if (g <= max_pal)
     while ((g << (p + 1)) <= 2 * Lx) ++p;
   return p;
 }
@@ -165,10 +175,10 @@ struct RowFill {
   uint32_t group, mask;  // sites per group (0: no near part), far count in a cursor
   bool split;            // smaller neighbours, then larger ones
 };
-__host__ __device__ inline RowFill row_fill(uint32_t g, uint32_t Lx, int64_t N) {
-  const unsigned p = near_levels(g, Lx);
+__host__ __device__ inline RowFill row_fill(uint32_t g, uint32_t Lx, int64_t N, uint32_t max_pal) {
+  const unsigned p = near_levels(g, Lx, max_pal);
   return p ? RowFill{g << p, 0xFFFFu, false}
-           : RowFill{0, 0xFFFFFFFFu, g > kFlowMaxPal && N >= kSplitSites};
+           : RowFill{0, 0xFFFFFFFFu, g > max_pal && N >= kSplitSites};
 }
 struct SwitchBufs {
   uint32_t* hslot;  // N * kSlotCap upper neighbours (j | flag) per site

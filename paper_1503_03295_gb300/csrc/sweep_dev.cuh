@@ -225,8 +225,8 @@ __device__ __forceinline__ int accept_df(const DevParams& P, int32_t xi, int32_t
 
 // The FP32-guarded form's screen: the same decision in plain FP32, from the FP32 spins and constants
 // (about 60 instructions per pair).  Bound as in accept_df, with kE32RelErr, c0 = kY32RelErr a1
-// (c0 / m < 2^((d >> 23) + 1 - 18), below 2^-6) and 2^-23 per product; it leaves about one site in
-// 10^4 to FP64.  N = {S', u}.
+// (c0 / m < 2^((d >> 23) + 1 - 18), below 2^-6) and 2^-23 per product; it leaves 1.5 to 2.5 sites in
+// 10^4 to FP64 (T = 0.8 to 0.3 D).  N = {S', u}.
 template <int kG, bool kExch>
 __device__ __forceinline__ int accept_f32(const DevParams& P, int32_t xi, int32_t yi, float4 S,
                                           float4 N, const float4* __restrict__ sw,

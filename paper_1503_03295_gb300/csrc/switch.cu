@@ -157,7 +157,7 @@ cudaError_t csr_fill(const DevParams& P, const SwitchBufs& b, uint32_t g, const 
   cudaError_t e = cudaMemsetAsync(b.lcur, 0, P.N * sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
   const unsigned nb = (unsigned)((P.N + 255) / 256);
-  const RowFill F = row_fill(g, (uint32_t)P.Lx, P.N);
+  const RowFill F = row_fill(g, (uint32_t)P.Lx, P.N, flow_max_pal(P.N));
   k_fill<<<nb, 256, 0, st>>>(P.N, F, b.hslot, b.hcnt, b.indeg, row_ptr, b.lcur, col);
   ++*launches;
   if (has_overflow) {
