@@ -67,7 +67,7 @@ typedef struct {
 typedef struct {
   double e_switched; /* H' of Eq. (4) (pseudointeractions of surviving pairs) + exchange */
   double e_exchange; /* -J sum_<ij> S_i.S_j */
-  double e_full;     /* full H of Eq. (6) by direct summation; NaN unless requested */
+  double e_full;     /* full H of Eq. (6); NaN unless requested */
   double mx, my, mz; /* magnetisation per spin */
   double m_abs;      /* |m| */
   double m_phi;      /* signed [(1/N) sum S_i x (r_i - r_c)/|r_i - r_c|]_z of Eq. (7) */
@@ -105,10 +105,13 @@ sco_status sco_colour(sco_ctx* c, int32_t* n_colours);
 sco_status sco_sweep(sco_ctx* c, int32_t n_mcs);
 
 /* Observables of the current state (Eqs. (4), (6), (7), Table 1).  want_full computes the
- * full H by O(N^2) direct summation (N <= 65536, else e_full = NaN).  Synchronises. */
+ * full H (N <= 65536, else e_full = NaN): by FP64 Fourier transforms where no side is above 1024
+ * and their workspace (at most 34 MB, kept with the context) can be had, else by O(N^2) direct
+ * summation.  Synchronises. */
 sco_status sco_observables(sco_ctx* c, sco_obs* out, int32_t want_full);
 
-/* Spin copies (SoA, 3*N doubles).  on_device != 0: xyz is a device pointer.  Synchronous. */
+/* Spin copies (SoA, 3*N doubles).  on_device != 0: xyz is a device pointer.  Synchronous.  Spins
+ * set with a component beyond 1 + 2^-10 are decided in FP64 and double-double throughout. */
 sco_status sco_get_spins(sco_ctx* c, double* xyz, int32_t on_device);
 sco_status sco_set_spins(sco_ctx* c, const double* xyz, int32_t on_device);
 

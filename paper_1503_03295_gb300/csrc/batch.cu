@@ -555,9 +555,9 @@ cudaError_t batch_colour(const BatchDev& B, const BatchLaunch& L, cudaStream_t s
   if ((e = cudaMemsetAsync(B.used, 0, (size_t)B.R * nw * sizeof(uint32_t), st)) != cudaSuccess)
     return e;
   FlowShape shape;
-  const bool flow = L.flow && L.kw_schedule == 0 && L.levels < kFlowMaxLevels &&
+  const bool flow = L.kw_schedule == 0 && L.levels < kFlowMaxLevels &&
                     flow_shape(B.R, B.Ntot, 0, &shape, &e);
-  if (L.flow && e != cudaSuccess) return e;
+  if (e != cudaSuccess) return e;
   kb_kw_init<<<B.nblocks, kBatchBlock, 0, st>>>(B, flow ? 1 : 0);
   ++*L.launches;
   if (flow) {

@@ -114,14 +114,14 @@ DevParams make_dev_params(const sco_params& p);
 
 // Launchers (batch.cu).  Each enqueues one phase for every replica on `st`.
 struct BatchLaunch {
-  int kw_schedule;  // 0: all levels in one kernel, buckets by colour; 1: one async kernel per level
+  int kw_schedule;  // 0: all levels in one kernel, by dataflow up to kFlowMaxPal colours, else buckets by
+                    // colour; 1: one async kernel per level
   int kw_low;       // 0: no block-local levels; 1: staged edges; 2: rows at every level
   uint32_t low_gmax;  // group-size cap of the block-local levels
   int low_grid;     // blocks of the block-local level kernel
   uint32_t low_ecap;  // its staged-edge capacity per group
   int kw_grid;     // blocks of the persistent KW kernel(s)
   int sweep_grid;  // blocks of the persistent sweep kernel
-  int flow;        // schedule 0: palettes up to kFlowMaxPal by the dataflow kernel
   unsigned levels;  // KW level launches per colouring (>= every replica's M)
   uint64_t* scan_tmp;
   int64_t* launches;

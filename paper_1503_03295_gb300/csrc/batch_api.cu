@@ -144,7 +144,6 @@ cudaError_t alloc_palette(sco_batch* b, uint32_t pal) {
 void set_grids(sco_batch* b) {
   const int sms = num_sms();
   b->L.kw_schedule = b->tune.kw_schedule;
-  b->L.flow = 1;
   b->L.kw_low = b->tune.kw_low;
   b->L.low_gmax = (uint32_t)b->tune.kw_low_group;
   if (batch_low_setup(b->R, b->L.low_gmax, &b->low_occ, &b->low_ecap) != cudaSuccess) {

@@ -8,9 +8,9 @@
 //   beta dE' = sum_{surviving j} [beta V(S', S_j) - L(S') - beta V(S, S_j) + L(S)]
 //              - beta J (S' - S) . sum_{nn j} S_j,
 //   L = log(1 - exp(beta (V - Vmax)))   (so that beta Vbar = beta V - L, Eq. (3)).
-// The decision is taken in FP64 (or FP32 in the FP32-guarded form) with a bound on the
-// rounding error of the margin; a site whose margin is inside the bound is settled by one
-// warp, in FP64 (after FP32) and then in double-double.
+// The decision is taken in float-float (in FP32 in the FP32-guarded form) with a bound on the
+// rounding error of the margin; a site whose margin is inside the bound, or whose terms are out of
+// range, is settled by one warp, in FP64 and then in double-double.
 #pragma once
 
 #include <cstdint>
